@@ -23,7 +23,7 @@ struct PoolDev {
   int type, capacity, group, window_us;
   int node0, n_nodes;   // GPU pools: first node in a gpu_busy row, node count
   int slot0, n_slots;   // demand slots in the prefix scan (GPU: 4 nested levels, else 1)
-  int lane_place;       // batched path: the pool is placed by k_place, one thread per scenario
+  int queue_place;      // batched path: grants are placed in queue order with the state in registers (CpuFresh, quota sums)
 };
 
 // per (scenario, pool) facts produced by the prefix kernel
@@ -60,8 +60,6 @@ struct Params {
   int* order;        // [S][N] action index at each partitioned position
   i64* tmin;         // [S][N] duration at the least level, partitioned order
   PoolMeta* meta;    // [S][P]
-  unsigned short* preq;  // what k_place reads per kept candidate: unit byte | multiplicity << 8 (partitioned order)
-  int* keepn;        // [S][P] candidates kept, -1 = placed elsewhere
   char* slabs; u64 slab_bytes; int n_workers;
   char* arena; u64 arena_bytes; u64* arena_top;
   int slot_tries;    // rounds of looking for a free arena slot (2 us apart) before a warp gives up
@@ -135,6 +133,8 @@ __device__ __forceinline__ i64 warp_sum64(i64 v) {      // 0 <= v, sum below 2^6
   const u32 c = __reduce_add_sync(TG_FULL, (u32)((u64)v >> 44));
   return (i64)((u64)a + ((u64)b << 22) + ((u64)c << 44));
 }
+// a value that is the same in every lane, so that the compiler knows it (uniform branches, no reconvergence code)
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(TG_FULL, v, 0); }
 __device__ __forceinline__ int warp_sum32(int v) { return (int)__reduce_add_sync(TG_FULL, (u32)v); }
 __device__ __forceinline__ int warp_min32(int v) { return __reduce_min_sync(TG_FULL, v); }
 __device__ __forceinline__ int warp_max32(int v) { return __reduce_max_sync(TG_FULL, v); }
@@ -157,6 +157,7 @@ __device__ __forceinline__ void gpu_caps(const PoolDev& pd, const u8* busy, int 
 // table and gives back (48 slots of at least 64 MiB when the arena allows, else down to 4
 // larger-as-possible ones); the rest is handed out by a bump pointer, never reused in a call.
 #define TG_ARENA_MAX_SLOTS 48
+#define TG_MIN_SLOT_BYTES (512u << 10)   // smaller slots are of no use to the tables of large boxes
 __device__ __forceinline__ int arena_n_slots(const Params& P) {
   u64 n = (P.arena_bytes / 8 * 7) >> 26;
   return n < 4 ? 4 : (n > TG_ARENA_MAX_SLOTS ? TG_ARENA_MAX_SLOTS : (int)n);

@@ -10,8 +10,8 @@
 // occupancy rows are still written).
 #pragma once
 #include "common.cuh"
-#include "sims.cuh"
-#include "select.cuh"
+#include "arrange.cuh"
+#include "evict.cuh"
 #include "place.cuh"
 #include "order_pin.cuh"
 
@@ -46,6 +46,7 @@ __device__ __forceinline__ int pool_busy_units(const Params& P, const ReplayWs& 
   if (pd.type == TG_POOL_API) b = pd.window_us > 0 ? Z.pst[((size_t)sc * P.P + j) * 2] : Z.pst[((size_t)sc * P.P + j) * 2 + 1];
   else {
     const int* ow = Z.owner + (size_t)sc * R.U + R.unit0[j];
+#pragma unroll 1
     for (int c = lane; c < pd.capacity; c += 32) b += ow[c] != -1;
     b = warp_sum32(b);
   }
@@ -59,12 +60,14 @@ __device__ __forceinline__ int pool_busy_units(const Params& P, const ReplayWs& 
 __device__ int replay_prefix(const Params& P, const ReplayWs& R, const ReplayState& Z, int sc, const int* wait, int nw,
                              int* dem, int* cap, int* aside, int* ncand, int lane) {
   const size_t row = (size_t)sc * P.N;
+#pragma unroll 1
   for (int j = 0; j < P.P; ++j) {
     const PoolDev& pd = P.pool[j];
     int c[4] = {0, 0, 0, 0};
     if (pd.type == TG_POOL_GPU) gpu_caps(pd, Z.nm + (size_t)sc * P.n_nodes_total, lane, c);
     else if (pd.type == TG_POOL_CPU) {
       int f = 0;
+#pragma unroll 1
       for (int d = lane; d < pd.capacity / pd.group; d += 32) f += Z.dfree[(size_t)sc * R.Dtot + R.dom0[j] + d];
       c[0] = warp_sum32(f);
     } else {
@@ -77,6 +80,7 @@ __device__ int replay_prefix(const Params& P, const ReplayWs& R, const ReplaySta
   __syncwarp();
   int n = 0;
   bool stop = false;
+#pragma unroll 1
   for (int i0 = 0; i0 < nw && !stop; i0 += 32) {
     // every lane decodes one waiting action, then the 32 are admitted one after the other
     int j = 0, lz = 0, units = 0;
@@ -95,9 +99,11 @@ __device__ int replay_prefix(const Params& P, const ReplayWs& R, const ReplaySta
       lz = P.pool[j].type == TG_POOL_GPU ? level_of(g, gang, rmin) : 0;
     }
     const int nb = min(32, nw - i0);
+#pragma unroll 1
     for (int b = 0; b < nb; ++b) {
       const int bj = __shfl_sync(TG_FULL, j, b), bl = __shfl_sync(TG_FULL, lz, b), bu = __shfl_sync(TG_FULL, units, b);
       bool over = false;
+#pragma unroll 1
       for (int l = 0; l <= bl; ++l) over |= dem[bj * 4 + l] + bu > cap[bj * 4 + l];
       int a0 = 0xff, c0 = 0, a1 = 0xff, c1 = 0;
       if (P.n_side > 0) {
@@ -131,6 +137,7 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   // m: members of the pool among the candidates (counted by the prefix); n_ac: members behind them, which
   // only an eviction step's estimate looks at (a single candidate is never evicted)
   int n_ac = 0;
+#pragma unroll 1
   for (int i0 = n & ~31; i0 < nw && m >= 2; i0 += 32) {
     const int i = i0 + lane;
     const bool mine = i < nw && i >= n && P.a_pool[row + wait[i]] == j;
@@ -150,6 +157,7 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   // fill them in queue order
   int cm = 0, ca = 0, first_ac = -1;
   bool elastic = false;
+#pragma unroll 1
   for (int i0 = 0; i0 < nw; i0 += 32) {
     const int i = i0 + lane;
     int a = -1; bool mine = false;
@@ -175,6 +183,7 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   // completion times (relative to now) of what runs on this pool seed the heap
   // (only an eviction step looks at the heap: with one candidate, or none that is elastic, nobody reads it)
   int ns = 0;
+#pragma unroll 1
   for (int i0 = 0; i0 < nr && elastic && m >= 2; i0 += 32) {
     const int i = i0 + lane;
     int a = -1; bool mine = false;
@@ -189,30 +198,37 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   __syncwarp();
   int keep = m;
   if (elastic) {
-    PoolTask T;
-    T.type = pd.type; T.group = pd.group;
-    T.cap[0] = T.cap[1] = T.cap[2] = T.cap[3] = 0;
-    if (pd.type == TG_POOL_GPU) gpu_caps(pd, Z.nm + (size_t)sc * P.n_nodes_total, lane, T.cap);
+    int cap[4] = {0, 0, 0, 0};
+    if (pd.type == TG_POOL_GPU) gpu_caps(pd, Z.nm + (size_t)sc * P.n_nodes_total, lane, cap);
     else if (pd.type == TG_POOL_CPU) {
       int f = 0;
+#pragma unroll 1
       for (int d = lane; d < pd.capacity / pd.group; d += 32) f += Z.dfree[(size_t)sc * R.Dtot + R.dom0[j] + d];
-      T.cap[0] = warp_sum32(f);
+      cap[0] = warp_sum32(f);
     } else {
       const int* ps = Z.pst + ((size_t)sc * P.P + j) * 2;
-      T.cap[0] = pd.capacity - (pd.window_us > 0 ? ps[0] : ps[1]) - aside_j;   // set aside for the other pools' candidates
+      cap[0] = pd.capacity - (pd.window_us > 0 ? ps[0] : ps[1]) - aside_j;   // set aside for the other pools' candidates
     }
-    T.m = m; T.cs = C.cs; T.cp = C.cp; T.cmask = C.cmask; T.cg = C.cg;
-    T.n_ac = n_ac; T.ac_tmin = ac_tmin;
-    T.ac_first.s = T.ac_first.p = 0; T.ac_first.mask = 1; T.ac_first.g = 1; T.ac_first.gang = 0;
+    Act first;
+    first.s = first.p = 0; first.mask = 1; first.g = 1; first.gang = 0;
     if (n_ac > 0) {
-      decode_levels(pd, P.a_unit[row + first_ac], P.a_mask[row + first_ac], T.ac_first.g, T.ac_first.gang, T.ac_first.mask);
-      T.ac_first.s = clamp_param(P.a_s[row + first_ac]); T.ac_first.p = clamp_param(P.a_p[row + first_ac]);
+      decode_levels(pd, P.a_unit[row + first_ac], P.a_mask[row + first_ac], first.g, first.gang, first.mask);
+      first.s = clamp_param(P.a_s[row + first_ac]); first.p = clamp_param(P.a_p[row + first_ac]);
     }
-    T.seeds = seeds; T.n_seeds = ns;
-    T.depth = P.depth;
-    T.rsel = C.rsel; T.rkeep = C.rkeep; T.rowcand = C.rowcand;
-    T.sim_base = 0; T.sim_cap = 0;
-    attach_warp_tree(T);
+    PoolTask& T = warp_task();
+    __syncwarp();
+    if (lane == 0) {
+      T.type = pd.type; T.group = pd.group;
+#pragma unroll 1
+      for (int l = 0; l < 4; ++l) T.cap[l] = cap[l];
+      T.m = m; T.cs = C.cs; T.cp = C.cp; T.cmask = C.cmask; T.cg = C.cg;
+      T.n_ac = n_ac; T.ac_tmin = ac_tmin; T.ac_first = first;
+      T.seeds = seeds; T.n_seeds = ns;
+      T.depth = P.depth;
+      T.rsel = C.rsel; T.rkeep = C.rkeep; T.rowcand = C.rowcand;
+      T.wk = warp_smem(); T.wk_bytes = WARP_WORK_BYTES;
+    }
+    __syncwarp();
     keep = evict_loop(P, T, slab, lane);
     if (keep < 0) return false;
   }
@@ -233,6 +249,7 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   } else {
     if (lane == 0) {
       int* ps = Z.pst + ((size_t)sc * P.P + j) * 2 + (pd.window_us > 0 ? 0 : 1);
+#pragma unroll 1
       for (int i = 0; i < keep; ++i) { C.pnode[i] = 0; C.poff[i] = *ps; *ps += (C.cg[i] & 0x7f) * C.rkeep[i]; }
     }
   }
@@ -240,6 +257,7 @@ __device__ bool replay_pool(const Params& P, const ReplayWs& R, const ReplayStat
   // start what was selected (Eq. 2: completion - arrival = waited so far + execution)
   i64 tot = 0;
   int started = 0;
+#pragma unroll 1
   for (int i = lane; i < keep; i += 32) {
     const size_t o = row + C.cidx[i];
     const int r = C.rkeep[i];
@@ -270,6 +288,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * KR_THREADS + threadIdx.x) >> 5;
   const int nw_warps = (gridDim.x * KR_THREADS) >> 5;
+#pragma unroll 1
   for (int sc = gw; sc < P.S; sc += nw_warps) {
     const size_t row = (size_t)sc * P.N;
     const int n_act = min(max(P.n_actions[sc], 0), P.N);
@@ -293,12 +312,15 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
     int* dfree = Z.dfree + (size_t)sc * R.Dtot;
     int* occ = R.occupancy ? R.occupancy + (size_t)sc * R.max_rounds * P.P : nullptr;
     // outputs and state start empty
+#pragma unroll 1
     for (int i = lane; i < P.N; i += 32) { P.o_alloc[row + i] = 0; P.o_node[row + i] = -1; P.o_off[row + i] = -1; P.o_act[row + i] = -1; }
     int status = 0;
+#pragma unroll 1
     for (int i = lane; i < n_act; i += 32) {
       const int j = P.a_pool[row + i];
       int g, gang; u32 eff;
       if (j >= P.P || !decode_levels(P.pool[j], P.a_unit[row + i], P.a_mask[row + i], g, gang, eff)) status |= TG_ST_BAD_ACTION;
+#pragma unroll 1
       for (int e = 0; e < P.n_side; ++e) {                  // further entries: a quota / concurrency pool other than j, 1 .. capacity
         const int k = P.a_side_pool[e * P.side_plane + row + i];
         if (k == 0xff) continue;
@@ -308,20 +330,25 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       }
       if (i > 0 && P.a_arrival && P.a_arrival[row + i - 1] > P.a_arrival[row + i]) status |= TG_ST_UNSORTED;
     }
+#pragma unroll 1
     for (int o = 16; o; o >>= 1) status |= __shfl_xor_sync(TG_FULL, status, o);
     if (status & TG_ST_BAD_ACTION) status = TG_ST_BAD_ACTION;
+#pragma unroll 1
     for (int j = 0; j < P.P; ++j) {
       const PoolDev& pd = P.pool[j];
       if (pd.type == TG_POOL_API) { if (lane < 2) Z.pst[((size_t)sc * P.P + j) * 2 + lane] = 0; if (lane == 0) Z.win[(size_t)sc * P.P + j] = 0; continue; }
+#pragma unroll 1
       for (int c = lane; c < pd.capacity; c += 32) {
         int v = -1;
         if (pd.type == TG_POOL_GPU && P.gpu_busy && (P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + c / pd.group] >> (c % pd.group) & 1)) v = -2;
         owner[R.unit0[j] + c] = v;
       }
       if (pd.type == TG_POOL_GPU)
+#pragma unroll 1
         for (int v = lane; v < pd.n_nodes; v += 32)
           nm[pd.node0 + v] = (P.gpu_busy ? P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + v] : 0) & ((1u << pd.group) - 1u);
       if (pd.type == TG_POOL_CPU)
+#pragma unroll 1
         for (int d = lane; d < pd.capacity / pd.group; d += 32) dfree[R.dom0[j] + d] = pd.group;
     }
     if (lane == 0) { P.o_total[sc] = 0; P.o_nsel[sc] = 0; P.o_status[sc] = status; }
@@ -338,10 +365,13 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       bool drained = false;
       // units in use per core / GPU pool, kept up to date by what starts and what is released
       int busy[TG_MAX_POOLS];
+#pragma unroll 1
       for (int j = 0; j < P.P; ++j) busy[j] = P.pool[j].type == TG_POOL_API ? 0 : pool_busy_units(P, R, Z, sc, j, lane);
+#pragma unroll 1
       while (r < R.max_rounds) {
         const i64 now = (i64)r * R.round_us;
         // 1. quota refill
+#pragma unroll 1
         for (int j = 0; j < P.P; ++j) {
           const PoolDev& pd = P.pool[j];
           if (pd.type == TG_POOL_API && pd.window_us > 0 && now / pd.window_us != Z.win[(size_t)sc * P.P + j]) {
@@ -354,6 +384,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         int kept = 0;
         bool gpu_released = false;
         i64 min_fin = TG_INF;                               // earliest completion among what keeps running
+#pragma unroll 1
         for (int i0 = 0; i0 < nr; i0 += 32) {
           const int i = i0 + lane;
           int a = -1; bool done = false;
@@ -368,6 +399,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (i < nr && !done) run[kept + __popc(bk & ((1u << lane) - 1u))] = a;
           kept += __popc(bk);
           u32 rest = bd;
+#pragma unroll 1
           while (rest) {
             const int b = __ffs(rest) - 1; rest &= rest - 1;
             const int fa = __shfl_sync(TG_FULL, a, b);
@@ -382,6 +414,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               }
             }
             if (P.n_side > 0 && lane == 0)                 // a concurrency pool held the action's further amounts until now
+#pragma unroll 1
               for (int e = 0; e < P.n_side; ++e) {
                 const int k = P.a_side_pool[e * P.side_plane + row + fa];
                 if (k != 0xff && P.pool[k].window_us == 0) Z.pst[((size_t)sc * P.P + k) * 2 + 1] -= P.a_side_units[e * P.side_plane + row + fa];
@@ -391,6 +424,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               const int freed = P.o_alloc[row + fa];
 #pragma unroll
               for (int jj = 0; jj < TG_MAX_POOLS; ++jj) if (jj == j) busy[jj] -= freed;
+#pragma unroll 1
               for (int c = lane; c < pd.capacity; c += 32) {
                 if (owner[R.unit0[j] + c] != fa) continue;
                 owner[R.unit0[j] + c] = -1;
@@ -404,11 +438,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         nr = kept;
         const int nr_before = nr;
         if (__any_sync(TG_FULL, gpu_released)) {            // node masks follow the owner map
+#pragma unroll 1
           for (int j = 0; j < P.P; ++j) {
             const PoolDev& pd = P.pool[j];
             if (pd.type != TG_POOL_GPU) continue;
+#pragma unroll 1
             for (int v = lane; v < pd.n_nodes; v += 32) {
               u32 mk = 0;
+#pragma unroll 1
               for (int b = 0; b < pd.group; ++b) mk |= (owner[R.unit0[j] + v * pd.group + b] != -1 ? 1u : 0u) << b;
               nm[pd.node0 + v] = (u8)mk;
             }
@@ -417,6 +454,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         }
         // 3. admit arrivals
         const int nw_admitted = nw;
+#pragma unroll 1
         while (next < n_act) {
           const int i = next + lane;
           const bool in = i < n_act && (P.a_arrival ? P.a_arrival[row + i] : 0) <= now;
@@ -451,6 +489,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           // Other queue orders (Section 4.2): the queue stays sorted by the policy's key, equal keys in arrival
           // order.  Each new arrival goes behind the last entry whose key is not larger; the tail moves up by one.
           u64* wkey = R.wkey + row;
+#pragma unroll 1
           for (int x = nw_admitted; x < nw; ++x) {
             const int a = wait[x];
             int g, gang; u32 eff;
@@ -458,10 +497,12 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
             const i64 T = duration(clamp_param(P.a_s[row + a]), clamp_param(P.a_p[row + a]), __ffs(eff));
             const u64 k = R.policy == 2 ? (u64)((1ll << 42) - T) : (u64)T;
             int p = 0;
+#pragma unroll 1
             for (int i0 = 0; i0 < x; i0 += 32) {
               const int i = i0 + lane;
               p += __popc(__ballot_sync(TG_FULL, i < x && wkey[i] <= k));
             }
+#pragma unroll 1
             for (int hi = x; hi > p;) {
               const int lo = max(p, hi - 32), i = lo + lane;
               int va = 0; u64 vk = 0;
@@ -483,6 +524,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           const int nr0 = nr;
           bool ok = true;
           if (n > 0)
+#pragma unroll 1
             for (int j = 0; j < P.P && ok; ++j) {
               if (ncand[j] == 0) continue;                  // no candidate has this pool as its key pool
               int add = 0;
@@ -493,7 +535,9 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (!ok) { if (lane == 0) P.o_status[sc] |= TG_ST_WORKSPACE; break; }
           if (P.n_side > 0 && nr > nr0) {                   // the started actions consume their further amounts
             __syncwarp();
+#pragma unroll 1
             for (int i = nr0 + lane; i < nr; i += 32)
+#pragma unroll 1
               for (int e = 0; e < P.n_side; ++e) {
                 const int k = P.a_side_pool[e * P.side_plane + row + run[i]];
                 if (k != 0xff)
@@ -504,6 +548,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           }
           if (nr > nr0) {                                   // drop the started actions from the queue
             int kw = 0;
+#pragma unroll 1
             for (int i0 = 0; i0 < nw; i0 += 32) {
               const int i = i0 + lane;
               int a = -1; bool stay = false;
@@ -519,6 +564,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           }
         }
         // 5. occupancy of this round
+#pragma unroll 1
         for (int j = 0; j < P.P; ++j) if (P.pool[j].type == TG_POOL_API) busy[j] = pool_busy_units(P, R, Z, sc, j, lane);
         if (occ && lane == 0) for (int j = 0; j < P.P; ++j) occ[(size_t)r * P.P + j] = busy[j];
         ++r;
@@ -528,6 +574,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           // (what was running before this round: the release scan's minimum; what started in it: the tail of the list)
           i64 t_next = next < n_act ? (P.a_arrival ? P.a_arrival[row + next] : 0) : TG_INF;
           t_next = min(t_next, min_fin);
+#pragma unroll 1
           for (int i = nr_before + lane; i < nr; i += 32) {
             const int a = run[i];
             t_next = min(t_next, (P.a_arrival ? P.a_arrival[row + a] : 0) + P.o_act[row + a]);
@@ -536,7 +583,9 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           i64 r_next = (t_next + R.round_us - 1) / R.round_us;
           if (r_next > R.max_rounds) r_next = R.max_rounds;
           // skipped rounds repeat this occupancy, except that quota usage restarts with its window
+#pragma unroll 1
           for (i64 rr = r + lane; rr < r_next; rr += 32)
+#pragma unroll 1
             for (int j = 0; j < P.P; ++j) {
               const PoolDev& pd = P.pool[j];
               int v = busy[j];
@@ -554,6 +603,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (hp.type == TG_POOL_API && hp.window_us > 0) t_next = (Z.win[(size_t)sc * P.P + blocked_pool] + 1) * (i64)hp.window_us;
           // (in a sorted queue an arrival with a smaller key becomes the head)
           if (ORDERED && next < n_act) t_next = min(t_next, P.a_arrival ? P.a_arrival[row + next] : 0);
+#pragma unroll 1
           for (int i = lane; i < nr; i += 32) {
             const int a = run[i];
             if (P.a_pool[row + a] == blocked_pool) t_next = min(t_next, (P.a_arrival ? P.a_arrival[row + a] : 0) + P.o_act[row + a]);
@@ -563,7 +613,9 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (r_next > R.max_rounds) r_next = R.max_rounds;
           if (r_next > r) {
             if (occ) {
+#pragma unroll 1
               for (i64 rr = r + lane; rr < r_next; rr += 32)
+#pragma unroll 1
                 for (int j = 0; j < P.P; ++j) {
                   const PoolDev& pd = P.pool[j];
                   int v = busy[j];
@@ -572,6 +624,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 }
               __syncwarp();
               // what ends on the other pools inside the jump leaves the rows from its round on
+#pragma unroll 1
               for (int i = lane; i < nr; i += 32) {
                 const int a = run[i];
                 const int j = P.a_pool[row + a];
@@ -580,6 +633,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 const i64 fin = (P.a_arrival ? P.a_arrival[row + a] : 0) + P.o_act[row + a];
                 i64 fr = (fin + R.round_us - 1) / R.round_us;
                 if (fr < r) fr = r;
+#pragma unroll 1
                 for (i64 rr = fr; rr < r_next; ++rr) atomicSub(&occ[(size_t)rr * P.P + j], P.o_alloc[row + a]);
               }
               __syncwarp();

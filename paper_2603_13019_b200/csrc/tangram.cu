@@ -11,30 +11,23 @@
 #include "prefix_kernel.cuh"
 #include "prefix_stream.cuh"
 #include "order_pin.cuh"
-#include "sims.cuh"
-#include "select.cuh"
+#include "arrange.cuh"
+#include "evict.cuh"
 #include "place.cuh"
 
 #define K2_THREADS 256
 #define TG_PROF_CALLS 256   // calls whose kernels can be timed between two queries
-#define TG_N_SIM_CLASSES 22
 #define TG_FILL_BLOCKS_PER_SM 4   // k_fill is a trickle beside the other kernels, not a flood
 #define TG_IO_CHUNKS 16
-#define TG_PROF_K 6         // timed intervals per call at most
+#define TG_PROF_K 3         // timed intervals per call at most
 #define TG_N_KERNELS 8
 
 // ---------------------------------------------------------------------------------------
-// Per-(scenario, pool) work of a round, one warp per task.  The pieces are shared by
-//   k_select            everything in one kernel (general path: any number of evictions,
-//                       running actions in the heap; used by the allocation-free entry point),
-//   k_solve / k_finish  the batched path: k_solve computes the optimal allocations of the full
-//                       candidate list and of the list without its last candidate; a pool
-//                       without elastic candidates, or whose first eviction step cannot pay
-//                       (eviction_cannot_pay), is placed and written at once.  For the others
-//                       k_sims (sims.cuh) runs the completion-heap simulations one thread
-//                       each, and k_finish compares the two objectives (Algorithm 1, lines
-//                       8-14), goes on evicting where the first eviction pays, places the
-//                       grants and writes the candidates' outputs (Eq. 2).
+// Per-(scenario, pool) work of a round, one warp per task: gather the pool's candidates, decide
+// them (arrange.cuh, evict.cuh), place what was granted, write the candidates' outputs (Eq. 2).
+//   k_pool     the batched path, behind k_head / k_stream; pools that the head kernel certified
+//              take a short way without any selection
+//   k_select   the allocation-free entry point, behind k_prefix
 // ---------------------------------------------------------------------------------------
 // Tasks are handed out by a counter so that long tasks do not pile up on the same warps.
 __device__ __forceinline__ int next_task(u64* counter, int lane) {
@@ -68,6 +61,7 @@ __device__ bool gather_candidates(const Params& P, int sc, int j, const PoolMeta
   if (!C.cg || !C.rkeep || !C.rsel || !C.cmask || !C.rowcand || !C.cp || !C.cs || !C.cidx || !C.pnode || !C.poff) return false;
   // four candidates per lane at a time: first all their indices, then all their records, so that a
   // pool of up to 128 candidates costs two rounds of loads instead of two per 32 candidates
+#pragma unroll 1
   for (int i0 = lane; i0 < m; i0 += 128) {
     int idx[4]; u8 un[4]; u32 mk[4]; i64 sv[4], pv[4];
 #pragma unroll
@@ -94,73 +88,72 @@ __device__ bool gather_candidates(const Params& P, int sc, int j, const PoolMeta
   return true;
 }
 
-// with_waiting = false leaves out the pool's waiting actions (k_solve estimates nothing itself).
-__device__ void make_task(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C, int lane,
-                          PoolTask& T, bool with_waiting = true) {
-  const PoolDev& pd = P.pool[j];
-  const size_t row = (size_t)sc * P.N;
-  const u8* busy_row = P.gpu_busy ? P.gpu_busy + (size_t)sc * P.n_nodes_total : nullptr;
-  T.type = pd.type; T.group = pd.group;
-  T.cap[0] = pd.capacity; T.cap[1] = T.cap[2] = T.cap[3] = 0;
-  if (pd.type == TG_POOL_GPU) gpu_caps(pd, busy_row, lane, T.cap);
-  if (P.n_side > 0 && pd.type == TG_POOL_API) T.cap[0] -= P.side_res[(size_t)sc * P.P + j];   // set aside for the other pools' candidates
-  T.m = mt.m; T.cs = C.cs; T.cp = C.cp; T.cmask = C.cmask; T.cg = C.cg;
-  T.n_ac = with_waiting ? mt.count - mt.m : 0;
-  T.ac_tmin = P.tmin + row + mt.base + mt.m;
-  T.ac_first.s = T.ac_first.p = 0; T.ac_first.mask = 1; T.ac_first.g = 1; T.ac_first.gang = 0;
-  if (T.n_ac > 0) {
-    int idx = mt.first_wait;
-    decode_levels(pd, P.a_unit[row + idx], P.a_mask[row + idx], T.ac_first.g, T.ac_first.gang, T.ac_first.mask);
-    T.ac_first.s = clamp_param(P.a_s[row + idx]); T.ac_first.p = clamp_param(P.a_p[row + idx]);
-  }
-  T.seeds = nullptr; T.n_seeds = 0;
-  T.depth = P.depth;
-  T.rsel = C.rsel; T.rkeep = C.rkeep; T.rowcand = C.rowcand;
-  T.sim_base = 0; T.sim_cap = 0;
-}
-
-// shared memory of the calling warp for winner trees inside the per-pool kernels
-#define WARP_TREE_SLOTS 448
-#define WARP_TREE_BYTES (WARP_TREE_SLOTS * 16)
+// the calling warp's scratch: work area and window in shared memory, slab in global memory
+#define WARP_WORK_BYTES 7424
 #define WARP_FAST_BYTES 2048
-#define WARP_SMEM_BYTES (WARP_TREE_BYTES + WARP_FAST_BYTES)
+#define WARP_TASK_BYTES 384
+#define WARP_SMEM_BYTES (WARP_WORK_BYTES + WARP_FAST_BYTES + WARP_TASK_BYTES)
+static_assert(sizeof(PoolTask) <= WARP_TASK_BYTES, "");
 #define K2_DYN_SMEM ((K2_THREADS / 32) * WARP_SMEM_BYTES + 16)
-__device__ __forceinline__ void attach_warp_tree(PoolTask& T) {
+__device__ __forceinline__ char* warp_smem() {
   extern __shared__ __align__(16) unsigned char k2_smem[];
-  const u32 start = ((u32)__cvta_generic_to_shared(k2_smem) + 15u) & ~15u;
-  T.sim_base = start + (threadIdx.x >> 5) * WARP_SMEM_BYTES;
-  T.sim_cap = WARP_TREE_SLOTS;
+  return (char*)(((u64)k2_smem + 15u) & ~(u64)15) + (threadIdx.x >> 5) * WARP_SMEM_BYTES;
 }
-// the calling warp's scratch: shared-memory window behind its tree area, then its global slab
+__device__ __forceinline__ PoolTask& warp_task() { return *(PoolTask*)(warp_smem() + WARP_WORK_BYTES + WARP_FAST_BYTES); }
 __device__ __forceinline__ Slab warp_slab(const Params& P, int gw) {
-  extern __shared__ __align__(16) unsigned char k2_smem[];
   Slab s;
   s.base = P.slabs + (u64)gw * P.slab_bytes; s.cap = P.slab_bytes; s.used = 0;
-  const u64 start = ((u64)k2_smem + 15u) & ~(u64)15;
-  s.fbase = (char*)start + (threadIdx.x >> 5) * WARP_SMEM_BYTES + WARP_TREE_BYTES;
+  s.fbase = warp_smem() + WARP_WORK_BYTES;
   s.fcap = WARP_FAST_BYTES; s.fused = 0;
   return s;
 }
 
+__device__ PoolTask& make_task(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C, int lane) {
+  const PoolDev& pd = P.pool[j];
+  const size_t row = (size_t)sc * P.N;
+  const u8* busy_row = P.gpu_busy ? P.gpu_busy + (size_t)sc * P.n_nodes_total : nullptr;
+  int cap[4] = {pd.capacity, 0, 0, 0};
+  if (pd.type == TG_POOL_GPU) gpu_caps(pd, busy_row, lane, cap);
+  if (P.n_side > 0 && pd.type == TG_POOL_API) cap[0] -= P.side_res[(size_t)sc * P.P + j];   // set aside for the other pools' candidates
+  Act first;
+  first.s = first.p = 0; first.mask = 1; first.g = 1; first.gang = 0;
+  const int n_ac = mt.count - mt.m;
+  if (n_ac > 0) {
+    const size_t o = row + mt.first_wait;
+    decode_levels(pd, P.a_unit[o], P.a_mask[o], first.g, first.gang, first.mask);
+    first.s = clamp_param(P.a_s[o]); first.p = clamp_param(P.a_p[o]);
+  }
+  PoolTask& T = warp_task();
+  __syncwarp();
+  if (lane == 0) {
+    T.type = pd.type; T.group = pd.group;
+#pragma unroll 1
+    for (int l = 0; l < 4; ++l) T.cap[l] = cap[l];
+    T.m = mt.m; T.cs = C.cs; T.cp = C.cp; T.cmask = C.cmask; T.cg = C.cg;
+    T.n_ac = n_ac; T.ac_tmin = P.tmin + row + mt.base + mt.m; T.ac_first = first;
+    T.seeds = nullptr; T.n_seeds = 0;
+    T.depth = P.depth;
+    T.rsel = C.rsel; T.rkeep = C.rkeep; T.rowcand = C.rowcand;
+    T.wk = warp_smem(); T.wk_bytes = WARP_WORK_BYTES;
+  }
+  __syncwarp();
+  return T;
+}
+
 // placement on a fresh copy of the pool's topology state, then the candidates' outputs
 __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C,
-                                int keep, Slab slab, int lane, bool defer = false) {
+                                int keep, Slab slab, int lane) {
   const int m = mt.m;
   const PoolDev& pd = P.pool[j];
   const size_t row = (size_t)sc * P.N;
   const u8* busy_row = P.gpu_busy ? P.gpu_busy + (size_t)sc * P.n_nodes_total : nullptr;
   const u8* missed = nullptr;                            // candidates whose chunk did not cache their service
-  defer = defer && pd.lane_place;
-  if (defer) {
-    // k_place will place this pool: leave it the kept requests in queue order
-    unsigned short* rq = P.preq + row + mt.cbase;
-    for (int i = lane; i < keep; i += 32) rq[i] = (unsigned short)(C.cg[i] | ((u32)C.rkeep[i] << 8));
-    if (lane == 0) P.keepn[(size_t)sc * P.P + j] = keep;
-  } else if (pd.type == TG_POOL_GPU && P.cache_slots > 0) {
+  if (pd.type == TG_POOL_GPU && P.cache_slots > 0) {
     // with a service cache: the chunk that caches the instance first, entries updated, misses noted in C.rsel
     u8* nm = (u8*)slab.take_fast(pd.n_nodes);
     if (!nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
     else {
+#pragma unroll 1
       for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
       __syncwarp();
       const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
@@ -170,33 +163,46 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
       missed = C.rsel;
     }
   } else if (pd.type == TG_POOL_GPU) {
-    if (pd.n_nodes <= 128) place_gpu_reg(pd, busy_row ? busy_row + pd.node0 : nullptr, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
+    const u8* br = busy_row ? busy_row + pd.node0 : nullptr;
+    if (pd.n_nodes <= 32) place_gpu_masks<1>(pd, br, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
+    else if (pd.n_nodes <= 128) place_gpu_masks<4>(pd, br, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
     else {
-    u8* nm = (u8*)slab.take_fast(pd.n_nodes);
-    if (!nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
-    else {
-      for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
-      __syncwarp();
-      place_gpu(pd, nm, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
-    }
+      u8* nm = (u8*)slab.take_fast(pd.n_nodes);
+      if (!nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
+      else {
+#pragma unroll 1
+        for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
+        __syncwarp();
+        place_gpu(pd, nm, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
+      }
     }
   } else if (pd.type == TG_POOL_CPU && pd.capacity / pd.group <= 128 && pd.group < 65536) {
-    place_cpu_fresh_reg(pd, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
+    CpuFresh<4> F(pd, lane);
+#pragma unroll 1
+    for (int i0 = 0; i0 < keep; i0 += 32) {
+      const int i = i0 + lane;
+      int node = -1, off = -1;
+      F.place(pd, i < keep ? (C.cg[i] & 0x7f) * C.rkeep[i] : 0, min(32, keep - i0), lane, node, off);
+      if (i < keep) { C.pnode[i] = node; C.poff[i] = off; }
+    }
   } else if (pd.type == TG_POOL_CPU) {
     const int D = pd.capacity / pd.group;
     int* dfree = (int*)slab.take_fast((u64)D * 4);
     if (!dfree) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
     else place_cpu_fresh(pd, dfree, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
   } else {
-    if (lane == 0) {
-      int used = 0;
-      for (int i = 0; i < keep; ++i) { C.pnode[i] = 0; C.poff[i] = used; used += (C.cg[i] & 0x7f) * C.rkeep[i]; }
+    int used = 0;                                        // Section 5.1: offset = units consumed before
+#pragma unroll 1
+    for (int i0 = 0; i0 < keep; i0 += 32) {
+      const int i = i0 + lane, u = i < keep ? (C.cg[i] & 0x7f) * C.rkeep[i] : 0;
+      const int incl = warp_incl_scan32(u, lane);
+      if (i < keep) { C.pnode[i] = 0; C.poff[i] = used + incl - u; }
+      used += __shfl_sync(TG_FULL, incl, 31);
     }
-    __syncwarp();
   }
-
   __syncwarp();
   i64 tot = 0; int cnt = 0;
+#pragma unroll 1
   for (int i = lane; i < m; i += 32) {
     const size_t o = row + C.cidx[i];
     if (i < keep) {
@@ -205,7 +211,7 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
       i64 act = (P.now - arr) + duration(C.cs[i], C.cp[i], r);
       if (missed && missed[i] && P.a_restore) act += clamp_param(P.a_restore[o]);   // restoration precedes execution
       P.o_alloc[o] = (C.cg[i] & 0x7f) * r; P.o_act[o] = act;
-      if (!defer) { P.o_node[o] = C.pnode[i]; P.o_off[o] = C.poff[i]; }
+      P.o_node[o] = C.pnode[i]; P.o_off[o] = C.poff[i];
       tot += act; ++cnt;
     } else {
       P.o_alloc[o] = 0; P.o_node[o] = -1; P.o_off[o] = -1; P.o_act[o] = -1;
@@ -218,9 +224,50 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
   }
 }
 
-__device__ void run_pool_task(const Params& P, int sc, int j, Slab slab, int lane) {
-  const PoolMeta mt = P.meta[(size_t)sc * P.P + j];
-  if (mt.m == 0) return;
+// A pool whose every candidate takes its best level (no elastic candidate, or all largest levels fit: the smallest
+// level that reaches the lowest duration, and no eviction can pay), of a type whose placement goes by queue order:
+// 32 candidates at a time through registers.  Bound by the chain of placements on a core pool (one warp
+// minimum per candidate).
+template <int NS>
+__device__ __forceinline__ void pool_best_levels(const Params& P, int sc, int j, const PoolMeta& mt, int lane) {
+  const PoolDev& pd = P.pool[j];
+  const size_t row = (size_t)sc * P.N;
+  const int* ord = P.order + row + mt.cbase;
+  const bool cpu = pd.type == TG_POOL_CPU;
+  CpuFresh<NS> F(pd, lane);
+  i64 tot = 0; int used = 0;
+#pragma unroll 1
+  for (int i0 = 0; i0 < mt.m; i0 += 32) {
+    const int i = i0 + lane;
+    const bool on = i < mt.m;
+    size_t o = row; int u = 0; i64 act = 0;
+    if (on) {
+      o += ord[i];
+      int g, gang; u32 eff;
+      decode_levels(pd, P.a_unit[o], P.a_mask[o], g, gang, eff);
+      const i64 s = clamp_param(P.a_s[o]), p = clamp_param(P.a_p[o]);
+      const int r = best_level(p, eff);
+      act = (P.now - (P.a_arrival ? P.a_arrival[o] : 0)) + duration(s, p, r);
+      u = g * r;
+      tot += act;
+    }
+    int node = 0, off = 0;
+    if (cpu) F.place(pd, u, min(32, mt.m - i0), lane, node, off);
+    else {
+      const int incl = warp_incl_scan32(u, lane);
+      off = used + incl - u;
+      used += __shfl_sync(TG_FULL, incl, 31);
+    }
+    if (on) { P.o_alloc[o] = u; P.o_act[o] = act; P.o_node[o] = node; P.o_off[o] = off; }
+  }
+  tot = warp_sum64(tot);                                 // (exact modulo 2^64, so also where an arrival lies behind now)
+  if (lane == 0) {
+    atomicAdd((u64*)&P.o_total[sc], (u64)tot);
+    atomicAdd(&P.o_nsel[sc], mt.m);
+  }
+}
+
+__device__ void run_pool_task(const Params& P, int sc, int j, const PoolMeta& mt, Slab slab, int lane) {
   CandArrays C;
   if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
     if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE);
@@ -228,10 +275,7 @@ __device__ void run_pool_task(const Params& P, int sc, int j, Slab slab, int lan
   }
   int keep = mt.m;
   if (mt.elastic) {
-    PoolTask T;
-    make_task(P, sc, j, mt, C, lane, T);
-    attach_warp_tree(T);
-    keep = evict_loop(P, T, slab, lane);
+    keep = evict_loop(P, make_task(P, sc, j, mt, C, lane), slab, lane);
     if (keep < 0) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
   }
   place_and_write(P, sc, j, mt, C, keep, slab, lane);
@@ -240,198 +284,38 @@ __device__ void run_pool_task(const Params& P, int sc, int j, Slab slab, int lan
 __global__ void __launch_bounds__(K2_THREADS) k_select(const __grid_constant__ Params P) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * K2_THREADS + threadIdx.x) >> 5;
-  const Slab slab = warp_slab(P, gw);
   const int n_tasks = P.S * P.P;
+#pragma unroll 1
   for (;;) {
     const int x = next_task(P.arena_top + 3, lane);
     if (x >= n_tasks) break;
-    run_pool_task(P, x % P.S, P.pool_order[x / P.S], slab, lane);   // pool-major, heaviest pools first
+    const int sc = x % P.S, j = P.pool_order[x / P.S];   // pool-major, heaviest pools first
+    const PoolMeta mt = P.meta[(size_t)sc * P.P + j];
+    if (mt.m > 0) run_pool_task(P, sc, j, mt, warp_slab(P, gw), lane);
   }
 }
 
-// The pools that the head kernel certified (no elastic candidate, or every candidate's largest level
-// fits: then each takes the smallest level that reaches its lowest duration and no eviction can
-// pay) need no selection at all.  One warp per such (scenario, pool), nothing but registers: the
-// candidates' allocations and predicted completion times (Eq. 2) are written, their requests are
-// left for the placement kernel.  Runs beside the streaming kernel, on a stream of its own.
-__global__ void __launch_bounds__(256) k_easy(const __grid_constant__ Params P, const HeadState* hst) {
-  const int lane = threadIdx.x & 31;
-  const long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (x >= (long long)P.S * P.P) return;
-  const int sc = (int)(x % P.S), j = P.pool_order[x / P.S], task = sc * P.P + j;
-  const PoolDev& pd = P.pool[j];
-  if (((hst[sc].need >> j) & 1u) || !pd.lane_place) return;
-  const PoolMeta mt = P.meta[task];
-  const int m = mt.m;
-  if (lane == 0) P.keepn[task] = m;
-  if (m == 0) return;
-  const size_t row = (size_t)sc * P.N;
-  const int* ord = P.order + row + mt.cbase;
-  unsigned short* rq = P.preq + row + mt.cbase;
-  i64 tot = 0; int cnt = 0;
-  for (int i = lane; i < m; i += 32) {
-    const size_t o = row + ord[i];
-    int g, gang; u32 eff;
-    decode_levels(pd, P.a_unit[o], P.a_mask[o], g, gang, eff);
-    const i64 s = clamp_param(P.a_s[o]), p = clamp_param(P.a_p[o]);
-    const int r = best_level(p, eff);
-    const i64 act = (P.now - (P.a_arrival ? P.a_arrival[o] : 0)) + duration(s, p, r);
-    P.o_alloc[o] = g * r; P.o_act[o] = act;
-    rq[i] = (unsigned short)((u32)g | ((u32)gang << 7) | ((u32)r << 8));
-    tot += act; ++cnt;
-  }
-  tot = warp_sum64(tot); cnt = warp_sum32(cnt);
-  if (lane == 0) {
-    atomicAdd((u64*)&P.o_total[sc], (u64)tot);
-    atomicAdd(&P.o_nsel[sc], cnt);
-  }
-}
-
-// workspace of the batched path, indexed like the partitioned arrays
-struct BatchWs {
-  TaskState* ts;   // [S][P]
-  i64* seed2;      // [S][cand_stride] durations of the first m-1 candidates under their optimal allocation
-  u8* rs1;         // [S][cand_stride] multiplicities of the optimal allocation of all m candidates
-  u8* rs2;         // [S][cand_stride] ... of the first m-1
-};
-
-__global__ void __launch_bounds__(K2_THREADS, 3) k_solve(const __grid_constant__ Params P, const BatchWs W, const HeadState* hst) {
+// All pools of a batched round, pool-major, the pools that may need a selection first.
+__global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ Params P, const HeadState* hst) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * K2_THREADS + threadIdx.x) >> 5;
   const int n_tasks = P.S * P.P;
+#pragma unroll 1
   for (;;) {
     const int x = next_task(P.arena_top + 1, lane);
     if (x >= n_tasks) break;
-    const int sc = x % P.S, j = P.pool_order[x / P.S], task = sc * P.P + j;
-    TaskState* st = W.ts + task;
-    if (!((hst[sc].need >> j) & 1u) && P.pool[j].lane_place) {   // certified by the head kernel: k_easy has it
-      if (lane == 0) st->flags = TS_DECIDED;
-      continue;
-    }
-    const PoolMeta mt = P.meta[task];
-    if (lane == 0) P.keepn[task] = -1;                   // nothing for k_place unless a decision says so
-    if (mt.m == 0) { if (lane == 0) st->flags = TS_DECIDED; continue; }
-    Slab slab = warp_slab(P, gw);
-    CandArrays C;
-    if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
-      if (lane == 0) { atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); st->flags = TS_DECIDED; }
-      continue;
-    }
-    // A pool is decided here unless its first eviction step needs the two estimates.
-    int keep = mt.m;
-    bool decided = true;
-    if (mt.elastic) {
-      PoolTask T;
-      make_task(P, sc, j, mt, C, lane, T, false);
-      attach_warp_tree(T);                               // scratch of the small-box DP
-      i64 opt0 = 0, opt1 = 0;
-      bool all_best;
-      bool ok = solve_prefix(P, T, mt.m, slab, lane, &opt0, &all_best);
-      if (ok) {
-        for (int i = lane; i < mt.m; i += 32) C.rkeep[i] = C.rsel[i];
-        __syncwarp();
-        if (mt.m >= 2 && !all_best) {                      // all at their best level: eviction_cannot_pay holds
-          ok = solve_prefix(P, T, mt.m - 1, slab, lane, &opt1);
-          if (ok && !eviction_cannot_pay(T, mt.m - 1, C.rkeep, C.rsel, lane)) {
-            decided = false;
-            const size_t pos = (size_t)sc * P.N + mt.base, cpos = (size_t)sc * P.N + mt.cbase;
-            for (int i = lane; i < mt.m; i += 32) {
-              W.rs1[cpos + i] = C.rkeep[i];
-              P.tmin[pos + i] = duration(C.cs[i], C.cp[i], C.rkeep[i]);   // heap seeds of the full list
-              if (i < mt.m - 1) {
-                W.rs2[cpos + i] = C.rsel[i];
-                W.seed2[cpos + i] = duration(C.cs[i], C.cp[i], C.rsel[i]);
-              }
-            }
-            if (lane == 0) {
-              st->opt[0] = opt0; st->opt[1] = opt1;
-              st->est[0] = 0;                              // stays if nothing waits behind the candidates
-              st->est[1] = TG_INF;
-              st->flags = TS_SOLVED;
-            }
-          }
-        }
-      }
-      if (!ok) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
-    }
-    if (decided) {
-      place_and_write(P, sc, j, mt, C, keep, slab, lane, true);
-      if (lane == 0) st->flags = TS_DECIDED;
-    }
-  }
-}
-
-// One pool whose first eviction step had to be estimated: compare the two objectives, go on
-// evicting where the first eviction pays, hand the result to the placement.
-__device__ void finish_task(const Params& P, const BatchWs& W, int x, int gw, int lane) {
-  const int sc = x % P.S, j = P.pool_order[x / P.S], task = sc * P.P + j;
-  const TaskState st = W.ts[task];
-  const PoolMeta mt = P.meta[task];
-  Slab slab = warp_slab(P, gw);
-  CandArrays C;
-  if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
-    if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE);
-    return;
-  }
-  int keep = mt.m;
-  if (!(st.flags & TS_SOLVED) || (st.flags & TS_FAILED)) keep = -1;
-  else {
-    const size_t pos = (size_t)sc * P.N + mt.cbase;
-    i64 obj = sat_add(st.opt[0], st.est[0]);
-    for (int i = lane; i < mt.m; i += 32) C.rkeep[i] = W.rs1[pos + i];
-    i64 nobj = sat_add(st.opt[1], st.est[1]);
-    if (nobj < obj) {                                    // the first eviction pays: go on
-      for (int i = lane; i < mt.m - 1; i += 32) C.rkeep[i] = W.rs2[pos + i];
-      __syncwarp();
-      PoolTask T;
-      make_task(P, sc, j, mt, C, lane, T);
-      attach_warp_tree(T);
-      keep = evict_resume(P, T, slab, lane, nobj, mt.m - 1);
-    }
-    __syncwarp();
-  }
-  if (keep < 0) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
-  place_and_write(P, sc, j, mt, C, keep, slab, lane, true);
-}
-
-// Work list of k_finish: the pools that k_solve left undecided, those that go on evicting first.
-// Each of the latter is a chain of dependent DPs and simulations, so they must start as early
-// as possible.  fl: [0] number of chain tasks, [1] number of other tasks, then the chain tasks
-// from the front and the others from the back of an array of S * P entries.
-__global__ void k_finish_list(const __grid_constant__ Params P, const BatchWs W, int* fl) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
-  const int n_tasks = P.S * P.P;
-  int kind = -1;                                          // 0 chain, 1 other
-  if (x < n_tasks) {
     const int sc = x % P.S, j = P.pool_order[x / P.S];
-    const TaskState* st = W.ts + (size_t)sc * P.P + j;
-    const int flags = st->flags;
-    if (!(flags & TS_DECIDED))
-      kind = ((flags & TS_SOLVED) && !(flags & TS_FAILED) &&
-              sat_add(st->opt[1], st->est[1]) < sat_add(st->opt[0], st->est[0])) ? 0 : 1;
-  }
-  for (int k = 0; k < 2; ++k) {
-    const u32 b = __ballot_sync(TG_FULL, kind == k);
-    if (!b) continue;
-    int at = 0;
-    if (lane == __ffs(b) - 1) at = atomicAdd(&fl[k], __popc(b));
-    at = __shfl_sync(TG_FULL, at, __ffs(b) - 1) + __popc(b & ((1u << lane) - 1u));
-    if (kind == k) fl[2 + (k == 0 ? at : n_tasks - 1 - at)] = x;
+    PoolMeta mt = P.meta[(size_t)sc * P.P + j];          // (a scenario with an invalid record has no candidates)
+    mt.m = uniform(mt.m); mt.count = uniform(mt.count); mt.elastic = uniform(mt.elastic);
+    if (mt.m == 0) continue;
+    if (!((hst[sc].need >> j) & 1u) && P.pool[j].queue_place) {
+      if (P.pool[j].type == TG_POOL_API || P.pool[j].capacity <= 64 * P.pool[j].group) pool_best_levels<2>(P, sc, j, mt, lane);
+      else pool_best_levels<4>(P, sc, j, mt, lane);
+    }
+    else run_pool_task(P, sc, j, mt, warp_slab(P, gw), lane);
   }
 }
 
-__global__ void __launch_bounds__(K2_THREADS) k_finish(const __grid_constant__ Params P, const BatchWs W, const int* fl) {
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * K2_THREADS + threadIdx.x) >> 5;
-  const int n_tasks = P.S * P.P, n_chain = fl[0], n_all = fl[0] + fl[1];
-  for (;;) {
-    const int y = next_task(P.arena_top + 2, lane);
-    if (y >= n_all) break;
-    finish_task(P, W, fl[2 + (y < n_chain ? y : n_tasks - 1 - (y - n_chain))], gw, lane);
-  }
-}
-
-#include "place_lane.cuh"
 #include "replay.cuh"
 
 // ---------------------------------------------------------------------------------------
@@ -453,17 +337,13 @@ struct tangram_round {
   int64_t launches;
   // workspace
   void* d_order; void* d_tmin; void* d_meta; void* d_slabs; void* d_arena; void* d_arena_top;
-  HeadState* hst; void* d_preq; void* d_keepn; int* d_fl; u32* d_ok_table; int* d_side_bad; int* d_side_res;
-  BatchWs W; int sim_blocks; SimLists L; int n_sm;
+  HeadState* hst; u32* d_ok_table; int* d_side_bad; int* d_side_res;
+  int n_sm;
   ReplayWs R;
   // host-buffer mode: copy-in, kernels and copy-out of successive chunks on streams of their own
   cudaStream_t io_in, io_comp, io_out;
   cudaEvent_t io_begin, io_end, io_in_done[TG_IO_CHUNKS], io_comp_done[TG_IO_CHUNKS];
-  // the capacity classes of k_sims are independent: they run on side streams between a fork
-  // and a join event so that their partial waves overlap
-  cudaStream_t sim_stream[TG_N_SIM_CLASSES + 1];
-  cudaEvent_t sim_fork, sim_join[TG_N_SIM_CLASSES + 1];
-  // the certified pools (k_easy and their placement) run beside the kernels that follow k_solve
+  // the output fill runs beside the other kernels of a round
   cudaStream_t side; cudaEvent_t side_fork, side_join;
   // sorted copy of the queue and of its results (tangram_schedule_batch_ordered), allocated at its first call
   char* d_sorted; int* d_perm; u64* d_wkey;
@@ -474,32 +354,8 @@ struct tangram_round {
   cudaEvent_t* ev; int ev_calls, ev_used; int ev_kernel[TG_PROF_CALLS][TG_PROF_K];
 };
 
-static const char* const g_kernel_names[TG_N_KERNELS] = {"k_head", "k_select", "k_replay", "k_solve",
-                                                          "k_sims", "k_finish", "k_place", "k_stream"};
-// capacity classes (slots per simulation) of the shared-memory simulation kernels
-static const int g_sim_caps[TG_N_SIM_CLASSES] = {16, 32, 48, 64, 80, 96, 112, 128, 144, 160, 176, 192, 224, 256,
-                                                 320, 384, 448, 512, 576, 608, 640, 672};
-#define TG_SMEM_PER_SM 233472   // shared memory an SM can split among resident blocks
-#define TG_SMEM_PER_BLOCK 232448
-
-typedef void (*sims_fn)(const Params, TaskState*, const i64*, const SimLists, int);
-// levels below the root of the 4-ary tree of a capacity class
-static int sim_levels(int cap) {
-  long long nodes = tree_nodes(cap), reach = 1, width = 1;
-  int d = 0;
-  while (reach < nodes) { width *= 4; reach += width; ++d; }
-  return d;
-}
-static sims_fn sim_kernel(int cap) {
-  switch (sim_levels(cap)) {
-    case 0: case 1: case 2: return k_sims1<2>;
-    case 3: return k_sims1<3>;
-    case 4: return k_sims1<4>;
-    default: return k_sims1<5>;
-  }
-}
-// shared memory of a block (32 trees interleaved by lane) of a capacity class
-static int sim_smem_bytes(int cap) { return tree_nodes(cap) * 8 * SIM_PER_WARP; }
+static const char* const g_kernel_names[TG_N_KERNELS] = {"k_head", "k_select", "k_replay", "k_pool",
+                                                          "k_stream", "k_order", "k_pin", "k_fill"};
 
 static cudaError_t fill_tables() {
   u64 recip[33];
@@ -552,11 +408,9 @@ static void fill_pool_order(Params& P) {
       if (P.pool[j].type == rank[r]) P.pool_order[k++] = j;
 }
 
-// pools that k_place can take: its per-thread state is a few hundred bytes of shared memory
-static int lane_place_ok(const PoolDev& d) {
-  if (d.type == TG_POOL_API) return 1;
-  if (d.type == TG_POOL_CPU) return d.capacity / d.group <= KPL_DOMAINS && d.group <= 255;
-  return d.n_nodes <= 64;
+// pools whose grants are placed one after the other in queue order with their state in registers
+static int queue_place_ok(const PoolDev& d) {
+  return d.type == TG_POOL_API || (d.type == TG_POOL_CPU && d.capacity / d.group <= 128 && d.group < 65536);
 }
 
 extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_round** out) {
@@ -592,8 +446,7 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     node0 += d.n_nodes;
     d.slot0 = slot0; d.n_slots = pd.type == TANGRAM_POOL_GPU ? 4 : 1;
     slot0 += d.n_slots;
-    d.lane_place = lane_place_ok(d);
-    if (desc->cache_slots > 0 && pd.type == TANGRAM_POOL_GPU) d.lane_place = 0;   // placed by the warp that decides the pool
+    d.queue_place = queue_place_ok(d);
   }
   r->desc.pools = r->pools;
   P.n_nodes_total = node0;
@@ -611,7 +464,7 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   if (e != cudaSuccess) { delete r; return cuda_fail(e, "device set-up"); }
 
   const size_t SN = (size_t)P.S * P.N, SC = (size_t)P.S * P.cand_stride;
-  P.n_workers = prop.multiProcessorCount * 3 * (K2_THREADS / 32);   // what k_solve keeps resident
+  P.n_workers = prop.multiProcessorCount * 2 * (K2_THREADS / 32);   // what k_pool keeps resident
   if ((int64_t)P.n_workers > (int64_t)P.S * P.P) P.n_workers = (int)align_up((size_t)P.S * P.P, K2_THREADS / 32);
   // every worker warp owns a slab that holds the candidate arrays, heaps and small DP tables of
   // the pool it is working on; larger DP tables come from the shared arena
@@ -631,26 +484,11 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   bad |= cudaMalloc(&r->d_slabs, (size_t)P.n_workers * slab) != cudaSuccess;
   bad |= cudaMalloc(&r->d_arena, P.arena_bytes) != cudaSuccess;
   bad |= cudaMalloc(&r->d_arena_top, 256) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->W.ts, (size_t)P.S * P.P * sizeof(TaskState)) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->W.seed2, SC * sizeof(i64)) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->W.rs1, SC) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->W.rs2, SC) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->d_preq, SC * sizeof(unsigned short)) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->d_keepn, (size_t)P.S * P.P * sizeof(int)) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->d_fl, ((size_t)P.S * P.P + 2) * sizeof(int)) != cudaSuccess;
   if (desc->side_costs > 0) {                              // cost vectors: flags and set-aside amounts
     bad |= cudaMalloc((void**)&r->d_side_bad, (size_t)P.S * sizeof(int)) != cudaSuccess;
     bad |= cudaMalloc((void**)&r->d_side_res, (size_t)P.S * P.P * sizeof(int)) != cudaSuccess;
   }
-  const long long n_sims = (long long)P.P * P.S * 2;
-  r->sim_blocks = (int)((n_sims + 31) / 32);
   r->n_sm = prop.multiProcessorCount;
-  r->L.n_groups = (int)((n_sims + SIM_PER_WARP - 1) / SIM_PER_WARP);
-  r->L.n_classes = TG_N_SIM_CLASSES;
-  for (int c = 0; c < TG_N_SIM_CLASSES; ++c) r->L.cap[c] = g_sim_caps[c];
-  bad |= cudaMalloc((void**)&r->L.count, 2 * 64 * sizeof(int)) != cudaSuccess;
-  bad |= cudaMalloc((void**)&r->L.list, (size_t)TG_N_SIM_CLASSES * r->L.n_groups * sizeof(int)) != cudaSuccess;
-  r->L.cursor = r->L.count ? r->L.count + 64 : nullptr;
   if (desc->max_rounds > 0) {                              // state of the trace replay
     ReplayWs& R = r->R;
     int u = 0, d = 0;
@@ -669,21 +507,11 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     bad |= cudaMalloc((void**)&R.pst, (size_t)P.S * P.P * 2 * sizeof(int)) != cudaSuccess;
     bad |= cudaMalloc((void**)&R.win, (size_t)P.S * P.P * sizeof(i64)) != cudaSuccess;
   }
-  bad |= cudaEventCreateWithFlags(&r->sim_fork, cudaEventDisableTiming) != cudaSuccess;
-  for (int c = 0; c <= TG_N_SIM_CLASSES; ++c) {
-    if (c == TG_N_SIM_CLASSES) {
-      // the fill's stream: highest priority, so that its few blocks get in between those of k_stream
-      int lo = 0, hi = 0;
-      bad |= cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess;
-      bad |= cudaStreamCreateWithPriority(&r->sim_stream[c], cudaStreamNonBlocking, hi) != cudaSuccess;
-    } else
-      bad |= cudaStreamCreateWithFlags(&r->sim_stream[c], cudaStreamNonBlocking) != cudaSuccess;
-    bad |= cudaEventCreateWithFlags(&r->sim_join[c], cudaEventDisableTiming) != cudaSuccess;
-  }
   {
+    // the fill's stream: highest priority, so that its few blocks get in between those of k_stream
     int lo = 0, hi = 0;
     bad |= cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess;
-    bad |= cudaStreamCreateWithPriority(&r->side, cudaStreamNonBlocking, lo) != cudaSuccess;
+    bad |= cudaStreamCreateWithPriority(&r->side, cudaStreamNonBlocking, hi) != cudaSuccess;
     bad |= cudaEventCreateWithFlags(&r->side_fork, cudaEventDisableTiming) != cudaSuccess;
     bad |= cudaEventCreateWithFlags(&r->side_join, cudaEventDisableTiming) != cudaSuccess;
   }
@@ -740,17 +568,12 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     P.ok_table = r->d_ok_table;
   }
   P.order = (int*)r->d_order; P.tmin = (i64*)r->d_tmin; P.meta = (PoolMeta*)r->d_meta;
-  P.preq = (unsigned short*)r->d_preq; P.keepn = (int*)r->d_keepn;
   P.n_side = desc->side_costs; P.side_plane = (u64)P.S * P.N;
   P.side_bad = r->d_side_bad; P.side_res = r->d_side_res;
   P.slabs = (char*)r->d_slabs; P.arena = (char*)r->d_arena; P.arena_top = (u64*)r->d_arena_top;
-  e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_DYN_SMEM + (KR_THREADS / 32) * KR_STATE_MAX);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_DYN_SMEM + (KR_THREADS / 32) * KR_STATE_MAX);
-  for (int c = 0; c < TG_N_SIM_CLASSES && e == cudaSuccess; ++c)
-    e = cudaFuncSetAttribute(sim_kernel(g_sim_caps[c]), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TG_SMEM_PER_BLOCK - 1024);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
   *out = r;
   return TANGRAM_OK;
@@ -799,11 +622,10 @@ extern "C" int tangram_kernel_time_ms(tangram_round* r, int kernel, double* tota
 }
 
 // events of the current call, or null when timing is off or the event pool is used up
-static cudaEvent_t* prof_begin(tangram_round* r, int k0, int k1, int k2, int k3, int k4 = -1, int k5 = -1) {
+static cudaEvent_t* prof_begin(tangram_round* r, int k0, int k1, int k2) {
   if (!r->ev || r->ev_used >= TG_PROF_CALLS) return nullptr;
   int c = r->ev_used++;
-  r->ev_kernel[c][0] = k0; r->ev_kernel[c][1] = k1; r->ev_kernel[c][2] = k2; r->ev_kernel[c][3] = k3;
-  r->ev_kernel[c][4] = k4; r->ev_kernel[c][5] = k5;
+  r->ev_kernel[c][0] = k0; r->ev_kernel[c][1] = k1; r->ev_kernel[c][2] = k2;
   return r->ev + c * (TG_PROF_K + 1);
 }
 
@@ -811,9 +633,7 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   if (!r) return;
   if (r->ev) tangram_set_profiling(r, 0);
   cudaFree(r->d_order); cudaFree(r->d_tmin); cudaFree(r->d_meta); cudaFree(r->d_slabs);
-  cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_preq); cudaFree(r->d_keepn); cudaFree(r->d_fl); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_sorted); cudaFree(r->d_perm); cudaFree(r->d_wkey);
-  cudaFree(r->W.ts); cudaFree(r->W.seed2); cudaFree(r->W.rs1); cudaFree(r->W.rs2);
-  cudaFree(r->L.count); cudaFree(r->L.list);
+  cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_sorted); cudaFree(r->d_perm); cudaFree(r->d_wkey);
   cudaFree(r->R.wait); cudaFree(r->R.run); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.dfree);
   cudaFree(r->R.pst); cudaFree(r->R.win);
   if (r->io_in) cudaStreamDestroy(r->io_in);
@@ -828,11 +648,6 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   if (r->side) cudaStreamDestroy(r->side);
   if (r->side_fork) cudaEventDestroy(r->side_fork);
   if (r->side_join) cudaEventDestroy(r->side_join);
-  if (r->sim_fork) cudaEventDestroy(r->sim_fork);
-  for (int c = 0; c <= TG_N_SIM_CLASSES; ++c) {
-    if (r->sim_stream[c]) cudaStreamDestroy(r->sim_stream[c]);
-    if (r->sim_join[c]) cudaEventDestroy(r->sim_join[c]);
-  }
   delete r;
 }
 
@@ -896,10 +711,7 @@ static void bind_device_io(Params& P, const tangram_actions* a, const tangram_re
 }
 
 // The kernels of one round for the scenarios that P describes, on stream st.
-static int run_pipeline(tangram_round* r, const Params& P, const BatchWs& W, const SimLists& L, cudaStream_t st,
-                        cudaEvent_t* ev) {
-  const int wblocks = P.n_workers / (K2_THREADS / 32);
-  const long long n_sims = (long long)P.P * P.S * 2;
+static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, cudaEvent_t* ev) {
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));          // arena top and the task counters
   if (ev) CK(cudaEventRecord(ev[0], st));
   if (P.n_side > 0) {
@@ -912,61 +724,20 @@ static int run_pipeline(tangram_round* r, const Params& P, const BatchWs& W, con
   if (P.n_side > 0) k_head<true><<<(P.S + 7) / 8, 256, 0, st>>>(P, r->hst);
   else k_head<false><<<(P.S + 7) / 8, 256, 0, st>>>(P, r->hst);
   if (ev) CK(cudaEventRecord(ev[1], st));
-  const unsigned place_grid = ((P.S + 31) / 32 * P.P + KPL_WARPS - 1) / KPL_WARPS;
   {                                                        // the output fill runs beside everything that follows
-    cudaStream_t fs = r->sim_stream[TG_N_SIM_CLASSES];
-    CK(cudaEventRecord(r->sim_fork, st));
-    CK(cudaStreamWaitEvent(fs, r->sim_fork, 0));
-    size_t blocks = ((size_t)P.S * ((P.N + 3) / 4) + 255) / 256;
-    if (blocks > (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM) blocks = (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM;
-    k_fill<<<(unsigned)blocks, 256, 0, fs>>>(P, r->hst);
-    CK(cudaEventRecord(r->sim_join[TG_N_SIM_CLASSES], fs));
-  }
-  // k_solve needs only what k_head left and could run beside k_stream; measured, the two get in each
-  // other's way on the SMs (1.6 ms together against 0.65 + 0.70 one after the other), so they do not
-  k_stream<<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
-  if (ev) CK(cudaEventRecord(ev[2], st));
-  k_solve<<<wblocks, K2_THREADS, K2_DYN_SMEM, st>>>(P, W, r->hst);
-  if (ev) CK(cudaEventRecord(ev[3], st));
-  CK(cudaMemsetAsync(L.count, 0, 2 * 64 * sizeof(int), st));
-  k_sim_classify<<<(L.n_groups + 7) / 8, 256, 0, st>>>(P, W.ts, L);
-  CK(cudaEventRecord(r->sim_fork, st));
-  for (int c = 0; c < TG_N_SIM_CLASSES; ++c) {
-    cudaStream_t ss = r->sim_stream[c];
-    CK(cudaStreamWaitEvent(ss, r->sim_fork, 0));
-    const int smem = sim_smem_bytes(g_sim_caps[c]);
-    int per_sm = TG_SMEM_PER_SM / (smem + 1024);
-    if (per_sm > 32) per_sm = 32;
-    if (per_sm < 1) per_sm = 1;
-    int grid = r->n_sm * per_sm;
-    if (grid > L.n_groups) grid = L.n_groups;
-    sim_kernel(g_sim_caps[c])<<<grid, 32, smem, ss>>>(P, W.ts, W.seed2, L, c);
-    CK(cudaEventRecord(r->sim_join[c], ss));
-    CK(cudaStreamWaitEvent(st, r->sim_join[c], 0));
-  }
-  k_sims_big<<<(int)((n_sims + 31) / 32), 32, 0, st>>>(P, W.ts, W.seed2, g_sim_caps[TG_N_SIM_CLASSES - 1], L.count + 63);
-  if (ev) CK(cudaEventRecord(ev[4], st));
-  {                                                        // the certified pools: decided and placed beside the continued evictions,
-                                                           // which are chains of dependent steps that leave most of the machine idle
     CK(cudaEventRecord(r->side_fork, st));
     CK(cudaStreamWaitEvent(r->side, r->side_fork, 0));
-    k_easy<<<(unsigned)(((size_t)P.S * P.P + 7) / 8), 256, 0, r->side>>>(P, r->hst);
-    k_place<<<place_grid, KPL_THREADS, 0, r->side>>>(P, r->hst, 0, 0);
+    size_t blocks = ((size_t)P.S * ((P.N + 3) / 4) + 255) / 256;
+    if (blocks > (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM) blocks = (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM;
+    k_fill<<<(unsigned)blocks, 256, 0, r->side>>>(P, r->hst);
     CK(cudaEventRecord(r->side_join, r->side));
   }
-  CK(cudaMemsetAsync(r->d_fl, 0, 2 * sizeof(int), st));
-  k_finish_list<<<(P.S * P.P + 255) / 256, 256, 0, st>>>(P, W, r->d_fl);
-  k_finish<<<wblocks, K2_THREADS, K2_DYN_SMEM, st>>>(P, W, r->d_fl);
-  if (ev) CK(cudaEventRecord(ev[5], st));
-  // A warp per GPU pool is the shorter chain as long as all those warps are resident at once; beyond
-  // that a thread per pool (32 pools per warp instruction) gets through the batch sooner.
-  const int gpu_apart = (long long)P.S * P.P <= (long long)r->n_sm * 64 * 2 ? 1 : 0;
-  k_place<<<place_grid, KPL_THREADS, 0, st>>>(P, r->hst, 1, gpu_apart);
-  if (gpu_apart) k_place_gpu<<<(unsigned)(((size_t)P.S * P.P + 7) / 8), 256, 0, st>>>(P, r->hst);
-  CK(cudaStreamWaitEvent(st, r->side_join, 0));
-  CK(cudaStreamWaitEvent(st, r->sim_join[TG_N_SIM_CLASSES], 0));   // the fill is part of the round
-  if (ev) CK(cudaEventRecord(ev[6], st));
-  r->launches += 11 + TG_N_SIM_CLASSES + gpu_apart;
+  k_stream<<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
+  if (ev) CK(cudaEventRecord(ev[2], st));
+  k_pool<<<P.n_workers / (K2_THREADS / 32), K2_THREADS, K2_DYN_SMEM, st>>>(P, r->hst);
+  CK(cudaStreamWaitEvent(st, r->side_join, 0));            // the fill is part of the round
+  if (ev) CK(cudaEventRecord(ev[3], st));
+  r->launches += 4;
   CK(cudaGetLastError());
   return TANGRAM_OK;
 }
@@ -981,7 +752,7 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   P.now = now_us;
   if (!r->desc.host_buffers) {
     bind_device_io(P, a, res);
-    return run_pipeline(r, P, r->W, r->L, st, prof_begin(r, 0, 7, 3, 4, 5, 6));
+    return run_pipeline(r, P, st, prof_begin(r, 0, 4, 3));
   }
   bind_stage(r, a, P);
   // Host buffers: scenarios go through in chunks, so that the copy-in of a chunk, the kernels
@@ -992,7 +763,7 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   if (C > P.S) C = P.S;
   if (C <= 1 || r->ev) {                                   // small batch, or per-kernel timing wanted
     int rc = copy_in(r, a, P, 0, P.S, st);
-    if (!rc) rc = run_pipeline(r, P, r->W, r->L, st, prof_begin(r, 0, 7, 3, 4, 5, 6));
+    if (!rc) rc = run_pipeline(r, P, st, prof_begin(r, 0, 4, 3));
     if (!rc) rc = copy_out(r, res, P, 0, P.S, st);
     return rc;
   }
@@ -1015,10 +786,8 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
     Q.o_alloc += o; Q.o_node += o; Q.o_off += o; Q.o_act += o;
     Q.o_total += s0; Q.o_nsel += s0; Q.o_status += s0;
     if ((int64_t)Q.n_workers > (int64_t)Q.S * P.P) Q.n_workers = (int)align_up((size_t)Q.S * P.P, K2_THREADS / 32);
-    SimLists L = r->L;
-    L.n_groups = (int)(((long long)P.P * Q.S * 2 + SIM_PER_WARP - 1) / SIM_PER_WARP);
     CK(cudaStreamWaitEvent(r->io_comp, r->io_in_done[c], 0));
-    rc = run_pipeline(r, Q, r->W, L, r->io_comp, nullptr);   // the workspace is reused chunk after chunk
+    rc = run_pipeline(r, Q, r->io_comp, nullptr);   // the workspace is reused chunk after chunk
     if (rc) return rc;
     CK(cudaEventRecord(r->io_comp_done[c], r->io_comp));
     CK(cudaStreamWaitEvent(r->io_out, r->io_comp_done[c], 0));
@@ -1082,7 +851,7 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
   }
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));
   int warps = P.n_workers < P.S ? P.n_workers : (int)align_up((size_t)P.S, K2_THREADS / 32);
-  cudaEvent_t* ev = prof_begin(r, 2, -1, -1, -1);
+  cudaEvent_t* ev = prof_begin(r, 2, -1, -1);
   if (ev) CK(cudaEventRecord(ev[0], st));
   {
     // a scenario's live state (owner of every unit, node masks, free cores per domain, quota counters) goes to
@@ -1196,7 +965,7 @@ extern "C" int tangram_schedule_batch_ordered(tangram_round* r, const tangram_ac
   Params Q = P;
   Q.a_pool = G.pool; Q.a_unit = G.unit; Q.a_mask = G.mask; Q.a_s = G.s; Q.a_p = G.p; Q.a_arrival = G.arrival;
   Q.o_alloc = (int*)(d + off_alloc); Q.o_node = (int*)(d + off_node); Q.o_off = (int*)(d + off_off); Q.o_act = (i64*)(d + off_act);
-  rc = run_pipeline(r, Q, r->W, r->L, st, nullptr);
+  rc = run_pipeline(r, Q, st, nullptr);
   if (rc) return rc;
   ScatterIo X;
   X.perm = r->d_perm; X.alloc = Q.o_alloc; X.node = Q.o_node; X.off = Q.o_off; X.act = Q.o_act;
