@@ -1022,12 +1022,58 @@ __device__ __forceinline__ i64 small_answer(const PoolTask& T, int nrows, int y,
   return bv;
 }
 
+// Two or three candidates: all combinations of their levels, one per lane (a replay's rounds seldom have more).
+#define FEW_MAX 3
+__device__ __forceinline__ bool solve_few(PoolTask& T0, int q, int lane) {
+  const int type = T0.type;
+  u32 mk[FEW_MAX]; i64 s[FEW_MAX], p[FEW_MAX]; int cg[FEW_MAX], nl[FEW_MAX], total = 1;
+#pragma unroll
+  for (int i = 0; i < FEW_MAX; ++i) {
+    mk[i] = i < q ? T0.cmask[i] : 1u; s[i] = i < q ? T0.cs[i] : 0; p[i] = i < q ? T0.cp[i] : 0; cg[i] = i < q ? (int)T0.cg[i] : 0;
+    nl[i] = __popc(mk[i]); total *= nl[i];
+  }
+  if (total > 256) return false;
+  i64 bv = TG_INF; int bu = INT_MAX; u32 bs = 0;
+#pragma unroll 1
+  for (int c = lane; c < total; c += 32) {
+    int rest = c, dem[4] = {0, 0, 0, 0};
+    i64 v = 0; u32 seq = 0;
+#pragma unroll
+    for (int i = 0; i < FEW_MAX; ++i) {
+      const int d = rest % nl[i];
+      rest /= nl[i];
+      u32 mm = mk[i];
+#pragma unroll 1
+      for (int k = 0; k < d; ++k) mm &= mm - 1;
+      const int r = __ffs(mm), g = cg[i] & 0x7f, cl = class_of(type, max(g, 1), cg[i] >> 7, r);
+#pragma unroll
+      for (int l = 0; l < 4; ++l) if (l <= cl) dem[l] += g * r;
+      v += duration(s[i], p[i], r);
+      seq |= (u32)r << (6 * i);                          // (a later candidate counts more)
+    }
+    bool fit = dem[0] <= T0.cap[0];
+    if (type == TG_POOL_GPU) {
+#pragma unroll
+      for (int l = 1; l < 4; ++l) fit &= dem[l] <= T0.cap[l];
+    }
+    if (fit && (v < bv || (v == bv && (dem[0] < bu || (dem[0] == bu && seq < bs))))) { bv = v; bu = dem[0]; bs = seq; }
+  }
+  const i64 v = warp_min64(bv);
+  const int u = warp_min32(bv == v ? bu : INT_MAX);
+  const u32 w = __reduce_min_sync(TG_FULL, bv == v && bu == u ? bs : 0xffffffffu);
+  if (lane < q) T0.rsel[lane] = (u8)((w >> (6 * lane)) & 63u);
+  if (lane == 0) T0.opt = v;
+  __syncwarp();
+  return v != TG_INF;
+}
+
 // Optimal allocation of candidates [0, q) -> T.rsel[0..q), duration sum -> T.opt.  Prefixes are asked for in descending
 // order.
 #define SOLVED_ALL_BEST 2   // every candidate got its best level (then so does every shorter prefix)
 #define SOLVED 1
 #define UNSOLVED 0          // the workspace is too small
 __device__ __noinline__ int solve_prefix(const Params& P, PoolTask& T0, int q, Slab slab, int lane) {
+  if (q <= FEW_MAX && solve_few(T0, q, lane)) return SOLVED;
   PoolTask T;                                            // (what is used of it, in registers)
   T.type = T0.type; T.cs = T0.cs; T.cp = T0.cp; T.cmask = T0.cmask; T.cg = T0.cg; T.rsel = T0.rsel; T.rowcand = T0.rowcand;
   T.wk = T0.wk; T.wk_bytes = T0.wk_bytes;

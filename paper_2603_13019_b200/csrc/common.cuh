@@ -69,8 +69,6 @@ struct Params {
 // ceil(2^64 / r) for r = 2..32: floor(p / r) == umul64hi(p, c_recip[r]) for 0 <= p <= 2^40,
 // because the rounding excess p * (r - 2^64 mod r) / (r * 2^64) stays below 2^-24 < 1/r.
 __constant__ u64 c_recip[33];
-// maximal free aligned blocks of a node, indexed by its busy mask: byte l = blocks of size 2^l
-__constant__ u32 c_fblocks[256];
 
 __device__ __forceinline__ i64 div_small(i64 p, int r) {
   return r == 1 ? p : (i64)__umul64hi((u64)p, c_recip[r]);
@@ -139,15 +137,39 @@ __device__ __forceinline__ int warp_sum32(int v) { return (int)__reduce_add_sync
 __device__ __forceinline__ int warp_min32(int v) { return __reduce_min_sync(TG_FULL, v); }
 __device__ __forceinline__ int warp_max32(int v) { return __reduce_max_sync(TG_FULL, v); }
 
+// maximal free aligned blocks of a node: bit = first GPU of such a block (busy: 8 bits, padded)
+struct NodeBlocks { u32 s1, s2, s4, s8; };
+__device__ __forceinline__ NodeBlocks node_blocks(u32 busy) {
+  const u32 fr = ~busy & 0xffu;
+  const u32 pr = fr & (fr >> 1) & 0x55u;          // bit 2k: GPUs 2k, 2k+1 free
+  const u32 nb = pr & (pr >> 2) & 0x11u;          // bit 4k: GPUs 4k .. 4k+3 free
+  const u32 oc = nb & (nb >> 4) & 1u;             // the whole node free
+  NodeBlocks b;
+  b.s1 = fr & ~(pr | (pr << 1));
+  b.s2 = pr & ~(nb | (nb << 2));
+  b.s4 = nb & ~(oc | (oc << 4));
+  b.s8 = oc;
+  return b;
+}
+__device__ __forceinline__ u32 node_levels(u32 busy) {   // bit l: a maximal free block of 2^l GPUs exists
+  const NodeBlocks b = node_blocks(busy);
+  return (b.s1 ? 1u : 0u) | (b.s2 ? 2u : 0u) | (b.s4 ? 4u : 0u) | (b.s8 ? 8u : 0u);
+}
+__device__ __forceinline__ int node_block_start(u32 busy, int bl) {
+  const NodeBlocks b = node_blocks(busy);
+  const u32 m = bl == 0 ? b.s1 : (bl == 1 ? b.s2 : (bl == 2 ? b.s4 : b.s8));
+  return __ffs(m) - 1;
+}
+
 // Free capacity per chunk level of a GPU pool: cap[l] = GPUs held in maximal free aligned
 // blocks of size >= 2^l.  `busy` may be null (all free).  Warp-cooperative.
 __device__ __forceinline__ void gpu_caps(const PoolDev& pd, const u8* busy, int lane, int cap[4]) {
   int F0 = 0, F1 = 0, F2 = 0, F3 = 0;
-  u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;   // GPUs beyond the node size count as busy
+  const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;   // GPUs beyond the node size count as busy
+#pragma unroll 1
   for (int v = lane; v < pd.n_nodes; v += 32) {
-    u32 b = (busy ? busy[pd.node0 + v] : 0u) | pad;
-    u32 f = c_fblocks[b & 0xffu];
-    F0 += f & 0xff; F1 += (f >> 8) & 0xff; F2 += (f >> 16) & 0xff; F3 += f >> 24;
+    const NodeBlocks b = node_blocks((busy ? busy[pd.node0 + v] : 0u) | pad);
+    F0 += __popc(b.s1); F1 += __popc(b.s2); F2 += __popc(b.s4); F3 += __popc(b.s8);
   }
   F0 = warp_sum32(F0); F1 = warp_sum32(F1); F2 = warp_sum32(F2); F3 = warp_sum32(F3);
   cap[3] = F3 * 8; cap[2] = cap[3] + F2 * 4; cap[1] = cap[2] + F1 * 2; cap[0] = cap[1] + F0;

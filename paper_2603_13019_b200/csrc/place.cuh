@@ -47,7 +47,7 @@ __device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, con
 #pragma unroll 1
           for (int v0 = 0; v0 < pd.n_nodes; v0 += 32) {
             int v = v0 + lane;
-            bool has = v < pd.n_nodes && ((c_fblocks[nm[v] | pad] >> (8 * bl)) & 0xffu) != 0;
+            bool has = v < pd.n_nodes && ((node_levels(nm[v] | pad) >> bl) & 1u) != 0;
             u32 b = __ballot_sync(TG_FULL, has);
             if (b) { node = v0 + __ffs(b) - 1; start = find_block(nm[node] | pad, bl, pd.group); break; }
           }
@@ -62,40 +62,6 @@ __device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, con
         __syncwarp();
       }
     }
-  }
-}
-
-// busy: one bit per core (word array); dfree: free cores per domain.  Both updated.
-__device__ void place_cpu(const PoolDev& pd, u32* busy, int* dfree, int keep, const u8* cg,
-                          const u8* r, int* pnode, int* poff, int lane) {
-  const int D = pd.capacity / pd.group;
-#pragma unroll 1
-  for (int i = 0; i < keep; ++i) {
-    const int k = (cg[i] & 0x7f) * r[i];
-    i64 key = TG_INF;
-#pragma unroll 1
-    for (int d = lane; d < D; d += 32) {
-      int f = dfree[d];
-      if (f >= k) key = min(key, ((i64)f << 32) | d);
-    }
-    key = warp_min64(key);
-    if (lane == 0) {
-      int lo = 0, hi = pd.capacity;
-      if (key != TG_INF) { int d = (int)(key & 0xffffffff); lo = d * pd.group; hi = lo + pd.group; }
-      int need = k, first = -1;
-#pragma unroll 1
-      for (int c = lo; c < hi && need > 0; ++c) {
-        u32 w = busy[c >> 5];
-        if (w == 0xffffffffu && (c & 31) == 0 && c + 32 <= hi) { c += 31; continue; }
-        if (w >> (c & 31) & 1u) continue;
-        busy[c >> 5] = w | (1u << (c & 31));
-        dfree[c / pd.group] -= 1;
-        if (first < 0) first = c;
-        --need;
-      }
-      pnode[i] = first >= 0 ? first / pd.group : -1; poff[i] = first;
-    }
-    __syncwarp();
   }
 }
 
@@ -147,67 +113,9 @@ __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u
   }
 }
 
-// CPU placement on a pool with cores in use (trace replay): owner[c] < 0 marks a free core,
-// dfree the free cores per domain.  Same rule as place_cpu; a grant writes ids[i] into owner.
-__device__ void place_cpu_owner(const PoolDev& pd, int* owner, int* dfree, int keep, const u8* cg,
-                                const u8* r, const int* ids, int* pnode, int* poff, int lane) {
-  const int D = pd.capacity / pd.group;
-#pragma unroll 1
-  for (int i = 0; i < keep; ++i) {
-    const int k = (cg[i] & 0x7f) * r[i];
-    i64 key = TG_INF;
-#pragma unroll 1
-    for (int d = lane; d < D; d += 32) {
-      int f = dfree[d];
-      if (f >= k) key = min(key, ((i64)f << 32) | d);
-    }
-    key = warp_min64(key);
-    int lo = 0, hi = pd.capacity;
-    if (key != TG_INF) { int d = (int)(key & 0xffffffff); lo = d * pd.group; hi = lo + pd.group; }
-    // lowest free cores of [lo, hi): 32 cores per pass, each lane claims by its rank among the free
-    int need = k, first = -1;
-#pragma unroll 1
-    for (int c0 = lo; c0 < hi && need > 0; c0 += 32) {
-      const int c = c0 + lane;
-      const bool fr = c < hi && owner[c] < 0;
-      const u32 b = __ballot_sync(TG_FULL, fr);
-      const int rank = __popc(b & ((1u << lane) - 1u));
-      if (fr && rank < need) { owner[c] = ids[i]; atomicSub(&dfree[c / pd.group], 1); }
-      if (b && first < 0) first = c0 + __ffs(b) - 1;
-      need -= min(need, __popc(b));
-    }
-    if (lane == 0) { pnode[i] = first >= 0 ? first / pd.group : -1; poff[i] = first; }
-    __syncwarp();
-  }
-}
-
 // ---- register-resident fast paths of a single round (fresh CPU pool, at most 128 domains /
 // ---- GPU nodes): the state lives in lane registers, the arg-min is one redux, and every lane
 // ---- keeps the result of "its" candidate of a block of 32 for a coalesced write.
-
-// maximal free aligned blocks of a node: bit = first GPU of such a block (busy: 8 bits, padded)
-struct NodeBlocks { u32 s1, s2, s4, s8; };
-__device__ __forceinline__ NodeBlocks node_blocks(u32 busy) {
-  const u32 fr = ~busy & 0xffu;
-  const u32 pr = fr & (fr >> 1) & 0x55u;          // bit 2k: GPUs 2k, 2k+1 free
-  const u32 nb = pr & (pr >> 2) & 0x11u;          // bit 4k: GPUs 4k .. 4k+3 free
-  const u32 oc = nb & (nb >> 4) & 1u;             // the whole node free
-  NodeBlocks b;
-  b.s1 = fr & ~(pr | (pr << 1));
-  b.s2 = pr & ~(nb | (nb << 2));
-  b.s4 = nb & ~(oc | (oc << 4));
-  b.s8 = oc;
-  return b;
-}
-__device__ __forceinline__ u32 node_levels(u32 busy) {   // bit l: a maximal free block of 2^l GPUs exists
-  const NodeBlocks b = node_blocks(busy);
-  return (b.s1 ? 1u : 0u) | (b.s2 ? 2u : 0u) | (b.s4 ? 4u : 0u) | (b.s8 ? 8u : 0u);
-}
-__device__ __forceinline__ int node_block_start(u32 busy, int bl) {
-  const NodeBlocks b = node_blocks(busy);
-  const u32 m = bl == 0 ? b.s1 : (bl == 1 ? b.s2 : (bl == 2 ? b.s4 : b.s8));
-  return __ffs(m) - 1;
-}
 
 // GPU placement with a service cache (Section 5.3, evict on execution).  The rule of place_gpu, and among
 // the free blocks of the level it picks, one whose granted chunk (the block's low end) caches the

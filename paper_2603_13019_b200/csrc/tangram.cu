@@ -19,6 +19,8 @@
 #define TG_PROF_CALLS 256   // calls whose kernels can be timed between two queries
 #define TG_FILL_BLOCKS_PER_SM 4   // k_fill is a trickle beside the other kernels, not a flood
 #define TG_IO_CHUNKS 16
+#define TG_SMEM_PER_SM 233472   // shared memory an SM can split among resident blocks
+#define TG_REPLAY_SMEM 114688    // a replay block takes at most that much (the rest of the SM's is L1)
 #define TG_PROF_K 3         // timed intervals per call at most
 #define TG_N_KERNELS 8
 
@@ -339,7 +341,7 @@ struct tangram_round {
   void* d_order; void* d_tmin; void* d_meta; void* d_slabs; void* d_arena; void* d_arena_top;
   HeadState* hst; u32* d_ok_table; int* d_side_bad; int* d_side_res;
   int n_sm;
-  ReplayWs R;
+  ReplayWs R; int replay_smem;
   // host-buffer mode: copy-in, kernels and copy-out of successive chunks on streams of their own
   cudaStream_t io_in, io_comp, io_out;
   cudaEvent_t io_begin, io_end, io_in_done[TG_IO_CHUNKS], io_comp_done[TG_IO_CHUNKS];
@@ -362,24 +364,7 @@ static cudaError_t fill_tables() {
   recip[0] = recip[1] = 0;
   // ceil(2^64 / r) = floor((2^64 - 1) / r) + 1 for every r >= 2
   for (int r = 2; r <= 32; ++r) recip[r] = 0xffffffffffffffffull / (u64)r + 1ull;
-  u32 fb[256];
-  for (int b = 0; b < 256; ++b) {
-    int F[4] = {0, 0, 0, 0};
-    // maximal free aligned blocks of an 8-GPU node with busy mask b
-    if (b == 0) F[3] = 1;
-    else
-      for (int h = 0; h < 8; h += 4) {
-        if (((b >> h) & 0xf) == 0) { F[2]++; continue; }
-        for (int q = h; q < h + 4; q += 2) {
-          if (((b >> q) & 0x3) == 0) { F[1]++; continue; }
-          for (int s = q; s < q + 2; ++s) if (!((b >> s) & 1)) F[0]++;
-        }
-      }
-    fb[b] = (u32)F[0] | ((u32)F[1] << 8) | ((u32)F[2] << 16) | ((u32)F[3] << 24);
-  }
-  cudaError_t e = cudaMemcpyToSymbol(c_recip, recip, sizeof(recip));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_fblocks, fb, sizeof(fb));
-  return e;
+  return cudaMemcpyToSymbol(c_recip, recip, sizeof(recip));
 }
 
 extern "C" const char* tangram_strerror(int code) {
@@ -500,7 +485,33 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     R.U = u ? u : 1; R.Dtot = d ? d : 1;
     R.round_us = desc->round_us > 0 ? desc->round_us : 1; R.max_rounds = desc->max_rounds;
     bad |= cudaMalloc((void**)&R.wait, SN * sizeof(int)) != cudaSuccess;
-    bad |= cudaMalloc((void**)&R.run, SN * sizeof(int)) != cudaSuccess;
+    // what a block (one scenario at a time) keeps in shared memory: live state, running actions, waiting records
+    {
+      const size_t state = align16((size_t)R.U * 4) + align16((size_t)node0 + 1) + align16((size_t)R.Dtot * 4) + 2 * align16((size_t)P.P * 8);
+      R.state_bytes = state <= KR_STATE_MAX ? (int)state : 0;
+      size_t running = 0;                                  // a running action holds a unit at least, quota calls aside
+      for (int j = 0; j < P.P; ++j) running += P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0 ? (size_t)P.N : (size_t)P.pool[j].capacity;
+      running = align_up(running < (size_t)P.N ? running : (size_t)P.N, 8);
+      size_t per_sm = ((size_t)P.S + r->n_sm - 1) / r->n_sm;
+      if (per_sm > 6) per_sm = 6;
+      size_t room = (size_t)TG_SMEM_PER_SM / per_sm - 1024;
+      if (room > TG_REPLAY_SMEM) room = TG_REPLAY_SMEM;
+      size_t left = room - KR_BASE_BYTES - (size_t)R.state_bytes;
+      R.rcap = running * KR_RUN_BYTES <= left / 2 ? (int)running : 0;
+      left -= (size_t)R.rcap * KR_RUN_BYTES;
+      size_t wc = left / KR_WAIT_BYTES;
+      if (wc > 2048) wc = 2048;
+      if (wc > align_up((size_t)P.N, 32)) wc = align_up((size_t)P.N, 32);
+      R.wcap = (int)(wc / 32 * 32);
+      r->replay_smem = KR_BASE_BYTES + R.state_bytes + (int)align16((size_t)R.rcap * KR_RUN_BYTES) + (int)align16((size_t)R.wcap * KR_WAIT_BYTES);
+      if (R.rcap == 0) {
+        bad |= cudaMalloc((void**)&R.run_fin, SN * sizeof(i64)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_idx, SN * sizeof(int)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_pu, SN * sizeof(u32)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_off, SN * sizeof(int)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_dom, SN * sizeof(int)) != cudaSuccess;
+      }
+    }
     bad |= cudaMalloc((void**)&R.owner, (size_t)P.S * R.U * sizeof(int)) != cudaSuccess;
     bad |= cudaMalloc((void**)&R.nm, (size_t)P.S * (node0 ? node0 : 1)) != cudaSuccess;
     bad |= cudaMalloc((void**)&R.dfree, (size_t)P.S * R.Dtot * sizeof(int)) != cudaSuccess;
@@ -572,8 +583,8 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   P.side_bad = r->d_side_bad; P.side_res = r->d_side_res;
   P.slabs = (char*)r->d_slabs; P.arena = (char*)r->d_arena; P.arena_top = (u64*)r->d_arena_top;
   e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_DYN_SMEM + (KR_THREADS / 32) * KR_STATE_MAX);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_DYN_SMEM + (KR_THREADS / 32) * KR_STATE_MAX);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
   *out = r;
   return TANGRAM_OK;
@@ -634,7 +645,7 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   if (r->ev) tangram_set_profiling(r, 0);
   cudaFree(r->d_order); cudaFree(r->d_tmin); cudaFree(r->d_meta); cudaFree(r->d_slabs);
   cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_sorted); cudaFree(r->d_perm); cudaFree(r->d_wkey);
-  cudaFree(r->R.wait); cudaFree(r->R.run); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.dfree);
+  cudaFree(r->R.wait); cudaFree(r->R.run_fin); cudaFree(r->R.run_idx); cudaFree(r->R.run_pu); cudaFree(r->R.run_off); cudaFree(r->R.run_dom); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.dfree);
   cudaFree(r->R.pst); cudaFree(r->R.win);
   if (r->io_in) cudaStreamDestroy(r->io_in);
   if (r->io_comp) cudaStreamDestroy(r->io_comp);
@@ -850,16 +861,9 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
     R.occupancy = res->occupancy; R.rounds_used = res->rounds_used;
   }
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));
-  int warps = P.n_workers < P.S ? P.n_workers : (int)align_up((size_t)P.S, K2_THREADS / 32);
+  const int blocks = P.n_workers < P.S ? P.n_workers : P.S;
   cudaEvent_t* ev = prof_begin(r, 2, -1, -1);
   if (ev) CK(cudaEventRecord(ev[0], st));
-  {
-    // a scenario's live state (owner of every unit, node masks, free cores per domain, quota counters) goes to
-    // shared memory when it is small
-    const size_t need = align16((size_t)R.U * 4) + align16((size_t)P.n_nodes_total + 1) + align16((size_t)R.Dtot * 4) +
-                        2 * align16((size_t)P.P * 8);
-    R.state_bytes = need <= KR_STATE_MAX ? (int)need : 0;
-  }
   if (pin) {
     // the kernel reads and rewrites the caller's pool_out: it starts as a copy of the pool column
     CK(cudaMemcpyAsync(pin->pool_out, a->pool, (size_t)P.S * P.N, cudaMemcpyDeviceToDevice, st));
@@ -868,8 +872,8 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
     R.max_traj = pin->max_trajectories; R.traj_node = pin->traj_node; R.mem_free = (i64*)pin->node_mem_free;
     R.pool_rw = pin->pool_out;
   }
-  if (policy || pin) k_replay<true><<<warps / (KR_THREADS / 32), KR_THREADS, KR_DYN_SMEM + (KR_THREADS / 32) * R.state_bytes, st>>>(P, R);
-  else k_replay<false><<<warps / (KR_THREADS / 32), KR_THREADS, KR_DYN_SMEM + (KR_THREADS / 32) * R.state_bytes, st>>>(P, R);
+  if (policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0)) k_replay<true><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
+  else k_replay<false><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   if (ev) CK(cudaEventRecord(ev[1], st));
   r->launches += 1;
   CK(cudaGetLastError());
