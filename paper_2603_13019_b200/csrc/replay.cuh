@@ -100,15 +100,6 @@ __device__ __forceinline__ u32 replay_meta(const Params& P, const ReplayQueue& Q
   return replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], 0, 0).meta;
 }
 
-// ceil(t / d) for 0 <= t < 2^52 by a reciprocal, corrected
-__device__ __forceinline__ i64 replay_ceil_div(i64 t, i64 d, double inv) {
-  i64 q = (i64)((double)t * inv);
-  q += q * d < t ? 1 : 0;
-  q += q * d < t ? 1 : 0;
-  q -= (q - 1) * d >= t ? 1 : 0;
-  return q;
-}
-
 // Live state of the scenario at hand: in the warp's shared memory, or in the arrays of ReplayWs where it is large.
 struct ReplayState { int* owner; u8* nm; int* dfree; int* pst; i64* win; };
 
@@ -349,9 +340,10 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       bool drained = false, gated = false;                 // gated: an arrival waits for a node (Section 5.2)
       i64 total = 0; int selected = 0;
       i64 min_fin = TG_INF;                                // earliest completion among what runs
-      const double inv_round = 1.0 / (double)R.round_us;
-      auto round_of = [&](i64 t) -> i64 {                  // first round at or after time t
-        return t < (1ll << 52) ? replay_ceil_div(t, R.round_us, inv_round) : (t - 1) / R.round_us + 1;
+      // first round at or after time t > now_t, the time of round r_t (a 32-bit division where the distance allows)
+      auto round_after = [&](i64 t, i64 now_t, int r_t) -> i64 {
+        const i64 d = max(t - now_t, 1ll);
+        return d <= 0xffffffffll && R.round_us <= 0xffffffffll ? (i64)r_t + (i64)(((u32)d - 1u) / (u32)R.round_us + 1u) : (i64)r_t + (d - 1) / R.round_us + 1;
       };
       // arrivals, 32 at a time: lane k holds record base + k
       int base = -32;
@@ -374,6 +366,8 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       int capreg = 0;                                      // lane v: free capacity of demand slot v
       u32 stale = ~0u;                                     // pools whose slots have to be worked out again
       bool windows = false;
+      // lane j: where pool j's units in use are counted if it is a quota / concurrency pool, else -1
+      const int api_at = lane < P.P && P.pool[lane].type == TG_POOL_API ? lane * 2 + (P.pool[lane].window_us > 0 ? 0 : 1) : -1;
 #pragma unroll 1
       for (int j = 0; j < P.P; ++j) windows |= P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0;
       while (r < R.max_rounds) {
@@ -800,7 +794,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         }
         // 5. occupancy of this round: lane j holds pool j's
         int in_use = busy;
-        if (lane < P.P && P.pool[lane].type == TG_POOL_API) in_use = Z.pst[lane * 2 + (P.pool[lane].window_us > 0 ? 0 : 1)];
+        if (api_at >= 0) in_use = Z.pst[api_at];
         if (occ && lane < P.P) occ[(size_t)r * P.P + lane] = in_use;
         ++r;
         if (next == n_act && nw == 0 && nr == 0) { drained = true; break; }
@@ -836,14 +830,15 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         }
         if (jump) {
           int r_next = R.max_rounds;
-          if (t_next < now + (i64)(R.max_rounds - r + 1) * R.round_us) r_next = min(r_next, (int)round_of(t_next));
+          if (t_next <= now) r_next = r;
+          else if (t_next < now + (i64)(R.max_rounds - r + 1) * R.round_us) r_next = min(r_next, (int)round_after(t_next, now, r - 1));
           if (r_next > r) {
             if (occ) {
               if (lane < P.P) {
                 // (this lane's pool; its usage restarts with its window)
                 int turn = r_next;
-                if (windows && P.pool[lane].type == TG_POOL_API && P.pool[lane].window_us > 0) {
-                  const i64 tr = round_of((Z.win[lane] + 1) * (i64)P.pool[lane].window_us);
+                if (windows && api_at >= 0 && !(api_at & 1)) {
+                  const i64 tr = round_after((Z.win[lane] + 1) * (i64)P.pool[lane].window_us, now, r - 1);
                   if (tr < (i64)turn) turn = (int)tr;
                 }
                 int* at = occ + (size_t)r * P.P + lane;
@@ -859,7 +854,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                   const u32 pu = run.pu[i];
                   const int j = (int)(pu >> 24);
                   if (P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0) continue;      // used quota is not given back
-                  const int fr = max(r, (int)round_of(fin));
+                  const int fr = max(r, (int)round_after(fin, now, r - 1));
 #pragma unroll 1
                   for (int rr = fr; rr < r_next; ++rr) atomicSub(&occ[(size_t)rr * P.P + j], (int)(pu & 0xffffffu));
                 }

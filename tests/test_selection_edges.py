@@ -51,3 +51,28 @@ def test_gang_requests_on_fragmented_nodes_match_oracle(oracle, nodes, m, tiny):
     rng = np.random.Generator(np.random.PCG64(nodes))
     a["gpu_busy"] = np.where(rng.random((6, nodes)) < 0.5, rng.integers(0, 256, (6, nodes)), 0).astype(np.uint8)
     assert_same(oracle.schedule_batch(pools, a), gpu_round(pools, a))
+
+
+@pytest.mark.parametrize("policy", [0, 1, 2])
+def test_replay_queues_beyond_shared_memory_match_oracle(oracle, policy):
+    # so many scenarios that a block keeps few waiting records in shared memory: with bursts of long actions on
+    # four cores the tail of every queue lives in global memory, and comes back as the queue drains
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, 2040, 1020), Pool(POOL_GPU, 8, 8))
+    S, N = 900, 420
+    rng = np.random.Generator(np.random.PCG64(policy))
+    gpu = rng.random((S, N)) < 0.4
+    a = dict(pool=gpu.astype(np.uint8), unit=np.where(gpu, 1 | GANG, 100).astype(np.uint8),
+             level_mask=np.where(gpu, 0x8B, np.where(rng.random((S, N)) < 0.5, 0x80, 0xC0)).astype(np.uint32),
+             s_us=rng.integers(5_000, 60_000, (S, N)).astype(np.int64), p_us=rng.integers(0, 60_000, (S, N)).astype(np.int64),
+             arrival_us=np.sort(rng.integers(0, 400_000, (S, N)), axis=1).astype(np.int64),
+             n_actions=np.full(S, N, np.int32), gpu_busy=None)
+    rnd = binding.Round(S, N, pools, round_us=10_000, max_rounds=3000)
+    g = rnd.replay_trace(binding.to_device(a), policy=policy)
+    torch.cuda.synchronize()
+    o = oracle.replay_trace(pools, a, round_us=10_000, max_rounds=3000, policy=policy, lo=0, hi=6)
+    for k in ("status", "n_selected", "total_act_us", "alloc_units", "place_node", "place_off", "act_us", "occupancy", "rounds_used"):
+        assert np.array_equal(o[k], g[k][:6].cpu().numpy()), k
+    assert np.all(o["n_selected"] == N)
+    rnd.destroy()
