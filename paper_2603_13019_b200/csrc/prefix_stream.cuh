@@ -96,13 +96,11 @@ __global__ void __launch_bounds__(256) k_side_check(const __grid_constant__ Para
 }
 
 // SIDE: the actions carry further cost-vector entries (Section 4.1); the plain instance keeps its registers.
+// ws: whose rows of the workspace are used (the scenario's own; the block's, where a block works a scenario off alone).
 template <bool SIDE>
-__global__ void __launch_bounds__(256) k_head(const __grid_constant__ Params P, HeadState* hst) {
-  const int lane = threadIdx.x & 31;
-  const int sc = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  if (sc >= P.S) return;
+__device__ __forceinline__ void head_walk(const Params& P, int sc, int ws, HeadState& hs_out, bool side_bad, int lane) {
   const size_t row = (size_t)sc * P.N;
-  const size_t prow = (size_t)sc * P.P * P.N;       // pool j's part starts at prow + j * N
+  const size_t prow = (size_t)ws * P.P * P.N;       // pool j's part starts at prow + j * N
   const int n_act = min(max(P.n_actions[sc], 0), P.N);
   const int D = P.V - P.P;                          // demand slots
 
@@ -203,7 +201,7 @@ __global__ void __launch_bounds__(256) k_head(const __grid_constant__ Params P, 
       if (lane == jj) { cnt += __popc(b); mreg += __popc(b & below_f); }
     }
     if (cand) {
-      P.order[(size_t)sc * P.cand_stride + P.cand_off[j] + pos] = i;
+      P.order[(size_t)ws * P.cand_stride + P.cand_off[j] + pos] = i;
       if (eff & (eff - 1)) el |= 1u << j;
     }
     for (int v = 0; v < D; ++v) {
@@ -243,25 +241,31 @@ __global__ void __launch_bounds__(256) k_head(const __grid_constant__ Params P, 
       if (((elw >> jj) & 1u) && (unfit & slots)) need |= 1u << jj;
     }
   }
-  const int anybad = (__any_sync(TG_FULL, bad) || (SIDE && P.side_bad[sc])) ? 1 : 0;
+  const int anybad = (__any_sync(TG_FULL, bad) || (SIDE && side_bad)) ? 1 : 0;
   if (SIDE) {
     const int sr = __shfl_sync(TG_FULL, sres, lane < P.P ? P.pool[lane].slot0 : 0);
-    if (lane < P.P) P.side_res[(size_t)sc * P.P + lane] = sr;
+    if (lane < P.P) P.side_res[(size_t)ws * P.P + lane] = sr;
   }
   if (lane < P.P) {
     PoolMeta mt;
-    mt.base = (i64)sc * (P.P - 1) * P.N + (i64)lane * P.N;   // row + base = prow + lane * N
-    mt.cbase = (i64)sc * (P.cand_stride - P.N) + P.cand_off[lane];   // row + cbase = sc * cand_stride + cand_off
+    mt.base = ((i64)ws * P.P + lane - sc) * P.N;      // row + base = prow + lane * N
+    mt.cbase = (i64)ws * P.cand_stride + P.cand_off[lane] - (i64)sc * P.N;
     // an invalid record among the actions seen here: nothing of the scenario is decided
     mt.count = anybad ? 0 : cnt; mt.m = anybad ? 0 : mreg; mt.elastic = anybad ? 0 : ((elw >> lane) & 1u);
     mt.first_wait = anybad ? -1 : fwreg;
-    P.meta[(size_t)sc * P.P + lane] = mt;
-    hst[sc].cur[lane] = cnt;
+    P.meta[(size_t)ws * P.P + lane] = mt;
+    hs_out.cur[lane] = cnt;
   }
   if (lane == 0) {
-    hst[sc].hs = hs; hst[sc].need = need; hst[sc].bad = anybad; hst[sc].n = n_pref;
+    hs_out.hs = hs; hs_out.need = need; hs_out.bad = anybad; hs_out.n = n_pref;
     P.o_status[sc] = anybad ? TG_ST_BAD_ACTION : 0; P.o_total[sc] = 0; P.o_nsel[sc] = 0;
   }
+}
+
+template <bool SIDE>
+__global__ void __launch_bounds__(256) k_head(const __grid_constant__ Params P, HeadState* hst) {
+  const int sc = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (sc < P.S) head_walk<SIDE>(P, sc, sc, hst[sc], SIDE && P.side_bad[sc], threadIdx.x & 31);
 }
 
 // exclusive scan of one int per thread over the CTA; *total = sum.  wsum: 8 ints of scratch.
@@ -278,33 +282,36 @@ __device__ __forceinline__ int ks_block_scan(int x, int* wsum, int t, int* total
   return off + incl - x;
 }
 
-__global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant__ Params P, const HeadState* hst) {
-  __shared__ int s_m[TG_MAX_POOLS], s_first[TG_MAX_POOLS], s_cur[TG_MAX_POOLS], s_scan[KS_THREADS / 32];
-  __shared__ int s_bad;
+struct StreamShared {
   // usable multiplicities by (pool, unit byte): a record's usable levels are its mask ANDed with the
   // entry, and a record with none is invalid (decode_levels, tabulated once per round description)
-  __shared__ __align__(16) u32 s_ok[TG_MAX_POOLS * 256];
-
-  const int sc = blockIdx.x, t = threadIdx.x;
+  __align__(16) u32 ok[TG_MAX_POOLS * 256];
+  int m[TG_MAX_POOLS], first[TG_MAX_POOLS], cur[TG_MAX_POOLS], scan[KS_THREADS / 32];
+  int bad;
+};
+// Everything behind the head, by a block of KS_THREADS.  The waiting lists' facts go to the pools' PoolMeta.
+__device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, const HeadState& H, StreamShared& X, int t) {
   const size_t row = (size_t)sc * P.N;
-  const size_t prow = (size_t)sc * P.P * P.N;
+  const size_t prow = (size_t)ws * P.P * P.N;
   const int n_act = min(max(P.n_actions[sc], 0), P.N);
-  const HeadState H = hst[sc];
   const u32 need = H.need;
-  const bool vec = (P.N % 16 == 0) && ((((size_t)P.a_pool | (size_t)P.a_unit | (size_t)P.a_mask) & 15) == 0);
+  // 128-bit loads need groups that start at multiples of 16 of the whole array, wherever the row begins: the first tile
+  // starts up to 15 records early and skips them
+  const bool vec = (((size_t)P.a_pool | (size_t)P.a_unit | (size_t)P.a_mask) & 15) == 0;
+  const int hs = H.hs, skew = vec ? (int)((row + hs) & 15) : 0;
   if (t < TG_MAX_POOLS) {
-    s_m[t] = t < P.P ? P.meta[(size_t)sc * P.P + t].m : 0;
-    s_first[t] = INT_MAX;
+    X.m[t] = t < P.P ? P.meta[(size_t)ws * P.P + t].m : 0;
+    X.first[t] = INT_MAX;
   }
-  for (int x = t; x < TG_MAX_POOLS * 256 / 4; x += KS_THREADS) ((uint4*)s_ok)[x] = ((const uint4*)P.ok_table)[x];
-  if (t == 0) s_bad = H.bad;
+  for (int x = t; x < TG_MAX_POOLS * 256 / 4; x += KS_THREADS) ((uint4*)X.ok)[x] = ((const uint4*)P.ok_table)[x];
+  if (t == 0) X.bad = H.bad;
   __syncthreads();
 
-  if (t < TG_MAX_POOLS) s_cur[t] = H.cur[t];          // actions of every pool seen so far
+  if (t < TG_MAX_POOLS) X.cur[t] = H.cur[t];          // actions of every pool seen so far
   __syncthreads();
-  for (int tile0 = H.hs; tile0 < n_act; tile0 += KS_TILE) {   // a bad scenario is streamed on: its rows are rewritten below
+  for (int tile0 = hs - skew; tile0 < n_act; tile0 += KS_TILE) {   // a bad scenario is streamed on: its rows are rewritten below
     const int i_first = tile0 + t * KS_ITEMS;
-    const bool full = vec && i_first + KS_ITEMS <= n_act;
+    const bool full = vec && i_first >= hs && i_first + KS_ITEMS <= n_act;
     __align__(16) u8 rp[KS_ITEMS], ru[KS_ITEMS];
     // validate; keep the least multiplicity of the records whose pool may need its list
     bool bad = false;
@@ -320,35 +327,36 @@ __global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant_
 #pragma unroll
         for (int k = 0; k < KS_ITEMS; ++k) {
           const int i = i_first + k;
-          rp[k] = i < n_act ? P.a_pool[row + i] : 0xff;
-          ru[k] = i < n_act ? P.a_unit[row + i] : 1;
-          rm[k] = i < n_act ? P.a_mask[row + i] : 1;
+          const bool on = i >= hs && i < n_act;
+          rp[k] = on ? P.a_pool[row + i] : 0xff;
+          ru[k] = on ? P.a_unit[row + i] : 1;
+          rm[k] = on ? P.a_mask[row + i] : 1;
         }
       }
 #pragma unroll
       for (int k = 0; k < KS_ITEMS / 4; ++k) rmin4[k] = 0;
 #pragma unroll
       for (int k = 0; k < KS_ITEMS; ++k) {
-        if (!full && i_first + k >= n_act) continue;
+        if (!full && (i_first + k < hs || i_first + k >= n_act)) continue;
         const int j = rp[k];
-        const u32 eff = j < TG_MAX_POOLS ? rm[k] & s_ok[j * 256 + ru[k]] : 0u;   // pools beyond the description hold zeros
+        const u32 eff = j < TG_MAX_POOLS ? rm[k] & X.ok[j * 256 + ru[k]] : 0u;   // pools beyond the description hold zeros
         bad |= eff == 0;
         if ((need >> j) & 1u) rmin4[k >> 2] |= (u32)__ffs(eff) << (8 * (k & 3));
       }
     }
-    if (bad) s_bad = 1;
+    if (bad) X.bad = 1;
     // waiting lists of the pools that may need them; a position follows from the pool bytes alone
     for (u32 nm = need; nm; nm &= nm - 1) {
       const int j = __ffs(nm) - 1;
       u32 mine = 0;
 #pragma unroll
       for (int k = 0; k < KS_ITEMS; ++k) if (rp[k] == j) mine |= 1u << k;
-      const int before = s_cur[j];
+      const int before = X.cur[j];
       int tot;
-      int pos = before + ks_block_scan(__popc(mine), s_scan, t, &tot);
-      if (t == 0) s_cur[j] = before + tot;               // read again only after the barrier that ends the tile
+      int pos = before + ks_block_scan(__popc(mine), X.scan, t, &tot);
+      if (t == 0) X.cur[j] = before + tot;               // read again only after the barrier that ends the tile
       if (!mine) continue;
-      const int m_j = s_m[j];
+      const int m_j = X.m[j];
       i64* dst = P.tmin + prow + (size_t)j * P.N;
       // the thread's listed records, four at a time: their s / p loads are in flight together
       const u64 rlo = (u64)rmin4[0] | ((u64)rmin4[1] << 32), rhi = (u64)rmin4[2] | ((u64)rmin4[3] << 32);
@@ -366,7 +374,7 @@ __global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant_
           if (kk[x] < 0) continue;
           const int rmin = (int)(((kk[x] < 8 ? rlo : rhi) >> (8 * (kk[x] & 7))) & 0xffu);
           if (rmin) dst[pos] = duration(clamp_param(sv[x]), clamp_param(pv[x]), rmin);   // 0: invalid record, the scenario is flagged
-          if (pos == m_j) s_first[j] = i_first + kk[x];   // the pool's first waiting action
+          if (pos == m_j) X.first[j] = i_first + kk[x];   // the pool's first waiting action
           ++pos;
         }
       }
@@ -374,52 +382,63 @@ __global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant_
     __syncthreads();
   }
   __syncthreads();
-  const bool bad = s_bad != 0;
+  const bool bad = X.bad != 0;
   // nobody will write the candidates of a bad scenario: their rows are "not scheduled" too
   if (bad) for (int i = t; i < min(H.n, P.N); i += KS_THREADS) {
     P.o_alloc[row + i] = 0; P.o_node[row + i] = -1; P.o_off[row + i] = -1; P.o_act[row + i] = -1;
   }
   if (t < P.P) {
-    PoolMeta* mt = P.meta + (size_t)sc * P.P + t;
+    PoolMeta* mt = P.meta + (size_t)ws * P.P + t;
     if (bad) { mt->count = 0; mt->m = 0; mt->first_wait = -1; }
     else if ((need >> t) & 1u) {
-      mt->count = s_cur[t];
-      if (s_first[t] != INT_MAX) mt->first_wait = s_first[t];
+      mt->count = X.cur[t];
+      if (X.first[t] != INT_MAX) mt->first_wait = X.first[t];
     } else mt->count = mt->m;                          // a list nobody reads counts as empty
   }
   // status, total and count were initialised by k_head; k_solve may be adding to them already
   if (t == 0 && bad) atomicOr(&P.o_status[sc], TG_ST_BAD_ACTION);
 }
 
+__global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant__ Params P, const HeadState* hst) {
+  __shared__ StreamShared X;
+  stream_queue(P, blockIdx.x, blockIdx.x, hst[blockIdx.x], X, threadIdx.x);
+}
+
 // "not scheduled" (Eq. 2 has no value for an action that stays queued): units 0, node -1, offset -1,
 // ACT -1 for every action behind its scenario's candidate prefix (the candidates' rows are written
 // by the kernels that decide them, which may run at the same time).  Consecutive threads take
 // consecutive groups of four actions, so a warp's store covers whole contiguous sectors.
+__device__ __forceinline__ void write_unscheduled(const Params& P, size_t o) {
+  P.o_alloc[o] = 0; P.o_node[o] = -1; P.o_off[o] = -1; P.o_act[o] = -1;
+}
+__device__ __forceinline__ void write_unscheduled4(const Params& P, size_t o) {
+  const int4 z = make_int4(0, 0, 0, 0), m1 = make_int4(-1, -1, -1, -1);
+  const longlong2 a1 = make_longlong2(-1, -1);
+  *(int4*)(P.o_alloc + o) = z; *(int4*)(P.o_node + o) = m1; *(int4*)(P.o_off + o) = m1;
+  *(longlong2*)(P.o_act + o) = a1; *(longlong2*)(P.o_act + o + 2) = a1;
+}
+__device__ __forceinline__ bool outputs_aligned(const Params& P) {
+  return (((size_t)P.o_alloc | (size_t)P.o_node | (size_t)P.o_off | (size_t)P.o_act) & 15) == 0;
+}
 __global__ void __launch_bounds__(256) k_fill(const __grid_constant__ Params P, const HeadState* hst) {
-  const bool vec = (P.N % 4 == 0) &&
-                   ((((size_t)P.o_alloc | (size_t)P.o_node | (size_t)P.o_off | (size_t)P.o_act) & 15) == 0);
   const u32 stride = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (vec) {
-    const u32 qpr = (u32)P.N / 4, quads = (u32)P.S * qpr;   // S * N <= 2^31
-    const int4 z = make_int4(0, 0, 0, 0), m1 = make_int4(-1, -1, -1, -1);
-    const longlong2 a1 = make_longlong2(-1, -1);
-    for (u32 q = tid; q < quads; q += stride) {
-      const u32 sc = q / qpr;
-      const int i0 = (int)(q - sc * qpr) * 4, n = hst[sc].n;
-      if (i0 + 4 <= n) continue;
-      const size_t o = (size_t)q * 4;
-      if (i0 >= n) {
-        *(int4*)(P.o_alloc + o) = z; *(int4*)(P.o_node + o) = m1; *(int4*)(P.o_off + o) = m1;
-        *(longlong2*)(P.o_act + o) = a1; *(longlong2*)(P.o_act + o + 2) = a1;
-      } else {
-        for (int k = n - i0; k < 4; ++k) { P.o_alloc[o + k] = 0; P.o_node[o + k] = -1; P.o_off[o + k] = -1; P.o_act[o + k] = -1; }
-      }
+  const u32 N = (u32)P.N, total = (u32)P.S * N;              // S * N <= 2^31
+  if (outputs_aligned(P)) {
+    // groups of four of the whole array; one may hold the end of a row and the beginning of the next
+    for (u32 q = tid; q <= (total - 1) / 4; q += stride) {
+      const u32 o = q * 4, sc = o / N, i0 = o - sc * N;
+      if (i0 + 4 <= N) {
+        const int left = (int)i0 - hst[sc].n;
+        if (left >= 0) { write_unscheduled4(P, o); continue; }
+        for (int k = max(-left, 0); k < 4; ++k) write_unscheduled(P, (size_t)o + k);
+      } else
+        for (u32 k = 0, s = sc, i = i0; k < 4 && o + k < total; ++k, ++i) {
+          if (i == N) { i = 0; ++s; }
+          if ((int)i >= hst[s].n) write_unscheduled(P, (size_t)o + k);
+        }
     }
   } else {
-    const size_t total = (size_t)P.S * P.N;
-    for (size_t o = tid; o < total; o += stride) {
-      if ((int)(o % P.N) < hst[o / P.N].n) continue;
-      P.o_alloc[o] = 0; P.o_node[o] = -1; P.o_off[o] = -1; P.o_act[o] = -1;
-    }
+    for (u32 o = tid; o < total; o += stride)
+      if ((int)(o % N) >= hst[o / N].n) write_unscheduled(P, o);
   }
 }
