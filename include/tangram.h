@@ -189,9 +189,9 @@ int tangram_replay_trace(tangram_round* round, const tangram_actions* actions,
  * image: every GPU that loads the library holds those bytes until the process exits, whether
  * or not this entry point is ever called.  A batch whose scratch does not fit is refused with
  * TANGRAM_ETOOBIG and nothing is launched: 12 bytes per action of n_scenarios * max_actions,
- * plus (39 + 16 * depth) * max_actions + 324 KiB for each of 8 to 32 worker warps (as many as
- * fit, at least 8), plus at least 4 MiB for large DP tables must fit.  At most 32 worker warps
- * run, so this call is slower on big batches; results are identical.  A scenario whose DP tables outgrow what is left of the
+ * plus (39 + 16 * depth) * max_actions + 324 KiB for each of 8 worker warps, plus at least
+ * 4 MiB for large DP tables must fit.  As many scenarios as the array has room for run at a time,
+ * a worker warp per pool, so this call is slower on big batches; results are identical.  A scenario whose DP tables outgrow what is left of the
  * array is marked TANGRAM_STATUS_WORKSPACE in `status`, exactly as with a round whose
  * workspace_bytes is too small; the other scenarios of the batch are unaffected.
  *

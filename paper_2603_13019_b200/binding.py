@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from dataclasses import dataclass
 from typing import Dict, Optional, Sequence
 
@@ -54,6 +55,10 @@ class _Result(C.Structure):
                 ("status", C.c_void_p), ("occupancy", C.c_void_p), ("rounds_used", C.c_void_p)]
 
 
+# the two structures as packed bytes: what the calls are given (a _Actions / _Result by reference does as well)
+_PACK_ACTIONS = struct.Struct(f"{len(_Actions._fields_)}P").pack
+_PACK_RESULT = struct.Struct(f"{len(_Result._fields_)}P").pack
+
 EXPORTS = ("tangram_round_create", "tangram_schedule_batch", "tangram_replay_trace",
            "tangram_round_destroy", "tangram_kernel_launches", "tangram_strerror",
            "tangram_last_cuda_error", "tangram_set_profiling", "tangram_kernel_time_ms",
@@ -74,9 +79,9 @@ def load_library(path: Optional[str] = None):
     lib.tangram_round_create.restype = C.c_int
     lib.tangram_round_create.argtypes = [C.POINTER(_RoundDesc), C.POINTER(C.c_void_p)]
     lib.tangram_schedule_batch.restype = C.c_int
-    lib.tangram_schedule_batch.argtypes = [C.c_void_p, C.POINTER(_Actions), C.c_int64, C.POINTER(_Result), C.c_void_p]
+    lib.tangram_schedule_batch.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_void_p]
     lib.tangram_replay_trace.restype = C.c_int
-    lib.tangram_replay_trace.argtypes = [C.c_void_p, C.POINTER(_Actions), C.POINTER(_Result), C.c_void_p]
+    lib.tangram_replay_trace.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
     lib.tangram_round_destroy.restype = None
     lib.tangram_round_destroy.argtypes = [C.c_void_p]
     lib.tangram_kernel_launches.restype = C.c_int64
@@ -92,19 +97,19 @@ def load_library(path: Optional[str] = None):
     lib.tangram_kernel_name.argtypes = [C.c_int]
     lib.tangram_schedule_batch_static.restype = C.c_int
     lib.tangram_order_queue.restype = C.c_int
-    lib.tangram_order_queue.argtypes = [C.c_void_p, C.POINTER(_Actions), C.c_int, C.c_void_p, C.c_void_p]
+    lib.tangram_order_queue.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p]
     lib.tangram_schedule_batch_ordered.restype = C.c_int
-    lib.tangram_schedule_batch_ordered.argtypes = [C.c_void_p, C.POINTER(_Actions), C.c_int, C.c_int64,
-                                                   C.POINTER(_Result), C.c_void_p]
+    lib.tangram_schedule_batch_ordered.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_int64,
+                                                   C.c_void_p, C.c_void_p]
     lib.tangram_replay_trace_ordered.restype = C.c_int
-    lib.tangram_replay_trace_ordered.argtypes = [C.c_void_p, C.POINTER(_Actions), C.c_int, C.POINTER(_Result), C.c_void_p]
+    lib.tangram_replay_trace_ordered.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p]
     lib.tangram_replay_trace_pinned.restype = C.c_int
-    lib.tangram_replay_trace_pinned.argtypes = [C.c_void_p, C.POINTER(_Actions), C.c_int, C.POINTER(_Pinning),
-                                                C.POINTER(_Result), C.c_void_p]
+    lib.tangram_replay_trace_pinned.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.POINTER(_Pinning),
+                                                C.c_void_p, C.c_void_p]
     lib.tangram_pin_trajectories.restype = C.c_int
-    lib.tangram_pin_trajectories.argtypes = [C.c_void_p, C.POINTER(_Actions), C.POINTER(_Pinning), C.c_void_p]
-    lib.tangram_schedule_batch_static.argtypes = [C.POINTER(_RoundDesc), C.POINTER(_Actions), C.c_int64,
-                                                  C.POINTER(_Result), C.c_void_p]
+    lib.tangram_pin_trajectories.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(_Pinning), C.c_void_p]
+    lib.tangram_schedule_batch_static.argtypes = [C.POINTER(_RoundDesc), C.c_void_p, C.c_int64,
+                                                  C.c_void_p, C.c_void_p]
     if path is None:
         _lib = lib
     return lib
@@ -118,16 +123,12 @@ class PoolDesc:
     window_us: int = 0
 
 
-def _dtypes():
-    import torch
-    ins = dict(pool=torch.uint8, unit=torch.uint8, level_mask=torch.int32, s_us=torch.int64,
-               p_us=torch.int64, arrival_us=torch.int64, n_actions=torch.int32, gpu_busy=torch.uint8,
-               service=torch.int16, restore_us=torch.int64, cache_tag=torch.int32, cache_use=torch.int64,
-               side_pool=torch.uint8, side_units=torch.int16)
-    outs = dict(alloc_units=torch.int32, place_node=torch.int32, place_off=torch.int32,
-                act_us=torch.int64, total_act_us=torch.int64, n_selected=torch.int32,
-                status=torch.int32, occupancy=torch.int32, rounds_used=torch.int32)
-    return ins, outs
+# columns of the two argument structures, in their order, with the dtypes (torch is imported on the first call)
+_INS = dict(pool="uint8", unit="uint8", level_mask="int32", s_us="int64", p_us="int64", arrival_us="int64",
+            n_actions="int32", gpu_busy="uint8", service="int16", restore_us="int64", cache_tag="int32",
+            cache_use="int64", side_pool="uint8", side_units="int16")
+_OUTS = dict(alloc_units="int32", place_node="int32", place_off="int32", act_us="int64", total_act_us="int64",
+             n_selected="int32", status="int32", occupancy="int32", rounds_used="int32")
 
 
 def _check(rc: int):
@@ -157,7 +158,23 @@ class Round:
         _check(self._lib.tangram_round_create(C.byref(desc), C.byref(h)))
         self._h = h
 
+        self._ins, self._outs = self._columns()
+
     # -- marshalling ---------------------------------------------------------------
+    def _columns(self):
+        """(name, dtype, elements) of every input and output column; elements None: never handed over."""
+        import torch
+        S, SN = self.n_scenarios, self.n_scenarios * self.max_actions
+        nodes = sum(p.capacity // p.group for p in self.pools if p.type == POOL_GPU)
+        sizes = dict(n_actions=S, gpu_busy=S * nodes, total_act_us=S, n_selected=S, status=S,
+                     occupancy=S * self.max_rounds * len(self.pools), rounds_used=S)
+        # the cache and cost-vector columns are only handed over when the round was created with them
+        cached = self.cache_slots != 0
+        sizes.update(service=SN if cached else None, restore_us=SN if cached else None)
+        sizes.update(dict.fromkeys(("cache_tag", "cache_use"), S * nodes * 8 * self.cache_slots if cached else None))
+        sizes.update(dict.fromkeys(("side_pool", "side_units"), SN * self.side_costs if self.side_costs != 0 else None))
+        return tuple(tuple((k, getattr(torch, d), sizes.get(k, SN)) for k, d in cols.items()) for cols in (_INS, _OUTS))
+
     def _ptr(self, name: str, t, dtype, numel: Optional[int]):
         if t is None:
             return None
@@ -171,45 +188,36 @@ class Round:
             raise TangramError(f"{name}: expected {numel} elements, got {t.numel()}")
         return t.data_ptr()
 
-    def _actions(self, a: Dict) -> _Actions:
-        ins, _ = _dtypes()
-        SN = self.n_scenarios * self.max_actions
-        nodes = sum(p.capacity // p.group for p in self.pools if p.type == POOL_GPU)
-        ncache = self.n_scenarios * nodes * 8 * self.cache_slots
-        sizes = dict(pool=SN, unit=SN, level_mask=SN, s_us=SN, p_us=SN, arrival_us=SN,
-                     n_actions=self.n_scenarios, gpu_busy=self.n_scenarios * nodes,
-                     service=SN, restore_us=SN, cache_tag=ncache, cache_use=ncache,
-                     side_pool=SN * self.side_costs, side_units=SN * self.side_costs)
-        # the cache and cost-vector columns are only handed over when the round was created with them
-        off = set()
-        if self.cache_slots == 0:
-            off |= {"service", "restore_us", "cache_tag", "cache_use"}
-        if self.side_costs == 0:
-            off |= {"side_pool", "side_units"}
-        return _Actions(*[self._ptr(k, None if k in off else a.get(k), ins[k], sizes[k]) for k in
-                          ("pool", "unit", "level_mask", "s_us", "p_us", "arrival_us", "n_actions", "gpu_busy",
-                           "service", "restore_us", "cache_tag", "cache_use", "side_pool", "side_units")])
+    def _pack(self, pack, columns, get) -> bytes:
+        # a small batch takes the GPU as long as this loop takes the host: one test per tensor, the
+        # reason looked up only when it fails
+        host, ptrs = self.host_buffers, []
+        for name, dtype, numel in columns:
+            t = None if numel is None else get(name)
+            if t is None:
+                ptrs.append(0)
+            elif t.dtype is dtype and t.numel() == numel and t.is_cuda != host and t.is_contiguous():
+                ptrs.append(t.data_ptr())
+            else:
+                ptrs.append(self._ptr(name, t, dtype, numel) or 0)
+        return pack(*ptrs)
+
+    def _actions(self, a: Dict) -> bytes:
+        return self._pack(_PACK_ACTIONS, self._ins, a.get)
 
     def new_result(self, replay: bool = False) -> Dict:
         """Output tensors of the right shapes (device, or pinned host in host-buffer mode)."""
         import torch
-        _, outs = _dtypes()
         S, N = self.n_scenarios, self.max_actions
         kw = dict(pin_memory=True) if self.host_buffers else dict(device="cuda")
         shapes = dict(alloc_units=(S, N), place_node=(S, N), place_off=(S, N), act_us=(S, N),
                       total_act_us=(S,), n_selected=(S,), status=(S,))
         if replay:
             shapes.update(occupancy=(S, self.max_rounds, len(self.pools)), rounds_used=(S,))
-        return {k: torch.empty(shp, dtype=outs[k], **kw) for k, shp in shapes.items()}
+        return {k: torch.empty(shp, dtype=getattr(torch, _OUTS[k]), **kw) for k, shp in shapes.items()}
 
-    def _result(self, r: Dict) -> _Result:
-        _, outs = _dtypes()
-        S, N = self.n_scenarios, self.max_actions
-        sizes = dict(alloc_units=S * N, place_node=S * N, place_off=S * N, act_us=S * N, total_act_us=S,
-                     n_selected=S, status=S, occupancy=S * self.max_rounds * len(self.pools), rounds_used=S)
-        return _Result(*[self._ptr(k, r.get(k), outs[k], sizes[k]) for k in
-                         ("alloc_units", "place_node", "place_off", "act_us", "total_act_us", "n_selected",
-                          "status", "occupancy", "rounds_used")])
+    def _result(self, r: Dict) -> bytes:
+        return self._pack(_PACK_RESULT, self._outs, r.get)
 
     @staticmethod
     def _stream(stream) -> int:
@@ -223,7 +231,7 @@ class Round:
         """tangram_schedule_batch: one round for every scenario, asynchronous on `stream`."""
         result = self.new_result() if result is None else result
         a, r = self._actions(actions), self._result(result)
-        _check(self._lib.tangram_schedule_batch(self._h, C.byref(a), int(now_us), C.byref(r), self._stream(stream)))
+        _check(self._lib.tangram_schedule_batch(self._h, a, int(now_us), r, self._stream(stream)))
         return result
 
     def replay_trace(self, actions: Dict, result: Optional[Dict] = None, stream=None, policy: int = 0) -> Dict:
@@ -232,9 +240,9 @@ class Round:
         result = self.new_result(replay=True) if result is None else result
         a, r = self._actions(actions), self._result(result)
         if policy:
-            _check(self._lib.tangram_replay_trace_ordered(self._h, C.byref(a), int(policy), C.byref(r), self._stream(stream)))
+            _check(self._lib.tangram_replay_trace_ordered(self._h, a, int(policy), r, self._stream(stream)))
         else:
-            _check(self._lib.tangram_replay_trace(self._h, C.byref(a), C.byref(r), self._stream(stream)))
+            _check(self._lib.tangram_replay_trace(self._h, a, r, self._stream(stream)))
         return result
 
     def order_queue(self, actions: Dict, policy: int, stream=None):
@@ -242,7 +250,7 @@ class Round:
         import torch
         perm = torch.empty((self.n_scenarios, self.max_actions), dtype=torch.int32, device="cuda")
         a = self._actions(actions)
-        _check(self._lib.tangram_order_queue(self._h, C.byref(a), int(policy), C.c_void_p(perm.data_ptr()),
+        _check(self._lib.tangram_order_queue(self._h, a, int(policy), C.c_void_p(perm.data_ptr()),
                                              self._stream(stream)))
         return perm
 
@@ -251,7 +259,7 @@ class Round:
         """tangram_schedule_batch_ordered: one round on every queue sorted by `policy`."""
         result = self.new_result() if result is None else result
         a, r = self._actions(actions), self._result(result)
-        _check(self._lib.tangram_schedule_batch_ordered(self._h, C.byref(a), int(policy), int(now_us), C.byref(r),
+        _check(self._lib.tangram_schedule_batch_ordered(self._h, a, int(policy), int(now_us), r,
                                                         self._stream(stream)))
         return result
 
@@ -270,7 +278,7 @@ class Round:
                        self._ptr("node_mem_free", actions["node_mem_free"], torch.int64, S * len(self.pools)),
                        out["pool"].data_ptr(), out["n_admitted"].data_ptr(), None)
         a = self._actions(actions)
-        _check(self._lib.tangram_pin_trajectories(self._h, C.byref(a), C.byref(pin), self._stream(stream)))
+        _check(self._lib.tangram_pin_trajectories(self._h, a, C.byref(pin), self._stream(stream)))
         return out
 
     def replay_trace_pinned(self, actions: Dict, policy: int = 0, result: Optional[Dict] = None, stream=None) -> Dict:
@@ -289,7 +297,7 @@ class Round:
                        result["pool"].data_ptr(), None,
                        self._ptr("traj_last", actions.get("traj_last"), torch.uint8, S * N))
         a, r = self._actions(actions), self._result(result)
-        _check(self._lib.tangram_replay_trace_pinned(self._h, C.byref(a), int(policy), C.byref(pin), C.byref(r),
+        _check(self._lib.tangram_replay_trace_pinned(self._h, a, int(policy), C.byref(pin), r,
                                                      self._stream(stream)))
         return result
 
@@ -346,6 +354,7 @@ def to_device(arrays: Dict, device: str = "cuda", pin: bool = False) -> Dict:
 
 
 STATIC_SCRATCH_BYTES = 32 << 20
+_STATIC_INS = ("pool", "unit", "level_mask", "s_us", "p_us", "arrival_us", "n_actions", "gpu_busy")
 
 
 def schedule_batch_static(pools: Sequence, actions: Dict, result: Dict, *, depth: int = 2, now_us: int = 0,
@@ -359,21 +368,18 @@ def schedule_batch_static(pools: Sequence, actions: Dict, result: Dict, *, depth
     stream capture.  Returns the C return code (0, or -4 when the batch is too large for the
     array) instead of raising, so that callers can fall back to a Round."""
     lib = load_library()
-    ins, outs = _dtypes()
     S, N = actions["pool"].shape
     arr = (_PoolDesc * len(pools))(*[_PoolDesc(p.type, p.capacity, p.group, p.window_us) for p in pools])
     desc = _RoundDesc(S, N, len(pools), depth, 0, 0, 0, 0, 0, 0, 0, arr)
 
     def ptr(t):
-        return None if t is None else t.data_ptr()
+        return 0 if t is None else t.data_ptr()
 
-    for k, t in list(actions.items()) + list(result.items()):
-        if t is not None and not (t.is_cuda and t.is_contiguous()):
-            raise TangramError(f"{k}: a contiguous device tensor is required")
-    a = _Actions(*([ptr(actions.get(k)) for k in
-                    ("pool", "unit", "level_mask", "s_us", "p_us", "arrival_us", "n_actions", "gpu_busy")] + [None] * 6))
-    r = _Result(*[ptr(result.get(k)) for k in
-                  ("alloc_units", "place_node", "place_off", "act_us", "total_act_us", "n_selected", "status",
-                   "occupancy", "rounds_used")])
-    return int(lib.tangram_schedule_batch_static(C.byref(desc), C.byref(a), int(now_us), C.byref(r),
+    for tensors in (actions, result):
+        for k, t in tensors.items():
+            if t is not None and not (t.is_cuda and t.is_contiguous()):
+                raise TangramError(f"{k}: a contiguous device tensor is required")
+    a = _PACK_ACTIONS(*[ptr(actions.get(k)) for k in _STATIC_INS], *[0] * 6)
+    r = _PACK_RESULT(*[ptr(result.get(k)) for k in _OUTS])
+    return int(lib.tangram_schedule_batch_static(C.byref(desc), a, int(now_us), r,
                                                  Round._stream(stream)))

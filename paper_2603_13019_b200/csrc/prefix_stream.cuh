@@ -45,8 +45,14 @@ __device__ __forceinline__ int warp_incl_scan32(int x, int lane) {
 }
 
 // Further entries of the cost vectors (Section 4.1): an entry has to name a quota / concurrency pool other
-// than the action's key pool and an amount of 1 .. its capacity.  One thread per action; a scenario with
-// a bad entry is flagged for k_head, which then decides nothing of it.
+// than the action's key pool and an amount of 1 .. its capacity.
+__device__ __forceinline__ bool side_entry_bad(const Params& P, int e, size_t o) {
+  const int k = P.a_side_pool[e * P.side_plane + o];
+  if (k == 0xff) return false;
+  const int c = P.a_side_units[e * P.side_plane + o];
+  return k >= P.P || P.pool[k < P.P ? k : 0].type != TG_POOL_API || k == P.a_pool[o] || c < 1 || c > P.pool[k < P.P ? k : 0].capacity;
+}
+// One thread per action; a scenario with a bad entry is flagged for k_head, which then decides nothing of it.
 __global__ void __launch_bounds__(256) k_side_check(const __grid_constant__ Params P) {
   // sixteen consecutive actions of one scenario per thread (128-bit loads) where the rows allow it
   const bool vec = (P.N % 16 == 0) && (P.side_plane % 16 == 0) &&
@@ -84,13 +90,7 @@ __global__ void __launch_bounds__(256) k_side_check(const __grid_constant__ Para
     const int sc = (int)(o / P.N), i = (int)(o - (size_t)sc * P.N);
     if (i >= min(max(P.n_actions[sc], 0), P.N)) continue;
     bool bad = false;
-    for (int e = 0; e < P.n_side; ++e) {
-      const int k = P.a_side_pool[e * P.side_plane + o];
-      if (k == 0xff) continue;
-      const int c = P.a_side_units[e * P.side_plane + o];
-      bad |= k >= P.P || P.pool[k < P.P ? k : 0].type != TG_POOL_API || k == P.a_pool[o] || c < 1 ||
-             c > P.pool[k < P.P ? k : 0].capacity;
-    }
+    for (int e = 0; e < P.n_side; ++e) bad |= side_entry_bad(P, e, o);
     if (bad) P.side_bad[sc] = 1;
   }
 }
@@ -303,7 +303,16 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
     X.m[t] = t < P.P ? P.meta[(size_t)ws * P.P + t].m : 0;
     X.first[t] = INT_MAX;
   }
-  for (int x = t; x < TG_MAX_POOLS * 256 / 4; x += KS_THREADS) ((uint4*)X.ok)[x] = ((const uint4*)P.ok_table)[x];
+  if (P.ok_table) {
+    for (int x = t; x < TG_MAX_POOLS * 256 / 4; x += KS_THREADS) ((uint4*)X.ok)[x] = ((const uint4*)P.ok_table)[x];
+  } else {
+#pragma unroll 1
+    for (int x = t; x < TG_MAX_POOLS * 256; x += KS_THREADS) {
+      int g, gang; u32 eff = 0;
+      if (x < P.P * 256) decode_levels(P.pool[x >> 8], (u8)(x & 255), 0xffffffffu, g, gang, eff);
+      X.ok[x] = eff;
+    }
+  }
   if (t == 0) X.bad = H.bad;
   __syncthreads();
 

@@ -8,7 +8,6 @@
 
 #include "../../include/tangram.h"
 #include "common.cuh"
-#include "prefix_kernel.cuh"
 #include "prefix_stream.cuh"
 #include "order_pin.cuh"
 #include "arrange.cuh"
@@ -19,6 +18,10 @@
 #define TG_PROF_CALLS 256   // calls whose kernels can be timed between two queries
 #define TG_FILL_BLOCKS_PER_SM 4   // k_fill is a trickle beside the other kernels, not a flood
 #define TG_IO_CHUNKS 16
+// Scenarios per SM up to which a round is one launch of k_round: as many blocks as an SM holds at once (128 registers
+// x 256 threads), so that no block waits for another.  Beyond that the head walks of eight scenarios share a block, and
+// pools that need a selection are handed out before the others.
+#define TG_FUSED_PER_SM 2
 #define TG_SMEM_PER_SM 233472   // shared memory an SM can split among resident blocks
 #define TG_REPLAY_SMEM 114688    // a replay block takes at most that much (the rest of the SM's is L1)
 #define TG_PROF_K 3         // timed intervals per call at most
@@ -29,7 +32,7 @@
 // them (arrange.cuh, evict.cuh), place what was granted, write the candidates' outputs (Eq. 2).
 //   k_pool     the batched path, behind k_head / k_stream; pools that the head kernel certified
 //              take a short way without any selection
-//   k_select   the allocation-free entry point, behind k_prefix
+//   k_round    small batches and the allocation-free entry point: the whole round, one block per scenario
 // ---------------------------------------------------------------------------------------
 // Tasks are handed out by a counter so that long tasks do not pile up on the same warps.
 __device__ __forceinline__ int next_task(u64* counter, int lane) {
@@ -110,13 +113,13 @@ __device__ __forceinline__ Slab warp_slab(const Params& P, int gw) {
   return s;
 }
 
-__device__ PoolTask& make_task(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C, int lane) {
+__device__ PoolTask& make_task(const Params& P, int sc, int ws, int j, const PoolMeta& mt, const CandArrays& C, int lane) {
   const PoolDev& pd = P.pool[j];
   const size_t row = (size_t)sc * P.N;
   const u8* busy_row = P.gpu_busy ? P.gpu_busy + (size_t)sc * P.n_nodes_total : nullptr;
   int cap[4] = {pd.capacity, 0, 0, 0};
   if (pd.type == TG_POOL_GPU) gpu_caps(pd, busy_row, lane, cap);
-  if (P.n_side > 0 && pd.type == TG_POOL_API) cap[0] -= P.side_res[(size_t)sc * P.P + j];   // set aside for the other pools' candidates
+  if (P.n_side > 0 && pd.type == TG_POOL_API) cap[0] -= P.side_res[(size_t)ws * P.P + j];   // set aside for the other pools' candidates
   Act first;
   first.s = first.p = 0; first.mask = 1; first.g = 1; first.gang = 0;
   const int n_ac = mt.count - mt.m;
@@ -269,7 +272,8 @@ __device__ __forceinline__ void pool_best_levels(const Params& P, int sc, int j,
   }
 }
 
-__device__ void run_pool_task(const Params& P, int sc, int j, const PoolMeta& mt, Slab slab, int lane) {
+// ws: whose rows of the workspace the pool's facts are in
+__device__ __forceinline__ void run_pool_task(const Params& P, int sc, int ws, int j, const PoolMeta& mt, Slab slab, int lane) {
   CandArrays C;
   if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
     if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE);
@@ -277,24 +281,20 @@ __device__ void run_pool_task(const Params& P, int sc, int j, const PoolMeta& mt
   }
   int keep = mt.m;
   if (mt.elastic) {
-    keep = evict_loop(P, make_task(P, sc, j, mt, C, lane), slab, lane);
+    keep = evict_loop(P, make_task(P, sc, ws, j, mt, C, lane), slab, lane);
     if (keep < 0) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
   }
   place_and_write(P, sc, j, mt, C, keep, slab, lane);
 }
 
-__global__ void __launch_bounds__(K2_THREADS) k_select(const __grid_constant__ Params P) {
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * K2_THREADS + threadIdx.x) >> 5;
-  const int n_tasks = P.S * P.P;
-#pragma unroll 1
-  for (;;) {
-    const int x = next_task(P.arena_top + 3, lane);
-    if (x >= n_tasks) break;
-    const int sc = x % P.S, j = P.pool_order[x / P.S];   // pool-major, heaviest pools first
-    const PoolMeta mt = P.meta[(size_t)sc * P.P + j];
-    if (mt.m > 0) run_pool_task(P, sc, j, mt, warp_slab(P, gw), lane);
-  }
+__device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int j, u32 need, int slab, int lane) {
+  PoolMeta mt = P.meta[(size_t)ws * P.P + j];            // (a scenario with an invalid record has no candidates)
+  mt.m = uniform(mt.m); mt.count = uniform(mt.count); mt.elastic = uniform(mt.elastic);
+  if (mt.m == 0) return;
+  if (!((need >> j) & 1u) && P.pool[j].queue_place) {
+    if (P.pool[j].type == TG_POOL_API || P.pool[j].capacity <= 64 * P.pool[j].group) pool_best_levels<2>(P, sc, j, mt, lane);
+    else pool_best_levels<4>(P, sc, j, mt, lane);
+  } else run_pool_task(P, sc, ws, j, mt, warp_slab(P, slab), lane);
 }
 
 // All pools of a batched round, pool-major, the pools that may need a selection first.
@@ -306,15 +306,57 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
   for (;;) {
     const int x = next_task(P.arena_top + 1, lane);
     if (x >= n_tasks) break;
-    const int sc = x % P.S, j = P.pool_order[x / P.S];
-    PoolMeta mt = P.meta[(size_t)sc * P.P + j];          // (a scenario with an invalid record has no candidates)
-    mt.m = uniform(mt.m); mt.count = uniform(mt.count); mt.elastic = uniform(mt.elastic);
-    if (mt.m == 0) continue;
-    if (!((hst[sc].need >> j) & 1u) && P.pool[j].queue_place) {
-      if (P.pool[j].type == TG_POOL_API || P.pool[j].capacity <= 64 * P.pool[j].group) pool_best_levels<2>(P, sc, j, mt, lane);
-      else pool_best_levels<4>(P, sc, j, mt, lane);
+    const int sc = x % P.S;
+    decide_pool(P, sc, sc, P.pool_order[x / P.S], hst[sc].need, gw, lane);
+  }
+}
+
+// The whole round of a small batch in one launch, one block per scenario: the first warp walks the head of the queue
+// while the others write "not scheduled" everywhere, all of them stream the rest of the queue, then every pool
+// gets a warp (wpb < n_pools of them where memory is short: the static entry).  A block's scratch is its own, so nothing depends on the number of scenarios.  What bounds a small
+// batch is latency, and one launch instead of four (and a memset) saves the gaps.  The last block to finish resets
+// the bump pointer of the arena for the next call.  1 x 64: 38.6 -> 26.8 us a call, 16 x 500 (static): 110 -> 84 us.
+#define TG_DONE_COUNTER 4           // word of arena_top that counts finished blocks
+template <bool SIDE>
+__global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__ Params P, int wpb) {
+  __shared__ StreamShared X;
+  __shared__ HeadState H;
+  __shared__ int s_side_bad;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, ws = blockIdx.x;
+#pragma unroll 1
+  for (int sc = blockIdx.x; sc < P.S; sc += gridDim.x) {
+    const size_t row = (size_t)sc * P.N;
+    if (SIDE) {
+      if (t == 0) s_side_bad = 0;
+      __syncthreads();
+      const int n = min(max(P.n_actions[sc], 0), P.N);
+      bool bad = false;
+#pragma unroll 1
+      for (int i = t; i < n; i += K2_THREADS)
+        for (int e = 0; e < P.n_side; ++e) bad |= side_entry_bad(P, e, row + i);
+      if (bad) s_side_bad = 1;
+      __syncthreads();
     }
-    else run_pool_task(P, sc, j, mt, warp_slab(P, gw), lane);
+    if (warp == 0) head_walk<SIDE>(P, sc, ws, H, SIDE && s_side_bad, lane);
+    else if (outputs_aligned(P)) {
+      const size_t lo = (row + 3) / 4 * 4, hi = (row + P.N) / 4 * 4;       // groups of four of the whole array
+      const size_t mid = lo < hi ? hi : lo;
+      for (size_t o = lo + (size_t)(t - 32) * 4; o < hi; o += (size_t)(K2_THREADS - 32) * 4) write_unscheduled4(P, o);
+      const size_t end = row + P.N;
+      if (t < 40) { const size_t o = row + (t - 32); if (t < 36 && o < lo && o < end) write_unscheduled(P, o); }
+      if (t >= 64 && t < 68) { const size_t o = mid + (t - 64); if (o < end) write_unscheduled(P, o); }
+    } else
+      for (int i = t - 32; i < P.N; i += K2_THREADS - 32) write_unscheduled(P, row + i);
+    __syncthreads();
+    stream_queue(P, sc, ws, H, X, t);
+    __syncthreads();
+#pragma unroll 1
+    for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
+    __syncthreads();
+  }
+  if (t == 0) {
+    __threadfence();
+    if (atomicAdd(P.arena_top + TG_DONE_COUNTER, 1ull) + 1 == gridDim.x) { P.arena_top[0] = 0; P.arena_top[TG_DONE_COUNTER] = 0; }
   }
 }
 
@@ -356,7 +398,7 @@ struct tangram_round {
   cudaEvent_t* ev; int ev_calls, ev_used; int ev_kernel[TG_PROF_CALLS][TG_PROF_K];
 };
 
-static const char* const g_kernel_names[TG_N_KERNELS] = {"k_head", "k_select", "k_replay", "k_pool",
+static const char* const g_kernel_names[TG_N_KERNELS] = {"k_head", "k_round", "k_replay", "k_pool",
                                                           "k_stream", "k_order", "k_pin", "k_fill"};
 
 static cudaError_t fill_tables() {
@@ -391,6 +433,14 @@ static void fill_pool_order(Params& P) {
   for (int r = 0; r < 3; ++r)
     for (int j = 0; j < P.P; ++j)
       if (P.pool[j].type == rank[r]) P.pool_order[k++] = j;
+}
+
+// a pool has at most min(max_actions, capacity) candidates
+static void fill_candidate_rows(Params& P) {
+  P.cand_off[0] = 0;
+  for (int j = 0; j < P.P; ++j)
+    P.cand_off[j + 1] = P.cand_off[j] + (int)align_up((size_t)(P.pool[j].capacity < P.N ? P.pool[j].capacity : P.N), 8);
+  P.cand_stride = P.cand_off[P.P];
 }
 
 // pools whose grants are placed one after the other in queue order with their state in registers
@@ -437,10 +487,7 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   P.n_nodes_total = node0;
   P.V = slot0 + desc->n_pools;
   fill_pool_order(P);
-  P.cand_off[0] = 0;
-  for (int j = 0; j < desc->n_pools; ++j)
-    P.cand_off[j + 1] = P.cand_off[j] + (int)align_up((size_t)(P.pool[j].capacity < P.N ? P.pool[j].capacity : P.N), 8);
-  P.cand_stride = P.cand_off[desc->n_pools];
+  fill_candidate_rows(P);
 
   cudaError_t e = cudaGetDevice(&r->device);
   cudaDeviceProp prop;
@@ -582,7 +629,10 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   P.n_side = desc->side_costs; P.side_plane = (u64)P.S * P.N;
   P.side_bad = r->d_side_bad; P.side_res = r->d_side_res;
   P.slabs = (char*)r->d_slabs; P.arena = (char*)r->d_arena; P.arena_top = (u64*)r->d_arena_top;
-  e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  e = cudaMemset(r->d_arena_top, 0, 256);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
@@ -722,7 +772,20 @@ static void bind_device_io(Params& P, const tangram_actions* a, const tangram_re
 }
 
 // The kernels of one round for the scenarios that P describes, on stream st.
-static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, cudaEvent_t* ev) {
+static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, bool timed) {
+  const bool fused = r->P.S <= TG_FUSED_PER_SM * r->n_sm && r->P.S * P.P <= P.n_workers;   // all blocks resident at once
+  if (fused) {
+    cudaEvent_t* ev = timed ? prof_begin(r, 1, -1, -1) : nullptr;
+    if (ev) CK(cudaEventRecord(ev[0], st));
+    const int smem = P.P * WARP_SMEM_BYTES + 16;
+    if (P.n_side > 0) k_round<true><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    else k_round<false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    if (ev) CK(cudaEventRecord(ev[1], st));
+    r->launches += 1;
+    CK(cudaGetLastError());
+    return TANGRAM_OK;
+  }
+  cudaEvent_t* ev = timed ? prof_begin(r, 0, 4, 3) : nullptr;
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));          // arena top and the task counters
   if (ev) CK(cudaEventRecord(ev[0], st));
   if (P.n_side > 0) {
@@ -763,7 +826,7 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   P.now = now_us;
   if (!r->desc.host_buffers) {
     bind_device_io(P, a, res);
-    return run_pipeline(r, P, st, prof_begin(r, 0, 4, 3));
+    return run_pipeline(r, P, st, true);
   }
   bind_stage(r, a, P);
   // Host buffers: scenarios go through in chunks, so that the copy-in of a chunk, the kernels
@@ -774,7 +837,7 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   if (C > P.S) C = P.S;
   if (C <= 1 || r->ev) {                                   // small batch, or per-kernel timing wanted
     int rc = copy_in(r, a, P, 0, P.S, st);
-    if (!rc) rc = run_pipeline(r, P, st, prof_begin(r, 0, 4, 3));
+    if (!rc) rc = run_pipeline(r, P, st, true);
     if (!rc) rc = copy_out(r, res, P, 0, P.S, st);
     return rc;
   }
@@ -798,7 +861,7 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
     Q.o_total += s0; Q.o_nsel += s0; Q.o_status += s0;
     if ((int64_t)Q.n_workers > (int64_t)Q.S * P.P) Q.n_workers = (int)align_up((size_t)Q.S * P.P, K2_THREADS / 32);
     CK(cudaStreamWaitEvent(r->io_comp, r->io_in_done[c], 0));
-    rc = run_pipeline(r, Q, r->io_comp, nullptr);   // the workspace is reused chunk after chunk
+    rc = run_pipeline(r, Q, r->io_comp, false);   // the workspace is reused chunk after chunk
     if (rc) return rc;
     CK(cudaEventRecord(r->io_comp_done[c], r->io_comp));
     CK(cudaStreamWaitEvent(r->io_out, r->io_comp_done[c], 0));
@@ -875,6 +938,7 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
   if (policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0)) k_replay<true><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   else k_replay<false><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   if (ev) CK(cudaEventRecord(ev[1], st));
+  CK(cudaMemsetAsync(P.arena_top, 0, 256, st));            // k_round starts from counters at zero
   r->launches += 1;
   CK(cudaGetLastError());
   if (r->desc.host_buffers) {
@@ -969,7 +1033,7 @@ extern "C" int tangram_schedule_batch_ordered(tangram_round* r, const tangram_ac
   Params Q = P;
   Q.a_pool = G.pool; Q.a_unit = G.unit; Q.a_mask = G.mask; Q.a_s = G.s; Q.a_p = G.p; Q.a_arrival = G.arrival;
   Q.o_alloc = (int*)(d + off_alloc); Q.o_node = (int*)(d + off_node); Q.o_off = (int*)(d + off_off); Q.o_act = (i64*)(d + off_act);
-  rc = run_pipeline(r, Q, st, nullptr);
+  rc = run_pipeline(r, Q, st, false);
   if (rc) return rc;
   ScatterIo X;
   X.perm = r->d_perm; X.alloc = Q.o_alloc; X.node = Q.o_node; X.off = Q.o_off; X.act = Q.o_act;
@@ -1020,6 +1084,7 @@ static int static_setup(int* dev_out) {
     unsigned char* ptr = nullptr;
     CK(cudaGetSymbolAddress((void**)&ptr, g_static_scratch));
     CK(fill_tables());
+    CK(cudaFuncSetAttribute(k_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
     g_static_ptr[dev] = ptr;
     g_static_ready[dev] = true;
   }
@@ -1054,47 +1119,46 @@ extern "C" int tangram_schedule_batch_static(const tangram_round_desc* desc, con
     node0 += d.n_nodes;
     d.slot0 = slot0; d.n_slots = pd.type == TANGRAM_POOL_GPU ? 4 : 1;
     slot0 += d.n_slots;
+    d.queue_place = queue_place_ok(d);
   }
   P.n_nodes_total = node0;
   P.V = slot0 + desc->n_pools;
   fill_pool_order(P);
+  fill_candidate_rows(P);
   P.now = now_us;
 
-  // carve the array: fixed parts first, then as many worker slabs as fit, the rest is the arena
+  // what a batch may need at most is fixed by the header; the scratch itself is per block, as many as fit
   const size_t SN = (size_t)P.S * P.N;
   const size_t budget = TANGRAM_STATIC_SCRATCH_BYTES, arena_min = (size_t)4 << 20;
-  size_t off = 0;
-  const size_t o_top = off;   off = align_up(off + 256, 256);
-  const size_t o_meta = off;  off = align_up(off + (size_t)P.S * P.P * sizeof(PoolMeta), 256);
-  const size_t o_order = off; off = align_up(off + SN * sizeof(int), 256);
-  const size_t o_tmin = off;  off = align_up(off + SN * sizeof(i64), 256);
-  size_t per_cand = 8 + 8 + 4 + 4 + 4 + 4 + 4 + 3 + 16 * (size_t)desc->depth;
-  size_t slab = align_up((size_t)P.N * per_cand + 64 * 1024 + (1 << 20) / 4 + 4096, 256);
-  const int wpb = K2_THREADS / 32;
-  if (off + arena_min + slab * wpb > budget) return TANGRAM_ETOOBIG;
-  size_t workers = (budget - off - arena_min) / slab / wpb * wpb;
-  size_t wanted = align_up((size_t)P.S * P.P, wpb);
-  if (workers > wanted) workers = wanted;
-  if (workers > 32) workers = 32;                       // keep most of the array for DP tables
-  const size_t o_slabs = off; off += workers * slab;
-  const size_t o_arena = off;
+  const size_t per_cand = 8 + 8 + 4 + 4 + 4 + 4 + 4 + 3 + 16 * (size_t)desc->depth;
+  const size_t slab = align_up((size_t)P.N * per_cand + 64 * 1024 + (1 << 20) / 4 + 4096, 256);
+  if (256 + align_up((size_t)P.S * P.P * sizeof(PoolMeta), 256) + align_up(SN * sizeof(int), 256) + align_up(SN * sizeof(i64), 256) +
+      arena_min + slab * (K2_THREADS / 32) > budget) return TANGRAM_ETOOBIG;
+  const size_t b_meta = align_up((size_t)P.P * sizeof(PoolMeta), 256), b_order = align_up((size_t)P.cand_stride * sizeof(int), 256),
+               b_tmin = align_up((size_t)P.P * P.N * sizeof(i64), 256), room = budget - arena_min - 256;
+  int wpb = P.P;                                           // the rows of one block are per pool: with many pools of long queues
+  while (wpb > 1 && b_meta + b_order + b_tmin + slab * wpb > room) --wpb;   // a block has fewer slabs than pools
+  const size_t per_block = b_meta + b_order + b_tmin + slab * wpb;
+  size_t blocks = room / per_block;
+  if (blocks > (size_t)P.S) blocks = (size_t)P.S;
+  if (blocks < 1) return TANGRAM_ETOOBIG;
+  const size_t o_meta = 256, o_order = o_meta + blocks * b_meta, o_tmin = o_order + blocks * b_order, o_slabs = o_tmin + blocks * b_tmin,
+               o_arena = o_slabs + blocks * slab * wpb;
 
   int dev = -1;
   int rc = static_setup(&dev);
   if (rc) return rc;
   unsigned char* base = g_static_ptr[dev];
-  P.arena_top = (u64*)(base + o_top); P.meta = (PoolMeta*)(base + o_meta);
+  P.arena_top = (u64*)base; P.meta = (PoolMeta*)(base + o_meta);
   P.order = (int*)(base + o_order); P.tmin = (i64*)(base + o_tmin);
-  P.slabs = (char*)(base + o_slabs); P.slab_bytes = slab; P.n_workers = (int)workers;
+  P.slabs = (char*)(base + o_slabs); P.slab_bytes = slab; P.n_workers = (int)blocks * wpb;
   P.arena = (char*)(base + o_arena); P.arena_bytes = budget - o_arena;
   P.slot_tries = 50000;
   bind_device_io(P, a, res);
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  CK(cudaMemsetAsync(P.arena_top, 0, 256, st));           // the only part that must start at zero
-  k_prefix<<<P.S, K1_THREADS, P.V * K1_THREADS * sizeof(int), st>>>(P);
-  CK(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
-  k_select<<<P.n_workers / wpb, K2_THREADS, K2_DYN_SMEM, st>>>(P);
+  CK(cudaMemsetAsync(P.arena_top, 0, 256, st));           // whatever an overlapping call may have left
+  k_round<false><<<(unsigned)blocks, K2_THREADS, wpb * WARP_SMEM_BYTES + 16, st>>>(P, wpb);
   CK(cudaGetLastError());
   return TANGRAM_OK;
 }

@@ -76,3 +76,37 @@ def test_replay_queues_beyond_shared_memory_match_oracle(oracle, policy):
         assert np.array_equal(o[k], g[k][:6].cpu().numpy()), k
     assert np.all(o["n_selected"] == N)
     rnd.destroy()
+
+
+def _copies(a, o, n):
+    S = a["n_actions"].shape[0]
+    pick = np.arange(n) % S
+    return {k: None if v is None else v[pick] for k, v in a.items()}, {k: v[pick] for k, v in o.items()}
+
+
+@pytest.mark.parametrize("n", [295, 296, 297, 301])
+@pytest.mark.parametrize("behind", [0, 29, 150])
+def test_batches_around_one_launch_match_oracle(oracle, n, behind):
+    # two blocks on each of 148 multiprocessors: the last batch that is one launch, and the first that is not
+    pools = (Pool(POOL_CPU, 40, 40), Pool(POOL_API, 1, 0, 0))
+    a = _round(n, pools, 33, [0b11, 0b1011, 0b1], 1, behind)
+    a["n_actions"] = np.array([0, 1, 33, 34, a["pool"].shape[1], a["pool"].shape[1] // 2], np.int32)
+    b, want = _copies(a, oracle.schedule_batch(pools, a), n)
+    assert_same(want, gpu_round(pools, b))
+
+
+@pytest.mark.parametrize("n", [3, 40000])
+def test_static_entry_point_with_fewer_warps_than_pools_matches_oracle(oracle, n):
+    # eight pools with rows of 40000 actions leave room for seven worker warps
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = tuple(Pool(POOL_CPU, 40 + j, 40 + j) for j in range(8))
+    rng = np.random.Generator(np.random.PCG64(n))
+    a = dict(pool=rng.integers(0, 8, (1, n)).astype(np.uint8), unit=np.ones((1, n), np.uint8),
+             level_mask=np.full((1, n), 0b1011, np.uint32), arrival_us=None, gpu_busy=None,
+             s_us=rng.integers(0, 50_000, (1, n)), p_us=rng.integers(0, 500_000, (1, n)), n_actions=np.full(1, n, np.int32))
+    want = oracle.schedule_batch(pools, a)
+    got = {k: torch.full(v.shape, -7, dtype=torch.int64 if v.dtype == np.int64 else torch.int32, device="cuda")
+           for k, v in want.items()}
+    assert binding.schedule_batch_static(pools, binding.to_device(a), got) == 0
+    assert_same(want, {k: v.cpu().numpy() for k, v in got.items()})
