@@ -57,6 +57,7 @@ struct Params {
   // outputs (device)
   int* o_alloc; int* o_node; int* o_off; i64* o_act; i64* o_total; int* o_nsel; int* o_status;
   // workspace
+  const int* perm;   // [S][N] the queue in the order it is taken (null: as it stands)
   int* order;        // [S][N] action index at each partitioned position
   i64* tmin;         // [S][N] duration at the least level, partitioned order
   PoolMeta* meta;    // [S][P]

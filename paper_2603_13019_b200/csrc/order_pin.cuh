@@ -1,11 +1,9 @@
 // Front ends of a round that change what the scheduler sees as its queue.
 //
-// k_order (Section 4.2: Algorithm 1 takes the queue in any order): one CTA per scenario sorts the
+// k_order (Section 4.2: Algorithm 1 takes the queue in any order): one block per scenario sorts the
 // queue by a policy key -- least-level duration (Eq. 1) ascending or descending, or arrival time --
-// with the queue position as second key, so equal keys keep their order.  Keys and positions live
-// in shared memory (8 or 12 B per action, padded to a power of two); the sort is a bitonic network.
-// k_gather / k_scatter move the records into sorted order and the results back to the actions' own
-// positions, so the kernels of the round run unchanged on the sorted queue.
+// with the queue position as second key, so equal keys keep their order.  The round then walks the queue through
+// the sorted positions (P.perm) and leaves records and results where the caller has them.
 //
 // k_pin (Section 5.2: per-node CPU scheduling): one warp per scenario walks the queue; the first
 // action of a trajectory pins it to the CPU node (= CPU pool) with the most free memory among those
@@ -14,12 +12,11 @@
 #pragma once
 #include "common.cuh"
 
-#define KO_THREADS 512
 #define KO_MAX_N 16384
+#define KO_MAX_THREADS 512
 
 struct OrderIo {
   int policy;            // 1: shortest least-level duration first, 2: longest first, 3: earliest arrival first
-  int n_pad;             // max_actions rounded up to a power of two
   int* perm;             // [S][N] action index at each sorted position
 };
 
@@ -32,159 +29,116 @@ __device__ __forceinline__ i64 warp_max64_from_m1(i64 v) {
   return (i64)(((u64)mhi << 32) | mlo) - 1;
 }
 
-__device__ __forceinline__ bool ko_less(u64 ka, u32 ia, u64 kb, u32 ib) { return ka < kb || (ka == kb && ia < ib); }
-
-// WIDE = false: duration keys stay below 2^42 and positions below 2^14, so key and position are one 64-bit
-// word (8 B per action); WIDE = true (arrival times, any 64-bit value): key and position side by side (12 B).
-template <bool WIDE>
-__global__ void __launch_bounds__(KO_THREADS) k_order(const __grid_constant__ Params P, const OrderIo O) {
-  extern __shared__ __align__(16) unsigned char ko_smem[];
-  u64* key = (u64*)ko_smem;
-  u32* idx = (u32*)(key + O.n_pad);                    // WIDE only
-  const int sc = blockIdx.x, t = threadIdx.x;
-  const size_t row = (size_t)sc * P.N;
-  const int n = min(max(P.n_actions[sc], 0), P.N);
-  for (int i = t; i < O.n_pad; i += KO_THREADS) {
-    u64 k = ~0ull;                                     // padding and the positions behind the queue stay where they are
-    if (i < n) {
-      if (WIDE) k = (u64)(P.a_arrival ? P.a_arrival[row + i] : 0) ^ 0x8000000000000000ull;
-      else {
-        const int j = P.a_pool[row + i];
-        int g, gang; u32 eff;
-        i64 T = 0;                                     // a record no pool can serve has key 0
-        if (j < P.P && decode_levels(P.pool[j], P.a_unit[row + i], P.a_mask[row + i], g, gang, eff))
-          T = duration(clamp_param(P.a_s[row + i]), clamp_param(P.a_p[row + i]), __ffs(eff));
-        k = O.policy == 2 ? (u64)((1ll << 42) - T) : (u64)T;
-      }
-    }
-    if (WIDE) { key[i] = k; idx[i] = (u32)i; }
-    else key[i] = i < n ? (k << 14) | (u64)i : (~0ull << 14) | (u64)i;
-  }
-  __syncthreads();
-  for (int size = 2; size <= O.n_pad; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int x = t; x < O.n_pad / 2; x += KO_THREADS) {
-        // pair (lo, lo + stride); ascending where bit `size` of lo is clear
-        const int lo = ((x & ~(stride - 1)) << 1) | (x & (stride - 1)), hi = lo + stride;
-        const u64 ka = key[lo], kb = key[hi];
-        const bool up = (lo & size) == 0;
-        if (WIDE) {
-          const u32 ia = idx[lo], ib = idx[hi];
-          if (ko_less(kb, ib, ka, ia) == up) { key[lo] = kb; key[hi] = ka; idx[lo] = ib; idx[hi] = ia; }
-        } else if ((kb < ka) == up) { key[lo] = kb; key[hi] = ka; }
-      }
-      __syncthreads();
-    }
-  }
-  for (int i = t; i < P.N; i += KO_THREADS) O.perm[row + i] = WIDE ? (int)idx[i] : (int)(key[i] & 0x3fffu);
+// The key an action is sorted by, smallest first.
+__device__ __forceinline__ u64 order_key(const Params& P, int policy, size_t o) {
+  if (policy == 3) return (u64)(P.a_arrival ? P.a_arrival[o] : 0) ^ 0x8000000000000000ull;
+  const int j = P.a_pool[o];
+  int g, gang; u32 eff;
+  i64 T = 0;                                           // a record no pool can serve has key 0
+  if (j < P.P && decode_levels(P.pool[j], P.a_unit[o], P.a_mask[o], g, gang, eff))
+    T = duration(clamp_param(P.a_s[o]), clamp_param(P.a_p[o]), __ffs(eff));
+  return policy == 2 ? (u64)((1ll << 42) - T) : (u64)T;
 }
 
-// The same sort for the duration keys when the padded queue gives every thread EPT >= 1 whole elements
-// (thread t holds positions t * EPT .. t * EPT + EPT - 1 in registers): compare-exchanges at strides below EPT
-// stay inside a thread, strides below 32 * EPT go through warp shuffles, and only the strides beyond that
-// through shared memory (one conflict-free store / load of every element per such stage).
+// One block per scenario, EPT actions per thread in registers: element e of a lane is position warp * 32 * EPT + 32 * e + lane
+// of the queue.  A radix sort from the low end, eight bits at a time: a warp ranks its elements by a match and its own
+// counters, one scan over (digit, warp) gives every warp its place for every digit, and one trip through shared
+// memory puts the elements there; each step keeps the order of equal digits.  Only digits in which the keys of the
+// queue differ are sorted (durations of minutes: four), and a queue that is in order already is left alone.  A bitonic network took
+// 66 compare steps for 2048 actions where this takes four passes.
+// Key and position share a 64-bit word (50 + 14 bits); where arrival times differ in higher bits than that, the
+// word holds the position alone and the key is read again in every pass.
 template <int EPT>
-__global__ void __launch_bounds__(KO_THREADS) k_order_regs(const __grid_constant__ Params P, const OrderIo O) {
+__global__ void __launch_bounds__(KO_MAX_THREADS) k_order(const __grid_constant__ Params P, const OrderIo O) {
   extern __shared__ __align__(16) unsigned char ko_smem[];
-  u64* sm = (u64*)ko_smem;                             // [EPT][KO_THREADS]
-  const int sc = blockIdx.x, t = threadIdx.x, lane = t & 31;
+  __shared__ u64 s_diff;
+  __shared__ int s_unsorted;
+  __shared__ u32 wsum[KO_MAX_THREADS / 32];
+  u64* buf = (u64*)ko_smem;                            // [EPT * blockDim.x]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+  u32* hist = (u32*)(buf + EPT * blockDim.x);          // [nw][256]
+  u32* mine = hist + warp * 256;
+  const int sc = blockIdx.x, wb = warp * 32 * EPT + lane;
   const size_t row = (size_t)sc * P.N;
   const int n = min(max(P.n_actions[sc], 0), P.N);
+  const u32 lt = (1u << lane) - 1u;
+  if (t == 0) { s_diff = 0; s_unsorted = 0; }
   u64 v[EPT];
 #pragma unroll
   for (int e = 0; e < EPT; ++e) {
-    const int i = t * EPT + e;
-    u64 k = ~0ull << 14;                               // padding and the positions behind the queue stay where they are
-    if (i < n) {
-      const int j = P.a_pool[row + i];
-      int g, gang; u32 eff;
-      i64 T = 0;                                       // a record no pool can serve has key 0
-      if (j < P.P && decode_levels(P.pool[j], P.a_unit[row + i], P.a_mask[row + i], g, gang, eff))
-        T = duration(clamp_param(P.a_s[row + i]), clamp_param(P.a_p[row + i]), __ffs(eff));
-      k = (O.policy == 2 ? (u64)((1ll << 42) - T) : (u64)T) << 14;
-    }
-    v[e] = k | (u64)i;
+    const int i = wb + 32 * e;
+    if (i < n) { v[e] = order_key(P, O.policy, row + i); buf[i] = v[e]; }
   }
-  for (int size = 2; size <= O.n_pad; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (stride < EPT) {
-        // cs is a compile-time copy of the stride, so that v[] stays in registers
-#pragma unroll
-        for (int cs = 1; cs < EPT; cs <<= 1) {
-          if (cs != stride) continue;
-#pragma unroll
-          for (int e = 0; e < EPT; ++e) {
-            if (e & cs) continue;
-            const bool up = ((t * EPT + e) & size) == 0;
-            const u64 a = v[e], b = v[e | cs];
-            if ((b < a) == up) { v[e] = b; v[e | cs] = a; }
-          }
-        }
-      } else if (stride < 32 * EPT) {
-        const int m = stride / EPT;                    // partner lane = lane ^ m
-        const bool lower = (lane & m) == 0;
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          const u64 o = __shfl_xor_sync(TG_FULL, v[e], m);
-          const bool up = ((t * EPT + e) & size) == 0;
-          const u64 lo_v = o < v[e] ? o : v[e], hi_v = o < v[e] ? v[e] : o;
-          v[e] = (lower == up) ? lo_v : hi_v;
-        }
-      } else {
-        const int m = stride / EPT;                    // partner thread = t ^ m
-        const bool lower = (t & m) == 0;
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) sm[e * KO_THREADS + t] = v[e];
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-          const u64 o = sm[e * KO_THREADS + (t ^ m)];
-          const bool up = ((t * EPT + e) & size) == 0;
-          const u64 lo_v = o < v[e] ? o : v[e], hi_v = o < v[e] ? v[e] : o;
-          v[e] = (lower == up) ? lo_v : hi_v;
-        }
-      }
-    }
-  }
-  // through shared memory once more, so that a warp writes consecutive positions
   __syncthreads();
+  u64 diff = 0;
+  bool unsorted = false;
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) ((u32*)sm)[t * EPT + e] = (u32)(v[e] & 0x3fffu);
+  for (int e = 0; e < EPT; ++e) {
+    const int i = wb + 32 * e;
+    if (i < n) { diff |= v[e] ^ buf[0]; unsorted |= i + 1 < n && buf[i + 1] < v[e]; }
+  }
+  if (unsorted) s_unsorted = 1;
+  const u32 dlo = __reduce_or_sync(TG_FULL, (u32)diff), dhi = __reduce_or_sync(TG_FULL, (u32)(diff >> 32));
+  if (lane == 0) atomicOr((unsigned long long*)&s_diff, ((u64)dhi << 32) | dlo);
   __syncthreads();
-  for (int i = t; i < P.N; i += KO_THREADS) O.perm[row + i] = (int)((u32*)sm)[i];
-}
+  diff = s_unsorted ? s_diff : 0;
+  const bool wide = (diff >> 50) != 0;
+#pragma unroll
+  for (int e = 0; e < EPT; ++e) v[e] = (wide ? 0 : v[e] << 14) | (u64)(u32)(wb + 32 * e);
 
-// the record columns in sorted order
-struct GatherIo {
-  const int* perm;
-  u8* pool; u8* unit; u32* mask; i64* s; i64* p; i64* arrival;     // staged copies (arrival may be null)
-};
-
-__global__ void __launch_bounds__(256) k_gather(const __grid_constant__ Params P, const GatherIo G) {
-  const size_t total = (size_t)P.S * P.N;
-  for (size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (size_t)gridDim.x * blockDim.x) {
-    const size_t row = o - o % P.N;
-    const size_t src = row + G.perm[o];
-    G.pool[o] = P.a_pool[src]; G.unit[o] = P.a_unit[src]; G.mask[o] = P.a_mask[src];
-    G.s[o] = P.a_s[src]; G.p[o] = P.a_p[src];
-    if (G.arrival) G.arrival[o] = P.a_arrival[src];
+#pragma unroll 1
+  for (int sh = 0; sh < 64; sh += 8) {
+    if (((diff >> sh) & 255) == 0) continue;
+    auto digit = [&](u64 x) -> u32 {
+      return (u32)((wide ? order_key(P, O.policy, row + (size_t)(x & 0x3fff)) : x >> 14) >> sh) & 255u;
+    };
+    u32 rank[EPT];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) mine[32 * x + lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+      if (wb - lane + 32 * e >= n) continue;           // nothing there for the whole warp
+      const bool on = wb + 32 * e < n;
+      const u32 d = on ? digit(v[e]) : 256u + lane;
+      const u32 peers = __match_any_sync(TG_FULL, d);
+      const u32 before = on ? mine[d] : 0;
+      rank[e] = before + __popc(peers & lt);
+      __syncwarp();
+      if (on && !(peers & lt)) mine[d] = before + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    // the digits in order, and for every digit the warps in order: where each warp's elements begin
+    const int dp = blockDim.x < 256 ? 256 / blockDim.x : 1;
+    u32 sum = 0;
+    if (t * dp < 256)
+#pragma unroll 1
+      for (int x = 0; x < dp; ++x)
+        for (int w = 0; w < nw; ++w) sum += hist[w * 256 + t * dp + x];
+    u32 incl = sum;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) { const u32 y = __shfl_up_sync(TG_FULL, incl, s); if (lane >= s) incl += y; }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    u32 off = incl - sum;
+    for (int w = 0; w < warp; ++w) off += wsum[w];
+    if (t * dp < 256)
+#pragma unroll 1
+      for (int x = 0; x < dp; ++x)
+        for (int w = 0; w < nw; ++w) { u32& h = hist[w * 256 + t * dp + x]; const u32 c = h; h = off; off += c; }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < EPT; ++e)
+      if (wb + 32 * e < n) buf[mine[digit(v[e])] + rank[e]] = v[e];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < EPT; ++e)
+      if (wb + 32 * e < n) v[e] = buf[wb + 32 * e];
   }
-}
-
-// the results back at the actions' own positions
-struct ScatterIo {
-  const int* perm;
-  const int* alloc; const int* node; const int* off; const i64* act;   // staged results, sorted order
-  int* o_alloc; int* o_node; int* o_off; i64* o_act;
-};
-
-__global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Params P, const ScatterIo X) {
-  const size_t total = (size_t)P.S * P.N;
-  for (size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (size_t)gridDim.x * blockDim.x) {
-    const size_t dst = o - o % P.N + X.perm[o];
-    X.o_alloc[dst] = X.alloc[o]; X.o_node[dst] = X.node[o]; X.o_off[dst] = X.off[o]; X.o_act[dst] = X.act[o];
-  }
+#pragma unroll
+  for (int e = 0; e < EPT; ++e)                        // the positions behind the queue stay where they are
+    if (wb + 32 * e < P.N) O.perm[row + wb + 32 * e] = (int)(v[e] & 0x3fff);
 }
 
 struct PinIo {

@@ -131,11 +131,15 @@ __device__ __forceinline__ void head_walk(const Params& P, int sc, int ws, HeadS
     nk0 = P.a_side_pool[row + lane]; nu0 = P.a_side_units[row + lane];
     if (P.n_side > 1) { nk1 = P.a_side_pool[P.side_plane + row + lane]; nu1 = P.a_side_units[P.side_plane + row + lane]; }
   }
-  if (lane < n_act) { nj = P.a_pool[row + lane]; nun = P.a_unit[row + lane]; nmk = P.a_mask[row + lane]; ns = P.a_s[row + lane]; np_ = P.a_p[row + lane]; }
+  int nsrc = lane;                                  // where in the row the queue's next action is
+  if (lane < n_act) {
+    if (P.perm) nsrc = P.perm[row + lane];
+    nj = P.a_pool[row + nsrc]; nun = P.a_unit[row + nsrc]; nmk = P.a_mask[row + nsrc]; ns = P.a_s[row + nsrc]; np_ = P.a_p[row + nsrc];
+  }
   for (int c0 = 0; c0 < n_act; c0 += 32) {
     const int i = c0 + lane;
     const bool present = i < n_act;
-    const int j = nj; const u32 un = nun, mk = nmk; const i64 s = ns, p = np_;
+    const int j = nj, src = nsrc; const u32 un = nun, mk = nmk; const i64 s = ns, p = np_;
     const int k0 = nk0, k1 = nk1;
     int su0 = nu0, su1 = nu1;
     if (SIDE) {
@@ -148,8 +152,11 @@ __device__ __forceinline__ void head_walk(const Params& P, int sc, int ws, HeadS
     }
     {
       const int i2 = i + 32;
-      nj = 0; nun = 0; nmk = 0; ns = 0; np_ = 0;
-      if (i2 < n_act) { nj = P.a_pool[row + i2]; nun = P.a_unit[row + i2]; nmk = P.a_mask[row + i2]; ns = P.a_s[row + i2]; np_ = P.a_p[row + i2]; }
+      nj = 0; nun = 0; nmk = 0; ns = 0; np_ = 0; nsrc = i2;
+      if (i2 < n_act) {
+        if (P.perm) nsrc = P.perm[row + i2];
+        nj = P.a_pool[row + nsrc]; nun = P.a_unit[row + nsrc]; nmk = P.a_mask[row + nsrc]; ns = P.a_s[row + nsrc]; np_ = P.a_p[row + nsrc];
+      }
     }
     bool valid = present && j < P.P;
     const u32 pi = __shfl_sync(TG_FULL, pinfo, valid ? j : 0);
@@ -201,7 +208,7 @@ __device__ __forceinline__ void head_walk(const Params& P, int sc, int ws, HeadS
       if (lane == jj) { cnt += __popc(b); mreg += __popc(b & below_f); }
     }
     if (cand) {
-      P.order[(size_t)ws * P.cand_stride + P.cand_off[j] + pos] = i;
+      P.order[(size_t)ws * P.cand_stride + P.cand_off[j] + pos] = src;
       if (eff & (eff - 1)) el |= 1u << j;
     }
     for (int v = 0; v < D; ++v) {
@@ -226,7 +233,8 @@ __device__ __forceinline__ void head_walk(const Params& P, int sc, int ws, HeadS
         P.tmin[prow + (size_t)j * P.N + pos] = duration(clamp_param(s), clamp_param(p), rmin);
       for (int jj = 0; jj < P.P; ++jj) {               // the pool's first waiting action
         const u32 b = __ballot_sync(TG_FULL, waits && j == jj && pos == mj);
-        if (lane == jj && b) fwreg = c0 + __ffs(b) - 1;
+        const int fw = __shfl_sync(TG_FULL, src, b ? __ffs(b) - 1 : 0);
+        if (lane == jj && b) fwreg = fw;
       }
       hs = min(c0 + 32, n_act); n_pref = c0 + f;
       break;
@@ -289,16 +297,61 @@ struct StreamShared {
   int m[TG_MAX_POOLS], first[TG_MAX_POOLS], cur[TG_MAX_POOLS], scan[KS_THREADS / 32];
   int bad;
 };
+// The waiting lists of a queue that is taken in another order than it stands in: four positions of the order per thread,
+// their records gathered from the row, which one block reads whole and so finds in L1.  Bound by the latency of those
+// gathers; copying the records into order first, and the results back, took twice the traffic of the round itself.
+__device__ __forceinline__ void stream_sorted(const Params& P, int sc, int ws, const HeadState& H, StreamShared& X, int t) {
+  const size_t row = (size_t)sc * P.N, prow = (size_t)ws * P.P * P.N;
+  const int n_act = min(max(P.n_actions[sc], 0), P.N);
+#pragma unroll 1
+  for (int tile0 = H.hs; tile0 < n_act; tile0 += KS_THREADS * 4) {
+    int src[4], pl[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { const int i = tile0 + 4 * t + k; src[k] = i < n_act ? P.perm[row + i] : -1; }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) pl[k] = src[k] >= 0 ? P.a_pool[row + src[k]] : 0xff;
+    i64 T[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      T[k] = 0;
+      if (pl[k] < P.P && ((H.need >> pl[k]) & 1u)) {
+        const u32 eff = P.a_mask[row + src[k]] & X.ok[pl[k] * 256 + P.a_unit[row + src[k]]];
+        if (eff) T[k] = duration(clamp_param(P.a_s[row + src[k]]), clamp_param(P.a_p[row + src[k]]), __ffs(eff));   // 0: the scenario is flagged
+      }
+    }
+#pragma unroll 1
+    for (u32 nm = H.need; nm; nm &= nm - 1) {
+      const int j = __ffs(nm) - 1;
+      const int mine = (pl[0] == j) + (pl[1] == j) + (pl[2] == j) + (pl[3] == j), before = X.cur[j];
+      int tot;
+      int pos = before + ks_block_scan(mine, X.scan, t, &tot);
+      if (t == 0) X.cur[j] = before + tot;
+      const int m_j = X.m[j];
+      i64* dst = P.tmin + prow + (size_t)j * P.N;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (pl[k] != j) continue;
+        dst[pos] = T[k];
+        if (pos == m_j) X.first[j] = src[k];
+        ++pos;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // Everything behind the head, by a block of KS_THREADS.  The waiting lists' facts go to the pools' PoolMeta.
+// SORTED: the queue is taken in the order P.perm.
+template <bool SORTED>
 __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, const HeadState& H, StreamShared& X, int t) {
   const size_t row = (size_t)sc * P.N;
   const size_t prow = (size_t)ws * P.P * P.N;
   const int n_act = min(max(P.n_actions[sc], 0), P.N);
-  const u32 need = H.need;
+  const u32 need = SORTED ? 0 : H.need;             // taken in another order: this pass only looks for invalid records
   // 128-bit loads need groups that start at multiples of 16 of the whole array, wherever the row begins: the first tile
   // starts up to 15 records early and skips them
   const bool vec = (((size_t)P.a_pool | (size_t)P.a_unit | (size_t)P.a_mask) & 15) == 0;
-  const int hs = H.hs, skew = vec ? (int)((row + hs) & 15) : 0;
+  const int hs = SORTED ? 0 : H.hs, skew = vec ? (int)((row + hs) & 15) : 0;
   if (t < TG_MAX_POOLS) {
     X.m[t] = t < P.P ? P.meta[(size_t)ws * P.P + t].m : 0;
     X.first[t] = INT_MAX;
@@ -390,6 +443,7 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
     }
     __syncthreads();
   }
+  if (SORTED && H.need) stream_sorted(P, sc, ws, H, X, t);
   __syncthreads();
   const bool bad = X.bad != 0;
   // nobody will write the candidates of a bad scenario: their rows are "not scheduled" too
@@ -399,7 +453,7 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
   if (t < P.P) {
     PoolMeta* mt = P.meta + (size_t)ws * P.P + t;
     if (bad) { mt->count = 0; mt->m = 0; mt->first_wait = -1; }
-    else if ((need >> t) & 1u) {
+    else if ((H.need >> t) & 1u) {
       mt->count = X.cur[t];
       if (X.first[t] != INT_MAX) mt->first_wait = X.first[t];
     } else mt->count = mt->m;                          // a list nobody reads counts as empty
@@ -408,9 +462,10 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
   if (t == 0 && bad) atomicOr(&P.o_status[sc], TG_ST_BAD_ACTION);
 }
 
+template <bool SORTED>
 __global__ void __launch_bounds__(KS_THREADS, 5) k_stream(const __grid_constant__ Params P, const HeadState* hst) {
   __shared__ StreamShared X;
-  stream_queue(P, blockIdx.x, blockIdx.x, hst[blockIdx.x], X, threadIdx.x);
+  stream_queue<SORTED>(P, blockIdx.x, blockIdx.x, hst[blockIdx.x], X, threadIdx.x);
 }
 
 // "not scheduled" (Eq. 2 has no value for an action that stays queued): units 0, node -1, offset -1,
@@ -437,17 +492,17 @@ __global__ void __launch_bounds__(256) k_fill(const __grid_constant__ Params P, 
     for (u32 q = tid; q <= (total - 1) / 4; q += stride) {
       const u32 o = q * 4, sc = o / N, i0 = o - sc * N;
       if (i0 + 4 <= N) {
-        const int left = (int)i0 - hst[sc].n;
+        const int left = (int)i0 - (P.perm ? 0 : hst[sc].n);   // with an order of its own the candidates are anywhere
         if (left >= 0) { write_unscheduled4(P, o); continue; }
         for (int k = max(-left, 0); k < 4; ++k) write_unscheduled(P, (size_t)o + k);
       } else
         for (u32 k = 0, s = sc, i = i0; k < 4 && o + k < total; ++k, ++i) {
           if (i == N) { i = 0; ++s; }
-          if ((int)i >= hst[s].n) write_unscheduled(P, (size_t)o + k);
+          if (P.perm || (int)i >= hst[s].n) write_unscheduled(P, (size_t)o + k);
         }
     }
   } else {
     for (u32 o = tid; o < total; o += stride)
-      if ((int)(o % N) >= hst[o / N].n) write_unscheduled(P, o);
+      if (P.perm || (int)(o % N) >= hst[o / N].n) write_unscheduled(P, o);
   }
 }

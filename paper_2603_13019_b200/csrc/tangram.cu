@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
 // batch is latency, and one launch instead of four (and a memset) saves the gaps.  The last block to finish resets
 // the bump pointer of the arena for the next call.  1 x 64: 38.6 -> 26.8 us a call, 16 x 500 (static): 110 -> 84 us.
 #define TG_DONE_COUNTER 4           // word of arena_top that counts finished blocks
-template <bool SIDE>
+template <bool SIDE, bool SORTED>
 __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__ Params P, int wpb) {
   __shared__ StreamShared X;
   __shared__ HeadState H;
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__
     } else
       for (int i = t - 32; i < P.N; i += K2_THREADS - 32) write_unscheduled(P, row + i);
     __syncthreads();
-    stream_queue(P, sc, ws, H, X, t);
+    stream_queue<SORTED>(P, sc, ws, H, X, t);
     __syncthreads();
 #pragma unroll 1
     for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
@@ -389,8 +389,8 @@ struct tangram_round {
   cudaEvent_t io_begin, io_end, io_in_done[TG_IO_CHUNKS], io_comp_done[TG_IO_CHUNKS];
   // the output fill runs beside the other kernels of a round
   cudaStream_t side; cudaEvent_t side_fork, side_join;
-  // sorted copy of the queue and of its results (tangram_schedule_batch_ordered), allocated at its first call
-  char* d_sorted; int* d_perm; u64* d_wkey;
+  // the sorted order of tangram_schedule_batch_ordered, allocated at its first call
+  int* d_perm; u64* d_wkey;
   // staging for host-buffer mode
   char* d_stage; size_t stage_bytes;
   size_t in_off[8], out_off[9];
@@ -631,8 +631,9 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   P.slabs = (char*)r->d_slabs; P.arena = (char*)r->d_arena; P.arena_top = (u64*)r->d_arena_top;
   e = cudaMemset(r->d_arena_top, 0, 256);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
@@ -694,7 +695,7 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   if (!r) return;
   if (r->ev) tangram_set_profiling(r, 0);
   cudaFree(r->d_order); cudaFree(r->d_tmin); cudaFree(r->d_meta); cudaFree(r->d_slabs);
-  cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_sorted); cudaFree(r->d_perm); cudaFree(r->d_wkey);
+  cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_perm); cudaFree(r->d_wkey);
   cudaFree(r->R.wait); cudaFree(r->R.run_fin); cudaFree(r->R.run_idx); cudaFree(r->R.run_pu); cudaFree(r->R.run_off); cudaFree(r->R.run_dom); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.dfree);
   cudaFree(r->R.pst); cudaFree(r->R.win);
   if (r->io_in) cudaStreamDestroy(r->io_in);
@@ -772,14 +773,28 @@ static void bind_device_io(Params& P, const tangram_actions* a, const tangram_re
 }
 
 // The kernels of one round for the scenarios that P describes, on stream st.
+static bool one_launch(const tangram_round* r) {           // all blocks of k_round are resident at once
+  return r->P.S <= TG_FUSED_PER_SM * r->n_sm && r->P.S * r->P.P <= r->P.n_workers;
+}
+
+static int launch_fill(tangram_round* r, const Params& P, cudaStream_t st) {
+  CK(cudaEventRecord(r->side_fork, st));
+  CK(cudaStreamWaitEvent(r->side, r->side_fork, 0));
+  size_t blocks = ((size_t)P.S * ((P.N + 3) / 4) + 255) / 256;
+  if (blocks > (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM) blocks = (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM;
+  k_fill<<<(unsigned)blocks, 256, 0, r->side>>>(P, r->hst);
+  CK(cudaEventRecord(r->side_join, r->side));
+  return TANGRAM_OK;
+}
+
 static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, bool timed) {
-  const bool fused = r->P.S <= TG_FUSED_PER_SM * r->n_sm && r->P.S * P.P <= P.n_workers;   // all blocks resident at once
-  if (fused) {
+  if (one_launch(r)) {
     cudaEvent_t* ev = timed ? prof_begin(r, 1, -1, -1) : nullptr;
     if (ev) CK(cudaEventRecord(ev[0], st));
     const int smem = P.P * WARP_SMEM_BYTES + 16;
-    if (P.n_side > 0) k_round<true><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
-    else k_round<false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    if (P.n_side > 0) k_round<true, false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    else if (P.perm) k_round<false, true><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    else k_round<false, false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
     if (ev) CK(cudaEventRecord(ev[1], st));
     r->launches += 1;
     CK(cudaGetLastError());
@@ -798,18 +813,13 @@ static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, bool
   if (P.n_side > 0) k_head<true><<<(P.S + 7) / 8, 256, 0, st>>>(P, r->hst);
   else k_head<false><<<(P.S + 7) / 8, 256, 0, st>>>(P, r->hst);
   if (ev) CK(cudaEventRecord(ev[1], st));
-  {                                                        // the output fill runs beside everything that follows
-    CK(cudaEventRecord(r->side_fork, st));
-    CK(cudaStreamWaitEvent(r->side, r->side_fork, 0));
-    size_t blocks = ((size_t)P.S * ((P.N + 3) / 4) + 255) / 256;
-    if (blocks > (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM) blocks = (size_t)r->n_sm * TG_FILL_BLOCKS_PER_SM;
-    k_fill<<<(unsigned)blocks, 256, 0, r->side>>>(P, r->hst);
-    CK(cudaEventRecord(r->side_join, r->side));
-  }
-  k_stream<<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
+  if (!P.perm) { const int rc = launch_fill(r, P, st); if (rc) return rc; }   // beside everything that follows
+  if (P.perm) k_stream<true><<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
+  else k_stream<false><<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
   if (ev) CK(cudaEventRecord(ev[2], st));
+  if (P.perm) CK(cudaStreamWaitEvent(st, r->side_join, 0));   // it wrote the candidates' rows as well
   k_pool<<<P.n_workers / (K2_THREADS / 32), K2_THREADS, K2_DYN_SMEM, st>>>(P, r->hst);
-  CK(cudaStreamWaitEvent(st, r->side_join, 0));            // the fill is part of the round
+  if (!P.perm) CK(cudaStreamWaitEvent(st, r->side_join, 0));  // the fill is part of the round
   if (ev) CK(cudaEventRecord(ev[3], st));
   r->launches += 4;
   CK(cudaGetLastError());
@@ -956,27 +966,18 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
 // ---------------------------------------------------------------------------------------
 // Other queue orders (Section 4.2) and trajectories pinned to CPU nodes (Section 5.2)
 // ---------------------------------------------------------------------------------------
-static int next_pow2(int v) { int p = 1; while (p < v) p <<= 1; return p; }
-
+// Threads and actions per thread of the sort: enough blocks on an SM to hide its barriers, and few idle threads on short queues.
 static int launch_order(tangram_round* r, const Params& P, int policy, int* perm, cudaStream_t st) {
   OrderIo O;
-  O.policy = policy; O.n_pad = next_pow2(P.N); O.perm = perm;
-  const bool wide = policy == 3;
-  if (!wide && O.n_pad >= KO_THREADS) {                  // whole elements per thread: the register version
-    const int ept = O.n_pad / KO_THREADS;
-    const size_t sm = (size_t)O.n_pad * 8;
-    void (*kern)(Params, OrderIo) = ept == 1 ? k_order_regs<1> : ept == 2 ? k_order_regs<2> : ept == 4 ? k_order_regs<4> :
-                                    ept == 8 ? k_order_regs<8> : ept == 16 ? k_order_regs<16> : k_order_regs<32>;
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    kern<<<P.S, KO_THREADS, sm, st>>>(P, O);
-    r->launches += 1;
-    CK(cudaGetLastError());
-    return TANGRAM_OK;
-  }
-  const size_t smem = (size_t)O.n_pad * (wide ? 12 : 8);
-  CK(cudaFuncSetAttribute(wide ? k_order<true> : k_order<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  if (wide) k_order<true><<<P.S, KO_THREADS, smem, st>>>(P, O);
-  else k_order<false><<<P.S, KO_THREADS, smem, st>>>(P, O);
+  O.policy = policy; O.perm = perm;
+  const int threads = P.N <= 512 ? 128 : P.N <= 2048 ? 256 : KO_MAX_THREADS;
+  int ept = 1;
+  while (ept * threads < P.N) ept <<= 1;
+  const size_t sm = (size_t)ept * threads * 8 + (size_t)threads / 32 * 1024;
+  void (*kern)(Params, OrderIo) = ept == 1 ? k_order<1> : ept == 2 ? k_order<2> : ept == 4 ? k_order<4> :
+                                  ept == 8 ? k_order<8> : ept == 16 ? k_order<16> : k_order<32>;
+  if (sm > 40 * 1024) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  kern<<<P.S, threads, sm, st>>>(P, O);
   r->launches += 1;
   CK(cudaGetLastError());
   return TANGRAM_OK;
@@ -1008,40 +1009,14 @@ extern "C" int tangram_schedule_batch_ordered(tangram_round* r, const tangram_ac
   Params P = r->P;
   P.now = now_us;
   bind_device_io(P, a, res);
-  const size_t SN = (size_t)P.S * P.N;
-  // sorted records (pool, unit, mask, s, p, arrival) and sorted results (alloc, node, off, act): 50 B per action
-  const size_t off_unit = align_up(SN, 256), off_mask = off_unit + align_up(SN, 256), off_s = off_mask + align_up(SN * 4, 256),
-               off_p = off_s + SN * 8, off_arr = off_p + SN * 8, off_alloc = off_arr + SN * 8, off_node = off_alloc + SN * 4,
-               off_off = off_node + SN * 4, off_act = align_up(off_off + SN * 4, 256), total = off_act + SN * 8;
-  if (!r->d_sorted) {
-    if (cudaMalloc((void**)&r->d_sorted, total) != cudaSuccess || cudaMalloc((void**)&r->d_perm, SN * sizeof(int)) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(r->d_sorted); cudaFree(r->d_perm); cudaFree(r->d_wkey); r->d_sorted = nullptr; r->d_perm = nullptr;
-      return TANGRAM_ENOMEM;
-    }
+  if (!r->d_perm && cudaMalloc((void**)&r->d_perm, (size_t)P.S * P.N * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError(); r->d_perm = nullptr;
+    return TANGRAM_ENOMEM;
   }
-  char* d = r->d_sorted;
-  int rc = launch_order(r, P, policy, r->d_perm, st);
-  if (rc) return rc;
-  GatherIo G;
-  G.perm = r->d_perm; G.pool = (u8*)d; G.unit = (u8*)(d + off_unit); G.mask = (u32*)(d + off_mask);
-  G.s = (i64*)(d + off_s); G.p = (i64*)(d + off_p); G.arrival = P.a_arrival ? (i64*)(d + off_arr) : nullptr;
-  size_t blocks = (SN + 255) / 256;
-  if (blocks > (size_t)r->n_sm * 32) blocks = (size_t)r->n_sm * 32;
-  k_gather<<<(unsigned)blocks, 256, 0, st>>>(P, G);
-  // the round itself, on the sorted copy; the per-scenario results go straight to the caller
-  Params Q = P;
-  Q.a_pool = G.pool; Q.a_unit = G.unit; Q.a_mask = G.mask; Q.a_s = G.s; Q.a_p = G.p; Q.a_arrival = G.arrival;
-  Q.o_alloc = (int*)(d + off_alloc); Q.o_node = (int*)(d + off_node); Q.o_off = (int*)(d + off_off); Q.o_act = (i64*)(d + off_act);
-  rc = run_pipeline(r, Q, st, false);
-  if (rc) return rc;
-  ScatterIo X;
-  X.perm = r->d_perm; X.alloc = Q.o_alloc; X.node = Q.o_node; X.off = Q.o_off; X.act = Q.o_act;
-  X.o_alloc = P.o_alloc; X.o_node = P.o_node; X.o_off = P.o_off; X.o_act = P.o_act;
-  k_scatter<<<(unsigned)blocks, 256, 0, st>>>(P, X);
-  r->launches += 2;
-  CK(cudaGetLastError());
-  return TANGRAM_OK;
+  P.perm = r->d_perm;
+  if (!one_launch(r)) { const int rc = launch_fill(r, P, st); if (rc) return rc; }   // beside the sort
+  const int rc = launch_order(r, P, policy, r->d_perm, st);
+  return rc ? rc : run_pipeline(r, P, st, false);
 }
 
 extern "C" int tangram_pin_trajectories(tangram_round* r, const tangram_actions* a, const tangram_pinning* pin,
@@ -1084,7 +1059,7 @@ static int static_setup(int* dev_out) {
     unsigned char* ptr = nullptr;
     CK(cudaGetSymbolAddress((void**)&ptr, g_static_scratch));
     CK(fill_tables());
-    CK(cudaFuncSetAttribute(k_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
+    CK(cudaFuncSetAttribute(k_round<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
     g_static_ptr[dev] = ptr;
     g_static_ready[dev] = true;
   }
@@ -1158,7 +1133,7 @@ extern "C" int tangram_schedule_batch_static(const tangram_round_desc* desc, con
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));           // whatever an overlapping call may have left
-  k_round<false><<<(unsigned)blocks, K2_THREADS, wpb * WARP_SMEM_BYTES + 16, st>>>(P, wpb);
+  k_round<false, false><<<(unsigned)blocks, K2_THREADS, wpb * WARP_SMEM_BYTES + 16, st>>>(P, wpb);
   CK(cudaGetLastError());
   return TANGRAM_OK;
 }

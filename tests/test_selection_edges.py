@@ -110,3 +110,19 @@ def test_static_entry_point_with_fewer_warps_than_pools_matches_oracle(oracle, n
            for k, v in want.items()}
     assert binding.schedule_batch_static(pools, binding.to_device(a), got) == 0
     assert_same(want, {k: v.cpu().numpy() for k, v in got.items()})
+
+
+@pytest.mark.parametrize("n", [1, 31, 128, 129, 512, 513, 2049, 16384])
+@pytest.mark.parametrize("lo,hi", [(0, 3), (-40, 40), (-2**62, 2**62), (7, 8)])
+def test_sorted_orders_match_oracle(oracle, n, lo, hi):
+    # edges of the sort's tiles; few, mixed-sign, 64-bit and equal arrival times; one queue in order already
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, 64, 64), Pool(POOL_API, 1, 0, 0))
+    rng = np.random.Generator(np.random.PCG64(n))
+    a = dict(pool=np.zeros((4, n), np.uint8), unit=np.ones((4, n), np.uint8), level_mask=np.full((4, n), 0b1011, np.uint32),
+             gpu_busy=None, s_us=rng.integers(0, 50, (4, n)), p_us=rng.integers(0, 1 << 40, (4, n)),
+             arrival_us=rng.integers(lo, hi, (4, n)), n_actions=np.array([n, n // 2, n, 0], np.int32))
+    a["arrival_us"][2].sort()
+    rnd, dev = binding.Round(4, n, pools), binding.to_device(a)
+    for policy in (1, 2, 3):
+        assert np.array_equal(oracle.order_queue(pools, a, policy), rnd.order_queue(dev, policy).cpu().numpy())
