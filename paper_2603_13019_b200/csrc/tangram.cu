@@ -970,10 +970,10 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
 static int launch_order(tangram_round* r, const Params& P, int policy, int* perm, cudaStream_t st) {
   OrderIo O;
   O.policy = policy; O.perm = perm;
-  const int threads = P.N <= 512 ? 128 : P.N <= 2048 ? 256 : KO_MAX_THREADS;
+  const int threads = P.N <= 512 ? 128 : P.N <= 1024 ? 256 : KO_MAX_THREADS;
   int ept = 1;
   while (ept * threads < P.N) ept <<= 1;
-  const size_t sm = (size_t)ept * threads * 8 + (size_t)threads / 32 * 1024;
+  const size_t sm = (size_t)ept * threads * 8 + ko_counter_bytes(ept, threads);
   void (*kern)(Params, OrderIo) = ept == 1 ? k_order<1> : ept == 2 ? k_order<2> : ept == 4 ? k_order<4> :
                                   ept == 8 ? k_order<8> : ept == 16 ? k_order<16> : k_order<32>;
   if (sm > 40 * 1024) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
