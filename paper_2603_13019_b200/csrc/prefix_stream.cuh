@@ -351,12 +351,13 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
   // 128-bit loads need groups that start at multiples of 16 of the whole array, wherever the row begins: the first tile
   // starts up to 15 records early and skips them
   const bool vec = (((size_t)P.a_pool | (size_t)P.a_unit | (size_t)P.a_mask) & 15) == 0;
-  const int hs = SORTED ? 0 : H.hs, skew = vec ? (int)((row + hs) & 15) : 0;
+  const int hs = SORTED && H.hs < n_act ? 0 : H.hs, skew = vec ? (int)((row + hs) & 15) : 0;
   if (t < TG_MAX_POOLS) {
     X.m[t] = t < P.P ? P.meta[(size_t)ws * P.P + t].m : 0;
     X.first[t] = INT_MAX;
   }
-  if (P.ok_table) {
+  if (hs >= n_act) {                                 // the head walk has seen every record: 8 KB of table for nothing
+  } else if (P.ok_table) {
     for (int x = t; x < TG_MAX_POOLS * 256 / 4; x += KS_THREADS) ((uint4*)X.ok)[x] = ((const uint4*)P.ok_table)[x];
   } else {
 #pragma unroll 1
