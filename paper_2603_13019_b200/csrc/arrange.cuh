@@ -85,7 +85,9 @@ __device__ __forceinline__ void slot_release(const Params& P, int s, int lane) {
 }
 
 // One (scenario, pool) at hand.  It lives in the warp's shared memory: the same for all lanes, and the routines
-// below are out of line (each with its own registers) and take what they need of it into locals.
+// below take what they need of it into locals.  They are inlined, one place each in every kernel: a warp that calls
+// waits for the instructions at the other end (a third of all warp cycles at 8192 x 1024 was waiting for instructions; k_pool at 16384 x
+// 4096 1555 us with the routines out of line, 1316 us inlined).
 struct PoolTask {
   // the pool
   int type, group;
@@ -620,7 +622,7 @@ __device__ __forceinline__ int solve_priced(const PoolTask& T0, const PoolTask& 
 // memory does not suffice or a value outgrows its field.
 #define SP_EMPTY 0xffffffffffffffffull
 __device__ __forceinline__ u64 sp_hash(u64 k) { k ^= k >> 29; k *= 0xbf58476d1ce4e5b9ull; k ^= k >> 32; return k; }
-__device__ __noinline__ int dp_sparse(const PoolTask& T, int nrows, const int ext[4], u32 kept,
+__device__ __forceinline__ int dp_sparse(const PoolTask& T, int nrows, const int ext[4], u32 kept,
                                       char* mem, u64 bytes, int lane) {
   // bit fields of a key
   int shift[4], width[4], total_bits = 0;
@@ -801,7 +803,7 @@ __device__ __noinline__ int dp_sparse(const PoolTask& T, int nrows, const int ex
 
 // The whole box of feasible extra-demand vectors (T.rowcand, T.rsel = least levels; maxex[l] = largest extra demand at
 // level l): where the states within a bound do not fit their table, or very many end states tie.  
-__device__ __noinline__ bool solve_box(const Params& P, const PoolTask& T, int q, int nrows, const int maxex[4], u32 kept, Slab slab,
+__device__ __forceinline__ bool solve_box(const Params& P, const PoolTask& T, int q, int nrows, const int maxex[4], u32 kept, Slab slab,
                                        int lane, i64* opt) {
   int ext[4], stride[4];
   u64 cells = 1;
@@ -1072,7 +1074,7 @@ __device__ __forceinline__ bool solve_few(PoolTask& T0, int q, int lane) {
 #define SOLVED_ALL_BEST 2   // every candidate got its best level (then so does every shorter prefix)
 #define SOLVED 1
 #define UNSOLVED 0          // the workspace is too small
-__device__ __noinline__ int solve_prefix(const Params& P, PoolTask& T0, int q, Slab slab, int lane) {
+__device__ __forceinline__ int solve_prefix(const Params& P, PoolTask& T0, int q, Slab slab, int lane) {
   if (q <= FEW_MAX && solve_few(T0, q, lane)) return SOLVED;
   PoolTask T;                                            // (what is used of it, in registers)
   T.type = T0.type; T.cs = T0.cs; T.cp = T0.cp; T.cmask = T0.cmask; T.cg = T0.cg; T.rsel = T0.rsel; T.rowcand = T0.rowcand;

@@ -474,7 +474,7 @@ __device__ __forceinline__ int ev_compare(const PoolTask& T, int q, const u8* ke
 }
 
 // heaps beyond 256 times: windows with the rests in shared memory, or in the slab where they do not fit
-__device__ __noinline__ int ev_compare_windows(const PoolTask& T, int q, const u8* kept, const u8* fewer, i64 fixed, Slab slab, u32 wk, int lane) {
+__device__ __forceinline__ int ev_compare_windows(const PoolTask& T, int q, const u8* kept, const u8* fewer, i64 fixed, Slab slab, u32 wk, int lane) {
   const u32 words = 2u * (u32)(T.n_seeds + q + 1) + 32u, stage = 2 * EV_BLOCK + 4;   // rests; staged durations
   if ((stage + words) * 4u <= T.wk_bytes) return ev_compare(T, q, kept, fewer, fixed, EvShared{wk + stage * 4u}, EvShared{wk}, lane);
   u32* g = (u32*)slab.take((u64)words * 4);
@@ -483,7 +483,7 @@ __device__ __noinline__ int ev_compare_windows(const PoolTask& T, int q, const u
 
 // Does evicting candidate q (the last of the q+1 kept, multiplicities rkeep) lower the objective (rsel, T0.opt: the
 // optimum without it)?  opt_kept: duration sum with it.  1 yes, 0 no, -1 workspace too small.
-__device__ __noinline__ int eviction_pays(const Params& P, const PoolTask& T0, int q, i64 opt_kept, Slab slab, int lane) {
+__device__ __forceinline__ int eviction_pays(const Params& P, const PoolTask& T0, int q, i64 opt_kept, Slab slab, int lane) {
   PoolTask T;                                            // (what is used of it, in registers)
   T.m = uniform(T0.m); T.n_ac = uniform(T0.n_ac); T.n_seeds = uniform(T0.n_seeds); T.depth = T0.depth;
   T.cs = T0.cs; T.cp = T0.cp; T.cmask = T0.cmask; T.ac_tmin = T0.ac_tmin; T.seeds = T0.seeds;

@@ -165,7 +165,7 @@ __device__ __forceinline__ void replay_place_gpu(const PoolDev& pd, u8* nm, int*
 // The selection of a pool with a choice to make: its candidates (among the first n positions) and, where an eviction
 // step can look at them, the waiting actions behind and the running ones are gathered into arrays.
 template <bool EXT>
-__device__ __noinline__ bool replay_select(const Params& P, const ReplayQueue Q, const ReplayRun run, const int* wait, int sc, int j,
+__device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue Q, const ReplayRun run, const int* wait, int sc, int j,
                                            int n, int nw, int nr, int m, i64 now, int cap0, int cap1, int cap2, int cap3, Slab& slab,
                                            CandArrays& C, int& keep, int lane) {
   const size_t row = (size_t)sc * P.N;
