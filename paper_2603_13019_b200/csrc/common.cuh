@@ -138,6 +138,14 @@ __device__ __forceinline__ int warp_sum32(int v) { return (int)__reduce_add_sync
 __device__ __forceinline__ int warp_min32(int v) { return __reduce_min_sync(TG_FULL, v); }
 __device__ __forceinline__ int warp_max32(int v) { return __reduce_max_sync(TG_FULL, v); }
 
+// decode_levels of a full mask, from the table where there is one
+__device__ __forceinline__ u32 usable_levels(const Params& P, int j, int unit) {
+  if (P.ok_table) return P.ok_table[j * 256 + unit];
+  int g, gang; u32 eff;
+  decode_levels(P.pool[j], (u8)unit, 0xffffffffu, g, gang, eff);
+  return eff;
+}
+
 // maximal free aligned blocks of a node: bit = first GPU of such a block (busy: 8 bits, padded)
 struct NodeBlocks { u32 s1, s2, s4, s8; };
 __device__ __forceinline__ NodeBlocks node_blocks(u32 busy) {

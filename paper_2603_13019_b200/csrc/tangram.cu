@@ -81,8 +81,8 @@ __device__ bool gather_candidates(const Params& P, int sc, int j, const PoolMeta
     for (int x = 0; x < 4; ++x) {
       const int i = i0 + 32 * x;
       if (i >= m) break;
-      int g, gang; u32 eff;
-      decode_levels(pd, un[x], mk[x], g, gang, eff);
+      const int g = un[x] & 0x7f, gang = (un[x] >> 7) && pd.type == TG_POOL_GPU;
+      const u32 eff = mk[x] & usable_levels(P, j, un[x]);
       C.cidx[i] = idx[x]; C.cmask[i] = eff; C.cg[i] = (u8)(g | (gang << 7));
       C.cs[i] = clamp_param(sv[x]); C.cp[i] = clamp_param(pv[x]);
       C.rkeep[i] = (u8)__ffs(eff);
@@ -248,8 +248,8 @@ __device__ __forceinline__ void pool_best_levels(const Params& P, int sc, int j,
     size_t o = row; int u = 0; i64 act = 0;
     if (on) {
       o += ord[i];
-      int g, gang; u32 eff;
-      decode_levels(pd, P.a_unit[o], P.a_mask[o], g, gang, eff);
+      const int unit = P.a_unit[o], g = unit & 0x7f;
+      const u32 eff = P.a_mask[o] & usable_levels(P, j, unit);
       const i64 s = clamp_param(P.a_s[o]), p = clamp_param(P.a_p[o]);
       const int r = best_level(p, eff);
       act = (P.now - (P.a_arrival ? P.a_arrival[o] : 0)) + duration(s, p, r);
