@@ -727,13 +727,17 @@ static void bind_stage(tangram_round* r, const tangram_actions* a, Params& P) {
   P.o_status = (int*)(d + r->out_off[6]);
 }
 
+#define IO_IN 8          // input columns, the per-action ones first
+#define IO_IN_ROWS 6
+#define IO_OUT 7         // output columns, the per-action ones first
+#define IO_OUT_ROWS 4
 // inputs of scenarios [s0, s1) host -> staging
-static int copy_in(tangram_round* r, const tangram_actions* a, const Params& P, int s0, int s1, cudaStream_t st) {
+static int copy_in(tangram_round* r, const tangram_actions* a, const Params& P, int s0, int s1, cudaStream_t st, int k0 = 0, int k1 = IO_IN) {
   char* d = r->d_stage;
   const void* src[8] = {a->pool, a->unit, a->level_mask, a->s_us, a->p_us, a->arrival_us, a->n_actions, a->gpu_busy};
   const size_t per[8] = {(size_t)P.N, (size_t)P.N, (size_t)P.N * 4, (size_t)P.N * 8, (size_t)P.N * 8, (size_t)P.N * 8,
                          4, (size_t)P.n_nodes_total};
-  for (int k = 0; k < 8; ++k)
+  for (int k = k0; k < k1; ++k)
     if (src[k] && per[k])
       CK(cudaMemcpyAsync(d + r->in_off[k] + per[k] * s0, (const char*)src[k] + per[k] * s0, per[k] * (s1 - s0),
                          cudaMemcpyHostToDevice, st));
@@ -741,12 +745,12 @@ static int copy_in(tangram_round* r, const tangram_actions* a, const Params& P, 
 }
 
 // results of scenarios [s0, s1) staging -> host
-static int copy_out(tangram_round* r, const tangram_result* res, const Params& P, int s0, int s1, cudaStream_t st) {
+static int copy_out(tangram_round* r, const tangram_result* res, const Params& P, int s0, int s1, cudaStream_t st, int k0 = 0, int k1 = IO_OUT) {
   char* d = r->d_stage;
   void* dst[7] = {res->alloc_units, res->place_node, res->place_off, res->act_us, res->total_act_us,
                   res->n_selected, res->status};
   const size_t per[7] = {(size_t)P.N * 4, (size_t)P.N * 4, (size_t)P.N * 4, (size_t)P.N * 8, 8, 4, 4};
-  for (int k = 0; k < 7; ++k)
+  for (int k = k0; k < k1; ++k)
     CK(cudaMemcpyAsync((char*)dst[k] + per[k] * s0, d + r->out_off[k] + per[k] * s0, per[k] * (s1 - s0),
                        cudaMemcpyDeviceToHost, st));
   return TANGRAM_OK;
@@ -842,7 +846,9 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   // Host buffers: scenarios go through in chunks, so that the copy-in of a chunk, the kernels
   // of the one before and the copy-out of the one before that overlap (three internal streams).
   const size_t bytes = (size_t)P.S * P.N * 42;
-  int C = (int)(bytes >> 26);                              // about 64 MiB of traffic per chunk
+  // A chunk costs about 80 us of calls and start-up.  On PCIe 5 two chunks pay from 16 MB on (67 MB: 1735 -> 1458 us), three
+  // at 189 MB (two 3846, three 3693, eight 4078 us), six or seven at 688 MB (ten 9867, six 9565 us).
+  int C = bytes < ((size_t)16 << 20) ? 1 : 2 + (int)(bytes >> 27);
   if (C > TG_IO_CHUNKS) C = TG_IO_CHUNKS;
   if (C > P.S) C = P.S;
   if (C <= 1 || r->ev) {                                   // small batch, or per-kernel timing wanted
@@ -855,10 +861,12 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
   CK(cudaStreamWaitEvent(r->io_in, r->io_begin, 0));
   CK(cudaStreamWaitEvent(r->io_comp, r->io_begin, 0));
   CK(cudaStreamWaitEvent(r->io_out, r->io_begin, 0));
+  int rc = copy_in(r, a, P, 0, P.S, r->io_in, IO_IN_ROWS, IO_IN);   // what is per scenario, for all chunks
+  if (rc) return rc;
   for (int c = 0; c < C; ++c) {
     const int s0 = (int)((long long)P.S * c / C), s1 = (int)((long long)P.S * (c + 1) / C);
     const size_t o = (size_t)s0 * P.N;
-    int rc = copy_in(r, a, P, s0, s1, r->io_in);
+    rc = copy_in(r, a, P, s0, s1, r->io_in, 0, IO_IN_ROWS);
     if (rc) return rc;
     CK(cudaEventRecord(r->io_in_done[c], r->io_in));
     Params Q = P;                                          // this chunk's view of everything per scenario
@@ -875,9 +883,11 @@ extern "C" int tangram_schedule_batch(tangram_round* r, const tangram_actions* a
     if (rc) return rc;
     CK(cudaEventRecord(r->io_comp_done[c], r->io_comp));
     CK(cudaStreamWaitEvent(r->io_out, r->io_comp_done[c], 0));
-    rc = copy_out(r, res, P, s0, s1, r->io_out);
+    rc = copy_out(r, res, P, s0, s1, r->io_out, 0, IO_OUT_ROWS);
     if (rc) return rc;
   }
+  rc = copy_out(r, res, P, 0, P.S, r->io_out, IO_OUT_ROWS, IO_OUT);
+  if (rc) return rc;
   CK(cudaEventRecord(r->io_end, r->io_out));
   CK(cudaStreamWaitEvent(st, r->io_end, 0));
   return TANGRAM_OK;
