@@ -459,7 +459,7 @@ __device__ __forceinline__ void stream_queue(const Params& P, int sc, int ws, co
       if (X.first[t] != INT_MAX) mt->first_wait = X.first[t];
     } else mt->count = mt->m;                          // a list nobody reads counts as empty
   }
-  // status, total and count were initialised by k_head; k_solve may be adding to them already
+  // (status, total and count were initialised by the head walk)
   if (t == 0 && bad) atomicOr(&P.o_status[sc], TG_ST_BAD_ACTION);
 }
 
