@@ -1180,11 +1180,18 @@ __device__ __forceinline__ int solve_prefix(const Params& P, PoolTask& T0, int q
   u64 cells = 1;                                         // of the box of feasible extra-demand vectors
 #pragma unroll
   for (int l = 0; l < 4; ++l) if (cells <= (1ull << 30)) cells *= ((kept >> l) & 1u) ? (u64)(max(maxex[l], 0) >> l) + 1 : 1;
-  // A box whose whole table would not fit the slab may need a slot of the arena.  Where the round's workspace is too
-  // small for one, such a pool is refused up front, whatever its data: the caller is told, not now and then.
+  // Gang requests couple the chunk sizes; the header asks that the table of such a pool's reachable states fits a slot
+  // of the workspace.  With slots below TG_MIN_SLOT_BYTES (workspace_bytes under 2.3 MB) that rule decides alone: a box
+  // whose table fits neither the slab nor the slot gets its status word whatever its durations.  All other pools need
+  // nothing but the slab, on any workspace.
   const bool dense_fits = slab.used + 2 * cells * sizeof(i64) + (u64)nrows * cells + 64 <= slab.cap;
-  if (!dense_fits && arena_slot_bytes(P) < TG_MIN_SLOT_BYTES) return UNSOLVED;
-  if (solve_priced(T0, T, nrows, uniform(T0.n_levels), Y, kept, slab, lane)) {
+  bool by_table = false;
+  if (!dense_fits && arena_slot_bytes(P) < TG_MIN_SLOT_BYTES) {
+#pragma unroll 1
+    for (int t = lane; t < nrows; t += 32) by_table |= (T.cg[T.rowcand[t]] >> 7) != 0;
+    by_table = __any_sync(TG_FULL, by_table);
+  }
+  if (!by_table && solve_priced(T0, T, nrows, uniform(T0.n_levels), Y, kept, slab, lane)) {
     i64 sum = 0;
 #pragma unroll 1
     for (int i = lane; i < q; i += 32) sum += duration(T.cs[i], T.cp[i], T.rsel[i]);

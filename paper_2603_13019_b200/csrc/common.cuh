@@ -188,7 +188,7 @@ __device__ __forceinline__ void gpu_caps(const PoolDev& pd, const u8* busy, int 
 // table and gives back (48 slots of at least 64 MiB when the arena allows, else down to 4
 // larger-as-possible ones); the rest is handed out by a bump pointer, never reused in a call.
 #define TG_ARENA_MAX_SLOTS 48
-#define TG_MIN_SLOT_BYTES (512u << 10)   // smaller slots are of no use to the tables of large boxes
+#define TG_MIN_SLOT_BYTES (512u << 10)   // in smaller slots few tables of large boxes fit (solve_prefix)
 __device__ __forceinline__ int arena_n_slots(const Params& P) {
   u64 n = (P.arena_bytes / 8 * 7) >> 26;
   return n < 4 ? 4 : (n > TG_ARENA_MAX_SLOTS ? TG_ARENA_MAX_SLOTS : (int)n);

@@ -537,8 +537,10 @@ __device__ __forceinline__ int evict_loop(const Params& P, PoolTask& T, Slab sla
   const int m = uniform(T.m);
   if (m == 1) { solve_single(T, lane); return 1; }
   u8* rkeep = T.rkeep; const u8* rsel = T.rsel;
-  // room for the small table of a pool of up to 256 elastic candidates (the routines below get the rest of the slab)
-  i64* cells = m <= 256 ? (i64*)slab.take((u64)m * (256 + 64)) : nullptr;
+  // room for the small table of a pool with one capacity and up to 256 elastic candidates (the routines below get the
+  // rest of the slab; a pool whose nested capacities bind never builds that table and keeps all of it)
+  const bool one_capacity = T.type != TG_POOL_GPU || T.cap[3] >= T.cap[0];
+  i64* cells = m <= 256 && one_capacity ? (i64*)slab.take((u64)m * (256 + 64)) : nullptr;
   if (lane < 4) T.lam[lane] = 0.f;
   if (lane == 0) { T.sq = 0; T.cell_rows = cells ? 0 : -1; T.cell_val = cells; T.cell_ch = (unsigned short*)(cells + (size_t)m * 32); }
   __syncwarp();

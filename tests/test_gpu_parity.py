@@ -263,3 +263,28 @@ def test_waiting_for_a_slot_ends(oracle):
             assert np.array_equal(o[k][sc], short[k][sc]), (sc, k)
     patient = _gpu_round_ws(pools, a, workspace_bytes=320 << 20, slot_wait_us=5_000_000)
     assert_same(o, patient)
+
+
+@pytest.mark.parametrize("nodes,N,max_mult", [(64, 260, 4), (96, 200, 8), (24, 300, 4)])
+def test_replica_requests_need_no_slot_of_the_workspace(oracle, nodes, N, max_mult):
+    # fragmented pools without gang requests: boxes far beyond a warp's slab, one MiB of workspace
+    w, a = contiguous_replica_round(7900 + nodes, 6, N, nodes, max_mult)
+    g = _gpu_round_ws(w.pools, a, workspace_bytes=1 << 20)
+    assert np.all(g["status"] == 0)
+    assert_same(oracle.schedule_batch(w.pools, a), g)
+
+
+@pytest.mark.parametrize("rows", [6, 8])
+def test_gang_table_that_fits_a_small_slot_is_solved(oracle, rows):
+    # alike gang requests reach few states of a box of 70000 cells: their table fits a slot of 229 KB (1 MiB of workspace)
+    busy = [0x00] * 4 + [0x0F] * 6 + [0x3F] * 5 + [0x7F] * 5
+    pools = (Pool(POOL_GPU, 8 * len(busy), 8),)
+    rng = np.random.Generator(np.random.PCG64(rows))
+    S = 6
+    a = dict(pool=np.zeros((S, rows), np.uint8), unit=np.full((S, rows), 1 | 0x80, np.uint8),
+             level_mask=np.full((S, rows), 0x8B, np.uint32), arrival_us=None, n_actions=np.full(S, rows, np.int32),
+             s_us=rng.integers(0, 50_000, (S, rows)), p_us=rng.integers(100_000, 500_000, (S, rows)),
+             gpu_busy=np.tile(np.array(busy, np.uint8), (S, 1)))
+    g = _gpu_round_ws(pools, a, workspace_bytes=1 << 20)
+    assert np.all(g["status"] == 0)
+    assert_same(oracle.schedule_batch(pools, a), g)
