@@ -18,7 +18,8 @@
 // Algorithm 3 / 4 only runs over the few that are not, on the few states (demand shifts against the
 // priced choices) whose accumulated excess stays <= U.  U starts small and is raised until a solution
 // within it is found, which then is the optimum: nothing outside could be better or tie.  The
-// result does not depend on the prices, only the work does.
+// result does not depend on the prices, only the work does.  Where nobody is a gang request, a method whose work
+// the extents bound takes over from passes that would cost more (dp_classes).
 //
 // Measured on B200 (fragmented 8-node pools with elastic gang requests, 500 scenarios x 200 actions):
 // the table over the product of the four extents has 1e3 .. 1e6 cells per row; the bounded states
@@ -115,6 +116,10 @@ struct PoolTask {
   // table of at most 32 cells over the elastic rows (small_table): values and choices, [row][32]; rows in it (0: not
   // built, -1: not possible)
   i64* cell_val; unsigned short* cell_ch; int cell_rows;
+  // nested capacities bind and nobody is an elastic gang request (dp_classes applies): upgrade steps and candidates
+  // with gaps in their levels; upgrades -1: another pool
+  int upgrades, gaps;
+  int limit;              // what a pass of bounded_dp may cost, in rows times 32 states
 };
 
 // a level as one number pair: units of multiplicity r and the chunk class they are asked for at
@@ -441,10 +446,329 @@ __device__ __forceinline__ int bounded_dp(const PoolTask& T, const int* frow, u3
   return 1;
 }
 
+// ---- replica requests only: one dimension per chunk size --------------------------------------
+// Without gang requests a row of chunk size 2^c only ever adds requests of that size, so the rows fall into four
+// classes that meet in nothing but the nested capacities (extra GPUs at sizes >= 2^l at most cap[l] - dmin[l]).  Per
+// class, f_c(x) = least duration sum with exactly x extra chunks; the classes are merged from the largest size down,
+//   G_c(e) = min over x of G_{c+1}((e - x) / 2) + f_c(x),   e in chunks of 2^c,
+// tables over each extent instead of one over their product.  The work depends on the extents and hardly on the
+// durations.  f_c: where every row's multiplicities are contiguous and its gains T(r) - T(r+1) do not grow (the
+// floor in Eq. 1 can break that), f_c(x) is the sum at the least levels minus the x largest gains (separable
+// convex resource allocation), and equal gains go to the earliest rows first (a later queue position gets less), so
+// one sort of the steps by (gain descending, row, step) serves every x; other classes go through Algorithm 3's
+// recurrence.  Two splits between classes that tie on a cell of the chosen path are not decided here.
+#define MG_GAIN_BITS 41
+#define MG_ROW_BITS 18
+#define MG_GAIN_MAX ((1ull << MG_GAIN_BITS) - 1ull)
+__device__ __forceinline__ u64 mg_key(i64 gain, int row, int step) {     // step 1-based, at most 31
+  return ((MG_GAIN_MAX - (u64)gain) << (MG_ROW_BITS + 5)) | ((u64)row << 5) | (u64)(step - 1);
+}
+__device__ __forceinline__ i64 mg_gain(u64 key) { return (i64)(MG_GAIN_MAX - (key >> (MG_ROW_BITS + 5))); }
+// contiguous multiplicities and gains that do not grow
+__device__ __forceinline__ bool mg_row_ok(i64 p, u32 mk) {
+  const int r0 = __ffs(mk), rx = 32 - __clz(mk);
+  if (__popc(mk) != rx - r0 + 1) return false;
+  i64 before = div_small(p, r0), last = TG_INF;
+#pragma unroll 1
+  for (int r = r0 + 1; r <= rx; ++r) {
+    const i64 now = div_small(p, r), gain = before - now;
+    if (gain > last) return false;
+    last = gain; before = now;
+  }
+  return true;
+}
+// ascending bitonic sort of n (a power of two) keys by the calling warp
+__device__ __forceinline__ void warp_sort_u64(u64* a, int n, int lane) {
+#pragma unroll 1
+  for (int k = 2; k <= n; k <<= 1)
+#pragma unroll 1
+    for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) {
+        const int l = i ^ j;
+        if (l > i) {
+          const u64 x = a[i], y = a[l];
+          if ((x > y) == ((i & k) == 0)) { a[i] = y; a[l] = x; }
+        }
+      }
+      __syncwarp();
+    }
+}
+
+// What dp_classes knows of one class; on the warp's slab, so that loops over the classes need no registers per class.
+struct ChunkClass {
+  int rows, most;          // rows; extra chunks they could use
+  int by_gain;             // the steps sorted by gain serve every count
+  int U;                   // extra chunks that may be given: min(most, units left >> class)
+  int E;                   // merged table: cells 0 .. E, in chunks of this size
+  int npad;                // sorted steps, padded to a power of two
+  i64 base;                // duration sum at the least levels
+  i64* f; u64* keys; u8* ch;
+  i64* G; int* sel; u8* tie;
+};
+#define DPC_MAX_CELLS 4096
+// Rows T.rowcand[0 .. T.nrows), none of them a gang request.  Returns 1 with the rows' multiplicities in T.rsel, 0 (T.rsel
+// untouched) where splits tie or the slab does not suffice.  This and solve_box are out of line, so that the usual path keeps its
+// registers (16384 x 4096, where nothing calls them: 0.3 % slower than without this routine, both inlined 1.5 %,
+// only this one out of line 0.7 %).
+__device__ __noinline__ int dp_classes(const PoolTask& T, Slab slab, int lane) {
+  const int nrows = T.nrows;
+  if (nrows >= (1 << MG_ROW_BITS)) return 0;
+  ChunkClass* C = (ChunkClass*)slab.take(4 * sizeof(ChunkClass));
+  if (!C) return 0;
+  int Umax = 0;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    int rows = 0, most = 0; i64 base = 0; bool convex = true;
+#pragma unroll 1
+    for (int t = lane; t < nrows; t += 32) {
+      const int i = T.rowcand[t];
+      if (ilog2(T.cg[i]) != c) continue;
+      const u32 mk = T.cmask[i];
+      ++rows; most += (32 - __clz(mk)) - __ffs(mk);
+      base += duration(T.cs[i], T.cp[i], __ffs(mk));
+      convex &= mg_row_ok(T.cp[i], mk);
+    }
+    rows = warp_sum32(rows); most = warp_sum32(most); base = warp_sum64(base);
+    const bool by_gain = __all_sync(TG_FULL, convex) && most >= 1;
+    const int E = max(T.cap[c] - T.dmin[c], 0) >> c, U = min(E, most);
+    if (U + 1 > DPC_MAX_CELLS || E + 1 > 2 * DPC_MAX_CELLS) return 0;
+    Umax = max(Umax, U);
+    int npad = 1;
+    while (npad < most) npad <<= 1;
+    i64* f = (i64*)slab.take((u64)(U + 1) * 8);
+    u64* keys = by_gain ? (u64*)slab.take((u64)npad * 8) : nullptr;
+    u8* ch = by_gain ? nullptr : (u8*)slab.take((u64)max(rows, 1) * (U + 1));
+    i64* G = (i64*)slab.take((u64)(E + 1) * 8);
+    int* sel = (int*)slab.take((u64)(E + 1) * 4);
+    u8* tie = (u8*)slab.take((u64)(E + 1));
+    if (!f || (by_gain ? !keys : !ch) || !G || !sel || !tie) return 0;
+    if (lane == 0) {
+      ChunkClass& k = C[c];
+      k.rows = rows; k.most = most; k.by_gain = by_gain; k.U = U; k.E = E; k.npad = npad; k.base = base;
+      k.f = f; k.keys = keys; k.ch = ch; k.G = G; k.sel = sel; k.tie = tie;
+    }
+  }
+  i64* work = (i64*)slab.take(2 * (u64)(Umax + 1) * 8);
+  if (!work) return 0;
+  __syncwarp();
+  // ---- per class: f_c(x), least duration sum with exactly x extra chunks
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const ChunkClass& k = C[c];
+    const int U = uniform(k.U);
+    i64* f = k.f;
+    if (k.by_gain) {
+      const int n = uniform(k.npad), most = uniform(k.most);
+      u64* srt = (u64)n * 8 <= T.wk_bytes ? (u64*)T.wk : k.keys;
+      int fill = 0;                                      // every row writes its steps behind those of the rows before it
+#pragma unroll 1
+      for (int t0 = 0; t0 < nrows; t0 += 32) {
+        const int t = t0 + lane;
+        int ex = 0, r0 = 1; i64 p = 0;
+        if (t < nrows) {
+          const int i = T.rowcand[t];
+          const u32 mk = T.cmask[i];
+          if (ilog2(T.cg[i]) == c) { r0 = __ffs(mk); ex = (32 - __clz(mk)) - r0; p = T.cp[i]; }
+        }
+        int incl = ex;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(TG_FULL, incl, o); if (lane >= o) incl += y; }
+        u64* dst = srt + fill + incl - ex;
+        i64 before = div_small(p, r0);
+#pragma unroll 1
+        for (int x = 1; x <= ex; ++x) {
+          const i64 now = div_small(p, r0 + x);
+          dst[x - 1] = mg_key(before - now, t, x);
+          before = now;
+        }
+        fill += __shfl_sync(TG_FULL, incl, 31);
+      }
+#pragma unroll 1
+      for (int x = most + lane; x < n; x += 32) srt[x] = ~0ull;
+      __syncwarp();
+      warp_sort_u64(srt, n, lane);
+      i64 run = k.base;                                  // f_c at the start of the block of 32
+#pragma unroll 1
+      for (int x0 = 0; x0 <= U; x0 += 32) {
+        // f_c(x0 + lane) = run - gains of the steps x0 .. x0 + lane - 1
+        const int x = x0 + lane;
+        const i64 g = x < U ? mg_gain(srt[x]) : 0;
+        i64 incl = g;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const i64 y = __shfl_up_sync(TG_FULL, incl, o); if (lane >= o) incl += y; }
+        if (x <= U) f[x] = run - (incl - g);
+        run -= __shfl_sync(TG_FULL, incl, 31);
+      }
+      if (srt != k.keys) {
+#pragma unroll 1
+        for (int x = lane; x < U; x += 32) k.keys[x] = srt[x];
+      }
+      __syncwarp();
+      continue;
+    }
+    i64* prev = work; i64* cur = work + (Umax + 1);
+#pragma unroll 1
+    for (int u = lane; u <= U; u += 32) prev[u] = u == 0 ? 0 : TG_INF;
+    __syncwarp();
+    u8* ch = k.ch;
+#pragma unroll 1
+    for (int t = 0; t < nrows; ++t) {
+      const int i = T.rowcand[t];
+      if (ilog2(T.cg[i]) != c) continue;
+      const u32 mk = T.cmask[i];
+      const int r0 = __ffs(mk);
+      const i64 s = T.cs[i], p = T.cp[i];
+#pragma unroll 1
+      for (int u = lane; u <= U; u += 32) {
+        i64 best = TG_INF; int bestr = 0;
+#pragma unroll 1
+        for (u32 mm = mk; mm; mm &= mm - 1) {
+          const int r = __ffs(mm), du = r - r0;
+          if (du > u) break;                             // levels ascend
+          const i64 pv = prev[u - du];
+          if (pv == TG_INF) continue;
+          const i64 cand = pv + duration(s, p, r);
+          if (cand < best) { best = cand; bestr = r; }
+        }
+        cur[u] = best; ch[u] = (u8)bestr;
+      }
+      __syncwarp();
+      i64* tmp = prev; prev = cur; cur = tmp;
+      ch += U + 1;
+    }
+#pragma unroll 1
+    for (int u = lane; u <= U; u += 32) f[u] = prev[u];
+    __syncwarp();
+  }
+  // ---- merge, largest chunks first
+#pragma unroll 1
+  for (int c = 3; c >= 0; --c) {
+    const ChunkClass& k = C[c];
+    const int E = uniform(k.E), U = uniform(k.U), Eup = c < 3 ? uniform(C[c + 1].E) : 0;
+    const i64* f = k.f;
+    const i64* up_G = c < 3 ? C[c + 1].G : nullptr;
+    const u8* up_tie = c < 3 ? C[c + 1].tie : nullptr;
+    i64* G = k.G; int* sel = k.sel; u8* tie = k.tie;
+#pragma unroll 1
+    for (int e = lane; e <= E; e += 32) {
+      i64 best = TG_INF; int bu = 0; bool tied = false;
+      if (c == 3) { if (e <= U) best = f[e]; }
+      else {
+        const int hi = min(Eup, e >> 1);
+#pragma unroll 1
+        for (int up = max(e - U + 1, 0) >> 1; up <= hi; ++up) {       // e - 2 up <= U
+          const i64 a = up_G[up], b = f[e - 2 * up];
+          if (a == TG_INF || b == TG_INF) continue;
+          const i64 cand = a + b;
+          if (cand < best) { best = cand; bu = up; tied = up_tie[up] != 0; }
+          else if (cand == best) tied = true;
+        }
+      }
+      G[e] = best; sel[e] = bu; tie[e] = tied ? 1 : 0;
+    }
+    __syncwarp();
+  }
+  // ---- best end cell: lowest value, then fewest extra GPUs
+  const i64* G0 = C[0].G;
+  const int E0 = uniform(C[0].E);
+  i64 bv = TG_INF;
+#pragma unroll 1
+  for (int e = lane; e <= E0; e += 32) bv = min(bv, G0[e]);
+  bv = warp_min64(bv);
+  if (bv == TG_INF) return 0;
+  int at = INT_MAX;
+#pragma unroll 1
+  for (int e = lane; e <= E0; e += 32) if (G0[e] == bv) at = min(at, e);
+  at = warp_min32(at);
+  if (C[0].tie[at]) return 0;
+  // ---- walk back: cells of the merged tables, then the rows of every class
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const ChunkClass& k = C[c];
+    const int up = c < 3 ? k.sel[at] : 0;
+    int u = at - 2 * up;                                 // extra chunks of this class
+    at = up;
+    if (k.by_gain) {
+      // the steps in front of the cut are taken: a row gets its steps up to the threshold key
+      const u64 thr = u >= 1 ? k.keys[u - 1] : 0ull;
+#pragma unroll 1
+      for (int t = lane; t < nrows; t += 32) {
+        const int i = T.rowcand[t];
+        if (ilog2(T.cg[i]) != c) continue;
+        const u32 mk = T.cmask[i];
+        const int r0 = __ffs(mk), ex = u >= 1 ? (32 - __clz(mk)) - r0 : 0;
+        const i64 p = T.cp[i];
+        i64 before = div_small(p, r0);
+        int take = 0;
+#pragma unroll 1
+        for (int x = 1; x <= ex; ++x) {
+          const i64 now = div_small(p, r0 + x);
+          if (mg_key(before - now, t, x) > thr) break;   // a row's keys ascend with the step
+          take = x; before = now;
+        }
+        T.rsel[i] = (u8)(r0 + take);
+      }
+    } else if (lane == 0) {
+      const u8* ch = k.ch + (u64)k.rows * (k.U + 1);
+#pragma unroll 1
+      for (int t = nrows - 1; t >= 0; --t) {
+        const int i = T.rowcand[t];
+        if (ilog2(T.cg[i]) != c) continue;
+        ch -= k.U + 1;
+        const int r = ch[u];
+        T.rsel[i] = (u8)r;
+        u -= r - __ffs(T.cmask[i]);
+      }
+    }
+  }
+  __syncwarp();
+  return 1;
+}
+
+// Once per task whose nested capacities bind: does dp_classes apply?  -> T.upgrades, T.gaps
+__device__ __forceinline__ void find_replicas(PoolTask& T, int lane) {
+  bool gang = false;
+  int gaps = 0, up = 0;
+#pragma unroll 1
+  for (int i = lane; i < T.m; i += 32) {
+    const u32 mk = T.cmask[i];
+    const int span = 32 - __clz(mk) - __ffs(mk);
+    gang |= (T.cg[i] >> 7) != 0 && span > 0;
+    gaps += __popc(mk) != span + 1 ? 1 : 0;
+    up += span;
+  }
+  gang = __any_sync(TG_FULL, gang);
+  gaps = warp_sum32(gaps); up = warp_sum32(up);
+  if (lane == 0) { T.upgrades = gang ? -1 : up; T.gaps = gaps; }
+  __syncwarp();
+}
+// Prices settle most boxes with few rows, but what a pass of bounded_dp costs is up to the durations; dp_classes costs what
+// the extents make of it.  In units of a row times 32 states (1500 to 3300 cycles) that is 40, one per 5 upgrade steps (sorts),
+// one per 9 rounds of the largest merge, 1.5 per 32 cells and row with gaps in its levels (recurrence).  A pass may cost
+// a quarter of it (at least 24: the first passes, of four rows): the state table is that much smaller.
+// Measured, us a call, lowest .. highest of 9 to 16 inputs (64 nodes, 30 % of the GPUs busy, levels 1..4):
+//                                       without dp_classes  at once         after one pass  with this limit
+//   1024 scenarios x 2048               790 .. 4140         800 .. 1014     757 .. 872      746 .. 895
+//   400 x 200                           1075 .. 4770        1600 .. 1900    1120 .. 1646    1083 .. 1792
+//   12 x 256, alike durations           495000              1140            1200            1270
+//   12 x 256, 128 nodes, levels 1 2 4 8 1090                6550            3110            1080
+//   12 x 256, levels 1 2 4 8            350                 680             650             630
+// (alike durations: the states outgrow every table but the arena's).  A pass that may cost half or all of dp_classes: 1540
+// and 1600 for the alike durations, 1118 .. 1750 and 1099 .. 2040 for 400 x 200.
+__device__ __forceinline__ void set_limit(PoolTask& T, int lane) {
+  const int Y0 = T.cap[0] - T.dmin[0], Y1 = T.cap[1] - T.dmin[1];
+  const int blocks = (min(Y0, 1 << 14) >> 5) + 1, span = min(min(Y1, T.upgrades), 1 << 14) >> 1;
+  const int cost = 40 + T.upgrades / 5 + blocks * span / 9 + min(T.gaps, 1 << 14) * blocks * 3 / 2;
+  if (lane == 0) T.limit = max(cost / 4, 24);
+  __syncwarp();
+}
+
 // The optimum under prices, over the elastic rows T.rowcand[0 .. nrows) with Y[l] units to give beyond everybody's
 // least level (Y[0] > 0).  lam: prices to start from and the prices found (all 0: none known).  T.rsel holds the
-// least level of every candidate on entry and the optimum on success.  Returns 0 if the state tables do not
-// suffice (the caller then goes through the general tables).
+// only level of every inelastic candidate on entry and the optimum on success.  T0.limit: what a pass may cost (INT_MAX:
+// anything); where it would cost more, dp_classes decides.  Returns 0 if the state tables do not suffice (the caller
+// then goes through the general tables).
 __device__ __forceinline__ int solve_priced(const PoolTask& T0, const PoolTask& T, int nrows, int n_levels, const int Y[4], u32 kept,
                                             Slab slab, int lane) {
   float lam[4] = {T0.lam[0], T0.lam[1], T0.lam[2], T0.lam[3]};
@@ -593,16 +917,24 @@ __device__ __forceinline__ int solve_priced(const PoolTask& T0, const PoolTask& 
     }
     if (kept != 1u && warp_sum32(reach) > 4000) return 0;   // (levels 2 and 3 move no further)
     __syncwarp();
+    const int per_row = T0.limit / max(nfree, 1);        // blocks of 32 states
     int got = -1;
 #pragma unroll 1
-    for (int where = 0; where < 2 && got < 0; ++where) { // the work area, then the slab
+    for (int where = 0; where < 2 && got < 0 && per_row > 0; ++where) { // the work area, then the slab
       const u64 half = where == 0 ? 0 : (room / 2) & ~(u64)15;
       BdTable B;
       if (!bd_table(B, where == 0 ? T.wk : slab.base + slab.used, where == 0 ? (u64)T.wk_bytes : half)) break;
+      B.cap = min(B.cap, 32 * min(per_row, 128));
       got = bounded_dp(T, frow, crow, lim, nfree, price, li, kept, slack, delta, B, (u8*)slab.base + slab.used + half, room - half, lane);
     }
-    if (got < 0) return 0;
     if (got > 0) return 1;
+    if (got < 0) {
+      if (T0.limit == INT_MAX) return 0;
+      if (dp_classes(T0, slab, lane)) return 1;
+      if (lane == 0) ((PoolTask&)T0).limit = INT_MAX;    // (splits tie: this pass once more, without a limit)
+      --pass;
+      continue;
+    }
     delta = max(nfree <= 16 ? 8 * delta : 2 * delta, (i64)16);
     if (feasible) delta = min(delta, s0);
   }
@@ -801,10 +1133,21 @@ __device__ __forceinline__ int dp_sparse(const PoolTask& T, int nrows, const int
   return 1;
 }
 
-// The whole box of feasible extra-demand vectors (T.rowcand, T.rsel = least levels; maxex[l] = largest extra demand at
-// level l): where the states within a bound do not fit their table, or very many end states tie.  
-__device__ __forceinline__ bool solve_box(const Params& P, const PoolTask& T, int q, int nrows, const int maxex[4], u32 kept, Slab slab,
-                                       int lane, i64* opt) {
+// The whole box of feasible extra-demand vectors (T.rowcand; T.maxex[l] = largest extra demand at level l), where the states
+// within a bound do not fit their table, or very many end states tie.  -> T.rsel, T.opt
+__device__ __noinline__ bool solve_box(const Params& P, PoolTask& T, int q, Slab slab, int lane) {
+  const int nrows = T.nrows;
+  int maxex[4] = {0, 0, 0, 0};
+  u32 kept = 1u;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    if (l > 0 && T.type != TG_POOL_GPU) continue;
+    maxex[l] = min(T.cap[l] - T.dmin[l], T.maxex[l]);
+    if (l > 0 && T.cap[l] < T.cap[l - 1]) kept |= 1u << l;
+  }
+#pragma unroll 1
+  for (int t = lane; t < nrows; t += 32) { const int i = T.rowcand[t]; T.rsel[i] = (u8)__ffs(T.cmask[i]); }
+  __syncwarp();
   int ext[4], stride[4];
   u64 cells = 1;
 #pragma unroll
@@ -827,7 +1170,9 @@ __device__ __forceinline__ bool solve_box(const Params& P, const PoolTask& T, in
     i64 sum = 0;
 #pragma unroll 1
     for (int i = lane; i < q; i += 32) sum += duration(T.cs[i], T.cp[i], T.rsel[i]);
-    *opt = warp_sum64(sum);
+    sum = warp_sum64(sum);
+    if (lane == 0) T.opt = sum;
+    __syncwarp();
     return true;
   }
   i64* prev = val; i64* cur = val + cells;
@@ -938,7 +1283,9 @@ __device__ __forceinline__ bool solve_box(const Params& P, const PoolTask& T, in
   i64 sum = 0;
 #pragma unroll 1
   for (int i = lane; i < q; i += 32) sum += duration(T.cs[i], T.cp[i], T.rsel[i]);
-  *opt = warp_sum64(sum);
+  sum = warp_sum64(sum);
+  if (lane == 0) T.opt = sum;
+  __syncwarp();
   return true;
 }
 
@@ -1191,6 +1538,7 @@ __device__ __forceinline__ int solve_prefix(const Params& P, PoolTask& T0, int q
     for (int t = lane; t < nrows; t += 32) by_table |= (T.cg[T.rowcand[t]] >> 7) != 0;
     by_table = __any_sync(TG_FULL, by_table);
   }
+  if (T0.upgrades >= 0) set_limit(T0, lane);
   if (!by_table && solve_priced(T0, T, nrows, uniform(T0.n_levels), Y, kept, slab, lane)) {
     i64 sum = 0;
 #pragma unroll 1
@@ -1200,12 +1548,5 @@ __device__ __forceinline__ int solve_prefix(const Params& P, PoolTask& T0, int q
     __syncwarp();
     return SOLVED;
   }
-#pragma unroll 1
-  for (int t = lane; t < nrows; t += 32) { const int i = T.rowcand[t]; T.rsel[i] = (u8)__ffs(T.cmask[i]); }
-  __syncwarp();
-  i64 opt = 0;
-  const bool ok = solve_box(P, T0, q, nrows, maxex, kept, slab, lane, &opt);
-  if (lane == 0) T0.opt = opt;
-  __syncwarp();
-  return ok ? SOLVED : UNSOLVED;
+  return solve_box(P, T0, q, slab, lane) ? SOLVED : UNSOLVED;
 }

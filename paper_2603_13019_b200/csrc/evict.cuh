@@ -542,8 +542,9 @@ __device__ __forceinline__ int evict_loop(const Params& P, PoolTask& T, Slab sla
   const bool one_capacity = T.type != TG_POOL_GPU || T.cap[3] >= T.cap[0];
   i64* cells = m <= 256 && one_capacity ? (i64*)slab.take((u64)m * (256 + 64)) : nullptr;
   if (lane < 4) T.lam[lane] = 0.f;
-  if (lane == 0) { T.sq = 0; T.cell_rows = cells ? 0 : -1; T.cell_val = cells; T.cell_ch = (unsigned short*)(cells + (size_t)m * 32); }
+  if (lane == 0) { T.upgrades = -1; T.limit = INT_MAX; T.sq = 0; T.cell_rows = cells ? 0 : -1; T.cell_val = cells; T.cell_ch = (unsigned short*)(cells + (size_t)m * 32); }
   __syncwarp();
+  if (!one_capacity) find_replicas(T, lane);
   i64 opt = 0;
   int keep = m;
 #pragma unroll 1

@@ -3,8 +3,8 @@ table, rows beyond its size and level lists beyond its width, against the oracle
 import numpy as np
 import pytest
 
-from test_gpu_parity import assert_same, gpu_round
-from workloads import POOL_API, POOL_CPU, POOL_GPU, GANG, Pool
+from test_gpu_parity import _gpu_round_ws, assert_same, gpu_round
+from workloads import POOL_API, POOL_CPU, POOL_GPU, GANG, Pool, contiguous_replica_round
 
 pytestmark = pytest.mark.gpu
 
@@ -51,6 +51,27 @@ def test_gang_requests_on_fragmented_nodes_match_oracle(oracle, nodes, m, tiny):
     rng = np.random.Generator(np.random.PCG64(nodes))
     a["gpu_busy"] = np.where(rng.random((6, nodes)) < 0.5, rng.integers(0, 256, (6, nodes)), 0).astype(np.uint8)
     assert_same(oracle.schedule_batch(pools, a), gpu_round(pools, a))
+
+
+@pytest.mark.parametrize("kind,S,nodes,N,seed", [
+    ("alike", 12, 64, 256, 320),     # more states within reach of the prices than a table holds
+    ("alike", 2, 256, 512, 768),     # more than 512 upgrade steps in a class: sorted in global memory
+    ("gaps", 6, 40, 120, 8168),      # levels 1, 2, 4, 8: the recurrence instead of the sorted gains
+    ("equal", 6, 64, 256, 8328),     # splits between chunk sizes tie in some pools
+])
+def test_alike_replica_requests_match_oracle(oracle, kind, S, nodes, N, seed):
+    # durations so close to each other that the prices settle nothing and a pass over the states within their reach costs
+    # more than the chunk sizes one by one; that way needs the slab only, so one MiB of workspace does
+    w, a = contiguous_replica_round(seed, S, N, nodes, 8)
+    rng = np.random.default_rng(seed % 8000)
+    a["p_us"] = rng.integers(400_000_000, 400_001_000, a["p_us"].shape)
+    if kind == "gaps":
+        a["level_mask"] = rng.choice(np.array([0x8B, 0xB, 0x5, 0x1], np.uint32), a["level_mask"].shape)
+    if kind == "equal":
+        a["p_us"] = 4000 * rng.integers(50, 52, a["p_us"].shape)
+    g = _gpu_round_ws(w.pools, a, workspace_bytes=1 << 20)
+    assert np.all(g["status"] == 0)
+    assert_same(oracle.schedule_batch(w.pools, a), g)
 
 
 @pytest.mark.parametrize("policy", [0, 1, 2])
