@@ -26,10 +26,10 @@ struct PoolDev {
   int queue_place;      // batched path: grants are placed in queue order with the state in registers (CpuFresh, quota sums)
 };
 
-// per (scenario, pool) facts produced by the prefix kernel
+// per (scenario, pool) facts produced by the head walk and the stream behind it
 struct PoolMeta {
   i64 base;       // the pool's list in `tmin` starts at scenario * max_actions + base
-  i64 cbase;      // the pool's candidates in order / preq / the solver's arrays start at scenario * max_actions + cbase
+  i64 cbase;      // the pool's candidates in `order` start at scenario * max_actions + cbase
   int count;      // actions of the pool in the queue (candidates only, if nobody will read its waiting list)
   int m;          // candidates of the pool (they occupy positions base .. base+m-1)
   int elastic;    // some candidate has more than one level

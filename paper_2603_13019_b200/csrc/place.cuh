@@ -67,7 +67,8 @@ __device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, con
 
 // CPU placement on a pool nobody occupies yet (a single round).  Cores are only ever taken
 // lowest id first, so the used cores of a domain are always a prefix of it: the free count per
-// domain is the whole state and a grant's first core follows from it.  Same rule as place_cpu.
+// domain is the whole state and a grant's first core follows from it.  The rule: the domain with the fewest free
+// cores that still fit, lowest index among equals; else ascending domains.
 __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u8* cg, const u8* r,
                                 int* pnode, int* poff, int lane) {
   const int D = pd.capacity / pd.group;
@@ -112,10 +113,6 @@ __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u
     }
   }
 }
-
-// ---- register-resident fast paths of a single round (fresh CPU pool, at most 128 domains /
-// ---- GPU nodes): the state lives in lane registers, the arg-min is one redux, and every lane
-// ---- keeps the result of "its" candidate of a block of 32 for a coalesced write.
 
 // GPU placement with a service cache (Section 5.3, evict on execution).  The rule of place_gpu, and among
 // the free blocks of the level it picks, one whose granted chunk (the block's low end) caches the
@@ -198,6 +195,10 @@ __device__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* c
     }
   }
 }
+
+// ---- register-resident fast paths of a single round (fresh CPU pool, at most 128 domains /
+// ---- GPU nodes): the state lives in lane registers, the arg-min is one redux, and every lane
+// ---- keeps the result of "its" candidate of a block of 32 for a coalesced write.
 
 // Same placement rule as place_gpu; requires pd.n_nodes <= 128.  busy_row: the pool's node masks before the round
 // (may be null).  Lane k and register s hold node 32 s + k; lv[l][s] has bit k set where that node has a maximal

@@ -103,7 +103,7 @@ __device__ __forceinline__ u32 replay_meta(const Params& P, const ReplayQueue& Q
 // Live state of the scenario at hand: in the warp's shared memory, or in the arrays of ReplayWs where it is large.
 struct ReplayState { int* owner; u8* nm; int* dfree; int* pst; i64* win; };
 
-// One grant on a core pool with cores in use (place_cpu_owner's rule: fewest free cores that still fit, lowest domain,
+// One grant on a core pool with cores in use (fewest free cores that still fit, lowest domain,
 // lowest cores first; else ascending domains).  fit: the domain, -1 where the grant spans several.
 __device__ __forceinline__ void replay_place_cpu(const PoolDev& pd, int* owner, int* dfree, int k, int id, int lane, int& node, int& off, int& fit) {
   const int D = pd.capacity / pd.group;

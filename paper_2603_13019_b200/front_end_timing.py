@@ -53,7 +53,7 @@ def main():
         out["sort_%s_ms" % name] = _timed(lambda: rnd.order_queue(dev, policy), args.steps, torch)
         out["ordered_round_%s_ms" % name] = _timed(lambda: rnd.schedule_batch_ordered(dev, policy, 0, res), args.steps, torch)
     rnd.destroy()
-    # per-node CPU scheduling: the core pool of cfg4 as eight nodes of 1024 cores, the GPU pool beside them
+    # per-node CPU scheduling: seven nodes of 1024 cores in place of the core pool of cfg4, the GPU pool beside them
     pools = tuple(Pool(POOL_CPU, 1024, 64) for _ in range(7)) + (Pool(POOL_GPU, 128, 8),)
     b = dict(a, pool=np.where(a["pool"] == 1, 7, 0).astype(np.uint8))
     b = add_trajectories(1, b, pools, max_traj=1024, mem_hi=16, pinned=0.5, mem_free_hi=20000)

@@ -98,7 +98,7 @@ def test_arrivals_and_host_buffers_match_oracle(oracle):
 
 
 def test_long_queue_spans_several_tiles(oracle):
-    # 9000 actions per scenario: the prefix kernel walks three tiles with carried prefix sums
+    # 9000 actions per scenario: the stream behind the prefix spans three tiles with carried positions
     pools = (Pool(POOL_CPU, 3008, 64), Pool(POOL_GPU, 512, 8), Pool(POOL_API, 2000, 0, 1_000_000))
     w, a = random_round(31, 6, 9000, pools, max_mult=4, ragged=False)
     a["n_actions"][:] = [9000, 8191, 4097, 4096, 100, 9000]
@@ -110,8 +110,8 @@ def test_long_queue_spans_several_tiles(oracle):
 
 @pytest.mark.parametrize("ties", [0.0, 0.6, 1.0])
 def test_fragmented_gpu_pool_of_replica_requests_matches_oracle(oracle, ties):
-    # replica requests only (no gang rows) on a fragmented pool: the per-size DPs merged through the
-    # nested capacities; with tiny durations different splits tie and the general loop takes over
+    # replica requests only (no gang rows) on a fragmented pool: prices, and the chunk sizes one by one where
+    # those would cost more; with tiny durations different splits tie and the prices take over again
     pools = (Pool(POOL_GPU, 192, 8),)
     w, a = random_round(4242 + int(ties * 10), 48, 220, pools, replicas=1.0, busy_fraction=0.35,
                         small_durations=ties, inelastic=0.2, max_mult=4)
@@ -193,9 +193,9 @@ def test_fragmented_pool_with_elastic_gang_requests_matches_oracle(oracle, seed,
 @pytest.mark.parametrize("seed,nodes,N,max_mult,tiny", [(0, 128, 800, 8, 0.0), (1, 160, 1000, 12, 0.3),
                                                          (2, 64, 500, 16, 0.0), (3, 96, 600, 31, 0.7)])
 def test_marginal_gain_classes_match_oracle(oracle, seed, nodes, N, max_mult, tiny):
-    # hundreds of candidates with contiguous multiplicities on a fragmented pool: the chunk-size classes
-    # are served from their sorted marginal gains (more than 512 steps in a class: sorted in global
-    # memory); tiny durations break the monotony of some rows' gains, whose classes keep their DP
+    # hundreds of candidates with contiguous multiplicities on a fragmented pool: prices settle most of
+    # these (pools that go by the sorted marginal gains of their chunk sizes: test_selection_edges.py);
+    # tiny durations break the monotony of some rows' gains
     w, a = contiguous_replica_round(7300 + seed, 5, N, nodes, max_mult, small_durations=tiny)
     for depth in (2, 1):
         o = oracle.schedule_batch(w.pools, a, depth=depth)
@@ -209,7 +209,7 @@ def test_gang_requests_with_a_large_feasible_box_match_oracle(oracle, seed, node
     # short queues on a large fragmented pool: every action is a candidate, there is far more room than
     # the least levels need but not enough for everybody's best level, and gang requests couple the
     # chunk sizes: the dense table over the four chunk-count ranges has millions of cells, of which
-    # the rows reach a few thousand (Algorithm 4 on the reachable states only)
+    # the rows reach a few thousand, and those within reach of the prices are fewer still
     pools = (Pool(POOL_GPU, 8 * nodes, 8),)
     w, a = random_round(6200 + seed, 6, N, pools, replicas=0.5, busy_fraction=0.35, inelastic=0.1, max_mult=8,
                         ragged=False)
@@ -252,8 +252,9 @@ def test_table_that_fits_no_slot_is_reported_per_scenario(oracle):
 
 
 def test_waiting_for_a_slot_ends(oracle):
-    # four slots for 40 scenarios whose tables all need one: with a wait of one millisecond some warps
-    # give up (status word, nothing else), with the default wait every warp gets its turn
+    # four slots for 40 scenarios of large boxes: with a wait of one millisecond a warp that needs a slot may
+    # give up (status word, nothing else), with a long wait every warp gets its turn (pools that are sure to
+    # need one: test_selection_edges.py)
     pools, a = _large_box_round(3, 40)
     o = oracle.schedule_batch(pools, a)
     short = _gpu_round_ws(pools, a, workspace_bytes=320 << 20, slot_wait_us=1000)

@@ -74,6 +74,45 @@ def test_alike_replica_requests_match_oracle(oracle, kind, S, nodes, N, seed):
     assert_same(oracle.schedule_batch(w.pools, a), g)
 
 
+def test_states_that_outgrow_the_priced_table_take_a_slot(oracle):
+    # an elastic gang request among replica requests of close durations: neither the prices nor the chunk sizes one by one
+    # settle it, the table of all reachable states in a slot of the workspace does.  Twelve copies for four slots:
+    # with a wait of a millisecond some give up, with a long one every copy gets its turn
+    w, a = contiguous_replica_round(96, 12, 64, 32, 8)
+    a["p_us"] = np.random.default_rng(96).integers(400_000_000, 400_001_000, a["p_us"].shape)
+    a["unit"][:, 0] = 1 | GANG
+    a["level_mask"][:, 0] = 0xB
+    a = {k: None if v is None else np.repeat(v[4:5], 12, axis=0) for k, v in a.items()}
+    want = oracle.schedule_batch(w.pools, a)
+    assert_same(want, _gpu_round_ws(w.pools, a))
+    short = _gpu_round_ws(w.pools, a, workspace_bytes=320 << 20, slot_wait_us=1000)
+    assert set(np.unique(short["status"])) == {0, 4}
+    solved = short["status"] == 0
+    assert_same({k: v[solved] for k, v in want.items()}, {k: v[solved] for k, v in short.items()})
+    assert_same(want, _gpu_round_ws(w.pools, a, workspace_bytes=320 << 20, slot_wait_us=5_000_000))
+
+
+def test_many_tied_end_states_take_the_dense_table(oracle):
+    # 70 gang requests and 40 requests for chunks of two, all with the same gain per GPU, share 70 GPUs: 36 splits tie on
+    # duration and units, more than a warp's lanes; long rows make a slab that holds the box
+    S, N, n = 3, 16384, 110
+    busy = np.array([0] * 27 + [0x3F] + [0x7F] * 2, np.uint8)
+    pools = (Pool(POOL_GPU, 8 * len(busy), 8),)
+    rng = np.random.default_rng(5)
+    a = dict(pool=np.zeros((S, N), np.uint8), unit=np.ones((S, N), np.uint8), level_mask=np.ones((S, N), np.uint32),
+             s_us=np.zeros((S, N), np.int64), p_us=np.zeros((S, N), np.int64), arrival_us=None,
+             n_actions=np.full(S, n, np.int32), gpu_busy=np.tile(busy, (S, 1)))
+    for sc in range(S):
+        gang = rng.permutation(n) < 70
+        a["unit"][sc, :n] = np.where(gang, 1 | GANG, 2)
+        a["level_mask"][sc, :n] = 3
+        a["p_us"][sc, :n] = np.where(gang, 80_000, 160_000)
+        a["s_us"][sc, :n] = rng.integers(0, 50_000, n)
+    g = gpu_round(pools, a)
+    assert np.all(g["status"] == 0)
+    assert_same(oracle.schedule_batch(pools, a), g)
+
+
 @pytest.mark.parametrize("policy", [0, 1, 2])
 def test_replay_queues_beyond_shared_memory_match_oracle(oracle, policy):
     # so many scenarios that a block keeps few waiting records in shared memory: with bursts of long actions on
