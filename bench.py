@@ -35,11 +35,11 @@ from workloads import CONFIGS, generate, make_workload  # noqa: E402
 ALGO_BYTES_PER_ACTION = 42        # 22 B read (pool, unit, mask, s, p) + 20 B written (alloc, node, off, act)
 METRIC = "actions scheduled/sec (1xB200)"
 # DRAM bytes per pending action (dram__bytes_read.sum + dram__bytes_write.sum of one launch / actions of the
-# launch) from the ncu capture summarised under profiles/ (cfg4 shape, 2048
-# scenarios); traffic grows in proportion to the actions, so a launch's traffic is this times its actions.
+# launch), captured by ncu on the whole workload (16384 scenarios; profiles/batched_round_cfg4.md), so that what stays in
+# L2 at the end of a launch is a small part; with fewer scenarios the figures are scaled by actions.
 # The k_stream interval of the per-kernel timing holds k_fill as well (it runs beside it).
-NCU_BYTES_PER_ACTION = {"cfg4": {"k_head": 1.72, "k_stream": 11.70 + 22.48}}
-NCU_TRAFFIC_SOURCE = "ncu on 2048 scenarios of the same shape, scaled by actions (profiles/)"
+NCU_BYTES_PER_ACTION = {"cfg4": {"k_head": 1.89, "k_stream": 23.45 + 17.80, "k_pool": 15.62}}
+NCU_TRAFFIC_SOURCE = "ncu on cfg4 at 16384 scenarios, scaled by actions (profiles/batched_round_cfg4.md)"
 
 
 def _peaks():
@@ -212,7 +212,7 @@ def main():
     rnd = binding.Round(S, N, w.pools, depth=w.depth, round_us=w.round_us, max_rounds=w.max_rounds, **extras)
     res = rnd.new_result(replay=w.replay)
     stream = torch.cuda.current_stream()
-    if args.order and not w.replay:                # the round on the sorted queue (sort, gather, round, scatter)
+    if args.order and not w.replay:                # the round on the sorted queue (sort, then the round through the permutation)
         _plain = rnd.schedule_batch
         rnd.schedule_batch = lambda a_, now_, res_, st_: rnd.schedule_batch_ordered(a_, args.order, now_, res_, st_)
     if w.replay:                                   # a step of a replay workload = the whole trace
