@@ -6,15 +6,20 @@
 //   4. runs the scheduler of Algorithm 1 on the queue with the running actions of a pool in
 //      its completion heap (Algorithm 2), using the same per-pool routines as a single round,
 //   5. starts what was selected and records the occupancy.
-// Rounds in which nothing can change are jumped over (their occupancy rows are still written).
+// Rounds in which nothing can start are jumped over: with an empty queue up to the next arrival (what ends
+// meanwhile is released then), behind a head of the queue that does not fit up to the next event on its pool.
 //
 // A scenario is one long chain of dependent rounds, each of which handles one or two actions, so what
-// counts is the latency of a round: the records of the waiting actions (decoded once, on arrival), the
-// running actions with their completion times, the owner of every core and GPU and the free counts sit in
-// the warp's shared memory, arrivals are read 32 at a time into lane registers, the demand of every pool
-// and chunk level is one lane's register, and pools without a choice to make (one candidate, or
-// none elastic) never build the arrays of the selection.  What was spent per worked round before: about
-// 15000 cycles, most of them dependent loads of scattered records and instruction fetch.
+// counts is the latency of a round, which is the number of dependent instructions in it:
+//   * the records of the waiting actions (decoded once, on arrival) and the running actions sit in the warp's shared
+//     memory in 16-byte pieces; arrivals are read 32 at a time, one batch ahead;
+//   * times are compared as round numbers (32 bits, one warp minimum), worked out when an action starts;
+//   * free cores are bit masks, a grant is a mask of one word wherever it can be, so everything that ends in a round
+//     is released at once, a lane each, by shared-memory atomics; only grants over several words or chunks are found
+//     again by their owner entries, one after the other;
+//   * the queue is a ring, so what starts leaves it by moving its head;
+//   * occupancy is recorded as differences (two atomics per action that nobody waits for), k_occupancy adds them up;
+//   * pools without a choice to make (one candidate, or none elastic) never build the arrays of the selection.
 #pragma once
 #include "common.cuh"
 #include "arrange.cuh"
@@ -25,47 +30,81 @@
 struct ReplayWs {
   int* wait;        // [S][N] waiting actions behind the first wcap, by queue position
   u64* wkey;        // [S][N] their sort keys (policy 1 / 2 only)
-  int* owner;       // [S][U]  action holding each core / GPU (-1 free, -2 occupied beforehand)
-  u8* nm;           // [S][nodes] GPU busy masks
+  u32* cores;       // [S][W][2] free cores of every domain word (bit = core)
   int* dfree;       // [S][Dtot] free cores per NUMA domain
-  int* pst;         // [S][P][2] quota used in the window / concurrency slots in use
-  i64* win;         // [S][P] current quota window
-  // running actions where they do not fit shared memory: completion, action, pool << 24 | units, lowest core, domain
-  i64* run_fin; int* run_idx; u32* run_pu; int* run_off; int* run_dom;
-  int unit0[TG_MAX_POOLS], dom0[TG_MAX_POOLS];   // first unit / domain of every pool in a row
-  int U, Dtot;
-  i64 round_us; int max_rounds;
-  int* occupancy; int* rounds_used;
+  int* owner;       // [S][U]  action holding each core / GPU of a grant over several words or chunks
+  u8* nm;           // [S][nodes] GPU busy masks
+  // running actions where they do not fit shared memory (ReplayRun)
+  uint4* run_at; i64* run_fin; int* run_end; u32* run_pu; int* run_idx;
+  // per pool: first unit / domain / word of a scenario's row, domains, words per domain (core pools)
+  int unit0[TG_MAX_POOLS], dom0[TG_MAX_POOLS], word0[TG_MAX_POOLS], n_dom[TG_MAX_POOLS], wpd[TG_MAX_POOLS];
+  int U, Dtot, W;
+  i64 round_us; u64 round_recip;      // round_recip: ceil(2^64 / round_us), 0 where round_at has to divide
+  int max_rounds;
+  int* occupancy; int* rounds_used;   // rounds_used: never null in the kernels
   int policy;       // 0: first come first served; 1 / 2: the queue is kept in shortest / longest least-level duration order
   // trajectories pinned to CPU nodes as their actions arrive (Section 5.2); trajectory == nullptr: none of it
   const int* trajectory; const u32* traj_mem; const u8* traj_last; int max_traj;
   int* traj_node; i64* mem_free; u8* pool_rw;   // pool_rw: the pool column the kernel reads (P.a_pool) and rewrites
-  int state_bytes;  // > 0: a scenario's live state (owner .. win) takes that many bytes of the warp's shared memory
+  int state_bytes;  // > 0: a scenario's live state (cores .. nm) takes that many bytes of the warp's shared memory
   int wcap, rcap;   // waiting records / running actions in shared memory (rcap 0: running actions in global memory)
 };
 
 __host__ __device__ __forceinline__ size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
+// bytes of the live state: masks and free counts, owners, node masks
+__host__ __device__ __forceinline__ size_t replay_state_bytes(const ReplayWs& R, int n_nodes) {
+  return align16((size_t)R.W * 8) + align16((size_t)R.Dtot * 4) + align16((size_t)R.U * 4) + align16((size_t)n_nodes + 1);
+}
 
 #define KR_THREADS 32
 #define KR_FAST_BYTES 8192        // shared-memory window of the selection's arrays
-#define KR_WAIT_BYTES 58          // per waiting record: s, p, least duration, arrival, key, action, packed meta, mask, queue, free list, unit
-#define KR_RUN_BYTES 24
+#define KR_WAIT_BYTES 60          // per waiting record: three 16-byte pieces, key, queue, free list
+#define KR_RUN_BYTES 36
 #define KR_STATE_MAX 16384
+#define KR_SLOT_BYTES 128         // free capacity of the 32 demand slots at most
 // shared memory of a block (one warp) without the parts sized by the round
-#define KR_BASE_BYTES (WARP_SMEM_BYTES + KR_FAST_BYTES + 64)
+#define KR_BASE_BYTES (WARP_SMEM_BYTES + KR_FAST_BYTES + KR_SLOT_BYTES + 64)
+#define KR_NEVER 0x7fffffff
 
-// Waiting records: slots that do not move, and the queue as slot numbers.  meta: pool (4 bits), first demand slot
-// (6), chunk class of the least level (2), units of the least level (13); bit 31: started in this round.
+// Waiting records: slots that do not move, and the queue as a ring of slot numbers.  sp: s, p; ta: least duration,
+// arrival; c: action, meta, mask, unit byte.  meta: pool (4 bits), first demand slot (6), chunk class of the least
+// level (2), units of the least level (13), elastic (1); bit 31: started in this round.
 struct ReplayQueue {
-  i64* s; i64* p; i64* tl; i64* arr; u64* key; int* idx; u32* meta; u32* mask; u8* cg; unsigned short* q; unsigned short* free;
-  int cap;
+  uint4* sp; uint4* ta; uint4* c; u64* key; unsigned short* q; unsigned short* free;
+  int cap, head;
+  __device__ __forceinline__ int at(int i) const { const int k = head + i; return k >= cap ? k - cap : k; }   // ring place of position i < cap
 };
 #define RQ_POOL(m) ((int)((m) & 15u))
 #define RQ_SLOT(m) ((int)(((m) >> 4) & 63u))
 #define RQ_CLASS(m) ((int)(((m) >> 10) & 3u))
 #define RQ_UNITS(m) ((int)(((m) >> 12) & 0x1fffu))
+#define RQ_ELASTIC 0x2000000u
 #define RQ_STARTED 0x80000000u
-struct ReplayRun { i64* fin; int* idx; u32* pu; int* off; int* dom; };   // dom: NUMA domain of a core grant, -1 where it spans several
+#define RQ_NOBODY 15u             // meta of a lane without a record: no pool, no demand
+
+// Running actions.  end: the round that releases it; pu: units (21 bits), first demand slot (5), pool (3), type (2), wide
+// (1); at: what it holds - mask (64 bits), word or node, domain.  A wide grant's units are the ones whose owner it is.
+struct ReplayRun { uint4* at; i64* fin; int* end; u32* pu; int* idx; };
+#define RR_UNITS(v) ((int)((v) & 0x1fffffu))
+#define RR_SLOT(v) ((int)(((v) >> 21) & 31u))
+#define RR_POOL(v) ((int)(((v) >> 26) & 7u))
+#define RR_TYPE(v) ((int)(((v) >> 29) & 3u))
+#define RR_WIDE 0x80000000u
+__device__ __forceinline__ u32 rr_pack(const PoolDev& pd, int j, int units, bool wide) {
+  return (u32)units | ((u32)pd.slot0 << 21) | ((u32)j << 26) | ((u32)pd.type << 29) | (wide ? RR_WIDE : 0u);
+}
+
+__device__ __forceinline__ i64 i64_of(u32 lo, u32 hi) { return (i64)(((u64)hi << 32) | lo); }
+
+// the first round at or after time t
+__device__ __forceinline__ int round_at(const ReplayWs& R, i64 t) {
+  if (t <= 0) return 0;
+  const u64 d = (u64)t - 1u;
+  // d * recip / 2^64 exceeds d / round_us by less than d * round_us / (round_us * 2^64) < 1 / round_us for d below 2^42 and
+  // round_us below 2^22 (where recip is set), so the floor is exact
+  const u64 q = R.round_recip && d < (1ull << 42) ? __umul64hi(d, R.round_recip) : d / (u64)R.round_us;
+  return q >= (u64)KR_NEVER - 1u ? KR_NEVER : (int)q + 1;
+}
 
 // A decoded record
 struct ReplayRec { i64 s, p, tl, arr; u32 meta, mask; u8 cg; };
@@ -77,89 +116,140 @@ __device__ __forceinline__ ReplayRec replay_decode(const Params& P, int j, u32 u
   const int rmin = __ffs(eff), c = pd.type == TG_POOL_GPU ? level_of(g, gang, rmin) : 0;
   r.s = clamp_param(s); r.p = clamp_param(p); r.tl = duration(r.s, r.p, rmin);
   r.mask = eff; r.cg = (u8)(g | (gang << 7));
-  r.meta = (u32)j | ((u32)pd.slot0 << 4) | ((u32)c << 10) | ((u32)(g * rmin) << 12);
+  r.meta = (u32)j | ((u32)pd.slot0 << 4) | ((u32)c << 10) | ((u32)(g * rmin) << 12) | (eff & (eff - 1) ? RQ_ELASTIC : 0u);
   return r;
 }
-// the waiting record at a queue position (any lane's own)
-__device__ __forceinline__ ReplayRec replay_rec(const Params& P, const ReplayQueue& Q, const int* wait, size_t row, int i, int& a) {
-  if (i < Q.cap) {
-    const int x = Q.q[i];
-    ReplayRec r;
-    r.s = Q.s[x]; r.p = Q.p[x]; r.tl = Q.tl[x]; r.arr = Q.arr[x]; r.meta = Q.meta[x]; r.mask = Q.mask[x]; r.cg = Q.cg[x];
-    a = Q.idx[x];
-    return r;
-  }
-  a = wait[i];
+__device__ __forceinline__ ReplayRec replay_load(const Params& P, size_t row, int a) {
   ReplayRec r = replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], P.a_s[row + a], P.a_p[row + a]);
   r.arr = P.a_arrival ? P.a_arrival[row + a] : 0;
   return r;
 }
-__device__ __forceinline__ u32 replay_meta(const Params& P, const ReplayQueue& Q, const int* wait, size_t row, int i) {
-  if (i < Q.cap) return Q.meta[Q.q[i]];
+__device__ __forceinline__ void replay_store(const ReplayQueue& Q, int x, const ReplayRec& r, int a) {
+  Q.sp[x] = make_uint4((u32)r.s, (u32)((u64)r.s >> 32), (u32)r.p, (u32)((u64)r.p >> 32));
+  Q.ta[x] = make_uint4((u32)r.tl, (u32)((u64)r.tl >> 32), (u32)r.arr, (u32)((u64)r.arr >> 32));
+  Q.c[x] = make_uint4((u32)a, r.meta, r.mask, (u32)r.cg);
+}
+// action, meta, mask and unit byte at a queue position (any lane's own); x: its slot where it is in shared memory
+__device__ __forceinline__ uint4 replay_facts(const Params& P, const ReplayQueue& Q, const int* wait, size_t row, int i, int& x) {
+  if (i < Q.cap) { x = Q.q[Q.at(i)]; return Q.c[x]; }
   const int a = wait[i];
-  return replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], 0, 0).meta;
+  const ReplayRec r = replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], 0, 0);
+  x = -1;
+  return make_uint4((u32)a, r.meta, r.mask, (u32)r.cg);
+}
+// ... and the rest of a record whose facts are known
+__device__ __forceinline__ ReplayRec replay_rec(const Params& P, const ReplayQueue& Q, size_t row, const uint4& c, int x) {
+  if (x < 0) return replay_load(P, row, (int)c.x);
+  const uint4 u = Q.sp[x], v = Q.ta[x];
+  ReplayRec r;
+  r.s = i64_of(u.x, u.y); r.p = i64_of(u.z, u.w); r.tl = i64_of(v.x, v.y); r.arr = i64_of(v.z, v.w);
+  r.meta = c.y; r.mask = c.z; r.cg = (u8)c.w;
+  return r;
 }
 
 // Live state of the scenario at hand: in the warp's shared memory, or in the arrays of ReplayWs where it is large.
-struct ReplayState { int* owner; u8* nm; int* dfree; int* pst; i64* win; };
+// slot: free capacity per demand slot, always in shared memory.
+struct ReplayState { u32* cores; int* dfree; int* owner; u8* nm; int* slot; };
 
-// One grant on a core pool with cores in use (fewest free cores that still fit, lowest domain,
-// lowest cores first; else ascending domains).  fit: the domain, -1 where the grant spans several.
-__device__ __forceinline__ void replay_place_cpu(const PoolDev& pd, int* owner, int* dfree, int k, int id, int lane, int& node, int& off, int& fit) {
-  const int D = pd.capacity / pd.group;
-  u32 best = 0xffffffffu; int dom = -1;
+// What a grant holds: a mask of one word (core pools) or node (GPU pools), or owner entries (wide).
+// node / off: NUMA domain or GPU node, and the first core or GPU.
+struct ReplayGrant { int node, off, word, dom; u32 lo, hi; bool wide; };
+
+// One grant of k cores on a pool with cores in use: fewest free cores that still fit, lowest domain, lowest cores first;
+// else ascending domains.  cores / dfree / owner: the pool's own rows.
+__device__ __forceinline__ ReplayGrant replay_take_cores(int group, int n_dom, int wpd, u32* cores, int* dfree, int* owner,
+                                                         int k, int id, int lane) {
+  ReplayGrant G;
+  G.node = G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = false;
+  int dom = -1;
+  if (n_dom <= 32 && group < (1 << 26)) {
+    const int f = lane < n_dom ? dfree[lane] : -1;
+    const u32 mn = __reduce_min_sync(TG_FULL, f >= k ? ((u32)f << 5) | (u32)lane : 0xffffffffu);
+    if (mn != 0xffffffffu) dom = (int)(mn & 31u);
+  } else {
+    u32 best = 0xffffffffu; int at = -1;
 #pragma unroll 1
-  for (int d = lane; d < D; d += 32) { const int f = dfree[d]; if (f >= k && (u32)f < best) { best = (u32)f; dom = d; } }
-  const u32 mn = __reduce_min_sync(TG_FULL, best);
-  int lo = 0, hi = pd.capacity, d1 = -1;
-  if (mn != 0xffffffffu) {
-    d1 = (int)__reduce_min_sync(TG_FULL, best == mn ? (u32)dom : 0xffffffffu);
-    lo = d1 * pd.group; hi = lo + pd.group;
+    for (int d = lane; d < n_dom; d += 32) { const int f = dfree[d]; if (f >= k && (u32)f < best) { best = (u32)f; at = d; } }
+    const u32 mn = __reduce_min_sync(TG_FULL, best);
+    if (mn != 0xffffffffu) dom = (int)__reduce_min_sync(TG_FULL, best == mn ? (u32)at : 0xffffffffu);
   }
-  int need = k, first = -1;
+  int need = k;
+  const int end = dom >= 0 ? (dom + 1) * wpd : n_dom * wpd;
 #pragma unroll 1
-  for (int c0 = lo; c0 < hi && need > 0; c0 += 32) {
-    const int c = c0 + lane;
-    const u32 b = __ballot_sync(TG_FULL, c < hi && owner[c] < 0);
-    const int rank = __popc(b & ((1u << lane) - 1u));
-    const bool mine = ((b >> lane) & 1u) && rank < need;
-    if (mine) owner[c] = id;
-    if (b && first < 0) first = c0 + __ffs(b) - 1;
-    const int got = min(need, __popc(b));
-    if (d1 < 0 && mine) atomicSub(&dfree[c / pd.group], 1);
+  for (int w = dom >= 0 ? dom * wpd : 0; w < end && need > 0; ++w) {
+    const uint2 m = *(const uint2*)(cores + 2 * w);
+    if ((m.x | m.y) == 0u) continue;
+    // the lowest `need` free cores of the word: every lane looks at two of them
+    const u32 below = (1u << lane) - 1u;
+    const int nlo = __popc(m.x);
+    const u32 lo = __ballot_sync(TG_FULL, ((m.x >> lane) & 1u) && __popc(m.x & below) < need);
+    const u32 hi = __ballot_sync(TG_FULL, ((m.y >> lane) & 1u) && nlo + __popc(m.y & below) < need);
+    const int got = __popc(lo) + __popc(hi);
+    const int d = wpd == 1 ? w : w / wpd, c0 = d * group + (wpd == 1 ? 0 : (w - d * wpd) * 64);   // the word's first core
+    if (G.off < 0) {
+      G.off = c0 + (lo ? __ffs(lo) - 1 : 31 + __ffs(hi)); G.node = d;
+      G.word = w; G.dom = d; G.lo = lo; G.hi = hi;
+      G.wide = got < need;
+      if (G.wide) G.dom = G.off;                           // (where the search for its cores begins)
+    }
+    if (G.wide) {
+      if ((lo >> lane) & 1u) owner[c0 + lane] = id;
+      if ((hi >> lane) & 1u) owner[c0 + 32 + lane] = id;
+    }
+    __syncwarp();
+    if (lane == 0) { *(uint2*)(cores + 2 * w) = make_uint2(m.x & ~lo, m.y & ~hi); dfree[d] -= got; }
     need -= got;
+    __syncwarp();
   }
-  if (d1 >= 0 && lane == 0) dfree[d1] -= k;
-  node = d1 >= 0 ? d1 : (first >= 0 ? first / pd.group : -1); off = first; fit = d1;
-  __syncwarp();
+  return G;
 }
 
 // One candidate alone on a GPU pool: nreq chunks of 2^lz GPUs (Section 5.3: smallest sufficient maximal free block,
 // lowest node, lowest start); node / off: the first chunk.
-__device__ __forceinline__ void replay_place_gpu(const PoolDev& pd, u8* nm, int* owner, int lz, int nreq, int id, int lane, int& node, int& off) {
+__device__ __forceinline__ ReplayGrant replay_take_gpus(const PoolDev& pd, u8* nm, int* owner, int lz, int nreq, int id, int lane) {
+  ReplayGrant G;
+  G.node = G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = nreq > 1;
   const int top = ilog2(pd.group), z = 1 << lz;
   const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
-  node = -1; off = -1;
 #pragma unroll 1
   for (int rep = 0; rep < nreq; ++rep) {
-    int at = -1, level = 4;
+    u32 best = 0xffffffffu;                                // level << 24 | node
 #pragma unroll 1
-    for (int v0 = 0; v0 < pd.n_nodes; v0 += 32) {
-      const u32 lev = v0 + lane < pd.n_nodes ? node_levels(nm[v0 + lane] | pad) & (~0u << lz) : 0u;
-      const int mine = lev ? __ffs(lev) - 1 : 4;           // the smallest sufficient block of the lane's node
-      const int best = __reduce_min_sync(TG_FULL, mine);
-      if (best < level) { level = best; at = v0 + __ffs(__ballot_sync(TG_FULL, mine == best)) - 1; }
-      if (level == lz) break;
+    for (int v = lane; v < pd.n_nodes; v += 32) {
+      const u32 lev = node_levels(nm[v] | pad) & (~0u << lz);   // the smallest sufficient block of the node
+      if (lev) best = min(best, ((u32)(__ffs(lev) - 1) << 24) | (u32)v);
     }
-    if (at < 0 || level > top) continue;                  // cannot happen: the selection fits
-    const u32 busy = nm[at] | pad;
-    const int start = node_block_start(busy, level);
+    best = __reduce_min_sync(TG_FULL, best);
+    const int at = (int)(best & 0xffffffu), level = (int)(best >> 24);
+    if (level > top) continue;                             // cannot happen: the selection fits
+    const u32 busy = nm[at];
+    const int start = node_block_start(busy | pad, level);
+    const u32 bits = ((1u << z) - 1u) << start;
     __syncwarp();
-    if (lane == 0) nm[at] |= (u8)(((1u << z) - 1u) << start);
-    if (lane < z) owner[at * pd.group + start + lane] = id;
-    if (rep == 0) { node = at; off = start; }
+    if (lane == 0) nm[at] = (u8)(busy | bits);
+    if (G.wide && lane < z) owner[at * pd.group + start + lane] = id;
+    if (rep == 0) { G.node = at; G.off = start; G.word = at; G.lo = bits; }
     __syncwarp();
   }
+  return G;
+}
+
+// free capacity of a GPU pool's four demand slots
+__device__ __forceinline__ void replay_gpu_slots(const PoolDev& pd, const u8* nm_row, int* slot, int lane) {
+  int c[4];
+  if (pd.n_nodes <= 32) {
+    // the four counts of free blocks in one word: at most 256, 128, 64 and 32
+    const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
+    u32 x = 0;
+    if (lane < pd.n_nodes) {
+      const NodeBlocks b = node_blocks(nm_row[pd.node0 + lane] | pad);
+      x = (u32)__popc(b.s1) | ((u32)__popc(b.s2) << 9) | ((u32)__popc(b.s4) << 17) | ((u32)__popc(b.s8) << 24);
+    }
+    x = __reduce_add_sync(TG_FULL, x);
+    c[3] = (int)(x >> 24) * 8; c[2] = c[3] + (int)((x >> 17) & 127u) * 4; c[1] = c[2] + (int)((x >> 9) & 255u) * 2; c[0] = c[1] + (int)(x & 511u);
+  } else gpu_caps(pd, nm_row, lane, c);
+  if (lane < 4) slot[pd.slot0 + lane] = pick4(c, lane);
+  __syncwarp();
 }
 
 // The selection of a pool with a choice to make: its candidates (among the first n positions) and, where an eviction
@@ -180,13 +270,14 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
 #pragma unroll 1
   for (int i0 = 0; i0 < n; i0 += 32) {
     const int i = i0 + lane;
-    int a = 0; ReplayRec r; r.meta = 15u;
-    if (i < n) r = replay_rec(P, Q, wait, row, i, a);
-    const bool mine = i < n && RQ_POOL(r.meta) == j;
+    int x = -1; uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u);
+    if (i < n) c = replay_facts(P, Q, wait, row, i, x);
+    const bool mine = RQ_POOL(c.y) == j;
     const u32 b = __ballot_sync(TG_FULL, mine);
     if (mine) {
+      const ReplayRec r = replay_rec(P, Q, row, c, x);
       const int k = cm + __popc(b & ((1u << lane) - 1u));
-      C.cidx[k] = a; C.cmask[k] = r.mask; C.cg[k] = r.cg; C.cs[k] = r.s; C.cp[k] = r.p;
+      C.cidx[k] = (int)c.x; C.cmask[k] = r.mask; C.cg[k] = r.cg; C.cs[k] = r.s; C.cp[k] = r.p;
       C.rkeep[k] = (u8)__ffs(r.mask); C.pnode[k] = -1; C.poff[k] = -1;
       elastic |= (r.mask & (r.mask - 1)) != 0;
     }
@@ -206,10 +297,10 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
 #pragma unroll 1
     for (int i0 = n; i0 < nw; i0 += 32) {
       const int i = i0 + lane;
-      int a; ReplayRec r; r.meta = 15u;
-      if (i < nw) r = replay_rec(P, Q, wait, row, i, a);
-      const u32 b = __ballot_sync(TG_FULL, i < nw && RQ_POOL(r.meta) == j);
-      if ((b >> lane) & 1u) ac[n_ac + __popc(b & ((1u << lane) - 1u))] = r.tl;
+      int x = -1; uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u);
+      if (i < nw) c = replay_facts(P, Q, wait, row, i, x);
+      const u32 b = __ballot_sync(TG_FULL, RQ_POOL(c.y) == j);
+      if ((b >> lane) & 1u) ac[n_ac + __popc(b & ((1u << lane) - 1u))] = replay_rec(P, Q, row, c, x).tl;
       if (first < 0 && b) first = i0 + __ffs(b) - 1;
       n_ac += __popc(b);
     }
@@ -217,7 +308,7 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
 #pragma unroll 1
     for (int i0 = 0; i0 < nr; i0 += 32) {
       const int i = i0 + lane;
-      const u32 b = __ballot_sync(TG_FULL, i < nr && (int)(run.pu[i] >> 24) == j);
+      const u32 b = __ballot_sync(TG_FULL, i < nr && RR_POOL(run.pu[i]) == j);
       if ((b >> lane) & 1u) { const i64 f = run.fin[i]; seeds[ns + __popc(b & ((1u << lane) - 1u))] = f > now ? f - now : 0; }
       ns += __popc(b);
     }
@@ -230,8 +321,9 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
     T.n_ac = n_ac; T.ac_tmin = ac;
     T.ac_first.s = T.ac_first.p = 0; T.ac_first.mask = 1; T.ac_first.g = 1; T.ac_first.gang = 0;
     if (first >= 0) {
-      int a;
-      const ReplayRec r = replay_rec(P, Q, wait, row, first, a);
+      int x;
+      const uint4 c = replay_facts(P, Q, wait, row, first, x);
+      const ReplayRec r = replay_rec(P, Q, row, c, x);
       T.ac_first.s = r.s; T.ac_first.p = r.p; T.ac_first.mask = r.mask; T.ac_first.g = r.cg & 0x7f; T.ac_first.gang = r.cg >> 7;
     }
     T.seeds = seeds; T.n_seeds = ns;
@@ -257,13 +349,11 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
   ReplayQueue Q;
   Q.cap = R.wcap;
   {
-    char* at = fast + KR_FAST_BYTES;
-    Q.s = (i64*)at; Q.p = Q.s + Q.cap; Q.tl = Q.p + Q.cap; Q.arr = Q.tl + Q.cap; Q.key = (u64*)(Q.arr + Q.cap);
-    at = (char*)(Q.key + (EXT ? Q.cap : 0));
-    Q.idx = (int*)at; Q.meta = (u32*)(Q.idx + Q.cap); Q.mask = Q.meta + Q.cap;
-    Q.q = (unsigned short*)(Q.mask + Q.cap); Q.free = Q.q + Q.cap; Q.cg = (u8*)(Q.free + Q.cap);
+    char* at = fast + KR_FAST_BYTES + KR_SLOT_BYTES;
+    Q.sp = (uint4*)at; Q.ta = Q.sp + Q.cap; Q.c = Q.ta + Q.cap; Q.key = (u64*)(Q.c + Q.cap);
+    Q.q = (unsigned short*)(Q.key + Q.cap); Q.free = Q.q + Q.cap;
   }
-  char* const run_at = fast + KR_FAST_BYTES + align16((size_t)Q.cap * KR_WAIT_BYTES);
+  char* const run_at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + align16((size_t)Q.cap * KR_WAIT_BYTES);
   char* const state_at = run_at + align16((size_t)R.rcap * KR_RUN_BYTES);
 #pragma unroll 1
   for (int sc = blockIdx.x; sc < P.S; sc += gridDim.x) {
@@ -271,24 +361,25 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
     const int n_act = uniform(min(max(P.n_actions[sc], 0), P.N));
     int* wait = R.wait + row; u64* wkey = EXT && R.wkey ? R.wkey + row : nullptr;
     ReplayRun run;
-    if (R.rcap > 0) { run.fin = (i64*)run_at; run.idx = (int*)(run.fin + R.rcap); run.pu = (u32*)(run.idx + R.rcap); run.off = (int*)(run.pu + R.rcap); run.dom = run.off + R.rcap; }
-    else { run.fin = R.run_fin + row; run.idx = R.run_idx + row; run.pu = R.run_pu + row; run.off = R.run_off + row; run.dom = R.run_dom + row; }
+    if (R.rcap > 0) {
+      run.at = (uint4*)run_at; run.fin = (i64*)(run.at + R.rcap); run.end = (int*)(run.fin + R.rcap); run.pu = (u32*)(run.end + R.rcap);
+      run.idx = (int*)(run.pu + R.rcap);
+    } else { run.at = R.run_at + row; run.fin = R.run_fin + row; run.end = R.run_end + row; run.pu = R.run_pu + row; run.idx = R.run_idx + row; }
     ReplayState Z;
+    Z.slot = (int*)(fast + KR_FAST_BYTES);
     if (R.state_bytes > 0) {
-      const size_t o_nm = align16((size_t)R.U * 4), o_df = o_nm + align16((size_t)P.n_nodes_total + 1),
-                   o_ps = o_df + align16((size_t)R.Dtot * 4), o_wn = o_ps + align16((size_t)P.P * 8);
-      Z.owner = (int*)state_at; Z.nm = (u8*)(state_at + o_nm); Z.dfree = (int*)(state_at + o_df);
-      Z.pst = (int*)(state_at + o_ps); Z.win = (i64*)(state_at + o_wn);
+      const size_t o_df = align16((size_t)R.W * 8), o_ow = o_df + align16((size_t)R.Dtot * 4), o_nm = o_ow + align16((size_t)R.U * 4);
+      Z.cores = (u32*)state_at; Z.dfree = (int*)(state_at + o_df); Z.owner = (int*)(state_at + o_ow); Z.nm = (u8*)(state_at + o_nm);
     } else {
-      Z.owner = R.owner + (size_t)sc * R.U; Z.nm = R.nm + (size_t)sc * P.n_nodes_total; Z.dfree = R.dfree + (size_t)sc * R.Dtot;
-      Z.pst = R.pst + (size_t)sc * P.P * 2; Z.win = R.win + (size_t)sc * P.P;
+      Z.cores = R.cores + (size_t)sc * R.W * 2; Z.dfree = R.dfree + (size_t)sc * R.Dtot; Z.owner = R.owner + (size_t)sc * R.U;
+      Z.nm = R.nm + (size_t)sc * ((P.n_nodes_total + 4) & ~3);
     }
     int* occ = R.occupancy ? R.occupancy + (size_t)sc * R.max_rounds * P.P : nullptr;
-    // outputs and state start empty
+    // outputs and state start empty (the occupancy rows were zeroed before)
 #pragma unroll 4
     for (int i = lane; i < P.N; i += 32) { P.o_alloc[row + i] = 0; P.o_node[row + i] = -1; P.o_off[row + i] = -1; P.o_act[row + i] = -1; }
     int status = 0;
-#pragma unroll 1
+#pragma unroll 2
     for (int i = lane; i < n_act; i += 32) {
       const int j = P.a_pool[row + i];
       int g, gang; u32 eff;
@@ -306,162 +397,191 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
     }
     status = __reduce_or_sync(TG_FULL, status);
     if (status & TG_ST_BAD_ACTION) status = TG_ST_BAD_ACTION;
-    int busy = 0;                                          // lane j: units in use of core / GPU pool j
 #pragma unroll 1
     for (int j = 0; j < P.P; ++j) {
       const PoolDev& pd = P.pool[j];
-      if (pd.type == TG_POOL_API) { if (lane < 2) Z.pst[j * 2 + lane] = 0; if (lane == 0) Z.win[j] = 0; continue; }
-      int taken = 0;
+      if (pd.type == TG_POOL_GPU) {
+        int taken = 0;
 #pragma unroll 1
-      for (int c = lane; c < pd.capacity; c += 32) {
-        int v = -1;
-        if (pd.type == TG_POOL_GPU && P.gpu_busy && (P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + c / pd.group] >> (c % pd.group) & 1)) { v = -2; ++taken; }
-        Z.owner[R.unit0[j] + c] = v;
+        for (int v = lane; v < pd.n_nodes; v += 32) {
+          const u32 b = (P.gpu_busy ? P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + v] : 0u) & ((1u << pd.group) - 1u);
+          Z.nm[pd.node0 + v] = (u8)b;
+          taken += __popc(b);
+        }
+        taken = warp_sum32(taken);
+        if (occ && lane == 0 && status == 0) occ[j] = taken;   // round 0's difference
+        __syncwarp();
+        replay_gpu_slots(pd, Z.nm, Z.slot, lane);
+      } else if (lane == 0) Z.slot[pd.slot0] = pd.capacity;
+      if (pd.type == TG_POOL_API) continue;
+#pragma unroll 1
+      for (int c = lane; c < pd.capacity; c += 32) Z.owner[R.unit0[j] + c] = -1;
+      if (pd.type != TG_POOL_CPU) continue;
+      const int wpd = R.wpd[j];
+#pragma unroll 1
+      for (int w = lane; w < R.n_dom[j] * wpd; w += 32) {
+        const int left = pd.group - (w % wpd) * 64;         // cores of the domain from this word on
+        const u64 m = left >= 64 ? ~0ull : (1ull << left) - 1ull;
+        *(uint2*)(Z.cores + 2 * (R.word0[j] + w)) = make_uint2((u32)m, (u32)(m >> 32));
       }
-      taken = warp_sum32(taken);
-      if (lane == j) busy = taken;
-      if (pd.type == TG_POOL_GPU)
 #pragma unroll 1
-        for (int v = lane; v < pd.n_nodes; v += 32)
-          Z.nm[pd.node0 + v] = (P.gpu_busy ? P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + v] : 0) & ((1u << pd.group) - 1u);
-      if (pd.type == TG_POOL_CPU)
-#pragma unroll 1
-        for (int d = lane; d < pd.capacity / pd.group; d += 32) Z.dfree[R.dom0[j] + d] = pd.group;
+      for (int d = lane; d < R.n_dom[j]; d += 32) Z.dfree[R.dom0[j] + d] = pd.group;
     }
 #pragma unroll 1
     for (int i = lane; i < Q.cap; i += 32) Q.free[i] = (unsigned short)i;
-    if (occ)
-#pragma unroll 4
-      for (int i = lane; i < R.max_rounds * P.P; i += 32) occ[i] = 0;
+    Q.head = 0;
     __syncwarp();
     int rounds = 0;
     if (status == 0) {
       int next = 0, nw = 0, nr = 0, r = 0, free_slots = Q.cap;
       bool drained = false, gated = false;                 // gated: an arrival waits for a node (Section 5.2)
       i64 total = 0; int selected = 0;
-      i64 min_fin = TG_INF;                                // earliest completion among what runs
-      // first round at or after time t > now_t, the time of round r_t (a 32-bit division where the distance allows)
-      auto round_after = [&](i64 t, i64 now_t, int r_t) -> i64 {
-        const i64 d = max(t - now_t, 1ll);
-        return d <= 0xffffffffll && R.round_us <= 0xffffffffll ? (i64)r_t + (i64)(((u32)d - 1u) / (u32)R.round_us + 1u) : (i64)r_t + (d - 1) / R.round_us + 1;
-      };
-      // arrivals, 32 at a time: lane k holds record base + k
-      int base = -32;
-      i64 b_arr = TG_INF; ReplayRec b_rec; b_rec.s = b_rec.p = b_rec.tl = b_rec.arr = 0; b_rec.meta = 0; b_rec.mask = 1; b_rec.cg = 1;
-      i64 next_arr = TG_INF;
-      auto refill = [&]() {                                // the records from `next` on
-        base = next;
-        const int i = base + lane;
-        b_arr = TG_INF;
+      int min_end = KR_NEVER;                              // the first round that releases something
+      // arrivals, 32 at a time: lane k holds record base + k; the next batch's columns are on their way
+      int base = 0;
+      int l_pool = 0; u32 l_unit = 1, l_mask = 1; i64 l_s = 0, l_p = 0, l_arr = 0;
+      auto fetch = [&](int from) {
+        const int i = from + lane;
         if (i < n_act) {
-          const int j = P.a_pool[row + i];
-          const u32 un = P.a_unit[row + i], mk = P.a_mask[row + i];
-          const i64 s = P.a_s[row + i], p = P.a_p[row + i];
-          b_arr = P.a_arrival ? P.a_arrival[row + i] : 0;
-          b_rec = replay_decode(P, j, un, mk, s, p);
+          l_pool = P.a_pool[row + i]; l_unit = P.a_unit[row + i]; l_mask = P.a_mask[row + i]; l_s = P.a_s[row + i]; l_p = P.a_p[row + i];
+          l_arr = P.a_arrival ? P.a_arrival[row + i] : 0;
         }
-        next_arr = __shfl_sync(TG_FULL, b_arr, 0);
       };
-      if (n_act > 0) refill();
-      int capreg = 0;                                      // lane v: free capacity of demand slot v
-      u32 stale = ~0u;                                     // pools whose slots have to be worked out again
-      bool windows = false;
-      // lane j: where pool j's units in use are counted if it is a quota / concurrency pool, else -1
-      const int api_at = lane < P.P && P.pool[lane].type == TG_POOL_API ? lane * 2 + (P.pool[lane].window_us > 0 ? 0 : 1) : -1;
-#pragma unroll 1
-      for (int j = 0; j < P.P; ++j) windows |= P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0;
+      ReplayRec b_rec; int b_at = KR_NEVER;                // b_at: the round that admits the lane's arrival
+      int next_at = KR_NEVER;
+      auto refill = [&](int from) {                        // the batch that was fetched becomes the current one
+        base = from;
+        b_rec = replay_decode(P, l_pool, l_unit, l_mask, l_s, l_p);
+        b_rec.arr = l_arr;
+        b_at = from + lane < n_act ? round_at(R, l_arr) : KR_NEVER;
+        next_at = __shfl_sync(TG_FULL, b_at, 0);
+        fetch(from + 32);
+      };
+      fetch(0);
+      refill(0);
+      // lane v < 32: free capacity of demand slot v is Z.slot[v]; lane j < P: where pool j's is, and the round in which its
+      // quota window turns
+      const int D = P.V - P.P;
+      const int my_slot = lane < P.P ? P.pool[lane].slot0 : 0;
+      const i64 my_window = lane < P.P && P.pool[lane].type == TG_POOL_API ? P.pool[lane].window_us : 0;
+      int my_turn = my_window > 0 ? round_at(R, my_window) : KR_NEVER;
+      int next_turn = warp_min32(my_turn);
       while (r < R.max_rounds) {
         const i64 now = (i64)r * R.round_us;
-        // 1. quota refill
-        if (windows)
-#pragma unroll 1
-          for (int j = 0; j < P.P; ++j) {
-            const PoolDev& pd = P.pool[j];
-            if (pd.type != TG_POOL_API || pd.window_us <= 0) continue;
-            const i64 w0 = Z.win[j];
-            if (now >= w0 * pd.window_us && now < (w0 + 1) * pd.window_us) continue;
-            __syncwarp();
-            if (lane == 0) { Z.win[j] = now / pd.window_us; Z.pst[j * 2] = 0; }
-            __syncwarp();
-            stale |= 1u << j;
+        // 1. quota refill: usage restarts with its window
+        if (r >= next_turn) {
+          if (r >= my_turn) {
+            const int cap = P.pool[lane].capacity, used = cap - Z.slot[my_slot];
+            if (occ && used) atomicSub(&occ[(size_t)my_turn * P.P + lane], used);
+            Z.slot[my_slot] = cap;
+            my_turn = round_at(R, (now / my_window + 1) * my_window);
           }
-        // 2. release what has finished; the running list is compacted in place
-        if (min_fin <= now) {
-          int kept = 0;
-          i64 mf = TG_INF;
+          next_turn = warp_min32(my_turn);
+          __syncwarp();
+        }
+        // 2. release what has finished, a lane each; the running list is compacted in place
+        while (min_end <= r) {
+          // (the memory of a trajectory that ends goes back in the order of the rounds)
+          const int until = EXT && R.traj_last ? min_end : r;
+          int kept = 0, me = KR_NEVER;
+          u32 touched = 0;                                 // GPU pools
 #pragma unroll 1
           for (int i0 = 0; i0 < nr; i0 += 32) {
             const int i = i0 + lane;
-            i64 fin = TG_INF; int a = 0, of = 0, dm = -1; u32 pu = 0;
-            if (i < nr) { fin = run.fin[i]; a = run.idx[i]; pu = run.pu[i]; of = run.off[i]; dm = run.dom[i]; }
-            const bool done = fin <= now, stay = i < nr && !done;
-            if (stay) mf = min(mf, fin);
-            const u32 bk = __ballot_sync(TG_FULL, stay);
-            u32 rest = __ballot_sync(TG_FULL, done);
-            if (rest || kept != i0) {
-              if (stay) { const int k = kept + __popc(bk & below); run.fin[k] = fin; run.idx[k] = a; run.pu[k] = pu; run.off[k] = of; run.dom[k] = dm; }
-            }
-            kept += __popc(bk);
-            __syncwarp();
+            const int end = i < nr ? run.end[i] : KR_NEVER;
+            const bool done = i < nr && end <= until, stay = i < nr && !done;
+            const u32 bd = __ballot_sync(TG_FULL, done), bk = __ballot_sync(TG_FULL, stay);
+            if (stay) me = min(me, end);
+            if (bd || kept != i0) {
+              uint4 at = make_uint4(0u, 0u, 0u, 0u); u32 pu = 0; int a = 0; i64 fin = 0;
+              if (i < nr) { at = run.at[i]; pu = run.pu[i]; a = run.idx[i]; fin = run.fin[i]; }
+              if (done) {
+                const int type = RR_TYPE(pu), units = RR_UNITS(pu), j = RR_POOL(pu);
+                if (type == TG_POOL_GPU) {
+                  touched |= 1u << j;
+                  if (!(pu & RR_WIDE)) {
+                    const u32 v = (u32)P.pool[j].node0 + at.z;
+                    atomicAnd((u32*)Z.nm + (v >> 2), ~(at.x << (8u * (v & 3u))));
+                  }
+                } else if (type == TG_POOL_CPU) {
+                  atomicAdd(&Z.slot[RR_SLOT(pu)], units);
+                  if (!(pu & RR_WIDE)) {
+                    u32* w = Z.cores + 2 * (R.word0[j] + (int)at.z);
+                    if (at.x) atomicOr(w, at.x);
+                    if (at.y) atomicOr(w + 1, at.y);
+                    atomicAdd(&Z.dfree[R.dom0[j] + (int)at.w], units);
+                  }
+                } else if (P.pool[j].window_us == 0) atomicAdd(&Z.slot[RR_SLOT(pu)], units);   // (used quota is not given back)
+                if (EXT)
 #pragma unroll 1
-            for (; rest; rest &= rest - 1) {
-              const int b = __ffs(rest) - 1;
-              const int fa = __shfl_sync(TG_FULL, a, b), fo = __shfl_sync(TG_FULL, of, b), fd = __shfl_sync(TG_FULL, dm, b);
-              const u32 fpu = __shfl_sync(TG_FULL, pu, b);
-              const int j = (int)(fpu >> 24), units = (int)(fpu & 0xffffffu);
-              const PoolDev& pd = P.pool[j];
-              stale |= 1u << j;
-              if (EXT && R.trajectory && R.traj_last && lane == 0 && pd.type == TG_POOL_CPU && R.traj_last[row + fa]) {
-                // the trajectory's last action has ended: its memory goes back to its node
-                const int t = R.trajectory[row + fa];
-                if (t >= 0 && t < R.max_traj) {
-                  int* tn = R.traj_node + (size_t)sc * R.max_traj;
-                  if (tn[t] >= 0) { R.mem_free[(size_t)sc * P.P + tn[t]] += (i64)R.traj_mem[row + fa]; tn[t] = -1; }
-                }
+                  for (int e = 0; e < P.n_side; ++e) {     // a concurrency pool held the action's further amounts until now
+                    const int k = P.a_side_pool[e * P.side_plane + row + a];
+                    if (k != 0xff && P.pool[k].window_us == 0) atomicAdd(&Z.slot[P.pool[k].slot0], (int)P.a_side_units[e * P.side_plane + row + a]);
+                  }
               }
-              if (EXT && P.n_side > 0) stale = ~0u;
-              if (EXT && P.n_side > 0 && lane == 0)        // a concurrency pool held the action's further amounts until now
 #pragma unroll 1
-                for (int e = 0; e < P.n_side; ++e) {
-                  const int k = P.a_side_pool[e * P.side_plane + row + fa];
-                  if (k != 0xff && P.pool[k].window_us == 0) Z.pst[k * 2 + 1] -= P.a_side_units[e * P.side_plane + row + fa];
-                }
-              if (pd.type == TG_POOL_API) { if (pd.window_us == 0 && lane == 0) Z.pst[j * 2 + 1] -= units; }
-              else {
-                if (lane == j) busy -= units;
+              for (u32 wide = __ballot_sync(TG_FULL, done && (pu & RR_WIDE)); wide; wide &= wide - 1) {
+                const int b = __ffs(wide) - 1, fa = __shfl_sync(TG_FULL, a, b);
+                const u32 fpu = __shfl_sync(TG_FULL, pu, b);
+                const int from = __shfl_sync(TG_FULL, (int)at.w, b), j = RR_POOL(fpu);
+                const PoolDev& pd = P.pool[j];
+                const bool cpu = pd.type == TG_POOL_CPU;
                 int* ow = Z.owner + R.unit0[j];
-                int left = units;
-                // (a core pool's grant starts at its lowest core; chunks of replicas can lie anywhere)
+                int left = RR_UNITS(fpu);
 #pragma unroll 1
-                for (int c0 = pd.type == TG_POOL_CPU ? fo & ~31 : 0; c0 < pd.capacity && left > 0; c0 += 32) {
+                for (int c0 = cpu ? from & ~31 : 0; c0 < pd.capacity && left > 0; c0 += 32) {
                   const int c = c0 + lane;
                   const bool mine = c < pd.capacity && ow[c] == fa;
                   const u32 mb = __ballot_sync(TG_FULL, mine);
                   if (!mb) continue;
-                  if (mine) ow[c] = -1;
                   left -= __popc(mb);
-                  if (pd.type == TG_POOL_CPU) {
-                    if (fd < 0) { if (mine) atomicAdd(&Z.dfree[R.dom0[j] + c / pd.group], 1); }
-                    else if (lane == 0) Z.dfree[R.dom0[j] + fd] += __popc(mb);
-                  }
-                  else if (lane < 32 / pd.group) {
-                    const u32 bits = (mb >> (lane * pd.group)) & ((1u << pd.group) - 1u);
-                    if (bits) Z.nm[pd.node0 + c0 / pd.group + lane] &= (u8)~bits;
+                  if (mine) {
+                    ow[c] = -1;
+                    const int d = c / pd.group, x = c - d * pd.group;
+                    if (cpu) {
+                      const int w = d * R.wpd[j] + (x >> 6);
+                      atomicOr(Z.cores + 2 * (R.word0[j] + w) + ((x >> 5) & 1), 1u << (x & 31));
+                      atomicAdd(&Z.dfree[R.dom0[j] + d], 1);
+                    } else {
+                      const u32 v = (u32)(pd.node0 + d);
+                      atomicAnd((u32*)Z.nm + (v >> 2), ~(1u << (x + 8 * (int)(v & 3u))));
+                    }
                   }
                 }
               }
+              if (EXT && R.trajectory && R.traj_last)
+#pragma unroll 1
+                for (u32 rest = bd; rest; rest &= rest - 1) {
+                  const int b = __ffs(rest) - 1, fa = __shfl_sync(TG_FULL, a, b);
+                  const u32 fpu = __shfl_sync(TG_FULL, pu, b);
+                  if (lane == 0 && RR_TYPE(fpu) == TG_POOL_CPU && R.traj_last[row + fa]) {
+                    // the trajectory's last action has ended: its memory goes back to its node
+                    const int t = R.trajectory[row + fa];
+                    if (t >= 0 && t < R.max_traj) {
+                      int* tn = R.traj_node + (size_t)sc * R.max_traj;
+                      if (tn[t] >= 0) { R.mem_free[(size_t)sc * P.P + tn[t]] += (i64)R.traj_mem[row + fa]; tn[t] = -1; }
+                    }
+                  }
+                }
               __syncwarp();
+              const int k = kept + __popc(bk & below);
+              if (stay && k != i) { run.at[k] = at; run.fin[k] = fin; run.end[k] = end; run.pu[k] = pu; run.idx[k] = a; }
             }
+            kept += __popc(bk);
+            __syncwarp();
           }
           nr = kept;
-          min_fin = warp_min64(mf);
+          min_end = warp_min32(me);
           gated = false;
+          touched = __reduce_or_sync(TG_FULL, touched);
+#pragma unroll 1
+          for (; touched; touched &= touched - 1) replay_gpu_slots(P.pool[__ffs(touched) - 1], Z.nm, Z.slot, lane);
         }
         // 3. admit arrivals
         bool was_gated = gated;
 #pragma unroll 1
-        while (next_arr <= now && !was_gated) {
-          int cnt = __popc(__ballot_sync(TG_FULL, base + lane >= next && b_arr <= now));   // sorted: the lanes from next - base on
+        while (next_at <= r && !was_gated) {
+          int cnt = __popc(__ballot_sync(TG_FULL, base + lane >= next && b_at <= r));   // sorted: the lanes from next - base on
           const int k0 = next - base;
           if (EXT && R.trajectory) {
             // per-node CPU scheduling: an arrival joins the queue once its trajectory has a node; the first one
@@ -495,7 +615,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
 #pragma unroll 1
               for (int i0 = 0; i0 < nw; i0 += 32) {
                 const int i = i0 + lane;
-                const u64 ki = i >= nw ? ~0ull : (i < Q.cap ? Q.key[Q.q[i]] : wkey[i]);
+                const u64 ki = i >= nw ? ~0ull : (i < Q.cap ? Q.key[Q.q[Q.at(i)]] : wkey[i]);
                 const u32 le = __ballot_sync(TG_FULL, i < nw && ki <= key);
                 p += __popc(le);
                 if (le != TG_FULL) break;                  // (sorted)
@@ -513,8 +633,8 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                   hi = lo;
                 }
                 if (p < Q.cap) {
-                  const int x = Q.q[Q.cap - 1];
-                  if (lane == 0) { wait[Q.cap] = Q.idx[x]; wkey[Q.cap] = Q.key[x]; Q.free[free_slots] = (unsigned short)x; }
+                  const int x = Q.q[Q.at(Q.cap - 1)];
+                  if (lane == 0) { wait[Q.cap] = (int)Q.c[x].x; wkey[Q.cap] = Q.key[x]; Q.free[free_slots] = (unsigned short)x; }
                   ++free_slots;
                   __syncwarp();
                 }
@@ -524,18 +644,15 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 for (int hi = min(nw, Q.cap - 1); hi > p;) {
                   const int lo = max(p, hi - 32), i = lo + lane;
                   unsigned short v = 0;
-                  if (i < hi) v = Q.q[i];
+                  if (i < hi) v = Q.q[Q.at(i)];
                   __syncwarp();
-                  if (i < hi) Q.q[i + 1] = v;
+                  if (i < hi) Q.q[Q.at(i + 1)] = v;
                   __syncwarp();
                   hi = lo;
                 }
                 const int x = Q.free[--free_slots];
                 __syncwarp();
-                if (lane == b) {
-                  Q.q[p] = (unsigned short)x; Q.s[x] = b_rec.s; Q.p[x] = b_rec.p; Q.tl[x] = b_rec.tl; Q.arr[x] = b_arr; Q.key[x] = key;
-                  Q.idx[x] = base + b; Q.meta[x] = b_rec.meta; Q.mask[x] = b_rec.mask; Q.cg[x] = b_rec.cg;
-                }
+                if (lane == b) { Q.q[Q.at(p)] = (unsigned short)x; Q.key[x] = key; replay_store(Q, x, b_rec, base + b); }
               } else if (lane == b) { wait[p] = base + b; wkey[p] = key; }
               __syncwarp();
               ++nw;
@@ -543,158 +660,173 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           } else {
             if (fits) {
               const int x = Q.free[free_slots - 1 - (lane - k0)];
-              Q.q[pos] = (unsigned short)x; Q.s[x] = b_rec.s; Q.p[x] = b_rec.p; Q.tl[x] = b_rec.tl; Q.arr[x] = b_arr;
-              Q.idx[x] = base + lane; Q.meta[x] = b_rec.meta; Q.mask[x] = b_rec.mask; Q.cg[x] = b_rec.cg;
+              Q.q[Q.at(pos)] = (unsigned short)x;
+              replay_store(Q, x, b_rec, base + lane);
             } else if (in) wait[pos] = base + lane;
-            free_slots -= __popc(__ballot_sync(TG_FULL, fits));
+            free_slots -= min(cnt, max(Q.cap - nw, 0));
             nw += cnt;
           }
           next += cnt;
           __syncwarp();
           if (next == base + 32 || next == n_act) {
-            next_arr = TG_INF;
-            if (next < n_act) refill();
-          } else next_arr = __shfl_sync(TG_FULL, b_arr, next - base);
+            next_at = KR_NEVER;
+            if (next < n_act) refill(next);
+          } else next_at = __shfl_sync(TG_FULL, b_at, next - base);
         }
         // 4. schedule
         int blocked_pool = -1;                             // pool of a head-of-line action that does not fit
-        bool any_started = false;
         if (nw > 0) {
+          const int capreg = lane < D ? Z.slot[lane] : 0;
+          // Candidate prefix (Algorithm 1, line 2): lane v adds up the demand on slot v, action by action
+          int n = 0, run_dem = 0, stop_pool = -1, aside = 0;
+          u32 present = 0;                                 // pools with candidates; << 8: with elastic ones
+          uint4 c0 = make_uint4(0u, RQ_NOBODY, 1u, 1u); int x0 = -1;   // the first 32 positions
 #pragma unroll 1
-          for (stale &= (1u << P.P) - 1u; stale; stale &= stale - 1u) {
-            const int j = __ffs(stale) - 1;
-            const PoolDev& pd = P.pool[j];
-            if (pd.type == TG_POOL_GPU) {
-              int c[4];
-              gpu_caps(pd, Z.nm, lane, c);
-              if (lane >= pd.slot0 && lane < pd.slot0 + 4) capreg = pick4(c, lane - pd.slot0);
-            } else {
-              const int used = pd.type == TG_POOL_CPU ? __shfl_sync(TG_FULL, busy, j) : Z.pst[j * 2 + (pd.window_us > 0 ? 0 : 1)];
-              if (lane == pd.slot0) capreg = pd.capacity - used;
-            }
-          }
-          // Candidate prefix (Algorithm 1, line 2): lane v adds up the demand on slot v, action by action; lane j counts
-          // the candidates of pool j and (cost vectors) what is set aside of it for the others
-          int n = 0, run_dem = 0, nc = 0, aside = 0;
-          bool stop = false;
-#pragma unroll 1
-          for (int i0 = 0; i0 < nw && !stop; i0 += 32) {
-            const int i = i0 + lane, nb = min(32, nw - i0);
-            const u32 meta = i < nw ? replay_meta(P, Q, wait, row, i) : 0u;
+          for (int i0 = 0; i0 < nw; i0 += 32) {
+            uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u); int x = -1;
+            if (i0 + lane < nw) c = replay_facts(P, Q, wait, row, i0 + lane, x);
+            if (i0 == 0) { c0 = c; x0 = x; }
+            const int nb = min(32, nw - i0);
             int k0 = 0xff, u0 = 0, k1 = 0xff, u1 = 0;      // further entries of the cost vector
-            if (EXT && P.n_side > 0 && i < nw) {
-              const int a = i < Q.cap ? Q.idx[Q.q[i]] : wait[i];
-              k0 = P.a_side_pool[row + a]; u0 = P.a_side_units[row + a];
-              if (P.n_side > 1) { k1 = P.a_side_pool[P.side_plane + row + a]; u1 = P.a_side_units[P.side_plane + row + a]; }
+            if (EXT && P.n_side > 0 && lane < nb) {
+              const size_t o = row + (int)c.x;
+              k0 = P.a_side_pool[o]; u0 = P.a_side_units[o];
+              if (P.n_side > 1) { k1 = P.a_side_pool[P.side_plane + o]; u1 = P.a_side_units[P.side_plane + o]; }
             }
+            // (lanes without a record ask for nothing; four steps at a time need one vote)
+            int over = 32;                                 // this slot's first action that does not fit
 #pragma unroll 1
-            for (int b = 0; b < nb; ++b) {
-              const u32 mb = __shfl_sync(TG_FULL, meta, b);
-              int dem = 0, sa = 0, aj = 0;
-              if (lane >= RQ_SLOT(mb) && lane <= RQ_SLOT(mb) + RQ_CLASS(mb)) dem = RQ_UNITS(mb);
-              if (EXT && P.n_side > 0) {
-                const int a0 = __shfl_sync(TG_FULL, k0, b), c0 = __shfl_sync(TG_FULL, u0, b);
-                const int a1 = __shfl_sync(TG_FULL, k1, b), c1 = __shfl_sync(TG_FULL, u1, b);
-                if (a0 != 0xff && lane == P.pool[a0].slot0) sa += c0;
-                if (a1 != 0xff && lane == P.pool[a1].slot0) sa += c1;
-                if (lane == a0) aj += c0;
-                if (lane == a1) aj += c1;
+            for (int b0 = 0; b0 < nb; b0 += 4) {
+#pragma unroll
+              for (int z = 0; z < 4; ++z) {
+                const int b = b0 + z;
+                const u32 mb = __shfl_sync(TG_FULL, c.y, b);
+                if ((u32)(lane - RQ_SLOT(mb)) <= (u32)RQ_CLASS(mb)) run_dem += RQ_UNITS(mb);
+                if (EXT && P.n_side > 0) {
+                  const int a0 = __shfl_sync(TG_FULL, k0, b), d0 = __shfl_sync(TG_FULL, u0, b);
+                  const int a1 = __shfl_sync(TG_FULL, k1, b), d1 = __shfl_sync(TG_FULL, u1, b);
+                  if (a0 != 0xff && lane == P.pool[a0].slot0) run_dem += d0;
+                  if (a1 != 0xff && lane == P.pool[a1].slot0) run_dem += d1;
+                }
+                if (run_dem > capreg) over = min(over, b);
               }
-              if (__any_sync(TG_FULL, dem + sa > 0 && run_dem + dem + sa > capreg)) { stop = true; break; }
-              run_dem += dem + sa; aside += aj;
-              if (lane == RQ_POOL(mb)) ++nc;
-              ++n;
+              if (__any_sync(TG_FULL, over < 32)) break;
             }
+            over = min(warp_min32(over), nb);
+            n += over;
+            u32 mine = 0;
+            if (lane < over) mine = (1u << RQ_POOL(c.y)) | (c.y & RQ_ELASTIC ? 256u << RQ_POOL(c.y) : 0u);
+            present |= __reduce_or_sync(TG_FULL, mine);
+            if (EXT && P.n_side > 0)                       // lane j: what is set aside of pool j for the others
+#pragma unroll 1
+              for (int j = 0; j < P.P; ++j) {
+                const int a = warp_sum32(lane < over ? (k0 == j ? u0 : 0) + (k1 == j ? u1 : 0) : 0);
+                if (lane == j) aside += a;
+              }
+            if (over < nb) { stop_pool = RQ_POOL(__shfl_sync(TG_FULL, c.y, over)); break; }
           }
-          if (n == 0) blocked_pool = RQ_POOL(uniform((int)replay_meta(P, Q, wait, row, 0)));
           const int nr0 = nr;
           bool ok = true;
+          int my_end = KR_NEVER;                           // first release among what this lane starts
+          // the lane's candidate starts (Eq. 2: completion - arrival = waited so far + execution)
+          auto start = [&](const PoolDev& pd, int j, int k, int a, int units, i64 fin, i64 arr, int node, int off) {
+            const size_t o = row + a;
+            const i64 act = fin - arr;
+            const int end = max(round_at(R, fin), r + 1);
+            P.o_alloc[o] = units; P.o_node[o] = node; P.o_off[o] = off; P.o_act[o] = act;
+            run.fin[k] = fin; run.end[k] = end; run.idx[k] = a;
+            if (occ) {
+              atomicAdd(&occ[(size_t)r * P.P + j], units);
+              if (end < R.max_rounds && (pd.type != TG_POOL_API || pd.window_us == 0)) atomicSub(&occ[(size_t)end * P.P + j], units);
+            }
+            total += act; my_end = min(my_end, end);
+          };
           // Algorithm 1, line 3: pool by pool
 #pragma unroll 1
-          for (u32 pools = __ballot_sync(TG_FULL, nc > 0); pools && ok; pools &= pools - 1) {
-            const int j = __ffs(pools) - 1, m = __shfl_sync(TG_FULL, nc, j);
+          for (u32 pools = present & 255u; pools && ok; pools &= pools - 1) {
+            const int j = __ffs(pools) - 1;
             const PoolDev& pd = P.pool[j];
             const int slot0 = pd.slot0, aside_j = EXT ? __shfl_sync(TG_FULL, aside, j) : 0;
-            const int cap0 = __shfl_sync(TG_FULL, capreg, slot0) - aside_j;
             int* ow = Z.owner + R.unit0[j];
-            int started_units = 0;
-            // elastic candidates?
-            bool el = false;
-            if (m > 1) {
+            int m = 0;
+            if (n <= 32) m = __popc(__ballot_sync(TG_FULL, lane < n && RQ_POOL(c0.y) == j));
+            else
 #pragma unroll 1
-              for (int i = lane; i < n; i += 32) {
-                int a;
-                const ReplayRec x = replay_rec(P, Q, wait, row, i, a);
-                el |= RQ_POOL(x.meta) == j && (x.mask & (x.mask - 1)) != 0;
+              for (int i0 = 0; i0 < n; i0 += 32) {
+                int x; u32 meta = RQ_NOBODY;
+                if (i0 + lane < n) meta = replay_facts(P, Q, wait, row, i0 + lane, x).y;
+                m += __popc(__ballot_sync(TG_FULL, RQ_POOL(meta) == j));
               }
-              el = __any_sync(TG_FULL, el);
-            }
+            const bool el = (present >> (8 + j)) & 1u;
             const bool cached = EXT && pd.type == TG_POOL_GPU && P.cache_slots > 0;
+            int units_now = 0;                             // what this lane's candidates take
             if ((m == 1 || (!el && pd.type != TG_POOL_GPU)) && !cached) {
               // Nothing to choose between candidates: each takes its level (a lone one DPArrange's answer in closed form: the
               // feasible level of least duration, the smallest among equals) and is placed in queue order.
               int seen = 0;
 #pragma unroll 1
               for (int i0 = 0; i0 < n && seen < m; i0 += 32) {
-                int a = 0; ReplayRec x; x.meta = 15u; x.s = x.p = 0; x.mask = 1; x.cg = 1;
-                if (i0 + lane < n) x = replay_rec(P, Q, wait, row, i0 + lane, a);
-                const bool mine = i0 + lane < n && RQ_POOL(x.meta) == j;
+                uint4 c = c0; int x = x0;
+                if (i0 > 0) {
+                  c = make_uint4(0u, RQ_NOBODY, 1u, 1u); x = -1;
+                  if (i0 + lane < n) c = replay_facts(P, Q, wait, row, i0 + lane, x);
+                }
+                const bool mine = i0 + lane < n && RQ_POOL(c.y) == j;
                 const u32 mb = __ballot_sync(TG_FULL, mine);
-                int rr = __ffs(x.mask), node = -1, off = -1, dom = -1;
-                if (m == 1 && mb) {
+                if (!mb) continue;
+                ReplayRec rec; rec.s = rec.p = rec.arr = 0;
+                if (mine) rec = replay_rec(P, Q, row, c, x);
+                int rr = __ffs(c.z);
+                if (m == 1 && el) {
                   const int b = __ffs(mb) - 1;
-                  const u32 mk = __shfl_sync(TG_FULL, x.mask, b), cg = __shfl_sync(TG_FULL, (u32)x.cg, b);
-                  if (mk & (mk - 1)) {
-                    const i64 s = __shfl_sync(TG_FULL, x.s, b), p = __shfl_sync(TG_FULL, x.p, b);
-                    const int g = cg & 0x7f, gang = cg >> 7, rl = lane + 1;
-                    bool fit = (mk >> lane) & 1u;
-                    const int c = fit && pd.type == TG_POOL_GPU ? level_of(g, gang, rl) : 0;
-                    const int room = __shfl_sync(TG_FULL, capreg, slot0 + c) - (c == 0 ? aside_j : 0);
-                    fit = fit && g * rl <= room;
-                    const i64 best = warp_min64(fit ? ((duration(s, p, rl) << 6) | (i64)rl) : TG_INF);
-                    if (lane == b && best != TG_INF) rr = (int)(best & 63);
-                  }
+                  const u32 mk = __shfl_sync(TG_FULL, c.z, b), cg = __shfl_sync(TG_FULL, c.w, b);
+                  const int g = cg & 0x7f, gang = cg >> 7, rl = lane + 1;
+                  bool fit = (mk >> lane) & 1u;
+                  const int cl = fit && pd.type == TG_POOL_GPU ? level_of(g, gang, rl) : 0;
+                  const int room = Z.slot[slot0 + cl] - (cl == 0 ? aside_j : 0);
+                  const u32 fits = __ballot_sync(TG_FULL, fit && g * rl <= room);
+                  if (lane == b && fits) rr = best_level(rec.p, fits);   // (durations do not grow with the level)
                 }
-                const int units = mine ? (x.cg & 0x7f) * rr : 0;
+                const int units = mine ? (int)(c.w & 0x7f) * rr : 0;
+                const i64 fin = now + duration(rec.s, rec.p, rr);
+                ReplayGrant G; G.node = 0; G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = false;
+                if (pd.type == TG_POOL_API) {
+                  // Section 5.1: the offset is what was in use before
+                  const int incl = warp_incl_scan32(units, lane);
+                  G.off = pd.capacity - Z.slot[slot0] + incl - units;
+                  const int all = __shfl_sync(TG_FULL, incl, 31);
+                  if (lane == 0) Z.slot[slot0] -= all;
+                } else
 #pragma unroll 1
-                for (u32 todo = mb; todo; todo &= todo - 1) {
-                  const int b = __ffs(todo) - 1;
-                  const int k = __shfl_sync(TG_FULL, units, b), id = __shfl_sync(TG_FULL, a, b);
-                  int nd = 0, of = 0, ft = -1;
-                  if (pd.type == TG_POOL_CPU) replay_place_cpu(pd, ow, Z.dfree + R.dom0[j], k, id, lane, nd, of, ft);
-                  else if (pd.type == TG_POOL_GPU) {
-                    const u32 cg = __shfl_sync(TG_FULL, (u32)x.cg, b);
-                    const int rb = __shfl_sync(TG_FULL, rr, b), g = cg & 0x7f, gang = cg >> 7;
-                    replay_place_gpu(pd, Z.nm + pd.node0, ow, ilog2(gang ? g * rb : g), gang ? 1 : rb, id, lane, nd, of);
-                  } else {
-                    int* ps = Z.pst + j * 2 + (pd.window_us > 0 ? 0 : 1);
-                    of = *ps;
-                    __syncwarp();
-                    if (lane == 0) *ps = of + k;
-                    __syncwarp();
+                  for (u32 todo = mb; todo; todo &= todo - 1) {
+                    const int b = __ffs(todo) - 1;
+                    const int k = __shfl_sync(TG_FULL, units, b), id = __shfl_sync(TG_FULL, (int)c.x, b);
+                    ReplayGrant g1;
+                    if (pd.type == TG_POOL_CPU)
+                      g1 = replay_take_cores(pd.group, R.n_dom[j], R.wpd[j], Z.cores + 2 * R.word0[j], Z.dfree + R.dom0[j], ow, k, id, lane);
+                    else {
+                      const int cg = __shfl_sync(TG_FULL, (int)c.w, b), rb = __shfl_sync(TG_FULL, rr, b), g = cg & 0x7f, gang = cg >> 7;
+                      g1 = replay_take_gpus(pd, Z.nm + pd.node0, ow, ilog2(gang ? g * rb : g), gang ? 1 : rb, id, lane);
+                    }
+                    if (lane == b) G = g1;
                   }
-                  if (lane == b) { node = nd; off = of; dom = ft; }
-                }
-                // start (Eq. 2: completion - arrival = waited so far + execution)
                 if (mine) {
-                  const size_t o = row + a;
-                  const i64 fin = now + duration(x.s, x.p, rr), act = fin - x.arr;
-                  P.o_alloc[o] = units; P.o_node[o] = node; P.o_off[o] = off; P.o_act[o] = act;
                   const int k = nr + __popc(mb & below);
-                  run.fin[k] = fin; run.idx[k] = a; run.pu[k] = ((u32)j << 24) | (u32)units; run.off[k] = off; run.dom[k] = dom;
-                  if (i0 + lane < Q.cap) Q.meta[Q.q[i0 + lane]] = x.meta | RQ_STARTED;
-                  total += act; min_fin = min(min_fin, fin);
-                  started_units += units;
+                  run.at[k] = make_uint4(G.lo, G.hi, (u32)G.word, (u32)G.dom); run.pu[k] = rr_pack(pd, j, units, G.wide);
+                  if (x >= 0) Q.c[x].y = c.y | RQ_STARTED;
+                  start(pd, j, k, (int)c.x, units, fin, rec.arr, G.node, G.off);
                 }
+                units_now += units;
                 nr += __popc(mb); seen += __popc(mb); selected += __popc(mb);
+                __syncwarp();
               }
             } else {
               Slab slab;
               slab.base = P.slabs + (u64)blockIdx.x * P.slab_bytes; slab.cap = P.slab_bytes; slab.used = 0;
               slab.fbase = fast; slab.fcap = KR_FAST_BYTES; slab.fused = 0;
               CandArrays C; int keep = 0;
-              ok = replay_select<EXT>(P, Q, run, wait, sc, j, n, nw, nr, m, now, cap0, __shfl_sync(TG_FULL, capreg, (slot0 + 1) & 31),
-                                      __shfl_sync(TG_FULL, capreg, (slot0 + 2) & 31), __shfl_sync(TG_FULL, capreg, (slot0 + 3) & 31), slab, C, keep, lane);
+              ok = replay_select<EXT>(P, Q, run, wait, sc, j, n, nw, nr, m, now, Z.slot[slot0] - aside_j, Z.slot[(slot0 + 1) & 31],
+                                      Z.slot[(slot0 + 2) & 31], Z.slot[(slot0 + 3) & 31], slab, C, keep, lane);
               if (!ok) break;
               const u8* missed = nullptr;                  // candidates whose chunk did not cache their service
               if (cached) {
@@ -707,71 +839,110 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               } else if (pd.type == TG_POOL_CPU) {
 #pragma unroll 1
                 for (int i = 0; i < keep; ++i) {
-                  int nd, of, ft;
-                  replay_place_cpu(pd, ow, Z.dfree + R.dom0[j], (C.cg[i] & 0x7f) * C.rkeep[i], C.cidx[i], lane, nd, of, ft);
-                  if (lane == 0) { C.pnode[i] = nd; C.poff[i] = of; C.rowcand[i] = ft; }
+                  const int units = (C.cg[i] & 0x7f) * C.rkeep[i];
+                  const ReplayGrant G = replay_take_cores(pd.group, R.n_dom[j], R.wpd[j], Z.cores + 2 * R.word0[j], Z.dfree + R.dom0[j], ow,
+                                                          units, C.cidx[i], lane);
+                  if (lane == 0) {
+                    C.pnode[i] = G.node; C.poff[i] = G.off;
+                    run.at[nr + i] = make_uint4(G.lo, G.hi, (u32)G.word, (u32)G.dom); run.pu[nr + i] = rr_pack(pd, j, units, G.wide);
+                  }
                 }
               } else if (lane == 0) {
-                int* ps = Z.pst + j * 2 + (pd.window_us > 0 ? 0 : 1);
+                int used = pd.capacity - Z.slot[slot0];
 #pragma unroll 1
-                for (int i = 0; i < keep; ++i) { C.pnode[i] = 0; C.poff[i] = *ps; *ps += (C.cg[i] & 0x7f) * C.rkeep[i]; }
+                for (int i = 0; i < keep; ++i) { C.pnode[i] = 0; C.poff[i] = used; used += (C.cg[i] & 0x7f) * C.rkeep[i]; }
+                Z.slot[slot0] = pd.capacity - used;
               }
               __syncwarp();
 #pragma unroll 1
               for (int i = lane; i < keep; i += 32) {
-                const size_t o = row + C.cidx[i];
-                const int rr = C.rkeep[i], units = (C.cg[i] & 0x7f) * rr;
+                const int g = C.cg[i] & 0x7f, gang = C.cg[i] >> 7, rr = C.rkeep[i], units = g * rr, a = C.cidx[i];
                 i64 fin = now + duration(C.cs[i], C.cp[i], rr);
-                if (EXT && missed && missed[i] && P.a_restore) fin += clamp_param(P.a_restore[o]);   // restoration precedes execution
-                const i64 act = fin - (P.a_arrival ? P.a_arrival[o] : 0);
-                P.o_alloc[o] = units; P.o_node[o] = C.pnode[i]; P.o_off[o] = C.poff[i]; P.o_act[o] = act;
-                run.fin[nr + i] = fin; run.idx[nr + i] = C.cidx[i]; run.pu[nr + i] = ((u32)j << 24) | (u32)units; run.off[nr + i] = C.poff[i]; run.dom[nr + i] = pd.type == TG_POOL_CPU ? C.rowcand[i] : -1;
-                total += act; min_fin = min(min_fin, fin);
-                started_units += units;
+                if (EXT && missed && missed[i] && P.a_restore) fin += clamp_param(P.a_restore[row + a]);   // restoration precedes execution
+                if (pd.type != TG_POOL_CPU) {
+                  run.at[nr + i] = make_uint4(((1u << (units & 31)) - 1u) << (C.poff[i] & 31), 0u, (u32)C.pnode[i], 0u);
+                  run.pu[nr + i] = rr_pack(pd, j, units, pd.type == TG_POOL_GPU && !gang && rr > 1);
+                }
+                start(pd, j, nr + i, a, units, fin, P.a_arrival ? P.a_arrival[row + a] : 0, C.pnode[i], C.poff[i]);
+                units_now += units;
               }
               // the kept ones are the pool's first `keep` in queue order
               int seen = 0;
 #pragma unroll 1
               for (int i0 = 0; i0 < n && seen < keep; i0 += 32) {
-                const int i = i0 + lane;
-                const u32 meta = i < n ? replay_meta(P, Q, wait, row, i) : 15u;
-                const u32 mb = __ballot_sync(TG_FULL, i < n && RQ_POOL(meta) == j);
-                if (((mb >> lane) & 1u) && seen + __popc(mb & below) < keep && i < Q.cap) Q.meta[Q.q[i]] = meta | RQ_STARTED;
+                int x = -1; u32 meta = RQ_NOBODY;
+                if (i0 + lane < n) meta = replay_facts(P, Q, wait, row, i0 + lane, x).y;
+                const bool mine = RQ_POOL(meta) == j;
+                const u32 mb = __ballot_sync(TG_FULL, mine);
+                if (mine && seen + __popc(mb & below) < keep && x >= 0) Q.c[x].y = meta | RQ_STARTED;
                 seen += __popc(mb);
               }
               nr += keep; selected += keep;
+              __syncwarp();
             }
-            started_units = warp_sum32(started_units);
-            if (lane == j && pd.type != TG_POOL_API) busy += started_units;
-            stale |= 1u << j;
+            if (pd.type == TG_POOL_GPU) replay_gpu_slots(pd, Z.nm, Z.slot, lane);
+            else if (pd.type == TG_POOL_CPU) {
+              const int all = warp_sum32(units_now);
+              if (lane == 0) Z.slot[slot0] -= all;
+            }
             __syncwarp();
           }
           if (!ok) { status = TG_ST_WORKSPACE; break; }
-          any_started = nr > nr0;
-          if (EXT && P.n_side > 0 && any_started) {         // the started actions consume their further amounts
-            stale = ~0u;
+          const int started = nr - nr0;
+          if (EXT && P.n_side > 0 && started) {             // the started actions consume their further amounts
 #pragma unroll 1
             for (int i = nr0 + lane; i < nr; i += 32)
 #pragma unroll 1
               for (int e = 0; e < P.n_side; ++e) {
-                const int k = P.a_side_pool[e * P.side_plane + row + run.idx[i]];
-                if (k != 0xff)
-                  atomicAdd(&Z.pst[k * 2 + (P.pool[k].window_us > 0 ? 0 : 1)], (int)P.a_side_units[e * P.side_plane + row + run.idx[i]]);
+                const size_t o = e * P.side_plane + row + run.idx[i];
+                const int k = P.a_side_pool[o];
+                if (k == 0xff) continue;
+                const int c = (int)P.a_side_units[o];
+                atomicSub(&Z.slot[P.pool[k].slot0], c);
+                if (occ) {
+                  atomicAdd(&occ[(size_t)r * P.P + k], c);
+                  if (P.pool[k].window_us == 0 && run.end[i] < R.max_rounds) atomicSub(&occ[(size_t)run.end[i] * P.P + k], c);
+                }
               }
             __syncwarp();
           }
-          if (any_started) {                                // drop the started actions from the queue
+          if (started) min_end = min(min_end, warp_min32(my_end));
+          // What does not fit behind candidates that all started does not fit until something ends on its pool: they hold at
+          // least what the prefix counted for them.
+          if (started == n) blocked_pool = stop_pool;
+          // the started actions leave the queue
+          if (started && nw <= Q.cap) {
+            int to_end = n;                                // the ones that stay move up behind the others, last first
+#pragma unroll 1
+            for (int i0 = (n - 1) & ~31; i0 >= 0; i0 -= 32) {
+              const int i = i0 + lane, x = i < n ? (int)Q.q[Q.at(i)] : 0;
+              const bool gone = i < n && (started == n || (Q.c[x].y & RQ_STARTED));
+              const u32 gb = __ballot_sync(TG_FULL, gone);
+              if (gone) Q.free[free_slots + __popc(gb & below)] = (unsigned short)x;
+              free_slots += __popc(gb);
+              if (started < n) {
+                const u32 sb = __ballot_sync(TG_FULL, i < n && !gone);
+                __syncwarp();
+                if (i < n && !gone) Q.q[Q.at(to_end - __popc(sb >> lane))] = (unsigned short)x;
+                to_end -= __popc(sb);
+                __syncwarp();
+              }
+            }
+            Q.head = Q.at(started < Q.cap ? started : 0);
+            nw -= started;
+            __syncwarp();
+          } else if (started) {                             // a queue that goes on in global memory
             int kw = 0;
 #pragma unroll 1
             for (int i0 = 0; i0 < nw; i0 += 32) {
               const int i = i0 + lane;
               bool stay = false; int x = 0, a = 0; u64 kk = 0;
-              if (i < min(nw, Q.cap)) { x = Q.q[i]; stay = !(Q.meta[x] & RQ_STARTED); }
+              if (i < min(nw, Q.cap)) { x = Q.q[Q.at(i)]; stay = !(Q.c[x].y & RQ_STARTED); }
               else if (i < nw) { a = wait[i]; stay = P.o_act[row + a] < 0; if (EXT && R.policy) kk = wkey[i]; }
               const u32 b = __ballot_sync(TG_FULL, stay), gone = __ballot_sync(TG_FULL, i < min(nw, Q.cap) && !stay);
               const int to = kw + __popc(b & below);
               __syncwarp();
-              if (stay && i < Q.cap) Q.q[to] = (unsigned short)x;
+              if (stay && i < Q.cap) Q.q[Q.at(to)] = (unsigned short)x;
               else if (stay && to >= Q.cap) { wait[to] = a; if (EXT && R.policy) wkey[to] = kk; }
               if ((gone >> lane) & 1u) Q.free[free_slots + __popc(gone & below)] = (unsigned short)x;
               free_slots += __popc(gone);
@@ -779,98 +950,90 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               const u32 mv = __ballot_sync(TG_FULL, stay && i >= Q.cap && to < Q.cap);
               if ((mv >> lane) & 1u) {                      // a record moves up into shared memory
                 const int y = Q.free[free_slots - 1 - __popc(mv & below)];
-                const ReplayRec rec = replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], P.a_s[row + a], P.a_p[row + a]);
-                Q.q[to] = (unsigned short)y; Q.s[y] = rec.s; Q.p[y] = rec.p; Q.tl[y] = rec.tl; Q.arr[y] = P.a_arrival ? P.a_arrival[row + a] : 0;
+                Q.q[Q.at(to)] = (unsigned short)y;
+                replay_store(Q, y, replay_load(P, row, a), a);
                 if (EXT) Q.key[y] = kk;
-                Q.idx[y] = a; Q.meta[y] = rec.meta; Q.mask[y] = rec.mask; Q.cg[y] = rec.cg;
               }
               free_slots -= __popc(mv);
               __syncwarp();
               kw += __popc(b);
             }
             nw = kw;
-            min_fin = warp_min64(min_fin);
           }
         }
-        // 5. occupancy of this round: lane j holds pool j's
-        int in_use = busy;
-        if (api_at >= 0) in_use = Z.pst[api_at];
-        if (occ && lane < P.P) occ[(size_t)r * P.P + lane] = in_use;
-        ++r;
-        if (next == n_act && nw == 0 && nr == 0) { drained = true; break; }
-        // Rounds in which nothing can change are jumped over, their rows repeat this occupancy (quota usage restarts
-        // with its window).
-        i64 t_next = TG_INF;
-        bool jump = false, partial = false;
+        // 5. the next round in which something can start
+        if (next == n_act && nw == 0 && nr == 0) { drained = true; ++r; break; }
+        int r_next = r + 1;
         if (nw == 0) {
-          // with an empty queue: to the next arrival or completion (a gated arrival waits for a completion)
-          jump = true;
-          t_next = min(gated ? TG_INF : next_arr, min_fin);
+          // empty queue: the next arrival (a gated one waits for a completion), after the last one the last completion
+          r_next = gated ? min_end : next_at;
+          if (next == n_act) {
+            int last = 0;
+#pragma unroll 1
+            for (int i = lane; i < nr; i += 32) last = max(last, run.end[i]);
+            r_next = warp_max32(last);
+          }
         } else if (blocked_pool >= 0) {
           // The action at the head of the queue does not fit, so nothing can start until an action that runs ends, a quota
           // window turns or (in a sorted queue) an arrival becomes the head.
-          jump = true;
-          const PoolDev& hp = P.pool[blocked_pool];
           if (EXT && (P.n_side > 0 || R.trajectory)) {
             // (the head may wait for any pool's amounts; an arrival would be pinned against the memory free at its time)
-            t_next = min(gated ? TG_INF : next_arr, min_fin);
-#pragma unroll 1
-            for (int j = 0; j < P.P; ++j)
-              if (P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0) t_next = min(t_next, (Z.win[j] + 1) * (i64)P.pool[j].window_us);
+            r_next = min(min(gated ? KR_NEVER : next_at, min_end), next_turn);
           } else {
-            // ... on its pool: arrivals join behind it, what ends on other pools leaves the rows from its round on
-            partial = true;
-            if (hp.type == TG_POOL_API && hp.window_us > 0) t_next = (Z.win[blocked_pool] + 1) * (i64)hp.window_us;
-            if (EXT && R.policy) t_next = min(t_next, next_arr);
+            // ... on its pool: arrivals join behind it
+            r_next = __shfl_sync(TG_FULL, my_turn, blocked_pool);
+            if (EXT && R.policy) r_next = min(r_next, next_at);
+            int e = KR_NEVER;
 #pragma unroll 1
             for (int i = lane; i < nr; i += 32)
-              if ((int)(run.pu[i] >> 24) == blocked_pool) t_next = min(t_next, run.fin[i]);
-            t_next = warp_min64(t_next);
+              if (RR_POOL(run.pu[i]) == blocked_pool) e = min(e, run.end[i]);
+            r_next = min(r_next, warp_min32(e));
           }
         }
-        if (jump) {
-          int r_next = R.max_rounds;
-          if (t_next <= now) r_next = r;
-          else if (t_next < now + (i64)(R.max_rounds - r + 1) * R.round_us) r_next = min(r_next, (int)round_after(t_next, now, r - 1));
-          if (r_next > r) {
-            if (occ) {
-              if (lane < P.P) {
-                // (this lane's pool; its usage restarts with its window)
-                int turn = r_next;
-                if (windows && api_at >= 0 && !(api_at & 1)) {
-                  const i64 tr = round_after((Z.win[lane] + 1) * (i64)P.pool[lane].window_us, now, r - 1);
-                  if (tr < (i64)turn) turn = (int)tr;
-                }
-                int* at = occ + (size_t)r * P.P + lane;
-#pragma unroll 1
-                for (int rr = r; rr < r_next; ++rr, at += P.P) *at = rr < turn ? in_use : 0;
-              }
-              if (partial) {
-                __syncwarp();
-#pragma unroll 1
-                for (int i = lane; i < nr; i += 32) {
-                  const i64 fin = run.fin[i];
-                  if (fin > (i64)(r_next - 1) * R.round_us) continue;
-                  const u32 pu = run.pu[i];
-                  const int j = (int)(pu >> 24);
-                  if (P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0) continue;      // used quota is not given back
-                  const int fr = max(r, (int)round_after(fin, now, r - 1));
-#pragma unroll 1
-                  for (int rr = fr; rr < r_next; ++rr) atomicSub(&occ[(size_t)rr * P.P + j], (int)(pu & 0xffffffu));
-                }
-                __syncwarp();
-              }
-            }
-            r = r_next;
-          }
-        }
+        r_next = max(r_next, r + 1);
+        // (the last round still gives back what ends by then)
+        if (r_next >= R.max_rounds) r_next = r < R.max_rounds - 1 ? R.max_rounds - 1 : R.max_rounds;
+        r = r_next;
       }
       rounds = drained ? r : R.max_rounds;
       if (!drained && r < R.max_rounds) rounds = r;
       total = warp_sum64(total);
       if (lane == 0) { P.o_total[sc] = total; P.o_nsel[sc] = selected; P.o_status[sc] = status; }
     } else if (lane == 0) { P.o_total[sc] = 0; P.o_nsel[sc] = 0; P.o_status[sc] = status; }
-    if (R.rounds_used && lane == 0) R.rounds_used[sc] = rounds;
+    if (lane == 0) R.rounds_used[sc] = rounds;
     __syncwarp();
   }
+}
+
+// Occupancy: running sums of the differences that k_replay left, in place, one block per scenario; rows behind the last
+// round are zero.  Every thread adds up KOCC_ROWS consecutive rounds of a pool.
+#define KOCC_ROWS 8
+__global__ void __launch_bounds__(256) k_occupancy(int n_pools, int max_rounds, const int* rounds_used, const int* status, int* occupancy) {
+  __shared__ int part[TG_MAX_POOLS][8];
+  __shared__ int carry[TG_MAX_POOLS];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int* occ = occupancy + (size_t)blockIdx.x * max_rounds * n_pools;
+  const int rounds = min(rounds_used[blockIdx.x], max_rounds);
+  if (t < TG_MAX_POOLS) carry[t] = 0;
+  __syncthreads();
+  for (int r0 = 0; r0 < rounds; r0 += 256 * KOCC_ROWS) {
+    const int first = r0 + t * KOCC_ROWS;
+    for (int j = 0; j < n_pools; ++j) {
+      int v[KOCC_ROWS], sum = 0;
+#pragma unroll
+      for (int k = 0; k < KOCC_ROWS; ++k) { v[k] = first + k < rounds ? occ[(size_t)(first + k) * n_pools + j] : 0; sum += v[k]; }
+      const int incl = warp_incl_scan32(sum, lane);
+      if (lane == 31) part[j][warp] = incl;
+      __syncthreads();
+      int run = carry[j] + incl - sum, all = 0;
+      for (int w = 0; w < 8; ++w) { if (w < warp) run += part[j][w]; all += part[j][w]; }
+#pragma unroll
+      for (int k = 0; k < KOCC_ROWS; ++k) { run += v[k]; if (first + k < rounds) occ[(size_t)(first + k) * n_pools + j] = run; }
+      __syncthreads();
+      if (t == 0) carry[j] += all;
+      __syncthreads();
+    }
+  }
+  if (status[blockIdx.x])                                  // (a replay that broke off leaves differences behind its last round)
+    for (size_t x = (size_t)rounds * n_pools + t; x < (size_t)max_rounds * n_pools; x += 256) occ[x] = 0;
 }

@@ -523,18 +523,21 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   r->n_sm = prop.multiProcessorCount;
   if (desc->max_rounds > 0) {                              // state of the trace replay
     ReplayWs& R = r->R;
-    int u = 0, d = 0;
+    int u = 0, d = 0, w = 0;
     for (int j = 0; j < P.P; ++j) {
-      R.unit0[j] = u; R.dom0[j] = d;
+      R.unit0[j] = u; R.dom0[j] = d; R.word0[j] = w;
       if (P.pool[j].type != TG_POOL_API) u += P.pool[j].capacity;
-      if (P.pool[j].type == TG_POOL_CPU) d += P.pool[j].capacity / P.pool[j].group;
+      if (P.pool[j].type != TG_POOL_CPU) continue;
+      R.n_dom[j] = P.pool[j].capacity / P.pool[j].group; R.wpd[j] = (P.pool[j].group + 63) / 64;
+      d += R.n_dom[j]; w += R.n_dom[j] * R.wpd[j];
     }
-    R.U = u ? u : 1; R.Dtot = d ? d : 1;
+    R.U = u ? u : 1; R.Dtot = d ? d : 1; R.W = w ? w : 1;
     R.round_us = desc->round_us > 0 ? desc->round_us : 1; R.max_rounds = desc->max_rounds;
+    R.round_recip = R.round_us > 1 && R.round_us < (1 << 22) ? ~0ull / (u64)R.round_us + 1ull : 0;
     bad |= cudaMalloc((void**)&R.wait, SN * sizeof(int)) != cudaSuccess;
     // what a block (one scenario at a time) keeps in shared memory: live state, running actions, waiting records
     {
-      const size_t state = align16((size_t)R.U * 4) + align16((size_t)node0 + 1) + align16((size_t)R.Dtot * 4) + 2 * align16((size_t)P.P * 8);
+      const size_t state = replay_state_bytes(R, node0);
       R.state_bytes = state <= KR_STATE_MAX ? (int)state : 0;
       size_t running = 0;                                  // a running action holds a unit at least, quota calls aside
       for (int j = 0; j < P.P; ++j) running += P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0 ? (size_t)P.N : (size_t)P.pool[j].capacity;
@@ -552,18 +555,20 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
       R.wcap = (int)(wc / 32 * 32);
       r->replay_smem = KR_BASE_BYTES + R.state_bytes + (int)align16((size_t)R.rcap * KR_RUN_BYTES) + (int)align16((size_t)R.wcap * KR_WAIT_BYTES);
       if (R.rcap == 0) {
+        bad |= cudaMalloc((void**)&R.run_at, SN * sizeof(uint4)) != cudaSuccess;
         bad |= cudaMalloc((void**)&R.run_fin, SN * sizeof(i64)) != cudaSuccess;
-        bad |= cudaMalloc((void**)&R.run_idx, SN * sizeof(int)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_end, SN * sizeof(int)) != cudaSuccess;
         bad |= cudaMalloc((void**)&R.run_pu, SN * sizeof(u32)) != cudaSuccess;
-        bad |= cudaMalloc((void**)&R.run_off, SN * sizeof(int)) != cudaSuccess;
-        bad |= cudaMalloc((void**)&R.run_dom, SN * sizeof(int)) != cudaSuccess;
+        bad |= cudaMalloc((void**)&R.run_idx, SN * sizeof(int)) != cudaSuccess;
       }
     }
-    bad |= cudaMalloc((void**)&R.owner, (size_t)P.S * R.U * sizeof(int)) != cudaSuccess;
-    bad |= cudaMalloc((void**)&R.nm, (size_t)P.S * (node0 ? node0 : 1)) != cudaSuccess;
-    bad |= cudaMalloc((void**)&R.dfree, (size_t)P.S * R.Dtot * sizeof(int)) != cudaSuccess;
-    bad |= cudaMalloc((void**)&R.pst, (size_t)P.S * P.P * 2 * sizeof(int)) != cudaSuccess;
-    bad |= cudaMalloc((void**)&R.win, (size_t)P.S * P.P * sizeof(i64)) != cudaSuccess;
+    bad |= cudaMalloc((void**)&R.rounds_used, (size_t)P.S * sizeof(int)) != cudaSuccess;
+    if (R.state_bytes == 0) {
+      bad |= cudaMalloc((void**)&R.cores, (size_t)P.S * R.W * 8) != cudaSuccess;
+      bad |= cudaMalloc((void**)&R.dfree, (size_t)P.S * R.Dtot * sizeof(int)) != cudaSuccess;
+      bad |= cudaMalloc((void**)&R.owner, (size_t)P.S * R.U * sizeof(int)) != cudaSuccess;
+      bad |= cudaMalloc((void**)&R.nm, (size_t)P.S * ((node0 + 4) & ~3)) != cudaSuccess;
+    }
   }
   {
     // the fill's stream: highest priority, so that its few blocks get in between those of k_stream
@@ -696,8 +701,8 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   if (r->ev) tangram_set_profiling(r, 0);
   cudaFree(r->d_order); cudaFree(r->d_tmin); cudaFree(r->d_meta); cudaFree(r->d_slabs);
   cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_perm); cudaFree(r->d_wkey);
-  cudaFree(r->R.wait); cudaFree(r->R.run_fin); cudaFree(r->R.run_idx); cudaFree(r->R.run_pu); cudaFree(r->R.run_off); cudaFree(r->R.run_dom); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.dfree);
-  cudaFree(r->R.pst); cudaFree(r->R.win);
+  cudaFree(r->R.wait); cudaFree(r->R.run_at); cudaFree(r->R.run_fin); cudaFree(r->R.run_end); cudaFree(r->R.run_pu); cudaFree(r->R.run_idx);
+  cudaFree(r->R.cores); cudaFree(r->R.dfree); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.rounds_used);
   if (r->io_in) cudaStreamDestroy(r->io_in);
   if (r->io_comp) cudaStreamDestroy(r->io_comp);
   if (r->io_out) cudaStreamDestroy(r->io_out);
@@ -938,15 +943,17 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
     int rc = copy_in(r, a, P, 0, P.S, st);
     if (rc) return rc;
     R.occupancy = res->occupancy ? (int*)(r->d_stage + r->out_off[7]) : nullptr;
-    R.rounds_used = res->rounds_used ? (int*)(r->d_stage + r->out_off[8]) : nullptr;
+    if (res->rounds_used) R.rounds_used = (int*)(r->d_stage + r->out_off[8]);
   } else {
     bind_device_io(P, a, res);
-    R.occupancy = res->occupancy; R.rounds_used = res->rounds_used;
+    R.occupancy = res->occupancy;
+    if (res->rounds_used) R.rounds_used = res->rounds_used;
   }
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));
   const int blocks = P.n_workers < P.S ? P.n_workers : P.S;
   cudaEvent_t* ev = prof_begin(r, 2, -1, -1);
   if (ev) CK(cudaEventRecord(ev[0], st));
+  if (R.occupancy) CK(cudaMemsetAsync(R.occupancy, 0, (size_t)P.S * R.max_rounds * P.P * sizeof(int), st));
   if (pin) {
     // the kernel reads and rewrites the caller's pool_out: it starts as a copy of the pool column
     CK(cudaMemcpyAsync(pin->pool_out, a->pool, (size_t)P.S * P.N, cudaMemcpyDeviceToDevice, st));
@@ -957,6 +964,7 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
   }
   if (policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0)) k_replay<true><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   else k_replay<false><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
+  if (R.occupancy) { k_occupancy<<<P.S, 256, 0, st>>>(P.P, R.max_rounds, R.rounds_used, P.o_status, R.occupancy); r->launches += 1; }
   if (ev) CK(cudaEventRecord(ev[1], st));
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));            // k_round starts from counters at zero
   r->launches += 1;
