@@ -351,41 +351,32 @@ __device__ __forceinline__ bool ev_behind_regs(const u32 (&a)[NS], const u32 (&b
   return __all_sync(TG_FULL, ok);
 }
 
-// The two heaps side by side (see ev_compare for the conventions).  wk: 64 NS + 2 EV_BLOCK + 4 words of shared memory.
-template <int NS>
-__device__ __forceinline__ int ev_compare_regs(const PoolTask& T, int q, const u8* kept, const u8* fewer, i64 fixed, u32 wk, int lane) {
-  const int ha = T.n_seeds + q + 1, n = T.m - q - 1 + T.n_ac;
+// The two heaps side by side (see ev_compare for the conventions).  a: heap of the longer prefix, in the first ha places; b:
+// of the shorter one, before the evicted candidate of duration `evicted`.  dur_of(k): duration of the k-th of n that wait behind
+// both, first_a: of the first one as `a` takes it; diff: the part of the difference that is no popped time.
+// wk: 64 NS + 2 EV_BLOCK + 4 words of shared memory.
+template <int NS, class Dur>
+__device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, int n, u32 evicted, u32 first_a, i64 diff, const Dur& dur_of, u32 wk,
+                                           int lane) {
   const EvShared dur = {wk + NS * 256u};
   const u32 above = lane == 31 ? 0u : TG_FULL << (lane + 1);
-  u32 a[NS], b[NS], last_a = 0, last_b;
-#pragma unroll
-  for (int j = 0; j < NS; ++j) {
-    const int i = j * 32 + lane, c = i - T.n_seeds;
-    a[j] = b[j] = EV_NONE;
-    if (i >= ha) continue;
-    if (c < 0) a[j] = b[j] = ev_key(T.seeds[i]);
-    else {
-      const i64 s = T.cs[c], p = T.cp[c];
-      a[j] = ev_key(duration(s, p, kept[c]));
-      if (c < q) b[j] = ev_key(duration(s, p, fewer[c]));
-    }
-  }
+  u32 last_a = 0, last_b;
   {                                                      // the evicted candidate
     const u32 lb = ev_local_min(b);
     last_b = __reduce_min_sync(TG_FULL, lb);
-    ev_replace(b, last_b, __ballot_sync(TG_FULL, lb == last_b), ev_key(rest_first(T, q)), above);
+    ev_replace(b, last_b, __ballot_sync(TG_FULL, lb == last_b), evicted, above);
   }
-  i64 diff = fixed + (i64)last_b;
+  diff += (i64)last_b;
   int wait = 0;                                          // blocks until the heaps are compared again
 #pragma unroll 1
   for (int k0 = 0; k0 < n; k0 += EV_BLOCK) {
     const int steps = min(EV_BLOCK, n - k0);
 #pragma unroll 1
-    for (int x = lane; x < steps; x += 32) dur.put(x, ev_key(rest_least(T, q + 1, k0 + x)));
+    for (int x = lane; x < steps; x += 32) dur.put(x, dur_of(k0 + x));
     __syncwarp();
     // The two chains, step by step side by side (warp-wide operations keep their order, so it is written this way).
     // A's first action takes its own level.
-    u32 da = k0 == 0 ? ev_key(rest_first(T, q + 1)) : dur.get(0);
+    u32 da = k0 == 0 ? first_a : dur.get(0);
     int k = 0;
 #pragma unroll 1
     for (; k + 4 <= steps; k += 4) {
@@ -414,6 +405,25 @@ __device__ __forceinline__ int ev_compare_regs(const PoolTask& T, int q, const u
   }
   if (last_b >= EV_SAT) return -1;
   return diff < 0 ? 1 : 0;
+}
+template <int NS>
+__device__ __forceinline__ int ev_compare_regs(const PoolTask& T, int q, const u8* kept, const u8* fewer, i64 fixed, u32 wk, int lane) {
+  const int ha = T.n_seeds + q + 1, n = T.m - q - 1 + T.n_ac;
+  u32 a[NS], b[NS];
+#pragma unroll
+  for (int j = 0; j < NS; ++j) {
+    const int i = j * 32 + lane, c = i - T.n_seeds;
+    a[j] = b[j] = EV_NONE;
+    if (i >= ha) continue;
+    if (c < 0) a[j] = b[j] = ev_key(T.seeds[i]);
+    else {
+      const i64 s = T.cs[c], p = T.cp[c];
+      a[j] = ev_key(duration(s, p, kept[c]));
+      if (c < q) b[j] = ev_key(duration(s, p, fewer[c]));
+    }
+  }
+  return ev_run_regs<NS>(a, b, ha, n, ev_key(rest_first(T, q)), n > 0 ? ev_key(rest_first(T, q + 1)) : 0u, fixed,
+                         [&](int k) { return ev_key(rest_least(T, q + 1, k)); }, wk, lane);
 }
 
 // The two heaps side by side.  fixed: the part of objective(q) - objective(q+1) that is no popped time.

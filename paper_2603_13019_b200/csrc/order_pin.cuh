@@ -235,27 +235,15 @@ struct PinIo {
   int* traj_node; i64* mem_free; u8* pool_out; int* n_admitted;
 };
 
-// One chunk of up to 32 consecutive queue actions, one per lane (`have`: the lane holds one; rec = its record
-// index).  Lane j < P keeps node j's free memory (mf) and cores (-1: not a CPU node).  The actions whose
+// One chunk of up to 32 consecutive queue actions, one per lane (`have`: the lane holds one, of pool pj; `mine`: an action of
+// the CPU manager, of trajectory t that needs `mem` and least-level cores `need`).  Lane j < P keeps node j's free memory (mf) and cores (-1: not a CPU node).  The actions whose
 // trajectory has no node yet are taken one after the other, lowest lane first.  Returns the lane of the first
 // action whose trajectory finds no node (32 if none); pool_of = the lane's pool afterwards (its trajectory's
 // node, or its own pool; untouched for a lane without an action); the actions from the returned lane on keep
 // their pools.
-__device__ __forceinline__ int pin_chunk(const Params& P, const u8* a_pool, size_t rec, bool have, const int* trajectory,
-                                         const u32* traj_mem, int max_traj, int* tn, i64& mf, int cores, int lane,
+__device__ __forceinline__ int pin_chunk(bool mine, int t, u32 mem, int need, int pj, bool have, int* tn, i64& mf, int cores, int lane,
                                          int& pool_of) {
-  int pj = 0xff, t = -1, node = -1, need = 0; u32 mem = 0;
-  bool mine = false;                                    // an action of the CPU manager with a trajectory
-  if (have) {
-    pj = a_pool[rec];
-    t = trajectory[rec];
-    mine = t >= 0 && t < max_traj && pj < P.P && P.pool[pj].type == TG_POOL_CPU;
-    if (mine) {
-      node = tn[t]; mem = traj_mem[rec];
-      const u32 mk = P.a_mask[rec];
-      need = (int)(P.a_unit[rec] & 0x7f) * (mk ? __ffs(mk) : 0);   // cores of the least level
-    }
-  }
+  int node = mine ? tn[t] : -1;
   int first_out = 32;
   u32 open = __ballot_sync(TG_FULL, mine && node < 0);
   while (open) {
@@ -297,7 +285,19 @@ __global__ void __launch_bounds__(256) k_pin(const __grid_constant__ Params P, c
     const int i = c0 + lane;
     int pool_of = i < P.N ? P.a_pool[row + i] : 0xff;
     if (admitted == n && c0 < n) {                      // (behind the admitted queue the pool column is copied)
-      const int out = pin_chunk(P, P.a_pool, row + i, i < n, X.trajectory, X.traj_mem, X.max_traj, tn, mf, cores, lane, pool_of);
+      int pj = 0xff, t = -1, need = 0; u32 mem = 0;
+      bool mine = false;                                // an action of the CPU manager with a trajectory
+      if (i < n) {
+        pj = P.a_pool[row + i];
+        t = X.trajectory[row + i];
+        mine = t >= 0 && t < X.max_traj && pj < P.P && P.pool[pj].type == TG_POOL_CPU;
+        if (mine) {
+          mem = X.traj_mem[row + i];
+          const u32 mk = P.a_mask[row + i];
+          need = (int)(P.a_unit[row + i] & 0x7f) * (mk ? __ffs(mk) : 0);
+        }
+      }
+      const int out = pin_chunk(mine, t, mem, need, pj, i < n, tn, mf, cores, lane, pool_of);
       if (out < 32) admitted = c0 + out;
     }
     if (i < P.N) X.pool_out[row + i] = (u8)pool_of;

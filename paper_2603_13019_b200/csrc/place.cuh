@@ -27,9 +27,7 @@ __device__ __forceinline__ int find_block(u32 busy, int bl, int group) {
 }
 
 // nm: node busy masks of the pool (updated).  keep candidates, multiplicities r[].
-// owner (may be null): one entry per GPU of the pool, receives ids[i] for every GPU granted.
-__device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r,
-                          int* pnode, int* poff, int lane, int* owner = nullptr, const int* ids = nullptr) {
+__device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r, int* pnode, int* poff, int lane) {
   const int top = ilog2(pd.group);
   const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
 #pragma unroll 1
@@ -57,7 +55,6 @@ __device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, con
         if (lane == 0) {
           nm[node] |= (u8)(((1u << z) - 1u) << start);
           if (rep == 0) { pnode[i] = node; poff[i] = start; }
-          if (owner) for (int b = 0; b < z; ++b) owner[node * pd.group + start + b] = ids[i];
         }
         __syncwarp();
       }

@@ -30,10 +30,9 @@
 struct ReplayWs {
   int* wait;        // [S][N] waiting actions behind the first wcap, by queue position
   u64* wkey;        // [S][N] their sort keys (policy 1 / 2 only)
-  u32* cores;       // [S][W][2] free cores of every domain word (bit = core)
-  int* dfree;       // [S][Dtot] free cores per NUMA domain
+  u32* words;       // [S][W] free cores of every domain word (two of them each), free GPUs of every node
+  int* dfree;       // [S][Dtot + 1] free cores per NUMA domain; the last one belongs to nobody
   int* owner;       // [S][U]  action holding each core / GPU of a grant over several words or chunks
-  u8* nm;           // [S][nodes] GPU busy masks
   // running actions where they do not fit shared memory (ReplayRun)
   uint4* run_at; i64* run_fin; int* run_end; u32* run_pu; int* run_idx;
   // per pool: first unit / domain / word of a scenario's row, domains, words per domain (core pools)
@@ -46,14 +45,14 @@ struct ReplayWs {
   // trajectories pinned to CPU nodes as their actions arrive (Section 5.2); trajectory == nullptr: none of it
   const int* trajectory; const u32* traj_mem; const u8* traj_last; int max_traj;
   int* traj_node; i64* mem_free; u8* pool_rw;   // pool_rw: the pool column the kernel reads (P.a_pool) and rewrites
-  int state_bytes;  // > 0: a scenario's live state (cores .. nm) takes that many bytes of the warp's shared memory
+  int state_bytes;  // > 0: a scenario's live state (words .. owner) takes that many bytes of the warp's shared memory
   int wcap, rcap;   // waiting records / running actions in shared memory (rcap 0: running actions in global memory)
 };
 
 __host__ __device__ __forceinline__ size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
-// bytes of the live state: masks and free counts, owners, node masks
-__host__ __device__ __forceinline__ size_t replay_state_bytes(const ReplayWs& R, int n_nodes) {
-  return align16((size_t)R.W * 8) + align16((size_t)R.Dtot * 4) + align16((size_t)R.U * 4) + align16((size_t)n_nodes + 1);
+// bytes of the live state: masks, free counts, owners (a release may touch the word behind the last one)
+__host__ __device__ __forceinline__ size_t replay_state_bytes(const ReplayWs& R) {
+  return align16((size_t)(R.W + 2) * 4) + align16((size_t)(R.Dtot + 1) * 4) + align16((size_t)R.U * 4);
 }
 
 #define KR_THREADS 32
@@ -63,35 +62,42 @@ __host__ __device__ __forceinline__ size_t replay_state_bytes(const ReplayWs& R,
 #define KR_STATE_MAX 16384
 #define KR_SLOT_BYTES 128         // free capacity of the 32 demand slots at most
 // shared memory of a block (one warp) without the parts sized by the round
-#define KR_BASE_BYTES (WARP_SMEM_BYTES + KR_FAST_BYTES + KR_SLOT_BYTES + 64)
+#define KR_TABLE_BYTES 2048       // per free mask of a node: its free blocks by size, and where a chunk of every size goes
+#define KR_BASE_BYTES (WARP_SMEM_BYTES + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES + 64)
 #define KR_NEVER 0x7fffffff
 
-// Waiting records: slots that do not move, and the queue as a ring of slot numbers.  sp: s, p; ta: least duration,
-// arrival; c: action, meta, mask, unit byte.  meta: pool (4 bits), first demand slot (6), chunk class of the least
-// level (2), units of the least level (13), elastic (1); bit 31: started in this round.
+// Waiting records, and the queue: a ring of records, or (LIST: a queue that is kept in another order) a ring of the
+// numbers of records that do not move.  sp: s, p; ta: least duration, arrival; c: action, meta, mask, unit byte
+// (bit 8: the last action of its trajectory).
+// meta: chunk class of the least level (2 bits) and pool (3), by which a demand slot's lane knows what it is charged; nobody
+// (1), elastic (1), started in this round (1), units of the least level (24).
+template <bool LIST>
 struct ReplayQueue {
   uint4* sp; uint4* ta; uint4* c; u64* key; unsigned short* q; unsigned short* free;
   int cap, head;
   __device__ __forceinline__ int at(int i) const { const int k = head + i; return k >= cap ? k - cap : k; }   // ring place of position i < cap
+  __device__ __forceinline__ int slot(int i) const { return LIST ? (int)q[at(i)] : at(i); }
 };
-#define RQ_POOL(m) ((int)((m) & 15u))
-#define RQ_SLOT(m) ((int)(((m) >> 4) & 63u))
-#define RQ_CLASS(m) ((int)(((m) >> 10) & 3u))
-#define RQ_UNITS(m) ((int)(((m) >> 12) & 0x1fffu))
-#define RQ_ELASTIC 0x2000000u
-#define RQ_STARTED 0x80000000u
-#define RQ_NOBODY 15u             // meta of a lane without a record: no pool, no demand
+#define RQ_CLASS(m) ((int)((m) & 3u))
+#define RQ_POOL(m) ((int)(((m) >> 2) & 15u))        // 8 and above: nobody
+#define RQ_ELASTIC 64u
+#define RQ_STARTED 128u
+#define RQ_UNITS(m) ((int)((m) >> 8))
+#define RQ_NOBODY 32u
 
-// Running actions.  end: the round that releases it; pu: units (21 bits), first demand slot (5), pool (3), type (2), wide
-// (1); at: what it holds - mask (64 bits), word or node, domain.  A wide grant's units are the ones whose owner it is.
+// Running actions.  end: the round that releases it; pu: the units it gives back (21 bits; none of a quota window's), first demand
+// slot (5), pool (3), wide (1), GPU (1), a trajectory's last (1); at: what it holds - masks of two words, the first one's number, domain.  A wide grant's
+// units are the ones whose owner it is, from at.x on.
 struct ReplayRun { uint4* at; i64* fin; int* end; u32* pu; int* idx; };
 #define RR_UNITS(v) ((int)((v) & 0x1fffffu))
 #define RR_SLOT(v) ((int)(((v) >> 21) & 31u))
 #define RR_POOL(v) ((int)(((v) >> 26) & 7u))
-#define RR_TYPE(v) ((int)(((v) >> 29) & 3u))
-#define RR_WIDE 0x80000000u
+#define RR_WIDE 0x20000000u
+#define RR_GPU 0x40000000u
+#define RR_LAST 0x80000000u
 __device__ __forceinline__ u32 rr_pack(const PoolDev& pd, int j, int units, bool wide) {
-  return (u32)units | ((u32)pd.slot0 << 21) | ((u32)j << 26) | ((u32)pd.type << 29) | (wide ? RR_WIDE : 0u);
+  const int back = pd.window_us > 0 ? 0 : units;          // used quota is not given back
+  return (u32)back | ((u32)pd.slot0 << 21) | ((u32)j << 26) | (pd.type == TG_POOL_GPU ? RR_GPU : 0u) | (wide ? RR_WIDE : 0u);
 }
 
 __device__ __forceinline__ i64 i64_of(u32 lo, u32 hi) { return (i64)(((u64)hi << 32) | lo); }
@@ -116,7 +122,7 @@ __device__ __forceinline__ ReplayRec replay_decode(const Params& P, int j, u32 u
   const int rmin = __ffs(eff), c = pd.type == TG_POOL_GPU ? level_of(g, gang, rmin) : 0;
   r.s = clamp_param(s); r.p = clamp_param(p); r.tl = duration(r.s, r.p, rmin);
   r.mask = eff; r.cg = (u8)(g | (gang << 7));
-  r.meta = (u32)j | ((u32)pd.slot0 << 4) | ((u32)c << 10) | ((u32)(g * rmin) << 12) | (eff & (eff - 1) ? RQ_ELASTIC : 0u);
+  r.meta = (u32)c | ((u32)j << 2) | (eff & (eff - 1) ? RQ_ELASTIC : 0u) | ((u32)(g * rmin) << 8);
   return r;
 }
 __device__ __forceinline__ ReplayRec replay_load(const Params& P, size_t row, int a) {
@@ -124,21 +130,24 @@ __device__ __forceinline__ ReplayRec replay_load(const Params& P, size_t row, in
   r.arr = P.a_arrival ? P.a_arrival[row + a] : 0;
   return r;
 }
-__device__ __forceinline__ void replay_store(const ReplayQueue& Q, int x, const ReplayRec& r, int a) {
+template <bool LIST>
+__device__ __forceinline__ void replay_store(const ReplayQueue<LIST>& Q, int x, const ReplayRec& r, int a, u32 last) {
   Q.sp[x] = make_uint4((u32)r.s, (u32)((u64)r.s >> 32), (u32)r.p, (u32)((u64)r.p >> 32));
   Q.ta[x] = make_uint4((u32)r.tl, (u32)((u64)r.tl >> 32), (u32)r.arr, (u32)((u64)r.arr >> 32));
-  Q.c[x] = make_uint4((u32)a, r.meta, r.mask, (u32)r.cg);
+  Q.c[x] = make_uint4((u32)a, r.meta, r.mask, (u32)r.cg | last);
 }
 // action, meta, mask and unit byte at a queue position (any lane's own); x: its slot where it is in shared memory
-__device__ __forceinline__ uint4 replay_facts(const Params& P, const ReplayQueue& Q, const int* wait, size_t row, int i, int& x) {
-  if (i < Q.cap) { x = Q.q[Q.at(i)]; return Q.c[x]; }
+template <bool LIST>
+__device__ __forceinline__ uint4 replay_facts(const Params& P, const ReplayQueue<LIST>& Q, const int* wait, size_t row, int i, int& x) {
+  if (i < Q.cap) { x = Q.slot(i); return Q.c[x]; }
   const int a = wait[i];
   const ReplayRec r = replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], 0, 0);
   x = -1;
   return make_uint4((u32)a, r.meta, r.mask, (u32)r.cg);
 }
 // ... and the rest of a record whose facts are known
-__device__ __forceinline__ ReplayRec replay_rec(const Params& P, const ReplayQueue& Q, size_t row, const uint4& c, int x) {
+template <bool LIST>
+__device__ __forceinline__ ReplayRec replay_rec(const Params& P, const ReplayQueue<LIST>& Q, size_t row, const uint4& c, int x) {
   if (x < 0) return replay_load(P, row, (int)c.x);
   const uint4 u = Q.sp[x], v = Q.ta[x];
   ReplayRec r;
@@ -148,117 +157,130 @@ __device__ __forceinline__ ReplayRec replay_rec(const Params& P, const ReplayQue
 }
 
 // Live state of the scenario at hand: in the warp's shared memory, or in the arrays of ReplayWs where it is large.
-// slot: free capacity per demand slot, always in shared memory.
-struct ReplayState { u32* cores; int* dfree; int* owner; u8* nm; int* slot; };
+// slot: free capacity per demand slot; node_of: by a node's free GPUs, x: its free blocks of 1, 2, 4 and 8 GPUs (9, 8, 7
+// and 6 bits, so that 32 nodes add up), y: a byte per chunk size, block level << 4 | first GPU of the smallest sufficient
+// block, 0xff where there is none.
+struct ReplayState { u32* words; int* dfree; int* owner; int* slot; uint2* node_of; };
 
-// What a grant holds: a mask of one word (core pools) or node (GPU pools), or owner entries (wide).
+__device__ __forceinline__ uint2 replay_node_entry(u32 free_mask) {
+  const u32 busy = ~free_mask & 0xffu;
+  const NodeBlocks b = node_blocks(busy);
+  const u32 lev = node_levels(busy);
+  u32 y = 0;
+  for (int lz = 3; lz >= 0; --lz) {
+    const u32 ok = lev & (~0u << lz);
+    const int l = __ffs(ok) - 1;
+    y = (y << 8) | (ok ? ((u32)l << 4) | (u32)node_block_start(busy, l) : 0xffu);
+  }
+  return make_uint2((u32)__popc(b.s1) | ((u32)__popc(b.s2) << 9) | ((u32)__popc(b.s4) << 17) | ((u32)__popc(b.s8) << 24), y);
+}
+
+// What a grant holds: masks of two words of the state (a core domain's, or a node's one), or owner entries (wide).
 // node / off: NUMA domain or GPU node, and the first core or GPU.
-struct ReplayGrant { int node, off, word, dom; u32 lo, hi; bool wide; };
+struct ReplayGrant { int node, off; uint4 at; bool wide; };
+
+// the lowest k of the 64 bits hi:lo (at least k are set); every lane looks at two of them
+__device__ __forceinline__ void lowest_bits(u32 lo, u32 hi, int k, int lane, u32& tlo, u32& thi) {
+  if (k == 1) { tlo = lo & (0u - lo); thi = lo ? 0u : hi & (0u - hi); return; }
+  const u32 below = (1u << lane) - 1u;
+  const int nlo = __popc(lo);
+  tlo = __ballot_sync(TG_FULL, ((lo >> lane) & 1u) && __popc(lo & below) < k);
+  thi = __ballot_sync(TG_FULL, ((hi >> lane) & 1u) && nlo + __popc(hi & below) < k);
+}
 
 // One grant of k cores on a pool with cores in use: fewest free cores that still fit, lowest domain, lowest cores first;
-// else ascending domains.  cores / dfree / owner: the pool's own rows.
-__device__ __forceinline__ ReplayGrant replay_take_cores(int group, int n_dom, int wpd, u32* cores, int* dfree, int* owner,
-                                                         int k, int id, int lane) {
+// else ascending domains.  For pools of many or large domains, and for grants that no domain holds; words / dfree /
+// owner: the pool's own rows, which begin at word w0 and domain d0 of the scenario's.
+__device__ __noinline__ ReplayGrant replay_take_cores(int group, int n_dom, int wpd, u32* words, int* dfree, int* owner, int w0, int d0,
+                                                      int k, int id, int lane) {
   ReplayGrant G;
-  G.node = G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = false;
-  int dom = -1;
-  if (n_dom <= 32 && group < (1 << 26)) {
-    const int f = lane < n_dom ? dfree[lane] : -1;
-    const u32 mn = __reduce_min_sync(TG_FULL, f >= k ? ((u32)f << 5) | (u32)lane : 0xffffffffu);
-    if (mn != 0xffffffffu) dom = (int)(mn & 31u);
-  } else {
-    u32 best = 0xffffffffu; int at = -1;
+  G.node = G.off = -1; G.at = make_uint4(0u, 0u, 0u, 0u); G.wide = false;
+  u32 best = 0xffffffffu; int at = -1, dom = -1;
 #pragma unroll 1
-    for (int d = lane; d < n_dom; d += 32) { const int f = dfree[d]; if (f >= k && (u32)f < best) { best = (u32)f; at = d; } }
-    const u32 mn = __reduce_min_sync(TG_FULL, best);
-    if (mn != 0xffffffffu) dom = (int)__reduce_min_sync(TG_FULL, best == mn ? (u32)at : 0xffffffffu);
-  }
+  for (int d = lane; d < n_dom; d += 32) { const int f = dfree[d]; if (f >= k && (u32)f < best) { best = (u32)f; at = d; } }
+  const u32 mn = __reduce_min_sync(TG_FULL, best);
+  if (mn != 0xffffffffu) dom = (int)__reduce_min_sync(TG_FULL, best == mn ? (u32)at : 0xffffffffu);
   int need = k;
   const int end = dom >= 0 ? (dom + 1) * wpd : n_dom * wpd;
 #pragma unroll 1
   for (int w = dom >= 0 ? dom * wpd : 0; w < end && need > 0; ++w) {
-    const uint2 m = *(const uint2*)(cores + 2 * w);
-    if ((m.x | m.y) == 0u) continue;
-    // the lowest `need` free cores of the word: every lane looks at two of them
-    const u32 below = (1u << lane) - 1u;
-    const int nlo = __popc(m.x);
-    const u32 lo = __ballot_sync(TG_FULL, ((m.x >> lane) & 1u) && __popc(m.x & below) < need);
-    const u32 hi = __ballot_sync(TG_FULL, ((m.y >> lane) & 1u) && nlo + __popc(m.y & below) < need);
-    const int got = __popc(lo) + __popc(hi);
-    const int d = wpd == 1 ? w : w / wpd, c0 = d * group + (wpd == 1 ? 0 : (w - d * wpd) * 64);   // the word's first core
+    const u32 mlo = words[2 * w], mhi = words[2 * w + 1];
+    if ((mlo | mhi) == 0u) continue;
+    u32 lo, hi;
+    const int got = min(need, __popc(mlo) + __popc(mhi));
+    lowest_bits(mlo, mhi, got, lane, lo, hi);
+    const int d = w / wpd, c0 = d * group + (w - d * wpd) * 64;        // the word's first core
     if (G.off < 0) {
       G.off = c0 + (lo ? __ffs(lo) - 1 : 31 + __ffs(hi)); G.node = d;
-      G.word = w; G.dom = d; G.lo = lo; G.hi = hi;
       G.wide = got < need;
-      if (G.wide) G.dom = G.off;                           // (where the search for its cores begins)
+      G.at = G.wide ? make_uint4((u32)G.off, 0u, 0u, 0u) : make_uint4(lo, hi, (u32)(w0 + 2 * w), (u32)(d0 + d));
     }
     if (G.wide) {
       if ((lo >> lane) & 1u) owner[c0 + lane] = id;
       if ((hi >> lane) & 1u) owner[c0 + 32 + lane] = id;
     }
     __syncwarp();
-    if (lane == 0) { *(uint2*)(cores + 2 * w) = make_uint2(m.x & ~lo, m.y & ~hi); dfree[d] -= got; }
+    if (lane == 0) { words[2 * w] = mlo & ~lo; words[2 * w + 1] = mhi & ~hi; dfree[d] -= got; }
     need -= got;
     __syncwarp();
   }
   return G;
 }
 
-// One candidate alone on a GPU pool: nreq chunks of 2^lz GPUs (Section 5.3: smallest sufficient maximal free block,
-// lowest node, lowest start); node / off: the first chunk.
-__device__ __forceinline__ ReplayGrant replay_take_gpus(const PoolDev& pd, u8* nm, int* owner, int lz, int nreq, int id, int lane) {
+// nreq chunks of 2^lz GPUs for one action (Section 5.3: smallest sufficient maximal free block, lowest node, lowest start);
+// node / off: the first chunk.  words / owner: the pool's own rows, which begin at word w0.
+__device__ __forceinline__ ReplayGrant replay_take_gpus(int group, int n_nodes, u32* words, const uint2* node_of, int* owner, int w0, int dummy,
+                                                        int lz, int nreq, int id, int lane) {
   ReplayGrant G;
-  G.node = G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = nreq > 1;
-  const int top = ilog2(pd.group), z = 1 << lz;
-  const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
+  G.node = G.off = -1; G.at = make_uint4(0u, 0u, (u32)w0, (u32)dummy); G.wide = nreq > 1;
 #pragma unroll 1
   for (int rep = 0; rep < nreq; ++rep) {
-    u32 best = 0xffffffffu;                                // level << 24 | node
+    u32 best = 0xffffffffu;                                // level | node | first GPU
+    if (n_nodes == 1) {
+      const u32 y = (node_of[words[0]].y >> (8 * lz)) & 0xffu;
+      if (y != 0xffu) best = y & 15u;
+    } else {
 #pragma unroll 1
-    for (int v = lane; v < pd.n_nodes; v += 32) {
-      const u32 lev = node_levels(nm[v] | pad) & (~0u << lz);   // the smallest sufficient block of the node
-      if (lev) best = min(best, ((u32)(__ffs(lev) - 1) << 24) | (u32)v);
+      for (int v = lane; v < n_nodes; v += 32) {
+        const u32 y = (node_of[words[v]].y >> (8 * lz)) & 0xffu;
+        if (y != 0xffu) best = min(best, ((y & 0xf0u) << 20) | ((u32)v << 4) | (y & 15u));
+      }
+      best = __reduce_min_sync(TG_FULL, best);
     }
-    best = __reduce_min_sync(TG_FULL, best);
-    const int at = (int)(best & 0xffffffu), level = (int)(best >> 24);
-    if (level > top) continue;                             // cannot happen: the selection fits
-    const u32 busy = nm[at];
-    const int start = node_block_start(busy | pad, level);
-    const u32 bits = ((1u << z) - 1u) << start;
+    if (best == 0xffffffffu) continue;                     // cannot happen: the selection fits
+    const int at = (int)((best >> 4) & 0xfffffu), start = (int)(best & 15u);
+    const u32 bits = ((1u << (1 << lz)) - 1u) << start;
     __syncwarp();
-    if (lane == 0) nm[at] = (u8)(busy | bits);
-    if (G.wide && lane < z) owner[at * pd.group + start + lane] = id;
-    if (rep == 0) { G.node = at; G.off = start; G.word = at; G.lo = bits; }
+    if (lane == 0) words[at] &= ~bits;
+    if (G.wide && lane < (1 << lz)) owner[at * group + start + lane] = id;
+    if (rep == 0) { G.node = at; G.off = start; if (!G.wide) { G.at.x = bits; G.at.z = (u32)(w0 + at); } }
     __syncwarp();
   }
   return G;
 }
 
 // free capacity of a GPU pool's four demand slots
-__device__ __forceinline__ void replay_gpu_slots(const PoolDev& pd, const u8* nm_row, int* slot, int lane) {
-  int c[4];
-  if (pd.n_nodes <= 32) {
-    // the four counts of free blocks in one word: at most 256, 128, 64 and 32
-    const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
-    u32 x = 0;
-    if (lane < pd.n_nodes) {
-      const NodeBlocks b = node_blocks(nm_row[pd.node0 + lane] | pad);
-      x = (u32)__popc(b.s1) | ((u32)__popc(b.s2) << 9) | ((u32)__popc(b.s4) << 17) | ((u32)__popc(b.s8) << 24);
-    }
-    x = __reduce_add_sync(TG_FULL, x);
-    c[3] = (int)(x >> 24) * 8; c[2] = c[3] + (int)((x >> 17) & 127u) * 4; c[1] = c[2] + (int)((x >> 9) & 255u) * 2; c[0] = c[1] + (int)(x & 511u);
-  } else gpu_caps(pd, nm_row, lane, c);
-  if (lane < 4) slot[pd.slot0 + lane] = pick4(c, lane);
+__device__ __forceinline__ void replay_gpu_slots(const PoolDev& pd, const u32* words, const uint2* node_of, int* slot, int lane) {
+  int f0 = 0, f1 = 0, f2 = 0, f3 = 0;
+#pragma unroll 1
+  for (int v0 = 0; v0 < pd.n_nodes; v0 += 32) {
+    u32 x;
+    if (pd.n_nodes == 1) x = node_of[words[0]].x;
+    else x = __reduce_add_sync(TG_FULL, v0 + lane < pd.n_nodes ? node_of[words[v0 + lane]].x : 0u);
+    f0 += (int)(x & 511u); f1 += (int)((x >> 9) & 255u); f2 += (int)((x >> 17) & 127u); f3 += (int)(x >> 24);
+  }
+  // GPUs in blocks of at least 2^lane
+  const int c = f3 * 8 + (lane <= 2 ? f2 * 4 : 0) + (lane <= 1 ? f1 * 2 : 0) + (lane == 0 ? f0 : 0);
+  if (lane < 4) slot[pd.slot0 + lane] = c;
   __syncwarp();
 }
 
 // The selection of a pool with a choice to make: its candidates (among the first n positions) and, where an eviction
 // step can look at them, the waiting actions behind and the running ones are gathered into arrays.
-template <bool EXT>
-__device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue Q, const ReplayRun run, const int* wait, int sc, int j,
+template <bool LIST>
+__device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue<LIST>& Q, const ReplayRun run, const int* wait, size_t row, int j,
                                            int n, int nw, int nr, int m, i64 now, int cap0, int cap1, int cap2, int cap3, Slab& slab,
                                            CandArrays& C, int& keep, int lane) {
-  const size_t row = (size_t)sc * P.N;
   const PoolDev& pd = P.pool[j];
   C.cg = (u8*)slab.take_fast(m); C.rsel = (u8*)slab.take_fast(m); C.rkeep = (u8*)slab.take_fast(m);
   C.cmask = (u32*)slab.take_fast((u64)m * 4); C.rowcand = (int*)slab.take_fast((u64)m * 4);
@@ -336,48 +358,124 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
   return keep >= 0;
 }
 
+// Two candidates (queue positions ba < bb < 32, in shared memory) on a pool with at most KR_PAIR_RUN actions running in all and
+// at most KR_PAIR_WAIT waiting behind the prefix: DPArrange's answer for both (lanes try b's levels, one after
+// the other a's), a's alone, and the eviction step between them, without any of the selection's arrays.  Returns how many
+// are kept, their levels in ra and rb, or 0: the general path decides (a time beyond 32 bits).  Most selections of a trace
+// are of two candidates: with the arrays 11400 cycles each on the `trace` cluster, and 3700 for placing them.
+#define KR_PAIR_RUN 30
+#define KR_PAIR_WAIT 1024
+template <bool LIST>
+__device__ __forceinline__ int replay_pair(const Params& P, const PoolDev& pd, const ReplayQueue<LIST>& Q, const ReplayRun& run, size_t row, int j, int ba,
+                                           int bb, int n, int nw, int nr, i64 now, const int* slot, int aside, u32* list, int lane, int& ra, int& rb) {
+  const int xa = Q.slot(ba), xb = Q.slot(bb);
+  const uint4 ca = Q.c[xa], cb = Q.c[xb];
+  const ReplayRec A = replay_rec(P, Q, row, ca, xa), B = replay_rec(P, Q, row, cb, xb);
+  const bool gpu = pd.type == TG_POOL_GPU;
+  const int ga = A.cg & 0x7f, anga = A.cg >> 7, gb = B.cg & 0x7f, angb = B.cg >> 7, r = lane + 1;
+  int cap[4] = {slot[0] - aside, 0, 0, 0};
+  if (gpu) { cap[1] = slot[1]; cap[2] = slot[2]; cap[3] = slot[3]; }
+  const bool has_b = (B.mask >> lane) & 1u;
+  const int ub = gb * r, lb = has_b && gpu ? level_of(gb, angb, r) : 0;
+  const i64 tb = duration(B.s, B.p, has_b ? r : 1);
+  i64 bv = TG_INF; u32 bt = 0xffffffffu;                  // duration sum; units << 12 | b's level << 6 | a's level
+#pragma unroll 1
+  for (u32 mk = A.mask; mk; mk &= mk - 1) {
+    const int x = __ffs(mk), ua = ga * x, la = gpu ? level_of(ga, anga, x) : 0;
+    const int m0 = cap[0] - ua, m1 = min(m0, cap[1] - (la >= 1 ? ua : 0)), m2 = min(m1, cap[2] - (la >= 2 ? ua : 0)),
+              m3 = min(m2, cap[3] - (la >= 3 ? ua : 0));
+    // (b's own class bounds it, a's the levels up to a's: a level that a charges and b does not has to hold a)
+    const bool a_fits = la == 0 ? m0 >= 0 : la == 1 ? m1 >= 0 : la == 2 ? m2 >= 0 : m3 >= 0;
+    const i64 v = duration(A.s, A.p, x) + tb;
+    const u32 t = ((u32)(ua + ub) << 12) | ((u32)r << 6) | (u32)x;
+    if (has_b && a_fits && ub <= (lb == 0 ? m0 : lb == 1 ? m1 : lb == 2 ? m2 : m3) && (v < bv || (v == bv && t < bt))) { bv = v; bt = t; }
+  }
+  const i64 both = warp_min64(bv);
+  const u32 t = __reduce_min_sync(TG_FULL, bv == both ? bt : 0xffffffffu);
+  const bool has_a = (A.mask >> lane) & 1u;
+  const int la = has_a && gpu ? level_of(ga, anga, r) : 0;
+  const u32 fits = __ballot_sync(TG_FULL, has_a && ga * r <= pick4(cap, la));
+  if (both == TG_INF || !fits) return 0;                  // (cannot happen: the prefix admitted them)
+  ra = (int)(t & 63u); rb = (int)((t >> 6) & 63u);
+  const int alone = best_level(A.p, fits);
+  const i64 t_alone = duration(A.s, A.p, alone), t_first = duration(B.s, B.p, nth_level(B.mask, min(P.depth, __popc(B.mask)) - 1));
+  if (ra == alone && duration(B.s, B.p, rb) <= t_first) return 2;      // eviction_cannot_pay
+  // ---- what waits on the pool behind them
+  int n_ac = 0, first = -1;
+#pragma unroll 1
+  for (int i0 = n; i0 < nw; i0 += 32) {
+    const int i = i0 + lane, x = i < nw ? Q.slot(i) : 0;
+    const bool mine = i < nw && RQ_POOL(Q.c[x].y) == j;
+    const u32 m = __ballot_sync(TG_FULL, mine);
+    if (mine) { const uint4 v = Q.ta[x]; list[n_ac + __popc(m & ((1u << lane) - 1u))] = ev_key(i64_of(v.x, v.y)); }
+    if (first < 0 && m) first = i0 + __ffs(m) - 1;
+    n_ac += __popc(m);
+  }
+  i64 fixed = t_alone - both + t_first, first_a = 0;
+  if (n_ac > 0) {
+    const int x = Q.slot(first);
+    const uint4 c = Q.c[x];
+    const ReplayRec F = replay_rec(P, Q, row, c, x);
+    first_a = duration(F.s, F.p, nth_level(F.mask, min(P.depth, __popc(F.mask)) - 1));
+    fixed += F.tl - first_a;
+  }
+  __syncwarp();
+  // ---- the heaps: what runs on the pool, and the candidates behind it
+  u32 a[1] = {EV_NONE}, b[1] = {EV_NONE};
+  if (lane < nr && RR_POOL(run.pu[lane]) == j) { const i64 f = run.fin[lane]; a[0] = b[0] = ev_key(f > now ? f - now : 0); }
+  if (lane == nr) { a[0] = ev_key(duration(A.s, A.p, ra)); b[0] = ev_key(t_alone); }
+  if (lane == nr + 1) a[0] = ev_key(duration(B.s, B.p, rb));
+  const int pays = ev_run_regs<1>(a, b, nr + 2, n_ac, ev_key(t_first), ev_key(first_a), fixed, [&](int k) { return list[k]; },
+                                  (u32)__cvta_generic_to_shared(warp_smem()), lane);
+  if (pays < 0) return 0;
+  if (pays) { ra = alone; return 1; }
+  return 2;
+}
+
 // EXT: the queue may be kept sorted by R.policy's key, trajectories pinned on arrival (R.trajectory), further cost-vector
-// entries (n_side) and a service cache; the plain instance carries none of their code.
-template <bool EXT>
+// entries (n_side) and a service cache; the plain instance carries none of their code.  SMEM: live state and running
+// actions are in shared memory; the other instance asks at run time.
+template <bool EXT, bool SMEM>
 __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant__ Params P, const __grid_constant__ ReplayWs R) {
   extern __shared__ __align__(16) unsigned char k2_smem[];
   const int lane = threadIdx.x;
   const u32 below = (1u << lane) - 1u;
-  char* const sm = (char*)(((u64)k2_smem + 15u) & ~(u64)15);
+  char* const sm = (char*)k2_smem;                         // (WARP_SMEM_BYTES from here are what warp_smem() hands out)
   char* const fast = sm + WARP_SMEM_BYTES;
   // per-warp arrays behind the selection's work area
-  ReplayQueue Q;
+  ReplayState Z;
+  Z.slot = (int*)(fast + KR_FAST_BYTES);
+  Z.node_of = (uint2*)(fast + KR_FAST_BYTES + KR_SLOT_BYTES);
+  ReplayQueue<EXT> Q;
   Q.cap = R.wcap;
   {
-    char* at = fast + KR_FAST_BYTES + KR_SLOT_BYTES;
+    char* at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES;
     Q.sp = (uint4*)at; Q.ta = Q.sp + Q.cap; Q.c = Q.ta + Q.cap; Q.key = (u64*)(Q.c + Q.cap);
     Q.q = (unsigned short*)(Q.key + Q.cap); Q.free = Q.q + Q.cap;
   }
-  char* const run_at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + align16((size_t)Q.cap * KR_WAIT_BYTES);
+  char* const run_at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES + align16((size_t)Q.cap * KR_WAIT_BYTES);
   char* const state_at = run_at + align16((size_t)R.rcap * KR_RUN_BYTES);
+#pragma unroll 1
+  for (int x = lane; x < 256; x += 32) Z.node_of[x] = replay_node_entry((u32)x);
 #pragma unroll 1
   for (int sc = blockIdx.x; sc < P.S; sc += gridDim.x) {
     const size_t row = (size_t)sc * P.N;
     const int n_act = uniform(min(max(P.n_actions[sc], 0), P.N));
     int* wait = R.wait + row; u64* wkey = EXT && R.wkey ? R.wkey + row : nullptr;
     ReplayRun run;
-    if (R.rcap > 0) {
+    if (SMEM || R.rcap > 0) {
       run.at = (uint4*)run_at; run.fin = (i64*)(run.at + R.rcap); run.end = (int*)(run.fin + R.rcap); run.pu = (u32*)(run.end + R.rcap);
       run.idx = (int*)(run.pu + R.rcap);
     } else { run.at = R.run_at + row; run.fin = R.run_fin + row; run.end = R.run_end + row; run.pu = R.run_pu + row; run.idx = R.run_idx + row; }
-    ReplayState Z;
-    Z.slot = (int*)(fast + KR_FAST_BYTES);
-    if (R.state_bytes > 0) {
-      const size_t o_df = align16((size_t)R.W * 8), o_ow = o_df + align16((size_t)R.Dtot * 4), o_nm = o_ow + align16((size_t)R.U * 4);
-      Z.cores = (u32*)state_at; Z.dfree = (int*)(state_at + o_df); Z.owner = (int*)(state_at + o_ow); Z.nm = (u8*)(state_at + o_nm);
-    } else {
-      Z.cores = R.cores + (size_t)sc * R.W * 2; Z.dfree = R.dfree + (size_t)sc * R.Dtot; Z.owner = R.owner + (size_t)sc * R.U;
-      Z.nm = R.nm + (size_t)sc * ((P.n_nodes_total + 4) & ~3);
-    }
+    if (SMEM || R.state_bytes > 0) {
+      Z.words = (u32*)state_at; Z.dfree = (int*)(state_at + align16((size_t)(R.W + 2) * 4));
+      Z.owner = (int*)((char*)Z.dfree + align16((size_t)(R.Dtot + 1) * 4));
+    } else { Z.words = R.words + (size_t)sc * (R.W + 2); Z.dfree = R.dfree + (size_t)sc * (R.Dtot + 1); Z.owner = R.owner + (size_t)sc * R.U; }
     int* occ = R.occupancy ? R.occupancy + (size_t)sc * R.max_rounds * P.P : nullptr;
+    int* const o_alloc = P.o_alloc + row; int* const o_node = P.o_node + row; int* const o_off = P.o_off + row; i64* const o_act = P.o_act + row;
     // outputs and state start empty (the occupancy rows were zeroed before)
 #pragma unroll 4
-    for (int i = lane; i < P.N; i += 32) { P.o_alloc[row + i] = 0; P.o_node[row + i] = -1; P.o_off[row + i] = -1; P.o_act[row + i] = -1; }
+    for (int i = lane; i < P.N; i += 32) { o_alloc[i] = 0; o_node[i] = -1; o_off[i] = -1; o_act[i] = -1; }
     int status = 0;
 #pragma unroll 2
     for (int i = lane; i < n_act; i += 32) {
@@ -397,21 +495,25 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
     }
     status = __reduce_or_sync(TG_FULL, status);
     if (status & TG_ST_BAD_ACTION) status = TG_ST_BAD_ACTION;
+    u32 gpu_pools = 0;
+    __syncwarp();
 #pragma unroll 1
     for (int j = 0; j < P.P; ++j) {
       const PoolDev& pd = P.pool[j];
       if (pd.type == TG_POOL_GPU) {
         int taken = 0;
+        u32* words = Z.words + R.word0[j];
 #pragma unroll 1
         for (int v = lane; v < pd.n_nodes; v += 32) {
           const u32 b = (P.gpu_busy ? P.gpu_busy[(size_t)sc * P.n_nodes_total + pd.node0 + v] : 0u) & ((1u << pd.group) - 1u);
-          Z.nm[pd.node0 + v] = (u8)b;
+          words[v] = ~b & ((1u << pd.group) - 1u);
           taken += __popc(b);
         }
         taken = warp_sum32(taken);
         if (occ && lane == 0 && status == 0) occ[j] = taken;   // round 0's difference
         __syncwarp();
-        replay_gpu_slots(pd, Z.nm, Z.slot, lane);
+        replay_gpu_slots(pd, words, Z.node_of, Z.slot, lane);
+        gpu_pools |= 1u << j;
       } else if (lane == 0) Z.slot[pd.slot0] = pd.capacity;
       if (pd.type == TG_POOL_API) continue;
 #pragma unroll 1
@@ -422,13 +524,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       for (int w = lane; w < R.n_dom[j] * wpd; w += 32) {
         const int left = pd.group - (w % wpd) * 64;         // cores of the domain from this word on
         const u64 m = left >= 64 ? ~0ull : (1ull << left) - 1ull;
-        *(uint2*)(Z.cores + 2 * (R.word0[j] + w)) = make_uint2((u32)m, (u32)(m >> 32));
+        Z.words[R.word0[j] + 2 * w] = (u32)m; Z.words[R.word0[j] + 2 * w + 1] = (u32)(m >> 32);
       }
 #pragma unroll 1
       for (int d = lane; d < R.n_dom[j]; d += 32) Z.dfree[R.dom0[j] + d] = pd.group;
     }
+    if (EXT)
 #pragma unroll 1
-    for (int i = lane; i < Q.cap; i += 32) Q.free[i] = (unsigned short)i;
+      for (int i = lane; i < Q.cap; i += 32) Q.free[i] = (unsigned short)i;
     Q.head = 0;
     __syncwarp();
     int rounds = 0;
@@ -440,19 +543,33 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       // arrivals, 32 at a time: lane k holds record base + k; the next batch's columns are on their way
       int base = 0;
       int l_pool = 0; u32 l_unit = 1, l_mask = 1; i64 l_s = 0, l_p = 0, l_arr = 0;
+      int l_traj = -1; u32 l_mem = 0, l_last = 0;          // (trajectories)
       auto fetch = [&](int from) {
         const int i = from + lane;
         if (i < n_act) {
+          if (EXT && R.trajectory) {
+            l_traj = R.trajectory[row + i]; l_mem = R.traj_mem[row + i];
+            l_last = R.traj_last && R.traj_last[row + i] ? 256u : 0u;
+          }
           l_pool = P.a_pool[row + i]; l_unit = P.a_unit[row + i]; l_mask = P.a_mask[row + i]; l_s = P.a_s[row + i]; l_p = P.a_p[row + i];
           l_arr = P.a_arrival ? P.a_arrival[row + i] : 0;
         }
       };
+      int b_traj = -1; u32 b_mem = 0, b_last = 0;
+      // lane j < P: free memory and cores of node j (-1 cores: not a CPU node)
+      i64 node_mem = 0; int node_cores = -1;
+      if (EXT && R.trajectory && lane < P.P) {
+        node_mem = R.mem_free[(size_t)sc * P.P + lane];
+        if (P.pool[lane].type == TG_POOL_CPU) node_cores = P.pool[lane].capacity;
+      }
+      int* const traj_node = EXT && R.trajectory ? R.traj_node + (size_t)sc * R.max_traj : nullptr;
       ReplayRec b_rec; int b_at = KR_NEVER;                // b_at: the round that admits the lane's arrival
       int next_at = KR_NEVER;
       auto refill = [&](int from) {                        // the batch that was fetched becomes the current one
         base = from;
         b_rec = replay_decode(P, l_pool, l_unit, l_mask, l_s, l_p);
         b_rec.arr = l_arr;
+        if (EXT) { b_traj = l_traj; b_mem = l_mem; b_last = l_last; }
         b_at = from + lane < n_act ? round_at(R, l_arr) : KR_NEVER;
         next_at = __shfl_sync(TG_FULL, b_at, 0);
         fetch(from + 32);
@@ -466,6 +583,12 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       const i64 my_window = lane < P.P && P.pool[lane].type == TG_POOL_API ? P.pool[lane].window_us : 0;
       int my_turn = my_window > 0 ? round_at(R, my_window) : KR_NEVER;
       int next_turn = warp_min32(my_turn);
+      u32 charged = 0;                                     // bit pool << 2 | class: such a request asks this lane's demand slot
+#pragma unroll 1
+      for (int j = 0; j < P.P; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (lane >= P.pool[j].slot0 && lane <= P.pool[j].slot0 + c && (c == 0 || P.pool[j].type == TG_POOL_GPU)) charged |= 1u << (4 * j + c);
       while (r < R.max_rounds) {
         const i64 now = (i64)r * R.round_us;
         // 1. quota refill: usage restarts with its window
@@ -482,36 +605,29 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         // 2. release what has finished, a lane each; the running list is compacted in place
         while (min_end <= r) {
           // (the memory of a trajectory that ends goes back in the order of the rounds)
-          const int until = EXT && R.traj_last ? min_end : r;
+          const int until = EXT && R.trajectory && R.traj_last ? min_end : r;
           int kept = 0, me = KR_NEVER;
-          u32 touched = 0;                                 // GPU pools
+          bool gpus = false;
 #pragma unroll 1
           for (int i0 = 0; i0 < nr; i0 += 32) {
             const int i = i0 + lane;
             const int end = i < nr ? run.end[i] : KR_NEVER;
-            const bool done = i < nr && end <= until, stay = i < nr && !done;
+            const bool done = end <= until, stay = i < nr && !done;
             const u32 bd = __ballot_sync(TG_FULL, done), bk = __ballot_sync(TG_FULL, stay);
             if (stay) me = min(me, end);
             if (bd || kept != i0) {
               uint4 at = make_uint4(0u, 0u, 0u, 0u); u32 pu = 0; int a = 0; i64 fin = 0;
               if (i < nr) { at = run.at[i]; pu = run.pu[i]; a = run.idx[i]; fin = run.fin[i]; }
               if (done) {
-                const int type = RR_TYPE(pu), units = RR_UNITS(pu), j = RR_POOL(pu);
-                if (type == TG_POOL_GPU) {
-                  touched |= 1u << j;
-                  if (!(pu & RR_WIDE)) {
-                    const u32 v = (u32)P.pool[j].node0 + at.z;
-                    atomicAnd((u32*)Z.nm + (v >> 2), ~(at.x << (8u * (v & 3u))));
-                  }
-                } else if (type == TG_POOL_CPU) {
-                  atomicAdd(&Z.slot[RR_SLOT(pu)], units);
-                  if (!(pu & RR_WIDE)) {
-                    u32* w = Z.cores + 2 * (R.word0[j] + (int)at.z);
-                    if (at.x) atomicOr(w, at.x);
-                    if (at.y) atomicOr(w + 1, at.y);
-                    atomicAdd(&Z.dfree[R.dom0[j] + (int)at.w], units);
-                  }
-                } else if (P.pool[j].window_us == 0) atomicAdd(&Z.slot[RR_SLOT(pu)], units);   // (used quota is not given back)
+                // (a GPU pool's slots are worked out again below; its domain, and a quota call's, is nobody's)
+                const int units = RR_UNITS(pu);
+                gpus |= (pu & RR_GPU) != 0;
+                atomicAdd(&Z.slot[RR_SLOT(pu)], units);
+                if (!(pu & RR_WIDE)) {
+                  atomicOr(Z.words + at.z, at.x);
+                  if (at.y) atomicOr(Z.words + at.z + 1, at.y);
+                  atomicAdd(Z.dfree + at.w, units);
+                }
                 if (EXT)
 #pragma unroll 1
                   for (int e = 0; e < P.n_side; ++e) {     // a concurrency pool held the action's further amounts until now
@@ -523,13 +639,13 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               for (u32 wide = __ballot_sync(TG_FULL, done && (pu & RR_WIDE)); wide; wide &= wide - 1) {
                 const int b = __ffs(wide) - 1, fa = __shfl_sync(TG_FULL, a, b);
                 const u32 fpu = __shfl_sync(TG_FULL, pu, b);
-                const int from = __shfl_sync(TG_FULL, (int)at.w, b), j = RR_POOL(fpu);
+                const int from = (int)__shfl_sync(TG_FULL, at.x, b), j = RR_POOL(fpu);
                 const PoolDev& pd = P.pool[j];
                 const bool cpu = pd.type == TG_POOL_CPU;
                 int* ow = Z.owner + R.unit0[j];
                 int left = RR_UNITS(fpu);
 #pragma unroll 1
-                for (int c0 = cpu ? from & ~31 : 0; c0 < pd.capacity && left > 0; c0 += 32) {
+                for (int c0 = from & ~31; c0 < pd.capacity && left > 0; c0 += 32) {
                   const int c = c0 + lane;
                   const bool mine = c < pd.capacity && ow[c] == fa;
                   const u32 mb = __ballot_sync(TG_FULL, mine);
@@ -538,30 +654,23 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                   if (mine) {
                     ow[c] = -1;
                     const int d = c / pd.group, x = c - d * pd.group;
-                    if (cpu) {
-                      const int w = d * R.wpd[j] + (x >> 6);
-                      atomicOr(Z.cores + 2 * (R.word0[j] + w) + ((x >> 5) & 1), 1u << (x & 31));
-                      atomicAdd(&Z.dfree[R.dom0[j] + d], 1);
-                    } else {
-                      const u32 v = (u32)(pd.node0 + d);
-                      atomicAnd((u32*)Z.nm + (v >> 2), ~(1u << (x + 8 * (int)(v & 3u))));
-                    }
+                    const int w = cpu ? 2 * (d * R.wpd[j] + (x >> 6)) + ((x >> 5) & 1) : d;
+                    atomicOr(Z.words + R.word0[j] + w, 1u << (x & 31));
+                    if (cpu) atomicAdd(&Z.dfree[R.dom0[j] + d], 1);
                   }
                 }
               }
-              if (EXT && R.trajectory && R.traj_last)
+              if (EXT)
 #pragma unroll 1
-                for (u32 rest = bd; rest; rest &= rest - 1) {
-                  const int b = __ffs(rest) - 1, fa = __shfl_sync(TG_FULL, a, b);
-                  const u32 fpu = __shfl_sync(TG_FULL, pu, b);
-                  if (lane == 0 && RR_TYPE(fpu) == TG_POOL_CPU && R.traj_last[row + fa]) {
-                    // the trajectory's last action has ended: its memory goes back to its node
-                    const int t = R.trajectory[row + fa];
-                    if (t >= 0 && t < R.max_traj) {
-                      int* tn = R.traj_node + (size_t)sc * R.max_traj;
-                      if (tn[t] >= 0) { R.mem_free[(size_t)sc * P.P + tn[t]] += (i64)R.traj_mem[row + fa]; tn[t] = -1; }
-                    }
-                  }
+                for (u32 rest = __ballot_sync(TG_FULL, done && (pu & RR_LAST)); rest; rest &= rest - 1) {
+                  // the trajectory's last action has ended: its memory goes back to its node
+                  const int fa = __shfl_sync(TG_FULL, a, __ffs(rest) - 1), t = R.trajectory[row + fa];
+                  const u32 mem = R.traj_mem[row + fa];
+                  const int node = t >= 0 && t < R.max_traj ? traj_node[t] : -1;
+                  if (lane == node) node_mem += (i64)mem;
+                  __syncwarp();
+                  if (lane == 0 && node >= 0) traj_node[t] = -1;
+                  __syncwarp();
                 }
               __syncwarp();
               const int k = kept + __popc(bk & below);
@@ -573,9 +682,12 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           nr = kept;
           min_end = warp_min32(me);
           gated = false;
-          touched = __reduce_or_sync(TG_FULL, touched);
+          if (__any_sync(TG_FULL, gpus))
 #pragma unroll 1
-          for (; touched; touched &= touched - 1) replay_gpu_slots(P.pool[__ffs(touched) - 1], Z.nm, Z.slot, lane);
+            for (u32 g = gpu_pools; g; g &= g - 1) {
+              const int j = __ffs(g) - 1;
+              replay_gpu_slots(P.pool[j], Z.words + R.word0[j], Z.node_of, Z.slot, lane);
+            }
         }
         // 3. admit arrivals
         bool was_gated = gated;
@@ -586,17 +698,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (EXT && R.trajectory) {
             // per-node CPU scheduling: an arrival joins the queue once its trajectory has a node; the first one
             // that finds none waits outside, with everything that arrived after it
-            __syncwarp();
-            i64 mf = 0; int cores = -1;
-            if (lane < P.P && P.pool[lane].type == TG_POOL_CPU) { mf = R.mem_free[(size_t)sc * P.P + lane]; cores = P.pool[lane].capacity; }
             int pool_of = 0xff;
             const bool have = lane >= k0 && lane < k0 + cnt;
-            const int out = pin_chunk(P, R.pool_rw, row + base + lane, have, R.trajectory, R.traj_mem, R.max_traj,
-                                      R.traj_node + (size_t)sc * R.max_traj, mf, cores, lane, pool_of);
-            if (lane < P.P && cores >= 0) R.mem_free[(size_t)sc * P.P + lane] = mf;
+            const int pj = RQ_POOL(b_rec.meta);
+            const bool mine = have && b_traj >= 0 && b_traj < R.max_traj && P.pool[pj].type == TG_POOL_CPU;
+            const int out = pin_chunk(mine, b_traj, b_mem, RQ_UNITS(b_rec.meta), pj, have, traj_node, node_mem, node_cores, lane, pool_of);
             if (have && lane < out) {
               R.pool_rw[row + base + lane] = (u8)pool_of;
-              b_rec.meta = (b_rec.meta & ~0x3ffu) | (u32)pool_of | ((u32)P.pool[pool_of].slot0 << 4);
+              b_rec.meta = (b_rec.meta & ~(7u << 2)) | ((u32)pool_of << 2);
             }
             __syncwarp();
             if (out < k0 + cnt) { cnt = out - k0; was_gated = true; gated = true; }   // the gate
@@ -652,18 +761,18 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 }
                 const int x = Q.free[--free_slots];
                 __syncwarp();
-                if (lane == b) { Q.q[Q.at(p)] = (unsigned short)x; Q.key[x] = key; replay_store(Q, x, b_rec, base + b); }
+                if (lane == b) { Q.q[Q.at(p)] = (unsigned short)x; Q.key[x] = key; replay_store(Q, x, b_rec, base + b, EXT ? b_last : 0u); }
               } else if (lane == b) { wait[p] = base + b; wkey[p] = key; }
               __syncwarp();
               ++nw;
             }
           } else {
             if (fits) {
-              const int x = Q.free[free_slots - 1 - (lane - k0)];
-              Q.q[Q.at(pos)] = (unsigned short)x;
-              replay_store(Q, x, b_rec, base + lane);
+              int x = Q.at(pos);
+              if (EXT) { const int y = Q.free[free_slots - 1 - (lane - k0)]; Q.q[x] = (unsigned short)y; x = y; }
+              replay_store(Q, x, b_rec, base + lane, EXT ? b_last : 0u);
             } else if (in) wait[pos] = base + lane;
-            free_slots -= min(cnt, max(Q.cap - nw, 0));
+            if (EXT) free_slots -= min(cnt, max(Q.cap - nw, 0));
             nw += cnt;
           }
           next += cnt;
@@ -701,7 +810,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               for (int z = 0; z < 4; ++z) {
                 const int b = b0 + z;
                 const u32 mb = __shfl_sync(TG_FULL, c.y, b);
-                if ((u32)(lane - RQ_SLOT(mb)) <= (u32)RQ_CLASS(mb)) run_dem += RQ_UNITS(mb);
+                if ((charged >> (mb & 31u)) & 1u) run_dem += RQ_UNITS(mb);
                 if (EXT && P.n_side > 0) {
                   const int a0 = __shfl_sync(TG_FULL, k0, b), d0 = __shfl_sync(TG_FULL, u0, b);
                   const int a1 = __shfl_sync(TG_FULL, k1, b), d1 = __shfl_sync(TG_FULL, u1, b);
@@ -729,15 +838,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           bool ok = true;
           int my_end = KR_NEVER;                           // first release among what this lane starts
           // the lane's candidate starts (Eq. 2: completion - arrival = waited so far + execution)
-          auto start = [&](const PoolDev& pd, int j, int k, int a, int units, i64 fin, i64 arr, int node, int off) {
-            const size_t o = row + a;
+          auto start = [&](const PoolDev& pd, int j, int k, int a, int units, i64 fin, i64 arr, const ReplayGrant& G, bool last) {
             const i64 act = fin - arr;
             const int end = max(round_at(R, fin), r + 1);
-            P.o_alloc[o] = units; P.o_node[o] = node; P.o_off[o] = off; P.o_act[o] = act;
-            run.fin[k] = fin; run.end[k] = end; run.idx[k] = a;
+            o_alloc[a] = units; o_node[a] = G.node; o_off[a] = G.off; o_act[a] = act;
+            run.at[k] = G.at; run.pu[k] = rr_pack(pd, j, units, G.wide) | (EXT && last && pd.type == TG_POOL_CPU ? RR_LAST : 0u); run.fin[k] = fin; run.end[k] = end; run.idx[k] = a;
             if (occ) {
               atomicAdd(&occ[(size_t)r * P.P + j], units);
-              if (end < R.max_rounds && (pd.type != TG_POOL_API || pd.window_us == 0)) atomicSub(&occ[(size_t)end * P.P + j], units);
+              if (end < R.max_rounds && pd.window_us == 0) atomicSub(&occ[(size_t)end * P.P + j], units);
             }
             total += act; my_end = min(my_end, end);
           };
@@ -759,9 +867,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               }
             const bool el = (present >> (8 + j)) & 1u;
             const bool cached = EXT && pd.type == TG_POOL_GPU && P.cache_slots > 0;
-            int units_now = 0;                             // what this lane's candidates take
-            if ((m == 1 || (!el && pd.type != TG_POOL_GPU)) && !cached) {
-              // Nothing to choose between candidates: each takes its level (a lone one DPArrange's answer in closed form: the
+            int units_now = 0;                             // core pools: what the candidates take
+            int pair = 0, ra = 1, rb = 1;                  // of two candidates: how many are kept, their levels
+            if (m == 2 && el && n <= 32 && !cached && nr <= KR_PAIR_RUN && nw <= Q.cap && nw - n <= KR_PAIR_WAIT) {
+              const u32 mb = __ballot_sync(TG_FULL, lane < n && RQ_POOL(c0.y) == j);
+              pair = replay_pair(P, pd, Q, run, row, j, __ffs(mb) - 1, 31 - __clz(mb), n, nw, nr, now, Z.slot + slot0, aside_j, (u32*)fast, lane, ra, rb);
+            }
+            if ((m == 1 || pair || (!el && (pd.type != TG_POOL_GPU || n <= 32))) && !cached) {
+              // Nothing left to choose: each candidate takes its level (a lone one DPArrange's answer in closed form: the
               // feasible level of least duration, the smallest among equals) and is placed in queue order.
               int seen = 0;
 #pragma unroll 1
@@ -771,52 +884,79 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                   c = make_uint4(0u, RQ_NOBODY, 1u, 1u); x = -1;
                   if (i0 + lane < n) c = replay_facts(P, Q, wait, row, i0 + lane, x);
                 }
-                const bool mine = i0 + lane < n && RQ_POOL(c.y) == j;
-                const u32 mb = __ballot_sync(TG_FULL, mine);
+                bool mine = i0 + lane < n && RQ_POOL(c.y) == j;
+                u32 mb = __ballot_sync(TG_FULL, mine);
                 if (!mb) continue;
+                if (pair == 1) { mb &= 0u - mb; mine = (mb >> lane) & 1u; }
                 ReplayRec rec; rec.s = rec.p = rec.arr = 0;
                 if (mine) rec = replay_rec(P, Q, row, c, x);
                 int rr = __ffs(c.z);
-                if (m == 1 && el) {
+                if (pair) rr = (mb & below) ? rb : ra;
+                else if (m == 1 && el) {
                   const int b = __ffs(mb) - 1;
                   const u32 mk = __shfl_sync(TG_FULL, c.z, b), cg = __shfl_sync(TG_FULL, c.w, b);
-                  const int g = cg & 0x7f, gang = cg >> 7, rl = lane + 1;
-                  bool fit = (mk >> lane) & 1u;
-                  const int cl = fit && pd.type == TG_POOL_GPU ? level_of(g, gang, rl) : 0;
+                  const int g = cg & 0x7f, gang = (cg >> 7) & 1, rl = lane + 1;
+                  const bool has = (mk >> lane) & 1u;
+                  const int cl = has && pd.type == TG_POOL_GPU ? level_of(g, gang, rl) : 0;
                   const int room = Z.slot[slot0 + cl] - (cl == 0 ? aside_j : 0);
-                  const u32 fits = __ballot_sync(TG_FULL, fit && g * rl <= room);
+                  const u32 fits = __ballot_sync(TG_FULL, has && g * rl <= room);
                   if (lane == b && fits) rr = best_level(rec.p, fits);   // (durations do not grow with the level)
                 }
                 const int units = mine ? (int)(c.w & 0x7f) * rr : 0;
                 const i64 fin = now + duration(rec.s, rec.p, rr);
-                ReplayGrant G; G.node = 0; G.off = -1; G.word = 0; G.dom = 0; G.lo = G.hi = 0; G.wide = false;
+                ReplayGrant G; G.node = 0; G.off = -1; G.at = make_uint4(0u, 0u, 0u, (u32)R.Dtot); G.wide = false;
                 if (pd.type == TG_POOL_API) {
                   // Section 5.1: the offset is what was in use before
                   const int incl = warp_incl_scan32(units, lane);
                   G.off = pd.capacity - Z.slot[slot0] + incl - units;
                   const int all = __shfl_sync(TG_FULL, incl, 31);
                   if (lane == 0) Z.slot[slot0] -= all;
-                } else
+                } else if (pd.type == TG_POOL_GPU) {       // largest chunks first, then queue position
+                  const int g = (int)(c.w & 0x7fu), gang = (int)(c.w >> 7) & 1, lz = ilog2(gang ? g * rr : g), nreq = gang ? 1 : rr;
 #pragma unroll 1
-                  for (u32 todo = mb; todo; todo &= todo - 1) {
-                    const int b = __ffs(todo) - 1;
-                    const int k = __shfl_sync(TG_FULL, units, b), id = __shfl_sync(TG_FULL, (int)c.x, b);
-                    ReplayGrant g1;
-                    if (pd.type == TG_POOL_CPU)
-                      g1 = replay_take_cores(pd.group, R.n_dom[j], R.wpd[j], Z.cores + 2 * R.word0[j], Z.dfree + R.dom0[j], ow, k, id, lane);
-                    else {
-                      const int cg = __shfl_sync(TG_FULL, (int)c.w, b), rb = __shfl_sync(TG_FULL, rr, b), g = cg & 0x7f, gang = cg >> 7;
-                      g1 = replay_take_gpus(pd, Z.nm + pd.node0, ow, ilog2(gang ? g * rb : g), gang ? 1 : rb, id, lane);
-                    }
+                  for (u32 todo = mb; todo;) {
+                    int b = __ffs(todo) - 1;
+                    if (todo & (todo - 1)) b = 31 - (int)(__reduce_max_sync(TG_FULL, (todo >> lane) & 1u ? ((u32)lz << 5) | (u32)(31 - lane) : 0u) & 31u);
+                    todo &= ~(1u << b);
+                    const ReplayGrant g1 = replay_take_gpus(pd.group, pd.n_nodes, Z.words + R.word0[j], Z.node_of, ow, R.word0[j], R.Dtot,
+                                                            __shfl_sync(TG_FULL, lz, b), __shfl_sync(TG_FULL, nreq, b), __shfl_sync(TG_FULL, (int)c.x, b), lane);
                     if (lane == b) G = g1;
                   }
-                if (mine) {
-                  const int k = nr + __popc(mb & below);
-                  run.at[k] = make_uint4(G.lo, G.hi, (u32)G.word, (u32)G.dom); run.pu[k] = rr_pack(pd, j, units, G.wide);
-                  if (x >= 0) Q.c[x].y = c.y | RQ_STARTED;
-                  start(pd, j, k, (int)c.x, units, fin, rec.arr, G.node, G.off);
+                } else {
+                  // lane d: free cores and masks of domain d
+                  const int n_dom = R.n_dom[j];
+                  u32* words = Z.words + R.word0[j]; int* dfree = Z.dfree + R.dom0[j];
+                  const bool direct = R.wpd[j] == 1 && n_dom <= 32;
+                  int f = -1; u32 lo = 0, hi = 0;
+                  auto load = [&]() { if (direct && lane < n_dom) { f = dfree[lane]; lo = words[2 * lane]; hi = words[2 * lane + 1]; } };
+                  auto save = [&]() { if (direct && lane < n_dom) { dfree[lane] = f; words[2 * lane] = lo; words[2 * lane + 1] = hi; } __syncwarp(); };
+                  load();
+#pragma unroll 1
+                  for (u32 todo = mb; todo; todo &= todo - 1) {
+                    const int b = __ffs(todo) - 1, k = __shfl_sync(TG_FULL, units, b);
+                    const u32 mn = __reduce_min_sync(TG_FULL, f >= k ? ((u32)f << 5) | (u32)lane : 0xffffffffu);
+                    units_now += k;
+                    if (mn != 0xffffffffu) {               // fewest free cores that still fit, lowest domain, lowest cores
+                      const int d = (int)(mn & 31u);
+                      u32 tlo, thi;
+                      lowest_bits(__shfl_sync(TG_FULL, lo, d), __shfl_sync(TG_FULL, hi, d), k, lane, tlo, thi);
+                      if (lane == d) { f -= k; lo &= ~tlo; hi &= ~thi; }
+                      if (lane == b) { G.node = d; G.at = make_uint4(tlo, thi, (u32)(R.word0[j] + 2 * d), (u32)(R.dom0[j] + d)); }
+                    } else {
+                      save();
+                      const ReplayGrant g1 = replay_take_cores(pd.group, n_dom, R.wpd[j], words, dfree, ow, R.word0[j], R.dom0[j],
+                                                               k, __shfl_sync(TG_FULL, (int)c.x, b), lane);
+                      if (lane == b) G = g1;
+                      load();
+                    }
+                  }
+                  save();
+                  if (G.off < 0) G.off = G.node * pd.group + (G.at.x ? __ffs(G.at.x) - 1 : 31 + __ffs(G.at.y));
                 }
-                units_now += units;
+                if (mine) {
+                  if (x >= 0) Q.c[x].y = c.y | RQ_STARTED;
+                  start(pd, j, nr + __popc(mb & below), (int)c.x, units, fin, rec.arr, G, c.w & 256u);
+                }
                 nr += __popc(mb); seen += __popc(mb); selected += __popc(mb);
                 __syncwarp();
               }
@@ -825,27 +965,50 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               slab.base = P.slabs + (u64)blockIdx.x * P.slab_bytes; slab.cap = P.slab_bytes; slab.used = 0;
               slab.fbase = fast; slab.fcap = KR_FAST_BYTES; slab.fused = 0;
               CandArrays C; int keep = 0;
-              ok = replay_select<EXT>(P, Q, run, wait, sc, j, n, nw, nr, m, now, Z.slot[slot0] - aside_j, Z.slot[(slot0 + 1) & 31],
-                                      Z.slot[(slot0 + 2) & 31], Z.slot[(slot0 + 3) & 31], slab, C, keep, lane);
+              ok = replay_select(P, Q, run, wait, row, j, n, nw, nr, m, now, Z.slot[slot0] - aside_j, Z.slot[(slot0 + 1) & 31],
+                                 Z.slot[(slot0 + 2) & 31], Z.slot[(slot0 + 3) & 31], slab, C, keep, lane);
               if (!ok) break;
               const u8* missed = nullptr;                  // candidates whose chunk did not cache their service
               if (cached) {
+                u8* nm = (u8*)slab.take_fast(pd.n_nodes);  // as busy masks
+                if (!nm) { ok = false; break; }
+#pragma unroll 1
+                for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = (u8)~Z.words[R.word0[j] + v];
+                __syncwarp();
                 const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
-                place_gpu_cache(pd, Z.nm + pd.node0, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel,
+                place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel,
                                 P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, now, lane, ow);
+#pragma unroll 1
+                for (int v = lane; v < pd.n_nodes; v += 32) Z.words[R.word0[j] + v] = ~(u32)nm[v] & ((1u << pd.group) - 1u);
                 missed = C.rsel;
               } else if (pd.type == TG_POOL_GPU) {
-                place_gpu(pd, Z.nm + pd.node0, keep, C.cg, C.rkeep, C.pnode, C.poff, lane, ow, C.cidx);
+                // Section 5.3: by size, largest first, then queue position
+#pragma unroll 1
+                for (int lz = 3; lz >= 0; --lz)
+#pragma unroll 1
+                  for (int i0 = 0; i0 < keep; i0 += 32) {
+                    const int i = i0 + lane;
+                    int nreq = 0;
+                    if (i < keep) {
+                      const int g = C.cg[i] & 0x7f, ri = C.rkeep[i];
+                      nreq = C.cg[i] >> 7 ? (g * ri == 1 << lz ? 1 : 0) : (g == 1 << lz ? ri : 0);
+                    }
+#pragma unroll 1
+                    for (u32 todo = __ballot_sync(TG_FULL, nreq > 0); todo; todo &= todo - 1) {
+                      const int b = __ffs(todo) - 1;
+                      const ReplayGrant G = replay_take_gpus(pd.group, pd.n_nodes, Z.words + R.word0[j], Z.node_of, ow, R.word0[j], R.Dtot, lz,
+                                                             __shfl_sync(TG_FULL, nreq, b), C.cidx[i0 + b], lane);
+                      if (lane == b) { C.pnode[i] = G.node; C.poff[i] = G.off; }
+                    }
+                  }
               } else if (pd.type == TG_POOL_CPU) {
 #pragma unroll 1
                 for (int i = 0; i < keep; ++i) {
                   const int units = (C.cg[i] & 0x7f) * C.rkeep[i];
-                  const ReplayGrant G = replay_take_cores(pd.group, R.n_dom[j], R.wpd[j], Z.cores + 2 * R.word0[j], Z.dfree + R.dom0[j], ow,
-                                                          units, C.cidx[i], lane);
-                  if (lane == 0) {
-                    C.pnode[i] = G.node; C.poff[i] = G.off;
-                    run.at[nr + i] = make_uint4(G.lo, G.hi, (u32)G.word, (u32)G.dom); run.pu[nr + i] = rr_pack(pd, j, units, G.wide);
-                  }
+                  const ReplayGrant G = replay_take_cores(pd.group, R.n_dom[j], R.wpd[j], Z.words + R.word0[j], Z.dfree + R.dom0[j], ow,
+                                                          R.word0[j], R.dom0[j], units, C.cidx[i], lane);
+                  if (lane == 0) { C.pnode[i] = G.node; C.poff[i] = G.off; run.at[nr + i] = G.at; C.rsel[i] = G.wide ? 1 : 0; }
+                  units_now += units;
                 }
               } else if (lane == 0) {
                 int used = pd.capacity - Z.slot[slot0];
@@ -856,15 +1019,17 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               __syncwarp();
 #pragma unroll 1
               for (int i = lane; i < keep; i += 32) {
-                const int g = C.cg[i] & 0x7f, gang = C.cg[i] >> 7, rr = C.rkeep[i], units = g * rr, a = C.cidx[i];
+                const int g = C.cg[i] & 0x7f, rr = C.rkeep[i], units = g * rr, a = C.cidx[i];
                 i64 fin = now + duration(C.cs[i], C.cp[i], rr);
                 if (EXT && missed && missed[i] && P.a_restore) fin += clamp_param(P.a_restore[row + a]);   // restoration precedes execution
-                if (pd.type != TG_POOL_CPU) {
-                  run.at[nr + i] = make_uint4(((1u << (units & 31)) - 1u) << (C.poff[i] & 31), 0u, (u32)C.pnode[i], 0u);
-                  run.pu[nr + i] = rr_pack(pd, j, units, pd.type == TG_POOL_GPU && !gang && rr > 1);
+                ReplayGrant G;
+                G.node = C.pnode[i]; G.off = C.poff[i]; G.wide = false; G.at = make_uint4(0u, 0u, 0u, (u32)R.Dtot);
+                if (pd.type == TG_POOL_CPU) { G.at = run.at[nr + i]; G.wide = C.rsel[i] != 0; }
+                else if (pd.type == TG_POOL_GPU) {
+                  G.wide = !(C.cg[i] >> 7) && rr > 1;      // chunks of replicas lie anywhere
+                  G.at.x = G.wide ? 0u : ((1u << units) - 1u) << G.off; G.at.z = (u32)(R.word0[j] + G.node);
                 }
-                start(pd, j, nr + i, a, units, fin, P.a_arrival ? P.a_arrival[row + a] : 0, C.pnode[i], C.poff[i]);
-                units_now += units;
+                start(pd, j, nr + i, a, units, fin, P.a_arrival ? P.a_arrival[row + a] : 0, G, EXT && R.trajectory && R.traj_last && R.traj_last[row + a]);
               }
               // the kept ones are the pool's first `keep` in queue order
               int seen = 0;
@@ -880,11 +1045,8 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               nr += keep; selected += keep;
               __syncwarp();
             }
-            if (pd.type == TG_POOL_GPU) replay_gpu_slots(pd, Z.nm, Z.slot, lane);
-            else if (pd.type == TG_POOL_CPU) {
-              const int all = warp_sum32(units_now);
-              if (lane == 0) Z.slot[slot0] -= all;
-            }
+            if (pd.type == TG_POOL_GPU) replay_gpu_slots(pd, Z.words + R.word0[j], Z.node_of, Z.slot, lane);
+            else if (pd.type == TG_POOL_CPU && lane == 0) Z.slot[slot0] -= units_now;
             __syncwarp();
           }
           if (!ok) { status = TG_ST_WORKSPACE; break; }
@@ -912,20 +1074,28 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
           if (started == n) blocked_pool = stop_pool;
           // the started actions leave the queue
           if (started && nw <= Q.cap) {
-            int to_end = n;                                // the ones that stay move up behind the others, last first
+            if (EXT || started < n) {
+              int to_end = n;                              // the ones that stay move up behind the others, last first
 #pragma unroll 1
-            for (int i0 = (n - 1) & ~31; i0 >= 0; i0 -= 32) {
-              const int i = i0 + lane, x = i < n ? (int)Q.q[Q.at(i)] : 0;
-              const bool gone = i < n && (started == n || (Q.c[x].y & RQ_STARTED));
-              const u32 gb = __ballot_sync(TG_FULL, gone);
-              if (gone) Q.free[free_slots + __popc(gb & below)] = (unsigned short)x;
-              free_slots += __popc(gb);
-              if (started < n) {
-                const u32 sb = __ballot_sync(TG_FULL, i < n && !gone);
-                __syncwarp();
-                if (i < n && !gone) Q.q[Q.at(to_end - __popc(sb >> lane))] = (unsigned short)x;
-                to_end -= __popc(sb);
-                __syncwarp();
+              for (int i0 = (n - 1) & ~31; i0 >= 0; i0 -= 32) {
+                const int i = i0 + lane, x = i < n ? Q.slot(i) : 0;
+                const bool gone = i < n && (started == n || (Q.c[x].y & RQ_STARTED));
+                const u32 gb = __ballot_sync(TG_FULL, gone);
+                if (EXT) {
+                  if (gone) Q.free[free_slots + __popc(gb & below)] = (unsigned short)x;
+                  free_slots += __popc(gb);
+                }
+                if (started < n) {
+                  const bool stay = i < n && !gone;
+                  const u32 sb = __ballot_sync(TG_FULL, stay);
+                  const int to = Q.at(stay ? to_end - __popc(sb >> lane) : 0);
+                  uint4 sp, ta, c;
+                  if (!EXT && stay) { sp = Q.sp[x]; ta = Q.ta[x]; c = Q.c[x]; }
+                  __syncwarp();
+                  if (stay) { if (EXT) Q.q[to] = (unsigned short)x; else { Q.sp[to] = sp; Q.ta[to] = ta; Q.c[to] = c; } }
+                  to_end -= __popc(sb);
+                  __syncwarp();
+                }
               }
             }
             Q.head = Q.at(started < Q.cap ? started : 0);
@@ -937,24 +1107,29 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
             for (int i0 = 0; i0 < nw; i0 += 32) {
               const int i = i0 + lane;
               bool stay = false; int x = 0, a = 0; u64 kk = 0;
-              if (i < min(nw, Q.cap)) { x = Q.q[Q.at(i)]; stay = !(Q.c[x].y & RQ_STARTED); }
-              else if (i < nw) { a = wait[i]; stay = P.o_act[row + a] < 0; if (EXT && R.policy) kk = wkey[i]; }
+              if (i < min(nw, Q.cap)) { x = Q.slot(i); stay = !(Q.c[x].y & RQ_STARTED); }
+              else if (i < nw) { a = wait[i]; stay = o_act[a] < 0; if (EXT && R.policy) kk = wkey[i]; }
               const u32 b = __ballot_sync(TG_FULL, stay), gone = __ballot_sync(TG_FULL, i < min(nw, Q.cap) && !stay);
               const int to = kw + __popc(b & below);
+              uint4 sp, ta, c;
+              if (!EXT && stay && i < Q.cap) { sp = Q.sp[x]; ta = Q.ta[x]; c = Q.c[x]; }
               __syncwarp();
-              if (stay && i < Q.cap) Q.q[Q.at(to)] = (unsigned short)x;
-              else if (stay && to >= Q.cap) { wait[to] = a; if (EXT && R.policy) wkey[to] = kk; }
-              if ((gone >> lane) & 1u) Q.free[free_slots + __popc(gone & below)] = (unsigned short)x;
-              free_slots += __popc(gone);
+              if (stay && i < Q.cap) {
+                const int y = Q.at(to);
+                if (EXT) Q.q[y] = (unsigned short)x; else { Q.sp[y] = sp; Q.ta[y] = ta; Q.c[y] = c; }
+              } else if (stay && to >= Q.cap) { wait[to] = a; if (EXT && R.policy) wkey[to] = kk; }
+              if (EXT) {
+                if ((gone >> lane) & 1u) Q.free[free_slots + __popc(gone & below)] = (unsigned short)x;
+                free_slots += __popc(gone);
+              }
               __syncwarp();
               const u32 mv = __ballot_sync(TG_FULL, stay && i >= Q.cap && to < Q.cap);
               if ((mv >> lane) & 1u) {                      // a record moves up into shared memory
-                const int y = Q.free[free_slots - 1 - __popc(mv & below)];
-                Q.q[Q.at(to)] = (unsigned short)y;
-                replay_store(Q, y, replay_load(P, row, a), a);
-                if (EXT) Q.key[y] = kk;
+                int y = Q.at(to);
+                if (EXT) { const int z = Q.free[free_slots - 1 - __popc(mv & below)]; Q.q[y] = (unsigned short)z; y = z; Q.key[y] = kk; }
+                replay_store(Q, y, replay_load(P, row, a), a, EXT && R.traj_last && R.traj_last[row + a] ? 256u : 0u);
               }
-              free_slots -= __popc(mv);
+              if (EXT) free_slots -= __popc(mv);
               __syncwarp();
               kw += __popc(b);
             }
@@ -997,6 +1172,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
       }
       rounds = drained ? r : R.max_rounds;
       if (!drained && r < R.max_rounds) rounds = r;
+      if (EXT && R.trajectory && lane < P.P) R.mem_free[(size_t)sc * P.P + lane] = node_mem;
       total = warp_sum64(total);
       if (lane == 0) { P.o_total[sc] = total; P.o_nsel[sc] = selected; P.o_status[sc] = status; }
     } else if (lane == 0) { P.o_total[sc] = 0; P.o_nsel[sc] = 0; P.o_status[sc] = status; }

@@ -527,17 +527,18 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     for (int j = 0; j < P.P; ++j) {
       R.unit0[j] = u; R.dom0[j] = d; R.word0[j] = w;
       if (P.pool[j].type != TG_POOL_API) u += P.pool[j].capacity;
+      if (P.pool[j].type == TG_POOL_GPU) w += P.pool[j].n_nodes;
       if (P.pool[j].type != TG_POOL_CPU) continue;
       R.n_dom[j] = P.pool[j].capacity / P.pool[j].group; R.wpd[j] = (P.pool[j].group + 63) / 64;
-      d += R.n_dom[j]; w += R.n_dom[j] * R.wpd[j];
+      d += R.n_dom[j]; w += 2 * R.n_dom[j] * R.wpd[j];
     }
-    R.U = u ? u : 1; R.Dtot = d ? d : 1; R.W = w ? w : 1;
+    R.U = u ? u : 1; R.Dtot = d; R.W = w;
     R.round_us = desc->round_us > 0 ? desc->round_us : 1; R.max_rounds = desc->max_rounds;
     R.round_recip = R.round_us > 1 && R.round_us < (1 << 22) ? ~0ull / (u64)R.round_us + 1ull : 0;
     bad |= cudaMalloc((void**)&R.wait, SN * sizeof(int)) != cudaSuccess;
     // what a block (one scenario at a time) keeps in shared memory: live state, running actions, waiting records
     {
-      const size_t state = replay_state_bytes(R, node0);
+      const size_t state = replay_state_bytes(R);
       R.state_bytes = state <= KR_STATE_MAX ? (int)state : 0;
       size_t running = 0;                                  // a running action holds a unit at least, quota calls aside
       for (int j = 0; j < P.P; ++j) running += P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0 ? (size_t)P.N : (size_t)P.pool[j].capacity;
@@ -564,10 +565,9 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     }
     bad |= cudaMalloc((void**)&R.rounds_used, (size_t)P.S * sizeof(int)) != cudaSuccess;
     if (R.state_bytes == 0) {
-      bad |= cudaMalloc((void**)&R.cores, (size_t)P.S * R.W * 8) != cudaSuccess;
-      bad |= cudaMalloc((void**)&R.dfree, (size_t)P.S * R.Dtot * sizeof(int)) != cudaSuccess;
+      bad |= cudaMalloc((void**)&R.words, (size_t)P.S * (R.W + 2) * sizeof(u32)) != cudaSuccess;
+      bad |= cudaMalloc((void**)&R.dfree, (size_t)P.S * (R.Dtot + 1) * sizeof(int)) != cudaSuccess;
       bad |= cudaMalloc((void**)&R.owner, (size_t)P.S * R.U * sizeof(int)) != cudaSuccess;
-      bad |= cudaMalloc((void**)&R.nm, (size_t)P.S * ((node0 + 4) & ~3)) != cudaSuccess;
     }
   }
   {
@@ -639,8 +639,6 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
   *out = r;
   return TANGRAM_OK;
@@ -702,7 +700,7 @@ extern "C" void tangram_round_destroy(tangram_round* r) {
   cudaFree(r->d_order); cudaFree(r->d_tmin); cudaFree(r->d_meta); cudaFree(r->d_slabs);
   cudaFree(r->d_ok_table); cudaFree(r->d_arena); cudaFree(r->d_arena_top); cudaFree(r->d_stage); cudaFree(r->hst); cudaFree(r->d_side_bad); cudaFree(r->d_side_res); cudaFree(r->d_perm); cudaFree(r->d_wkey);
   cudaFree(r->R.wait); cudaFree(r->R.run_at); cudaFree(r->R.run_fin); cudaFree(r->R.run_end); cudaFree(r->R.run_pu); cudaFree(r->R.run_idx);
-  cudaFree(r->R.cores); cudaFree(r->R.dfree); cudaFree(r->R.owner); cudaFree(r->R.nm); cudaFree(r->R.rounds_used);
+  cudaFree(r->R.words); cudaFree(r->R.dfree); cudaFree(r->R.owner); cudaFree(r->R.rounds_used);
   if (r->io_in) cudaStreamDestroy(r->io_in);
   if (r->io_comp) cudaStreamDestroy(r->io_comp);
   if (r->io_out) cudaStreamDestroy(r->io_out);
@@ -962,8 +960,11 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
     R.max_traj = pin->max_trajectories; R.traj_node = pin->traj_node; R.mem_free = (i64*)pin->node_mem_free;
     R.pool_rw = pin->pool_out;
   }
-  if (policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0)) k_replay<true><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
-  else k_replay<false><<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
+  // (the attribute is set here, so that a round that never replays does not load these kernels)
+  const bool ext = policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0);
+  void (*kern)(Params, ReplayWs) = R.rcap == 0 || R.state_bytes == 0 ? k_replay<true, false> : ext ? k_replay<true, true> : k_replay<false, true>;
+  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, r->replay_smem));
+  kern<<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   if (R.occupancy) { k_occupancy<<<P.S, 256, 0, st>>>(P.P, R.max_rounds, R.rounds_used, P.o_status, R.occupancy); r->launches += 1; }
   if (ev) CK(cudaEventRecord(ev[1], st));
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));            // k_round starts from counters at zero
