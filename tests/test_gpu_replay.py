@@ -112,3 +112,33 @@ def test_long_running_sets_match_oracle(oracle):
     g = gpu_replay(pools, a, 2, 10_000, 600)
     assert_same(o, g)
     assert o["occupancy"][:, :, 0].max() > 448 and np.all(o["n_selected"] == N)
+
+
+STATES = {
+    # domains of several mask words, more nodes than lanes
+    "wide": ((Pool(POOL_CPU, 900, 300), Pool(POOL_GPU, 320, 8)), 10_000, 1.0),
+    # one core per domain: every grant of more spans domains, more domains than lanes
+    "spanning": ((Pool(POOL_CPU, 40, 1), Pool(POOL_GPU, 6, 2), Pool(POOL_CPU, 33, 11)), 10_000, 1.0),
+    # live state and running actions in global memory; a window shorter than a round, a concurrency limit
+    "global": ((Pool(POOL_CPU, 6000, 60), Pool(POOL_API, 3, 0, 4_000), Pool(POOL_API, 4, 0, 0), Pool(POOL_GPU, 16, 4)), 10_000, 1.0),
+    # times beyond 32 bits: a step between two candidates that has to be decided exactly
+    "long": ((Pool(POOL_CPU, 6, 3), Pool(POOL_GPU, 8, 8)), 4_000_000, 2e4),
+    # round lengths around the ones whose reciprocal is used
+    "round": ((Pool(POOL_CPU, 24, 8), Pool(POOL_GPU, 8, 8)), (1 << 22) - 1, 20.0),
+    "rounds": ((Pool(POOL_CPU, 24, 8), Pool(POOL_GPU, 8, 8)), 1 << 22, 20.0),
+}
+
+
+@pytest.mark.parametrize("name", STATES)
+def test_replay_state_layouts_match_oracle(oracle, name):
+    pools, round_us, scale = STATES[name]
+    w, a = random_round(sum(map(ord, name)), 12, 150, pools, small_durations=0.1, busy_fraction=0.2, max_mult=6)
+    a["s_us"] = (a["s_us"] * scale).astype(np.int64)
+    a["p_us"] = (a["p_us"] * scale).astype(np.int64)
+    a["level_mask"] |= 1                            # (no head of the queue that never fits)
+    rng = np.random.default_rng(len(name))
+    a["arrival_us"] = np.cumsum(rng.integers(0, int(6000 * scale), a["pool"].shape), axis=1).astype(np.int64)
+    for max_rounds in (3000, 60):                   # (60: cut off with actions waiting and running)
+        o = oracle.replay_trace(pools, a, depth=2, round_us=round_us, max_rounds=max_rounds)
+        assert_same(o, gpu_replay(pools, a, 2, round_us, max_rounds))
+    assert o["n_selected"].sum() > 0
