@@ -284,36 +284,36 @@ __device__ __forceinline__ bool eviction_cannot_pay(const PoolTask& T, int q, co
   return duration(T.cs[q], T.cp[q], kept[q]) <= rest_first(T, q);
 }
 
-// ---- heaps of up to 256 times: 32 NS of them in lane registers, in no order -----------------------
-// One pop: every lane's own minimum, one warp minimum over those, and the (highest) lane that holds it puts the new
-// time in its place.  No order is kept, so nothing moves; the chain is local minimum, warp minimum, vote, select: 66
-// cycles per pop on B200 with two heaps of three registers side by side.  (Not waiting for the vote and mending
-// ties one step later was slower, 90: the branch costs more than the vote.)
+// ---- heaps of up to 256 times: 32 NS of them in lane registers -----------------------------------
+// Every lane keeps its own times in ascending order, the lanes among each other are in none.  One pop: a warp minimum over
+// the lanes' first times, and the (highest) lane that holds it sorts the new time in among its own; the chain is warp
+// minimum, vote, insertion.  (Not waiting for the vote and mending ties one step later was slower: the branch costs
+// more than the vote.  Without an order every step looks for a lane's minimum and its place: 16384 x 4096 1936 us a call
+// against 1780, 64 nodes of 8 GPUs, 1024 x 2048, 762 against 589; the insertion in a branch 866.)
 template <int NS>
-__device__ __forceinline__ u32 ev_local_min(const u32 (&key)[NS]) {
-  u32 lm = key[0];
+__device__ __forceinline__ void ev_order(u32 (&key)[NS]) {
 #pragma unroll
-  for (int j = 1; j < NS; ++j) lm = min(lm, key[j]);
-  return lm;
+  for (int i = 1; i < NS; ++i)
+#pragma unroll
+    for (int j = NS - 1; j >= i; --j) { const u32 x = key[j - 1], y = key[j]; key[j - 1] = min(x, y); key[j] = max(x, y); }
 }
-// above: the lanes above this one.  Which register holds the minimum is found while the vote is on its way.
+// above: the lanes above this one
 template <int NS>
 __device__ __forceinline__ void ev_replace(u32 (&key)[NS], u32 mn, u32 holders, u32 d, u32 above) {
-  const u32 c = min(mn, EV_SAT - d) + d;                 // d <= EV_SAT
-  bool here[NS], seen = false;
+  // (a lane whose time stays sorts that one in again: no branch; every place on its own: no chain through the registers)
+  const u32 c = key[0] == mn && (holders & above) == 0u ? min(mn, EV_SAT - d) + d : key[0];      // d <= EV_SAT
 #pragma unroll
-  for (int j = 0; j < NS; ++j) { here[j] = key[j] == mn && !seen; seen |= key[j] == mn; }
-  const bool own = (holders & above) == 0u;
-#pragma unroll
-  for (int j = 0; j < NS; ++j) if (here[j] && own) key[j] = c;
+  for (int j = 0; j < NS; ++j) {
+    const u32 x = j == 0 ? c : max(c, key[j]);
+    key[j] = j + 1 < NS ? min(x, key[j + 1]) : x;
+  }
 }
 
 template <int NS>
 __device__ __forceinline__ void ev_step(u32 (&a)[NS], u32 (&b)[NS], u32 da, u32 db, u32 above, u32& ma, u32& mb) {
-  const u32 lb = ev_local_min(b), la = ev_local_min(a);
-  mb = __reduce_min_sync(TG_FULL, lb);
-  ma = __reduce_min_sync(TG_FULL, la);
-  const u32 hb = __ballot_sync(TG_FULL, lb == mb), ha = __ballot_sync(TG_FULL, la == ma);
+  mb = __reduce_min_sync(TG_FULL, b[0]);
+  ma = __reduce_min_sync(TG_FULL, a[0]);
+  const u32 hb = __ballot_sync(TG_FULL, b[0] == mb), ha = __ballot_sync(TG_FULL, a[0] == ma);
   ev_replace(b, mb, hb, db, above);
   ev_replace(a, ma, ha, da, above);
 }
@@ -361,11 +361,9 @@ __device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, i
   const EvShared dur = {wk + NS * 256u};
   const u32 above = lane == 31 ? 0u : TG_FULL << (lane + 1);
   u32 last_a = 0, last_b;
-  {                                                      // the evicted candidate
-    const u32 lb = ev_local_min(b);
-    last_b = __reduce_min_sync(TG_FULL, lb);
-    ev_replace(b, last_b, __ballot_sync(TG_FULL, lb == last_b), evicted, above);
-  }
+  ev_order(a); ev_order(b);
+  last_b = __reduce_min_sync(TG_FULL, b[0]);             // the evicted candidate
+  ev_replace(b, last_b, __ballot_sync(TG_FULL, b[0] == last_b), evicted, above);
   diff += (i64)last_b;
   int wait = 0;                                          // blocks until the heaps are compared again
 #pragma unroll 1
