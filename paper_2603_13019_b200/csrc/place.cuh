@@ -26,6 +26,7 @@ __device__ __forceinline__ int find_block(u32 busy, int bl, int group) {
   return -1;
 }
 
+// One request after the other: where the list of place_gpu_lists finds no room.
 // nm: node busy masks of the pool (updated).  keep candidates, multiplicities r[].
 __device__ void place_gpu(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r, int* pnode, int* poff, int lane) {
   const int top = ilog2(pd.group);
@@ -193,73 +194,100 @@ __device__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* c
   }
 }
 
-// ---- register-resident fast paths of a single round (fresh CPU pool, at most 128 domains /
-// ---- GPU nodes): the state lives in lane registers, the arg-min is one redux, and every lane
-// ---- keeps the result of "its" candidate of a block of 32 for a coalesced write.
+// ---- fast paths of a single round: GPU requests size by size, core pools of at most 128 domains with their
+// ---- state in lane registers (the arg-min is one redux, every lane keeps the result of "its" candidate of a block of 32).
 
-// Same placement rule as place_gpu; requires pd.n_nodes <= 128.  busy_row: the pool's node masks before the round
-// (may be null).  Lane k and register s hold node 32 s + k; lv[l][s] has bit k set where that node has a maximal
-// free block of 2^l GPUs, the same in every lane, so that the lowest node of a level is one bit scan.
-template <int NS>
-__device__ __forceinline__ void place_gpu_masks(const PoolDev& pd, const u8* busy_row, int keep, const u8* cg, const u8* r,
-                                                int* pnode, int* poff, int lane) {
-  const int top = ilog2(pd.group), n_nodes = pd.n_nodes;
+// Same placement rule as place_gpu, all requests of one size at once.  While requests of size z are served, a block of
+// level L is only touched once every smaller sufficient block is used up, and then from its low end on; so the places that
+// are taken, in the order in which they are taken, are the free z-aligned places by (level of their block, node, start),
+// and the k-th request gets the k-th of them.  First every candidate gets the rank of its first request among those of its
+// size (pnode / poff hold size and rank meanwhile), then, size by size from the largest down, every node finds the ranks of
+// its places by a scan over the nodes and lists the ones that are taken, then the candidates look theirs up.
+// ONE: at most 32 nodes, their masks stay in registers; else in nm.  list: room for all requests (see gpu_requests).
+// One request after the other, with the nodes' levels as bit masks in registers, took about 80 instructions each, 18 % of the
+// selection kernel's cycles at 16384 x 4096: 1780 us a call against 1692, 4096 x 1024 279 against 252.
+template <bool ONE>
+__device__ __forceinline__ void place_gpu_lists(const PoolDev& pd, const u8* busy_row, u8* nm, u32* list, const int R[4], int keep, int* pnode, int* poff,
+                                                int lane) {
+  const int n_nodes = pd.n_nodes;
   const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
-  u32 nm[NS], lv[4][NS];
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const int v = lane + 32 * s;
-    nm[s] = v < n_nodes ? ((busy_row ? busy_row[v] : 0u) | pad) : 0xffu;
-    const u32 lev = node_levels(nm[s]);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) lv[l][s] = __ballot_sync(TG_FULL, (lev >> l) & 1u);
-  }
+  u32 reg = 0xffu;
+  if (ONE) { if (lane < n_nodes) reg = (busy_row ? busy_row[lane] : 0u) | pad; }
+  else
 #pragma unroll 1
-  for (int lz = top; lz >= 0; --lz) {
-    const int z = 1 << lz;
+    for (int v = lane; v < n_nodes; v += 32) nm[v] = (u8)((busy_row ? busy_row[v] : 0u) | pad);
+  const int at[4] = {R[3] + R[2] + R[1], R[3] + R[2], R[3], 0};          // where a size's part of the list begins
 #pragma unroll 1
-    for (int i0 = 0; i0 < keep; i0 += 32) {
-      const int i = i0 + lane;
-      int nreq = 0;
-      if (i < keep) {
-        const int g = cg[i] & 0x7f, gang = cg[i] >> 7, ri = r[i];
-        nreq = gang ? (g * ri == z ? 1 : 0) : (g == z ? ri : 0);
-      }
-      int myn = -1, myo = -1;
-      u32 bm = __ballot_sync(TG_FULL, nreq > 0);
+  for (int lz = 3; lz >= 0; --lz) {
+    const int want = pick4(R, lz);
+    u32* const mine = list + pick4(at, lz);
+    const u32 zm = (1u << (1 << lz)) - 1u;
+    int done = 0;                                        // places listed so far
 #pragma unroll 1
-      while (bm) {
-        const int b = __ffs(bm) - 1; bm &= bm - 1;
-        const int cnt = __shfl_sync(TG_FULL, nreq, b);
+    for (int L = lz; L < 4 && done < want; ++L)
 #pragma unroll 1
-        for (int rep = 0; rep < cnt; ++rep) {
-          // smallest sufficient block level, lowest node
-          int bl = -1, s = 0; u32 m = 0;
+      for (int v0 = 0; v0 < n_nodes && done < want; v0 += 32) {
+        const int v = v0 + lane;
+        u32 busy = ONE ? reg : (v < n_nodes ? nm[v] : 0xffu);
+        const NodeBlocks nb = node_blocks(busy);
+        u32 s = L == 0 ? nb.s1 : (L == 1 ? nb.s2 : (L == 2 ? nb.s4 : nb.s8));
+        if (!__any_sync(TG_FULL, s != 0u)) continue;
+        const int cnt = __popc(s) << (L - lz);
+        int incl = cnt;
 #pragma unroll
-          for (int l = 3; l >= 0; --l)
-#pragma unroll
-            for (int q = NS - 1; q >= 0; --q) if (l >= lz && lv[l][q]) { bl = l; s = q; m = lv[l][q]; }
-          if (bl < 0) continue;                         // cannot happen: the selection fits
-          const int k = __ffs(m) - 1;
-          u32 busy = 0;
-#pragma unroll
-          for (int q = 0; q < NS; ++q) if (q == s) busy = nm[q];
-          busy = __shfl_sync(TG_FULL, busy, k);
-          const int start = node_block_start(busy, bl);
-          busy |= ((1u << z) - 1u) << start;
-          const u32 lev = node_levels(busy), bit = 1u << k;
-#pragma unroll
-          for (int q = 0; q < NS; ++q)
-            if (q == s) {
-              if (lane == k) nm[q] = busy;
-#pragma unroll
-              for (int l = 0; l < 4; ++l) lv[l][q] = ((lev >> l) & 1u) ? lv[l][q] | bit : lv[l][q] & ~bit;
-            }
-          if (rep == 0 && lane == b) { myn = 32 * s + k; myo = start; }
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(TG_FULL, incl, o); if (lane >= o) incl += y; }
+        int k = done + incl - cnt;                       // rank of the node's first place
+        done += __shfl_sync(TG_FULL, incl, 31);
+        const int per = 1 << (L - lz);
+#pragma unroll 1
+        for (; s && k < want; s &= s - 1u) {
+          const int st = __ffs(s) - 1;
+#pragma unroll 1
+          for (int x = 0; x < per && k < want; ++x, ++k) {
+            const int p = st + (x << lz);
+            mine[k] = ((u32)v << 3) | (u32)p;
+            busy |= zm << p;
+          }
         }
+        if (ONE) reg = busy; else if (v < n_nodes) nm[v] = (u8)busy;
       }
-      if (i < keep && myn >= 0) { pnode[i] = myn; poff[i] = myo; }
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i < keep; i += 32) {
+    const u32 e = list[pick4(at, pnode[i]) + poff[i]];
+    pnode[i] = (int)(e >> 3); poff[i] = (int)(e & 7u);
+  }
+}
+// Requests per size -> R; every candidate's size and the rank of its first request among those of that size -> pnode, poff.
+__device__ __forceinline__ void gpu_requests(int keep, const u8* cg, const u8* r, int* pnode, int* poff, int R[4], int lane) {
+  R[0] = R[1] = R[2] = R[3] = 0;
+  const u32 below = (1u << lane) - 1u;
+#pragma unroll 1
+  for (int i0 = 0; i0 < keep; i0 += 32) {
+    const int i = i0 + lane;
+    int n = 0, c = -1;
+    if (i < keep) {
+      const int g = cg[i] & 0x7f, gang = cg[i] >> 7, ri = r[i];
+      n = gang ? 1 : ri; c = ilog2(gang ? g * ri : g);
     }
+    const bool several = __any_sync(TG_FULL, n > 1);
+    int rank = 0;
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const u32 b = __ballot_sync(TG_FULL, c == z);
+      int before = __popc(b & below), all = __popc(b);
+      if (several && b) {
+        const int x = c == z ? n : 0;
+        int incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(TG_FULL, incl, o); if (lane >= o) incl += y; }
+        before = incl - x; all = __shfl_sync(TG_FULL, incl, 31);
+      }
+      if (c == z) rank = R[z] + before;
+      R[z] += all;
+    }
+    if (i < keep) { pnode[i] = c; poff[i] = rank; }
   }
 }
 

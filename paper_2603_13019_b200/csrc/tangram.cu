@@ -169,17 +169,20 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
     }
   } else if (pd.type == TG_POOL_GPU) {
     const u8* br = busy_row ? busy_row + pd.node0 : nullptr;
-    if (pd.n_nodes <= 32) place_gpu_masks<1>(pd, br, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
-    else if (pd.n_nodes <= 128) place_gpu_masks<4>(pd, br, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
+    int R[4];
+    gpu_requests(keep, C.cg, C.rkeep, C.pnode, C.poff, R, lane);
+    const u64 bytes = (u64)(R[0] + R[1] + R[2] + R[3]) * 4;
+    u32* list = bytes <= WARP_WORK_BYTES ? (u32*)warp_smem() : (u32*)slab.take(bytes);   // (the selection is done with its work area)
+    u8* nm = pd.n_nodes > 32 ? (u8*)slab.take_fast(pd.n_nodes) : nullptr;
+    __syncwarp();
+    if (pd.n_nodes > 32 && !nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
+    else if (list && pd.n_nodes <= 32) place_gpu_lists<true>(pd, br, nullptr, list, R, keep, C.pnode, C.poff, lane);
+    else if (list) place_gpu_lists<false>(pd, br, nm, list, R, keep, C.pnode, C.poff, lane);
     else {
-      u8* nm = (u8*)slab.take_fast(pd.n_nodes);
-      if (!nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
-      else {
 #pragma unroll 1
-        for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
-        __syncwarp();
-        place_gpu(pd, nm, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
-      }
+      for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = br ? br[v] : 0;
+      __syncwarp();
+      place_gpu(pd, nm, keep, C.cg, C.rkeep, C.pnode, C.poff, lane);
     }
   } else if (pd.type == TG_POOL_CPU && pd.capacity / pd.group <= 128 && pd.group < 65536) {
     CpuFresh<4> F(pd, lane);

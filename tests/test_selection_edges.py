@@ -186,3 +186,37 @@ def test_sorted_orders_match_oracle(oracle, n, lo, hi):
     rnd, dev = binding.Round(4, n, pools), binding.to_device(a)
     for policy in (1, 2, 3):
         assert np.array_equal(oracle.order_queue(pools, a, policy), rnd.order_queue(dev, policy).cpu().numpy())
+
+
+@pytest.mark.parametrize("m", [68, 69])
+def test_rows_around_the_shared_table_match_oracle(oracle, m):
+    # m elastic candidates, ten spare cores; the last ones pay to be evicted in one scenario, everything ties in another
+    pools = (Pool(POOL_CPU, m + 10, m + 10), Pool(POOL_API, 1, 0, 0))
+    a = _round(m, pools, m, [0b1011], 1, 150)
+    a["p_us"][1, :m] = 50_000
+    a["s_us"][1] = 1000
+    a["p_us"][2, m - 4:m] = 4_000_000
+    assert_same(oracle.schedule_batch(pools, a), gpu_round(pools, a))
+
+
+@pytest.mark.parametrize("gpus,group,busy", [(8, 8, 0.0), (256, 8, 0.3), (264, 8, 0.3), (1032, 8, 0.1), (4800, 8, 0.2), (140, 4, 0.3),
+                                             (70, 2, 0.2), (33, 1, 0.3)])
+def test_gpu_placement_at_the_edges_match_oracle(oracle, gpus, group, busy):
+    # one node, 32 and 33 nodes, more than 128; more requests than the warp's work area lists (4800 GPUs, mostly single requests)
+    S, N = 4, gpus + 40
+    pools = (Pool(POOL_GPU, gpus, group),)
+    rng = np.random.default_rng(gpus)
+    top = int(np.log2(group))
+    unit = (1 << np.minimum(rng.geometric(0.7, (S, N)) - 1, top)).astype(np.uint8)
+    gang = rng.random((S, N)) < 0.5
+    mask = np.where(gang, 1, np.where(rng.random((S, N)) < 0.2, 4, 1))
+    a = dict(pool=np.zeros((S, N), np.uint8), unit=np.where(gang, unit | GANG, unit).astype(np.uint8), level_mask=mask.astype(np.uint32),
+             s_us=rng.integers(0, 20_000, (S, N)).astype(np.int64), p_us=rng.integers(0, 200_000, (S, N)).astype(np.int64),
+             arrival_us=None, n_actions=np.full(S, N, np.int32), gpu_busy=(rng.random((S, gpus // group, group)) < busy))
+    a["gpu_busy"] = (a["gpu_busy"] << np.arange(group)).sum(2).astype(np.uint8)
+    a["gpu_busy"][rng.random(a["gpu_busy"].shape) < 0.6] = 0
+    a["gpu_busy"][0] = 0
+    a["level_mask"][1] = np.where(gang[1] & (unit[1] * 2 <= group), 3, a["level_mask"][1])     # elastic gangs
+    o = oracle.schedule_batch(pools, a)
+    assert_same(o, gpu_round(pools, a))
+    assert o["n_selected"].sum() > gpus // 4
