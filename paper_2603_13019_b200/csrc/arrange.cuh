@@ -1298,6 +1298,7 @@ __device__ __noinline__ bool solve_box(const Params& P, PoolTask& T, int q, Slab
 // About 100 cycles per row: bound by the chain of shuffle, add and compare from row to row.
 #define CELL_LEVELS 6
 #define CELL_FAR (1ll << 61)        // an unreachable cell
+#define CELL_SHARED_ROWS 68         // rows whose choices fit the work area (7424 bytes)
 __device__ __forceinline__ bool small_table(const PoolTask& T, int nrows, i64* val, unsigned short* ch, int lane) {
   i64 prev = lane == 0 ? 0 : CELL_FAR;
 #pragma unroll 1
@@ -1512,8 +1513,12 @@ __device__ __forceinline__ int solve_prefix(const Params& P, PoolTask& T0, int q
     i64* val = T0.cell_val; unsigned short* ch = T0.cell_ch;
     int built = uniform(T0.cell_rows);
     if (built < nrows) {
+      // the choices behind the staged levels in the work area, which the simulations of up to 256 times leave alone: read
+      // back from the slab, every eight rows of the walk wait for the L2 (15000 cycles for 43 rows; cost vectors 2048 x 4096
+      // 403 us a call against 388, 16384 x 4096 1692 against 1685)
+      if (nrows <= CELL_SHARED_ROWS && T0.n_seeds + T0.m <= 256) ch = (unsigned short*)(T.wk + 32 * CELL_LEVELS * 16);
       built = small_table(T, nrows, val, ch, lane) ? nrows : -1;
-      if (lane == 0) T0.cell_rows = built;
+      if (lane == 0) { T0.cell_rows = built; T0.cell_ch = ch; }
     }
     if (built > 0) {
       const i64 change = small_answer(T, nrows, Y[0], val, ch, lane);
