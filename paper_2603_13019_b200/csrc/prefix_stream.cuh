@@ -15,9 +15,8 @@
 // an estimate the least-level durations (Eq. 1) of the waiting actions are appended, in queue
 // order, to the pool's list in `tmin`.
 //
-// k_fill writes "not scheduled" to every output row behind the candidate prefix (128-bit
-// stores).  Nothing else touches those rows, so it runs on a stream of its own beside all
-// kernels that follow k_head.
+// The output rows behind the candidate prefix get "not scheduled" from the selection kernel, which leaves the memory
+// idle (fill_part); of an ordered round k_fill writes all rows beside the sort, on a stream of its own.
 //
 // Partitioned arrays (order, tmin and the solver's arrays) give every (scenario, pool) its own
 // row of max_actions entries, so a position never depends on another pool's count and the
@@ -485,25 +484,33 @@ __device__ __forceinline__ void write_unscheduled4(const Params& P, size_t o) {
 __device__ __forceinline__ bool outputs_aligned(const Params& P) {
   return (((size_t)P.o_alloc | (size_t)P.o_node | (size_t)P.o_off | (size_t)P.o_act) & 15) == 0;
 }
-__global__ void __launch_bounds__(256) k_fill(const __grid_constant__ Params P, const HeadState* hst) {
-  const u32 stride = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const u32 N = (u32)P.N, total = (u32)P.S * N;              // S * N <= 2^31
+__global__ void __launch_bounds__(256) k_fill(const __grid_constant__ Params P) {
+  const u32 stride = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x, total = (u32)P.S * (u32)P.N;   // S * N <= 2^31
   if (outputs_aligned(P)) {
-    // groups of four of the whole array; one may hold the end of a row and the beginning of the next
-    for (u32 q = tid; q <= (total - 1) / 4; q += stride) {
-      const u32 o = q * 4, sc = o / N, i0 = o - sc * N;
-      if (i0 + 4 <= N) {
-        const int left = (int)i0 - (P.perm ? 0 : hst[sc].n);   // with an order of its own the candidates are anywhere
-        if (left >= 0) { write_unscheduled4(P, o); continue; }
-        for (int k = max(-left, 0); k < 4; ++k) write_unscheduled(P, (size_t)o + k);
-      } else
-        for (u32 k = 0, s = sc, i = i0; k < 4 && o + k < total; ++k, ++i) {
-          if (i == N) { i = 0; ++s; }
-          if (P.perm || (int)i >= hst[s].n) write_unscheduled(P, (size_t)o + k);
-        }
-    }
-  } else {
-    for (u32 o = tid; o < total; o += stride)
-      if (P.perm || (int)(o % N) >= hst[o / N].n) write_unscheduled(P, o);
+    for (u32 q = tid; q < total / 4; q += stride) write_unscheduled4(P, (size_t)q * 4);
+    if (tid < total % 4) write_unscheduled(P, (size_t)(total - 1 - tid));
+  } else
+    for (u32 o = tid; o < total; o += stride) write_unscheduled(P, o);
+}
+
+// The rows of scenario sc from action n on, by one warp.  Written by a kernel beside k_stream they took the memory that
+// that one needs: k_stream 549 us with that kernel beside it, 339 alone, at 16384 x 4096, and the
+// call 1675 against 1556.
+__device__ __forceinline__ void fill_rows(const Params& P, int sc, int n, int lane) {
+  const size_t row = (size_t)sc * P.N, o0 = row + (size_t)min(n, P.N), o1 = row + P.N;
+  const size_t a0 = (o0 + 3) & ~(size_t)3, a1 = o1 & ~(size_t)3;           // groups of four of the whole array
+  if (a0 >= a1 || !outputs_aligned(P)) {
+    for (size_t o = o0 + lane; o < o1; o += 32) write_unscheduled(P, o);
+    return;
   }
+  if (o0 + lane < a0) write_unscheduled(P, o0 + lane);
+  if (a1 + lane < o1) write_unscheduled(P, a1 + lane);
+  const u32 groups = (u32)((a1 - a0) / 4);
+  const int4 z = make_int4(0, 0, 0, 0), m1 = make_int4(-1, -1, -1, -1);
+  int4* const al = (int4*)P.o_alloc + a0 / 4; int4* const nd = (int4*)P.o_node + a0 / 4; int4* const of = (int4*)P.o_off + a0 / 4;
+  int4* const ac = (int4*)P.o_act + a0 / 2;
+#pragma unroll 2
+  for (u32 g = lane; g < groups; g += 32) { al[g] = z; nd[g] = m1; of[g] = m1; }
+#pragma unroll 4
+  for (u32 g = lane; g < 2 * groups; g += 32) ac[g] = m1;
 }

@@ -289,3 +289,27 @@ def test_gang_table_that_fits_a_small_slot_is_solved(oracle, rows):
     g = _gpu_round_ws(pools, a, workspace_bytes=1 << 20)
     assert np.all(g["status"] == 0)
     assert_same(oracle.schedule_batch(pools, a), g)
+
+
+@pytest.mark.parametrize("S,N,pools", [
+    (2400, 5, (Pool(POOL_CPU, 4, 2), Pool(POOL_GPU, 8, 8))),      # more scenarios than warps: with the first pool's tasks
+    (2400, 131, (Pool(POOL_GPU, 8, 4),)),
+    (600, 3, (Pool(POOL_GPU, 8, 8),)),                            # fewer: tasks behind the pools'
+    (600, 64, (Pool(POOL_CPU, 8, 4), Pool(POOL_API, 3, 0, 0))),
+])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_rows_that_stay_queued_match_oracle(oracle, S, N, pools, shift):
+    # every row of every output is written, whatever lay there, at any length and alignment of a row
+    import torch
+    from paper_2603_13019_b200 import binding
+    w, a = random_round(S + N, S, N, pools, small_durations=0.2, max_mult=4)
+    a["n_actions"][:2] = (0, N)
+    rnd = binding.Round(S, N, pools)
+    out = {}
+    for k, v in rnd.new_result().items():
+        flat = torch.full((v.numel() + shift,), 77, dtype=v.dtype, device="cuda")
+        out[k] = flat[shift:].view(v.shape)
+    rnd.schedule_batch(binding.to_device(a), 0, out)
+    torch.cuda.synchronize()
+    assert_same(oracle.schedule_batch(pools, a), {k: v.cpu().numpy() for k, v in out.items()})
+    rnd.destroy()
