@@ -119,65 +119,87 @@ __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u
 // [node][8][K] (tag 0 = empty, time of last use).  A grant makes the instance the most recently used
 // one on every GPU of the chunk; on a miss a GPU overwrites an empty entry (lowest index), else its
 // least recently used one (lowest index among equals), and miss[i] is set: candidate i then runs its
-// restoration time longer.  svc: the scenario's service column (may be null), ids: action indices.
-__device__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r, const int* ids,
-                                int* pnode, int* poff, u8* miss, const unsigned short* svc, u32* ctag, i64* cuse,
-                                int K, i64 now, int lane, int* owner = nullptr) {
-  const int top = ilog2(pd.group);
+// restoration time longer.  svc: the scenario's service column (may be null), ids: action indices, scratch: keep ints.
+// Per request, a lane looks at one GPU's entries and votes, four nodes a vote, then a lane per node finds the node's best block
+// by bit operations on free and holding GPUs, one warp minimum picks among them, and the chunk's GPUs update their
+// entries a lane each.  Bound by that chain; the entries work in shared memory (mem) where they fit, 38 nodes of two per
+// GPU in the selection's work area.  A lane that walked a node's chunks entry by entry in global memory took 3600 cycles a
+// request: 4096 x 1024 with two entries per GPU 400 us a call against 357.
+__device__ __forceinline__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r, const int* ids,
+                                                int* pnode, int* poff, u8* miss, int* scratch, const unsigned short* svc, u32* tag_row, i64* use_row,
+                                                int K, i64 now, int lane, char* mem, int mem_bytes, int* owner = nullptr) {
+  const int entries = pd.n_nodes * 8 * K;
+  u32* ctag = tag_row; i64* cuse = use_row;
+  const bool near = entries * 12 <= mem_bytes;
+  if (near) {
+    cuse = (i64*)mem; ctag = (u32*)(cuse + entries);
+#pragma unroll 2
+    for (int e = lane; e < entries; e += 32) { cuse[e] = use_row[e]; ctag[e] = tag_row[e]; }
+  }
+  const int top = ilog2(pd.group), n_nodes = pd.n_nodes;
   const u32 pad = (~((1u << pd.group) - 1u)) & 0xffu;
 #pragma unroll 1
-  for (int i = lane; i < keep; i += 32) miss[i] = 0;
+  for (int i = lane; i < keep; i += 32) { miss[i] = 0; scratch[i] = svc ? (int)svc[ids[i]] : 0xffff; }
   __syncwarp();
 #pragma unroll 1
   for (int lz = top; lz >= 0; --lz) {
     const int z = 1 << lz;
 #pragma unroll 1
-    for (int i = 0; i < keep; ++i) {
-      const int g = cg[i] & 0x7f, gang = cg[i] >> 7, ri = r[i];
-      const int nreq = gang ? (g * ri == z ? 1 : 0) : (g == z ? ri : 0);
-      if (nreq == 0) continue;
-      const u32 sv = svc ? svc[ids[i]] : 0xffffu;
-      const u32 tag = sv == 0xffffu ? 0u : ((sv << 3) | (u32)lz) + 1u;
+    for (int i0 = 0; i0 < keep; i0 += 32) {
+      int nreq = 0;
+      if (i0 + lane < keep) {
+        const int g = cg[i0 + lane] & 0x7f, gang = cg[i0 + lane] >> 7, ri = r[i0 + lane];
+        nreq = gang ? (g * ri == z ? 1 : 0) : (g == z ? ri : 0);
+      }
 #pragma unroll 1
-      for (int rep = 0; rep < nreq; ++rep) {
-        u32 kmin = 0xffffffffu;
+      for (u32 todo = __ballot_sync(TG_FULL, nreq > 0); todo; todo &= todo - 1u) {
+        const int b = __ffs(todo) - 1, i = i0 + b, cnt = __shfl_sync(TG_FULL, nreq, b);
+        const u32 sv = (u32)scratch[i], tag = sv == 0xffffu ? 0u : ((sv << 3) | (u32)lz) + 1u;
 #pragma unroll 1
-        for (int bl = lz; bl <= top && kmin == 0xffffffffu; ++bl) {
-          u32 key = 0xffffffffu;
+        for (int rep = 0; rep < cnt; ++rep) {
+          u32 best = 0xffffffffu;                        // block level | does not cache it | node | first GPU
 #pragma unroll 1
-          for (int v = lane; v < pd.n_nodes; v += 32) {
-            const NodeBlocks nb = node_blocks(nm[v] | pad);
-            u32 starts = bl == 0 ? nb.s1 : (bl == 1 ? nb.s2 : (bl == 2 ? nb.s4 : nb.s8));
+          for (int v0 = 0; v0 < n_nodes; v0 += 32) {
+            u32 hold = 0;                                // GPUs of the lane's node that remember the tag
+            if (tag)
 #pragma unroll 1
-            while (starts) {
-              const int st = __ffs(starts) - 1; starts &= starts - 1;
-              bool hit = tag != 0;
-#pragma unroll 1
-              for (int b = st; b < st + z && hit; ++b) {
+              for (int q = 0; q < 8 && v0 + 4 * q < n_nodes; ++q) {
+                const int at = (v0 + 4 * q) * 8 + lane;
                 bool has = false;
+                if (at < n_nodes * 8)
 #pragma unroll 1
-                for (int k = 0; k < K; ++k) has |= ctag[(size_t)(v * 8 + b) * K + k] == tag;
-                hit = has;
+                  for (int k = 0; k < K; ++k) has |= ctag[(size_t)at * K + k] == tag;
+                const u32 w = __ballot_sync(TG_FULL, has);
+                if ((lane >> 2) == q) hold = (w >> (8 * (lane & 3))) & 0xffu;
               }
-              key = min(key, (hit ? 0u : 1u << 30) | ((u32)v << 4) | (u32)st);
-            }
+            const int v = v0 + lane;
+            const NodeBlocks nb = node_blocks(v < n_nodes ? nm[v] | pad : 0xffu);
+            // the node's smallest sufficient level, the blocks of that level, and the ones whose low end caches the tag
+            const u32 s = lz <= 0 && nb.s1 ? nb.s1 : (lz <= 1 && nb.s2 ? nb.s2 : (lz <= 2 && nb.s4 ? nb.s4 : nb.s8));
+            const u32 lev = lz <= 0 && nb.s1 ? 0u : (lz <= 1 && nb.s2 ? 1u : (lz <= 2 && nb.s4 ? 2u : 3u));
+            u32 all = hold;                              // GPUs from which on z of them hold it
+            if (lz >= 1) all &= all >> 1;
+            if (lz >= 2) all &= all >> 2;
+            if (lz >= 3) all &= all >> 4;
+            const u32 hits = s & all;
+            if (s) best = min(best, (lev << 30) | (hits ? 0u : 1u << 29) | ((u32)v << 4) | (u32)(__ffs(hits ? hits : s) - 1));
           }
-          kmin = __reduce_min_sync(TG_FULL, key);
-        }
-        if (kmin == 0xffffffffu) continue;              // cannot happen: the selection fits
-        const int node = (int)((kmin >> 4) & 0x3ffffffu), start = (int)(kmin & 15u);
-        const bool hit = (kmin >> 30) == 0;
-        __syncwarp();
-        if (lane == 0) {
-          nm[node] |= (u8)(((1u << z) - 1u) << start);
-          if (rep == 0) { pnode[i] = node; poff[i] = start; }
-          if (owner) for (int b = 0; b < z; ++b) owner[node * pd.group + start + b] = ids[i];
-          if (tag) {
-            if (!hit) miss[i] = 1;
-#pragma unroll 1
-            for (int b = start; b < start + z; ++b) {
-              u32* tg = ctag + (size_t)(node * 8 + b) * K;
-              i64* us = cuse + (size_t)(node * 8 + b) * K;
+          best = __reduce_min_sync(TG_FULL, best);
+          if (best == 0xffffffffu) continue;              // cannot happen: the selection fits
+          const int node = (int)((best >> 4) & 0x1ffffffu), start = (int)(best & 15u);
+          const bool hit = ((best >> 29) & 1u) == 0u;
+          __syncwarp();
+          if (lane == 0) {
+            nm[node] |= (u8)(((1u << z) - 1u) << start);
+            if (rep == 0) { pnode[i] = node; poff[i] = start; }
+            if (tag && !hit) miss[i] = 1;
+          }
+          if (lane < z) {
+            const int gpu = start + lane;
+            if (owner) owner[node * pd.group + gpu] = ids[i];
+            if (tag) {
+              u32* tg = ctag + (size_t)(node * 8 + gpu) * K;
+              i64* us = cuse + (size_t)(node * 8 + gpu) * K;
               int at = -1;
 #pragma unroll 1
               for (int k = 0; k < K && at < 0; ++k) if (tg[k] == tag) at = k;
@@ -187,11 +209,14 @@ __device__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* c
               tg[at] = tag; us[at] = now;
             }
           }
+          __syncwarp();
         }
-        __syncwarp();
       }
     }
   }
+  if (near)
+#pragma unroll 2
+    for (int e = lane; e < entries; e += 32) { use_row[e] = cuse[e]; tag_row[e] = ctag[e]; }
 }
 
 // ---- fast paths of a single round: GPU requests size by size, core pools of at most 128 domains with their

@@ -976,8 +976,9 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = (u8)~Z.words[R.word0[j] + v];
                 __syncwarp();
                 const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
-                place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel,
-                                P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, now, lane, ow);
+                place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
+                                P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, now, lane,
+                                warp_smem(), WARP_WORK_BYTES, ow);
 #pragma unroll 1
                 for (int v = lane; v < pd.n_nodes; v += 32) Z.words[R.word0[j] + v] = ~(u32)nm[v] & ((1u << pd.group) - 1u);
                 missed = C.rsel;

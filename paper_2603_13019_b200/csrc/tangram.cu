@@ -145,15 +145,17 @@ __device__ PoolTask& make_task(const Params& P, int sc, int ws, int j, const Poo
   return T;
 }
 
-// placement on a fresh copy of the pool's topology state, then the candidates' outputs
-__device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C,
+// placement on a fresh copy of the pool's topology state, then the candidates' outputs.  CACHE: GPU pools have a service
+// cache; instances of their own, since the others are slower with its code in them (16384 x 4096 1555 us a call against 1510)
+template <bool CACHE>
+__device__ __forceinline__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& mt, const CandArrays& C,
                                 int keep, Slab slab, int lane) {
   const int m = mt.m;
   const PoolDev& pd = P.pool[j];
   const size_t row = (size_t)sc * P.N;
   const u8* busy_row = P.gpu_busy ? P.gpu_busy + (size_t)sc * P.n_nodes_total : nullptr;
   const u8* missed = nullptr;                            // candidates whose chunk did not cache their service
-  if (pd.type == TG_POOL_GPU && P.cache_slots > 0) {
+  if (CACHE && pd.type == TG_POOL_GPU) {
     // with a service cache: the chunk that caches the instance first, entries updated, misses noted in C.rsel
     u8* nm = (u8*)slab.take_fast(pd.n_nodes);
     if (!nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
@@ -162,9 +164,9 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
       for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
       __syncwarp();
       const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
-      place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel,
-                      P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase,
-                      P.cache_slots, P.now, lane);
+      place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
+                      P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, P.now, lane,
+                      warp_smem(), WARP_WORK_BYTES);   // (the selection is done with its work area)
       missed = C.rsel;
     }
   } else if (pd.type == TG_POOL_GPU) {
@@ -217,7 +219,7 @@ __device__ void place_and_write(const Params& P, int sc, int j, const PoolMeta& 
       int r = C.rkeep[i];
       i64 arr = P.a_arrival ? P.a_arrival[o] : 0;
       i64 act = (P.now - arr) + duration(C.cs[i], C.cp[i], r);
-      if (missed && missed[i] && P.a_restore) act += clamp_param(P.a_restore[o]);   // restoration precedes execution
+      if (CACHE && missed && missed[i] && P.a_restore) act += clamp_param(P.a_restore[o]);   // restoration precedes execution
       P.o_alloc[o] = (C.cg[i] & 0x7f) * r; P.o_act[o] = act;
       P.o_node[o] = C.pnode[i]; P.o_off[o] = C.poff[i];
       tot += act; ++cnt;
@@ -276,6 +278,7 @@ __device__ __forceinline__ void pool_best_levels(const Params& P, int sc, int j,
 }
 
 // ws: whose rows of the workspace the pool's facts are in
+template <bool CACHE>
 __device__ __forceinline__ void run_pool_task(const Params& P, int sc, int ws, int j, const PoolMeta& mt, Slab slab, int lane) {
   CandArrays C;
   if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
@@ -287,9 +290,10 @@ __device__ __forceinline__ void run_pool_task(const Params& P, int sc, int ws, i
     keep = evict_loop(P, make_task(P, sc, ws, j, mt, C, lane), slab, lane);
     if (keep < 0) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
   }
-  place_and_write(P, sc, j, mt, C, keep, slab, lane);
+  place_and_write<CACHE>(P, sc, j, mt, C, keep, slab, lane);
 }
 
+template <bool CACHE>
 __device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int j, u32 need, int slab, int lane) {
   PoolMeta mt = P.meta[(size_t)ws * P.P + j];            // (a scenario with an invalid record has no candidates)
   mt.m = uniform(mt.m); mt.count = uniform(mt.count); mt.elastic = uniform(mt.elastic);
@@ -297,7 +301,7 @@ __device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int
   if (!((need >> j) & 1u) && P.pool[j].queue_place) {
     if (P.pool[j].type == TG_POOL_API || P.pool[j].capacity <= 64 * P.pool[j].group) pool_best_levels<2>(P, sc, j, mt, lane);
     else pool_best_levels<4>(P, sc, j, mt, lane);
-  } else run_pool_task(P, sc, ws, j, mt, warp_slab(P, slab), lane);
+  } else run_pool_task<CACHE>(P, sc, ws, j, mt, warp_slab(P, slab), lane);
 }
 
 // All pools of a batched round, pool-major, the pools that may need a selection first.  The rows that stay queued are
@@ -305,6 +309,7 @@ __device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int
 // second one of those, as tasks behind all others, which idle warps find while the longest pools are decided.  Spread
 // over all pools, or with the second ones on, they meet the short tasks, which wait for memory themselves: 16384 x 4096 k_pool
 // 1188 us against 1109 (1014 without the rows).  Bulk copies of constant blocks in shared memory instead of stores: 1110.
+template <bool CACHE>
 __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ Params P, const HeadState* hst) {
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * K2_THREADS + threadIdx.x) >> 5;
@@ -317,7 +322,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
     if (x >= n_tasks) break;
     const int sc = x % P.S, k = x / P.S;
     if (fill && k == (with_first ? 0 : P.P)) fill_rows(P, sc, hst[sc].n, lane);
-    if (k < P.P) decide_pool(P, sc, sc, P.pool_order[k], hst[sc].need, gw, lane);
+    if (k < P.P) decide_pool<CACHE>(P, sc, sc, P.pool_order[k], hst[sc].need, gw, lane);
   }
 }
 
@@ -327,7 +332,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
 // batch is latency, and one launch instead of four (and a memset) saves the gaps.  The last block to finish resets
 // the bump pointer of the arena for the next call.  1 x 64: 38.6 -> 26.8 us a call, 16 x 500 (static): 110 -> 84 us.
 #define TG_DONE_COUNTER 4           // word of arena_top that counts finished blocks
-template <bool SIDE, bool SORTED>
+template <bool SIDE, bool SORTED, bool CACHE>
 __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__ Params P, int wpb) {
   __shared__ StreamShared X;
   __shared__ HeadState H;
@@ -361,7 +366,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__
     stream_queue<SORTED>(P, sc, ws, H, X, t);
     __syncthreads();
 #pragma unroll 1
-    for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
+    for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool<CACHE>(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
     __syncthreads();
   }
   if (t == 0) {
@@ -456,6 +461,12 @@ static void fill_candidate_rows(Params& P) {
 // pools whose grants are placed one after the other in queue order with their state in registers
 static int queue_place_ok(const PoolDev& d) {
   return d.type == TG_POOL_API || (d.type == TG_POOL_CPU && d.capacity / d.group <= 128 && d.group < 65536);
+}
+
+static bool has_cache(const Params& P) { return P.cache_slots > 0 && P.n_nodes_total > 0; }
+static const void* round_kernel(bool cache, bool side, bool sorted) {
+  if (cache) return side ? (const void*)k_round<true, false, true> : (const void*)k_round<false, false, true>;
+  return side ? (const void*)k_round<true, false, false> : sorted ? (const void*)k_round<false, true, false> : (const void*)k_round<false, false, false>;
 }
 
 extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_round** out) {
@@ -645,10 +656,11 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   P.side_bad = r->d_side_bad; P.side_res = r->d_side_res;
   P.slabs = (char*)r->d_slabs; P.arena = (char*)r->d_arena; P.arena_top = (u64*)r->d_arena_top;
   e = cudaMemset(r->d_arena_top, 0, 256);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pool, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_round<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  // the instances that this round's calls can take (a sorted queue has no cache and no further costs)
+  const bool cache = has_cache(P);
+  const void* kern[3] = {cache ? (const void*)k_pool<true> : (const void*)k_pool<false>, round_kernel(cache, false, false),
+                         cache || desc->side_costs > 0 ? round_kernel(cache, true, false) : round_kernel(false, false, true)};
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaFuncSetAttribute(kern[k], cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
   *out = r;
   return TANGRAM_OK;
@@ -810,9 +822,8 @@ static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, bool
     cudaEvent_t* ev = timed ? prof_begin(r, 1, -1, -1) : nullptr;
     if (ev) CK(cudaEventRecord(ev[0], st));
     const int smem = P.P * WARP_SMEM_BYTES + 16;
-    if (P.n_side > 0) k_round<true, false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
-    else if (P.perm) k_round<false, true><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
-    else k_round<false, false><<<P.S, K2_THREADS, smem, st>>>(P, P.P);
+    void (*kern)(Params, int) = (void (*)(Params, int))round_kernel(has_cache(P), P.n_side > 0, P.perm != nullptr);
+    kern<<<P.S, K2_THREADS, smem, st>>>(P, P.P);
     if (ev) CK(cudaEventRecord(ev[1], st));
     r->launches += 1;
     CK(cudaGetLastError());
@@ -835,7 +846,8 @@ static int run_pipeline(tangram_round* r, const Params& P, cudaStream_t st, bool
   else k_stream<false><<<P.S, KS_THREADS, 0, st>>>(P, r->hst);
   if (ev) CK(cudaEventRecord(ev[2], st));
   if (P.perm) CK(cudaStreamWaitEvent(st, r->side_join, 0));   // it wrote the candidates' rows as well
-  k_pool<<<P.n_workers / (K2_THREADS / 32), K2_THREADS, K2_DYN_SMEM, st>>>(P, r->hst);
+  if (has_cache(P)) k_pool<true><<<P.n_workers / (K2_THREADS / 32), K2_THREADS, K2_DYN_SMEM, st>>>(P, r->hst);
+  else k_pool<false><<<P.n_workers / (K2_THREADS / 32), K2_THREADS, K2_DYN_SMEM, st>>>(P, r->hst);
   if (ev) CK(cudaEventRecord(ev[3], st));
   r->launches += 3;
   CK(cudaGetLastError());
@@ -1087,7 +1099,7 @@ static int static_setup(int* dev_out) {
     unsigned char* ptr = nullptr;
     CK(cudaGetSymbolAddress((void**)&ptr, g_static_scratch));
     CK(fill_tables());
-    CK(cudaFuncSetAttribute(k_round<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
+    CK(cudaFuncSetAttribute(k_round<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM));
     g_static_ptr[dev] = ptr;
     g_static_ready[dev] = true;
   }
@@ -1161,7 +1173,7 @@ extern "C" int tangram_schedule_batch_static(const tangram_round_desc* desc, con
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CK(cudaMemsetAsync(P.arena_top, 0, 256, st));           // whatever an overlapping call may have left
-  k_round<false, false><<<(unsigned)blocks, K2_THREADS, wpb * WARP_SMEM_BYTES + 16, st>>>(P, wpb);
+  k_round<false, false, false><<<(unsigned)blocks, K2_THREADS, wpb * WARP_SMEM_BYTES + 16, st>>>(P, wpb);
   CK(cudaGetLastError());
   return TANGRAM_OK;
 }
