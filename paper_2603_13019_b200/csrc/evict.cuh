@@ -309,6 +309,9 @@ __device__ __forceinline__ void ev_replace(u32 (&key)[NS], u32 mn, u32 holders, 
   }
 }
 
+__device__ __forceinline__ void ev_load(u32 (&d)[2], u32 at) {
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(d[0]), "=r"(d[1]) : "r"(at) : "memory");
+}
 template <int NS>
 __device__ __forceinline__ void ev_step(u32 (&a)[NS], u32 (&b)[NS], u32 da, u32 db, u32 above, u32& ma, u32& mb) {
   mb = __reduce_min_sync(TG_FULL, b[0]);
@@ -374,23 +377,29 @@ __device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, i
     __syncwarp();
     // The two chains, step by step side by side (warp-wide operations keep their order, so it is written this way).
     // A's first action takes its own level.
-    u32 da = k0 == 0 ? first_a : dur.get(0);
+    // The next durations are loaded while these are worked on.  Two steps per turn of the loop: where all warps are busy they wait
+    // for instructions, and the text of this loop counts (16384 x 4096, 66 slots: four steps 1585 us a call, two 1510, one
+    // 1600), for 0.5 to 2 % where a few pools set the time (4096 x 1024: four 251, two 256; 64 nodes, 1024 x 2048: 527 and 550).
+    // Two for some register counts and four for others gained less than either.
+    u32 d[2];
+    ev_load(d, dur.base);
+    u32 da = k0 == 0 ? first_a : d[0];
     int k = 0;
 #pragma unroll 1
-    for (; k + 4 <= steps; k += 4) {
-      u32 d[4];
-      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(dur.base + (u32)k * 4u) : "memory");
-      if (k > 0) da = d[0];
+    for (; k + 2 <= steps; k += 2) {
+      u32 next[2];
+      ev_load(next, dur.base + (u32)k * 4u + 8u);          // (behind the last ones lies room for a block more)
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
+      for (int z = 0; z < 2; ++z) {
         ev_step(a, b, z == 0 ? da : d[z], d[z], above, last_a, last_b);
         diff += (i64)last_b - (i64)last_a;
       }
+      da = d[0] = next[0]; d[1] = next[1];
     }
 #pragma unroll 1
     for (; k < steps; ++k) {
-      const u32 d = dur.get(k);
-      ev_step(a, b, k > 0 ? d : da, d, above, last_a, last_b);
+      const u32 e = dur.get(k);
+      ev_step(a, b, k > 0 ? e : da, e, above, last_a, last_b);
       diff += (i64)last_b - (i64)last_a;
     }
     __syncwarp();
