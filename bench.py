@@ -37,7 +37,7 @@ METRIC = "actions scheduled/sec (1xB200)"
 # DRAM bytes per pending action (dram__bytes_read.sum + dram__bytes_write.sum of one launch / actions of the
 # launch), captured by ncu on the whole workload (16384 scenarios; profiles/batched_round_cfg4.md), so that what stays in
 # L2 at the end of a launch is a small part; with fewer scenarios the figures are scaled by actions.
-NCU_BYTES_PER_ACTION = {"cfg4": {"k_head": 1.89, "k_stream": 23.45, "k_pool": 33.42}}
+NCU_BYTES_PER_ACTION = {"cfg4": {"k_head": 1.89, "k_stream": 23.47, "k_pool": 35.78}}
 NCU_TRAFFIC_SOURCE = "ncu on cfg4 at 16384 scenarios, scaled by actions (profiles/batched_round_cfg4.md)"
 
 
