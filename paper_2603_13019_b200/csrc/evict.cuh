@@ -312,6 +312,10 @@ __device__ __forceinline__ void ev_replace(u32 (&key)[NS], u32 mn, u32 holders, 
 __device__ __forceinline__ void ev_load(u32 (&d)[2], u32 at) {
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(d[0]), "=r"(d[1]) : "r"(at) : "memory");
 }
+__device__ __forceinline__ void ev_load(u32 (&d)[4], u32 at) {
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(at) : "memory");
+}
+
 template <int NS>
 __device__ __forceinline__ void ev_step(u32 (&a)[NS], u32 (&b)[NS], u32 da, u32 db, u32 above, u32& ma, u32& mb) {
   mb = __reduce_min_sync(TG_FULL, b[0]);
@@ -358,7 +362,7 @@ __device__ __forceinline__ bool ev_behind_regs(const u32 (&a)[NS], const u32 (&b
 // of the shorter one, before the evicted candidate of duration `evicted`.  dur_of(k): duration of the k-th of n that wait behind
 // both, first_a: of the first one as `a` takes it; diff: the part of the difference that is no popped time.
 // wk: 64 NS + 2 EV_BLOCK + 4 words of shared memory.
-template <int NS, class Dur>
+template <int NS, int U, class Dur>
 __device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, int n, u32 evicted, u32 first_a, i64 diff, const Dur& dur_of, u32 wk,
                                            int lane) {
   const EvShared dur = {wk + NS * 256u};
@@ -377,24 +381,26 @@ __device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, i
     __syncwarp();
     // The two chains, step by step side by side (warp-wide operations keep their order, so it is written this way).
     // A's first action takes its own level.
-    // The next durations are loaded while these are worked on.  Two steps per turn of the loop: where all warps are busy they wait
-    // for instructions, and the text of this loop counts (16384 x 4096, 66 slots: four steps 1585 us a call, two 1510, one
-    // 1600), for 0.5 to 2 % where a few pools set the time (4096 x 1024: four 251, two 256; 64 nodes, 1024 x 2048: 527 and 550).
-    // Two for some register counts and four for others gained less than either.
-    u32 d[2];
+    // The next durations are loaded while these are worked on.  U steps per turn of the loop: two in k_pool, where all warps are
+    // busy and wait for instructions, so that the text of this loop counts (16384 x 4096, 66 slots: four steps 1585 us a call,
+    // two 1510, one 1600), for 0.5 to 2 % where a few pools set the time (4096 x 1024: four 251, two 256; 64 nodes,
+    // 1024 x 2048: 527 and 550); four in k_round and k_replay, where few warps wait for this chain.
+    u32 d[U];
     ev_load(d, dur.base);
     u32 da = k0 == 0 ? first_a : d[0];
     int k = 0;
 #pragma unroll 1
-    for (; k + 2 <= steps; k += 2) {
-      u32 next[2];
-      ev_load(next, dur.base + (u32)k * 4u + 8u);          // (behind the last ones lies room for a block more)
+    for (; k + U <= steps; k += U) {
+      u32 next[U];
+      ev_load(next, dur.base + (u32)(k + U) * 4u);          // (behind the last ones lies room for a block more)
 #pragma unroll
-      for (int z = 0; z < 2; ++z) {
+      for (int z = 0; z < U; ++z) {
         ev_step(a, b, z == 0 ? da : d[z], d[z], above, last_a, last_b);
         diff += (i64)last_b - (i64)last_a;
       }
-      da = d[0] = next[0]; d[1] = next[1];
+      da = next[0];
+#pragma unroll
+      for (int z = 0; z < U; ++z) d[z] = next[z];
     }
 #pragma unroll 1
     for (; k < steps; ++k) {
@@ -413,7 +419,7 @@ __device__ __forceinline__ int ev_run_regs(u32 (&a)[NS], u32 (&b)[NS], int ha, i
   if (last_b >= EV_SAT) return -1;
   return diff < 0 ? 1 : 0;
 }
-template <int NS>
+template <int NS, int U>
 __device__ __forceinline__ int ev_compare_regs(const PoolTask& T, int q, const u8* kept, const u8* fewer, i64 fixed, u32 wk, int lane) {
   const int ha = T.n_seeds + q + 1, n = T.m - q - 1 + T.n_ac;
   u32 a[NS], b[NS];
@@ -429,7 +435,7 @@ __device__ __forceinline__ int ev_compare_regs(const PoolTask& T, int q, const u
       if (c < q) b[j] = ev_key(duration(s, p, fewer[c]));
     }
   }
-  return ev_run_regs<NS>(a, b, ha, n, ev_key(rest_first(T, q)), n > 0 ? ev_key(rest_first(T, q + 1)) : 0u, fixed,
+  return ev_run_regs<NS, U>(a, b, ha, n, ev_key(rest_first(T, q)), n > 0 ? ev_key(rest_first(T, q + 1)) : 0u, fixed,
                          [&](int k) { return ev_key(rest_least(T, q + 1, k)); }, wk, lane);
 }
 
@@ -500,6 +506,7 @@ __device__ __forceinline__ int ev_compare_windows(const PoolTask& T, int q, cons
 
 // Does evicting candidate q (the last of the q+1 kept, multiplicities rkeep) lower the objective (rsel, T0.opt: the
 // optimum without it)?  opt_kept: duration sum with it.  1 yes, 0 no, -1 workspace too small.
+template <int U>
 __device__ __forceinline__ int eviction_pays(const Params& P, const PoolTask& T0, int q, i64 opt_kept, Slab slab, int lane) {
   PoolTask T;                                            // (what is used of it, in registers)
   T.m = uniform(T0.m); T.n_ac = uniform(T0.n_ac); T.n_seeds = uniform(T0.n_seeds); T.depth = T0.depth;
@@ -514,12 +521,12 @@ __device__ __forceinline__ int eviction_pays(const Params& P, const PoolTask& T0
     if (n > 0) fixed += rest_least(T, q + 1, 0) - rest_first(T, q + 1);
     const u32 wk = (u32)__cvta_generic_to_shared(T.wk);
     int got = -1;
-    if (ha <= 32) got = ev_compare_regs<1>(T, q, kept, fewer, fixed, wk, lane);
-    else if (ha <= 64) got = ev_compare_regs<2>(T, q, kept, fewer, fixed, wk, lane);
-    else if (ha <= 96) got = ev_compare_regs<3>(T, q, kept, fewer, fixed, wk, lane);
-    else if (ha <= 128) got = ev_compare_regs<4>(T, q, kept, fewer, fixed, wk, lane);
-    else if (ha <= 192) got = ev_compare_regs<6>(T, q, kept, fewer, fixed, wk, lane);
-    else if (ha <= 256) got = ev_compare_regs<8>(T, q, kept, fewer, fixed, wk, lane);
+    if (ha <= 32) got = ev_compare_regs<1, U>(T, q, kept, fewer, fixed, wk, lane);
+    else if (ha <= 64) got = ev_compare_regs<2, U>(T, q, kept, fewer, fixed, wk, lane);
+    else if (ha <= 96) got = ev_compare_regs<3, U>(T, q, kept, fewer, fixed, wk, lane);
+    else if (ha <= 128) got = ev_compare_regs<4, U>(T, q, kept, fewer, fixed, wk, lane);
+    else if (ha <= 192) got = ev_compare_regs<6, U>(T, q, kept, fewer, fixed, wk, lane);
+    else if (ha <= 256) got = ev_compare_regs<8, U>(T, q, kept, fewer, fixed, wk, lane);
     else got = ev_compare_windows(T0, q, kept, fewer, fixed, slab, wk, lane);
     if (got >= 0) return got;
   }
@@ -550,6 +557,7 @@ __device__ __forceinline__ void solve_single(const PoolTask& T, int lane) {
 
 // Greedy eviction (Algorithm 1, lines 8-14) from the full candidate list.  The accepted multiplicities are in
 // T.rkeep; returns the number of candidates kept, or -1 if the workspace is too small.
+template <int U>
 __device__ __forceinline__ int evict_loop(const Params& P, PoolTask& T, Slab slab, int lane) {
   const int m = uniform(T.m);
   if (m == 1) { solve_single(T, lane); return 1; }
@@ -570,7 +578,7 @@ __device__ __forceinline__ int evict_loop(const Params& P, PoolTask& T, Slab sla
     if (got == UNSOLVED) return -1;
     if (q < m) {
       if (eviction_cannot_pay(T, q, rkeep, rsel, lane)) break;
-      const int pays = eviction_pays(P, T, q, opt, slab, lane);
+      const int pays = eviction_pays<U>(P, T, q, opt, slab, lane);
       if (pays < 0) return -1;
       if (!pays) break;
     }

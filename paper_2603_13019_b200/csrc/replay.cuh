@@ -354,7 +354,7 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
     T.wk = warp_smem(); T.wk_bytes = WARP_WORK_BYTES;
   }
   __syncwarp();
-  keep = evict_loop(P, T, slab, lane);
+  keep = evict_loop<4>(P, T, slab, lane);
   return keep >= 0;
 }
 
@@ -425,7 +425,7 @@ __device__ __forceinline__ int replay_pair(const Params& P, const PoolDev& pd, c
   if (lane < nr && RR_POOL(run.pu[lane]) == j) { const i64 f = run.fin[lane]; a[0] = b[0] = ev_key(f > now ? f - now : 0); }
   if (lane == nr) { a[0] = ev_key(duration(A.s, A.p, ra)); b[0] = ev_key(t_alone); }
   if (lane == nr + 1) a[0] = ev_key(duration(B.s, B.p, rb));
-  const int pays = ev_run_regs<1>(a, b, nr + 2, n_ac, ev_key(t_first), ev_key(first_a), fixed, [&](int k) { return list[k]; },
+  const int pays = ev_run_regs<1, 4>(a, b, nr + 2, n_ac, ev_key(t_first), ev_key(first_a), fixed, [&](int k) { return list[k]; },
                                   (u32)__cvta_generic_to_shared(warp_smem()), lane);
   if (pays < 0) return 0;
   if (pays) { ra = alone; return 1; }

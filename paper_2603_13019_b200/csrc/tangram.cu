@@ -278,7 +278,7 @@ __device__ __forceinline__ void pool_best_levels(const Params& P, int sc, int j,
 }
 
 // ws: whose rows of the workspace the pool's facts are in
-template <bool CACHE>
+template <bool CACHE, int U>
 __device__ __forceinline__ void run_pool_task(const Params& P, int sc, int ws, int j, const PoolMeta& mt, Slab slab, int lane) {
   CandArrays C;
   if (!gather_candidates(P, sc, j, mt, slab, lane, C)) {
@@ -287,13 +287,13 @@ __device__ __forceinline__ void run_pool_task(const Params& P, int sc, int ws, i
   }
   int keep = mt.m;
   if (mt.elastic) {
-    keep = evict_loop(P, make_task(P, sc, ws, j, mt, C, lane), slab, lane);
+    keep = evict_loop<U>(P, make_task(P, sc, ws, j, mt, C, lane), slab, lane);
     if (keep < 0) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
   }
   place_and_write<CACHE>(P, sc, j, mt, C, keep, slab, lane);
 }
 
-template <bool CACHE>
+template <bool CACHE, int U>
 __device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int j, u32 need, int slab, int lane) {
   PoolMeta mt = P.meta[(size_t)ws * P.P + j];            // (a scenario with an invalid record has no candidates)
   mt.m = uniform(mt.m); mt.count = uniform(mt.count); mt.elastic = uniform(mt.elastic);
@@ -301,7 +301,7 @@ __device__ __forceinline__ void decide_pool(const Params& P, int sc, int ws, int
   if (!((need >> j) & 1u) && P.pool[j].queue_place) {
     if (P.pool[j].type == TG_POOL_API || P.pool[j].capacity <= 64 * P.pool[j].group) pool_best_levels<2>(P, sc, j, mt, lane);
     else pool_best_levels<4>(P, sc, j, mt, lane);
-  } else run_pool_task<CACHE>(P, sc, ws, j, mt, warp_slab(P, slab), lane);
+  } else run_pool_task<CACHE, U>(P, sc, ws, j, mt, warp_slab(P, slab), lane);
 }
 
 // All pools of a batched round, pool-major, the pools that may need a selection first.  The rows that stay queued are
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
     if (x >= n_tasks) break;
     const int sc = x % P.S, k = x / P.S;
     if (fill && k == (with_first ? 0 : P.P)) fill_rows(P, sc, hst[sc].n, lane);
-    if (k < P.P) decide_pool<CACHE>(P, sc, sc, P.pool_order[k], hst[sc].need, gw, lane);
+    if (k < P.P) decide_pool<CACHE, 2>(P, sc, sc, P.pool_order[k], hst[sc].need, gw, lane);
   }
 }
 
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__
     stream_queue<SORTED>(P, sc, ws, H, X, t);
     __syncthreads();
 #pragma unroll 1
-    for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool<CACHE>(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
+    for (int x = warp; x < P.P && warp < wpb; x += wpb) decide_pool<CACHE, 4>(P, sc, ws, P.pool_order[x], H.need, ws * wpb + warp, lane);
     __syncthreads();
   }
   if (t == 0) {
