@@ -136,14 +136,19 @@ __device__ __forceinline__ void replay_store(const ReplayQueue<LIST>& Q, int x, 
   Q.ta[x] = make_uint4((u32)r.tl, (u32)((u64)r.tl >> 32), (u32)r.arr, (u32)((u64)r.arr >> 32));
   Q.c[x] = make_uint4((u32)a, r.meta, r.mask, (u32)r.cg | last);
 }
-// action, meta, mask and unit byte at a queue position (any lane's own); x: its slot where it is in shared memory
+// a record's bit 8: the action is marked as the last one of its trajectory (traces with trajectories, and so LIST, only)
 template <bool LIST>
-__device__ __forceinline__ uint4 replay_facts(const Params& P, const ReplayQueue<LIST>& Q, const int* wait, size_t row, int i, int& x) {
+__device__ __forceinline__ u32 replay_last(const ReplayWs& R, size_t row, int a) {
+  return LIST && R.traj_last && R.traj_last[row + a] ? 256u : 0u;
+}
+// action, meta, mask, unit byte and bit 8 at a queue position (any lane's own); x: its slot where it is in shared memory
+template <bool LIST>
+__device__ __forceinline__ uint4 replay_facts(const Params& P, const ReplayWs& R, const ReplayQueue<LIST>& Q, const int* wait, size_t row, int i, int& x) {
   if (i < Q.cap) { x = Q.slot(i); return Q.c[x]; }
   const int a = wait[i];
   const ReplayRec r = replay_decode(P, P.a_pool[row + a], P.a_unit[row + a], P.a_mask[row + a], 0, 0);
   x = -1;
-  return make_uint4((u32)a, r.meta, r.mask, (u32)r.cg);
+  return make_uint4((u32)a, r.meta, r.mask, (u32)r.cg | replay_last<LIST>(R, row, a));
 }
 // ... and the rest of a record whose facts are known
 template <bool LIST>
@@ -278,7 +283,7 @@ __device__ __forceinline__ void replay_gpu_slots(const PoolDev& pd, const u32* w
 // The selection of a pool with a choice to make: its candidates (among the first n positions) and, where an eviction
 // step can look at them, the waiting actions behind and the running ones are gathered into arrays.
 template <bool LIST>
-__device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue<LIST>& Q, const ReplayRun run, const int* wait, size_t row, int j,
+__device__ __forceinline__ bool replay_select(const Params& P, const ReplayWs& R, const ReplayQueue<LIST>& Q, const ReplayRun run, const int* wait, size_t row, int j,
                                            int n, int nw, int nr, int m, i64 now, int cap0, int cap1, int cap2, int cap3, Slab& slab,
                                            CandArrays& C, int& keep, int lane) {
   const PoolDev& pd = P.pool[j];
@@ -293,7 +298,7 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
   for (int i0 = 0; i0 < n; i0 += 32) {
     const int i = i0 + lane;
     int x = -1; uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u);
-    if (i < n) c = replay_facts(P, Q, wait, row, i, x);
+    if (i < n) c = replay_facts(P, R, Q, wait, row, i, x);
     const bool mine = RQ_POOL(c.y) == j;
     const u32 b = __ballot_sync(TG_FULL, mine);
     if (mine) {
@@ -320,7 +325,7 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
     for (int i0 = n; i0 < nw; i0 += 32) {
       const int i = i0 + lane;
       int x = -1; uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u);
-      if (i < nw) c = replay_facts(P, Q, wait, row, i, x);
+      if (i < nw) c = replay_facts(P, R, Q, wait, row, i, x);
       const u32 b = __ballot_sync(TG_FULL, RQ_POOL(c.y) == j);
       if ((b >> lane) & 1u) ac[n_ac + __popc(b & ((1u << lane) - 1u))] = replay_rec(P, Q, row, c, x).tl;
       if (first < 0 && b) first = i0 + __ffs(b) - 1;
@@ -344,7 +349,7 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayQueue
     T.ac_first.s = T.ac_first.p = 0; T.ac_first.mask = 1; T.ac_first.g = 1; T.ac_first.gang = 0;
     if (first >= 0) {
       int x;
-      const uint4 c = replay_facts(P, Q, wait, row, first, x);
+      const uint4 c = replay_facts(P, R, Q, wait, row, first, x);
       const ReplayRec r = replay_rec(P, Q, row, c, x);
       T.ac_first.s = r.s; T.ac_first.p = r.p; T.ac_first.mask = r.mask; T.ac_first.g = r.cg & 0x7f; T.ac_first.gang = r.cg >> 7;
     }
@@ -549,7 +554,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         if (i < n_act) {
           if (EXT && R.trajectory) {
             l_traj = R.trajectory[row + i]; l_mem = R.traj_mem[row + i];
-            l_last = R.traj_last && R.traj_last[row + i] ? 256u : 0u;
+            l_last = replay_last<EXT>(R, row, i);
           }
           l_pool = P.a_pool[row + i]; l_unit = P.a_unit[row + i]; l_mask = P.a_mask[row + i]; l_s = P.a_s[row + i]; l_p = P.a_p[row + i];
           l_arr = P.a_arrival ? P.a_arrival[row + i] : 0;
@@ -793,7 +798,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
 #pragma unroll 1
           for (int i0 = 0; i0 < nw; i0 += 32) {
             uint4 c = make_uint4(0u, RQ_NOBODY, 1u, 1u); int x = -1;
-            if (i0 + lane < nw) c = replay_facts(P, Q, wait, row, i0 + lane, x);
+            if (i0 + lane < nw) c = replay_facts(P, R, Q, wait, row, i0 + lane, x);
             if (i0 == 0) { c0 = c; x0 = x; }
             const int nb = min(32, nw - i0);
             int k0 = 0xff, u0 = 0, k1 = 0xff, u1 = 0;      // further entries of the cost vector
@@ -862,7 +867,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
 #pragma unroll 1
               for (int i0 = 0; i0 < n; i0 += 32) {
                 int x; u32 meta = RQ_NOBODY;
-                if (i0 + lane < n) meta = replay_facts(P, Q, wait, row, i0 + lane, x).y;
+                if (i0 + lane < n) meta = replay_facts(P, R, Q, wait, row, i0 + lane, x).y;
                 m += __popc(__ballot_sync(TG_FULL, RQ_POOL(meta) == j));
               }
             const bool el = (present >> (8 + j)) & 1u;
@@ -882,7 +887,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 uint4 c = c0; int x = x0;
                 if (i0 > 0) {
                   c = make_uint4(0u, RQ_NOBODY, 1u, 1u); x = -1;
-                  if (i0 + lane < n) c = replay_facts(P, Q, wait, row, i0 + lane, x);
+                  if (i0 + lane < n) c = replay_facts(P, R, Q, wait, row, i0 + lane, x);
                 }
                 bool mine = i0 + lane < n && RQ_POOL(c.y) == j;
                 u32 mb = __ballot_sync(TG_FULL, mine);
@@ -965,7 +970,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               slab.base = P.slabs + (u64)blockIdx.x * P.slab_bytes; slab.cap = P.slab_bytes; slab.used = 0;
               slab.fbase = fast; slab.fcap = KR_FAST_BYTES; slab.fused = 0;
               CandArrays C; int keep = 0;
-              ok = replay_select(P, Q, run, wait, row, j, n, nw, nr, m, now, Z.slot[slot0] - aside_j, Z.slot[(slot0 + 1) & 31],
+              ok = replay_select(P, R, Q, run, wait, row, j, n, nw, nr, m, now, Z.slot[slot0] - aside_j, Z.slot[(slot0 + 1) & 31],
                                  Z.slot[(slot0 + 2) & 31], Z.slot[(slot0 + 3) & 31], slab, C, keep, lane);
               if (!ok) break;
               const u8* missed = nullptr;                  // candidates whose chunk did not cache their service
@@ -1030,14 +1035,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                   G.wide = !(C.cg[i] >> 7) && rr > 1;      // chunks of replicas lie anywhere
                   G.at.x = G.wide ? 0u : ((1u << units) - 1u) << G.off; G.at.z = (u32)(R.word0[j] + G.node);
                 }
-                start(pd, j, nr + i, a, units, fin, P.a_arrival ? P.a_arrival[row + a] : 0, G, EXT && R.trajectory && R.traj_last && R.traj_last[row + a]);
+                start(pd, j, nr + i, a, units, fin, P.a_arrival ? P.a_arrival[row + a] : 0, G, replay_last<EXT>(R, row, a) != 0u);
               }
               // the kept ones are the pool's first `keep` in queue order
               int seen = 0;
 #pragma unroll 1
               for (int i0 = 0; i0 < n && seen < keep; i0 += 32) {
                 int x = -1; u32 meta = RQ_NOBODY;
-                if (i0 + lane < n) meta = replay_facts(P, Q, wait, row, i0 + lane, x).y;
+                if (i0 + lane < n) meta = replay_facts(P, R, Q, wait, row, i0 + lane, x).y;
                 const bool mine = RQ_POOL(meta) == j;
                 const u32 mb = __ballot_sync(TG_FULL, mine);
                 if (mine && seen + __popc(mb & below) < keep && x >= 0) Q.c[x].y = meta | RQ_STARTED;
@@ -1128,7 +1133,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               if ((mv >> lane) & 1u) {                      // a record moves up into shared memory
                 int y = Q.at(to);
                 if (EXT) { const int z = Q.free[free_slots - 1 - __popc(mv & below)]; Q.q[y] = (unsigned short)z; y = z; Q.key[y] = kk; }
-                replay_store(Q, y, replay_load(P, row, a), a, EXT && R.traj_last && R.traj_last[row + a] ? 256u : 0u);
+                replay_store(Q, y, replay_load(P, row, a), a, replay_last<EXT>(R, row, a));
               }
               if (EXT) free_slots -= __popc(mv);
               __syncwarp();

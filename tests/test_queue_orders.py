@@ -294,3 +294,35 @@ def test_traces_with_trajectories_pinned_on_arrival_match_oracle(oracle, seed, p
     assert np.array_equal(o["node_mem_free"], dev["node_mem_free"].cpu().numpy())
     assert (o["alloc_units"] > 0).sum() > 500 and (o["pool"] != a["pool"]).sum() > 30
     rnd.destroy()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cores,policy", [(600, 0), (600, LJF), (1200, 0), (1200, SJF)])
+def test_memory_of_trajectories_that_start_from_a_long_queue_comes_back(oracle, cores, policy):
+    # 2 x cores one-core, one-action trajectories arrive and start in one round: more than a block keeps waiting records of
+    # (2048 at most) in shared memory, so the last ones start from global memory.  They take all of the nodes' memory;
+    # the arrivals behind them wait until it is given back.
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, cores, 60), Pool(POOL_CPU, cores, 60))
+    S, burst = 3, 2 * cores
+    N = burst + 300
+    rng = np.random.default_rng(cores + policy)
+    arrival = np.concatenate([np.zeros((S, burst), np.int64), np.sort(rng.integers(20_000, 2_000_000, (S, 300)), axis=1)], axis=1)
+    a = dict(pool=np.zeros((S, N), np.uint8), unit=np.ones((S, N), np.uint8), level_mask=np.ones((S, N), np.uint32), gpu_busy=None,
+             s_us=rng.integers(5_000, 900_000, (S, N)), p_us=np.zeros((S, N), np.int64), arrival_us=arrival,
+             n_actions=np.full(S, N, np.int32), trajectory=np.tile(np.arange(N, dtype=np.int32), (S, 1)),
+             traj_mem=np.full((S, N), 3, np.uint32), traj_last=np.ones((S, N), np.uint8),
+             traj_node=np.full((S, N), -1, np.int32), node_mem_free=np.full((S, 2), 3 * cores, np.int64))
+    o = oracle.replay_trace_pinned(pools, a, round_us=10_000, max_rounds=600, policy=policy)
+    rnd = binding.Round(S, N, pools, round_us=10_000, max_rounds=600)
+    dev = binding.to_device(a)
+    dev["traj_mem"] = dev["traj_mem"].view(torch.int32)
+    g = rnd.replay_trace_pinned(dev, policy=policy)
+    torch.cuda.synchronize()
+    assert np.array_equal(o["node_mem_free"], dev["node_mem_free"].cpu().numpy())
+    assert np.array_equal(o["traj_node"], dev["traj_node"].cpu().numpy())
+    for k in KEYS + ("rounds_used", "occupancy", "pool"):
+        assert np.array_equal(o[k], g[k].cpu().numpy()), k
+    assert np.all(o["node_mem_free"] == 3 * cores) and np.all(o["traj_node"] == -1) and np.all(o["n_selected"] == N)
+    rnd.destroy()
