@@ -244,6 +244,7 @@ struct PinIo {
 __device__ __forceinline__ int pin_chunk(bool mine, int t, u32 mem, int need, int pj, bool have, int* tn, i64& mf, int cores, int lane,
                                          int& pool_of) {
   int node = mine ? tn[t] : -1;
+  __syncwarp();                                         // (lane 0 writes tn below)
   int first_out = 32;
   u32 open = __ballot_sync(TG_FULL, mine && node < 0);
   while (open) {

@@ -791,6 +791,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
         int blocked_pool = -1;                             // pool of a head-of-line action that does not fit
         if (nw > 0) {
           const int capreg = lane < D ? Z.slot[lane] : 0;
+          __syncwarp();                                    // (before other lanes write the slots, in this round or the next worked one)
           // Candidate prefix (Algorithm 1, line 2): lane v adds up the demand on slot v, action by action
           int n = 0, run_dem = 0, stop_pool = -1, aside = 0;
           u32 present = 0;                                 // pools with candidates; << 8: with elastic ones
@@ -912,10 +913,11 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
                 ReplayGrant G; G.node = 0; G.off = -1; G.at = make_uint4(0u, 0u, 0u, (u32)R.Dtot); G.wide = false;
                 if (pd.type == TG_POOL_API) {
                   // Section 5.1: the offset is what was in use before
-                  const int incl = warp_incl_scan32(units, lane);
-                  G.off = pd.capacity - Z.slot[slot0] + incl - units;
+                  const int incl = warp_incl_scan32(units, lane), free_now = Z.slot[slot0];
+                  G.off = pd.capacity - free_now + incl - units;
                   const int all = __shfl_sync(TG_FULL, incl, 31);
-                  if (lane == 0) Z.slot[slot0] -= all;
+                  __syncwarp();                            // every lane has read the slot (a shuffle orders no memory)
+                  if (lane == 0) Z.slot[slot0] = free_now - all;
                 } else if (pd.type == TG_POOL_GPU) {       // largest chunks first, then queue position
                   const int g = (int)(c.w & 0x7fu), gang = (int)(c.w >> 7) & 1, lz = ilog2(gang ? g * rr : g), nreq = gang ? 1 : rr;
 #pragma unroll 1

@@ -142,3 +142,26 @@ def test_replay_state_layouts_match_oracle(oracle, name):
         o = oracle.replay_trace(pools, a, depth=2, round_us=round_us, max_rounds=max_rounds)
         assert_same(o, gpu_replay(pools, a, 2, round_us, max_rounds))
     assert o["n_selected"].sum() > 0
+
+
+@pytest.mark.parametrize("policy", [0, 1])
+def test_grants_of_calls_in_bursts_match_oracle(oracle, policy):
+    # a quota and a concurrency pool, up to 90 calls a burst: many of a round are granted at once, 32 at a time, and every
+    # offset is what was in use before; bursts of one and two elastic calls among them
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_API, 120, 0, 50_000), Pool(POOL_API, 90, 0, 0), Pool(POOL_CPU, 8, 4))
+    S, N = 8, 600
+    rng = np.random.default_rng(40 + policy)
+    burst = np.stack([np.repeat(np.arange(N), rng.choice([1, 2, 40, 90], N))[:N] for _ in range(S)])
+    a = dict(pool=rng.choice(3, (S, N), p=[0.5, 0.45, 0.05]).astype(np.uint8), unit=rng.integers(1, 4, (S, N)).astype(np.uint8),
+             level_mask=np.where((rng.random((S, N)) < 0.5) | (burst % 2 == 0), 1, 0b1011).astype(np.uint32),
+             s_us=rng.integers(0, 30_000, (S, N)), p_us=rng.integers(0, 60_000, (S, N)), arrival_us=burst * 7_000,
+             n_actions=np.full(S, N, np.int32), gpu_busy=None)
+    o = oracle.replay_trace(pools, a, round_us=10_000, max_rounds=3000, policy=policy)
+    rnd = binding.Round(S, N, pools, round_us=10_000, max_rounds=3000)
+    g = rnd.replay_trace(binding.to_device(a), policy=policy)
+    torch.cuda.synchronize()
+    assert_same(o, {k: v.cpu().numpy() for k, v in g.items()})
+    assert np.all(o["n_selected"] == N) and (o["place_off"][a["pool"] == 0] > 40).any()
+    rnd.destroy()
