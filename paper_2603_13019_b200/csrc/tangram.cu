@@ -469,6 +469,12 @@ static const void* round_kernel(bool cache, bool side, bool sorted) {
   return side ? (const void*)k_round<true, false, false> : sorted ? (const void*)k_round<false, true, false> : (const void*)k_round<false, false, false>;
 }
 
+// the replay's instance for a round: with the code of the extensions or not (see k_replay)
+static const void* replay_kernel(const ReplayWs& R, bool ext) {
+  if (R.rcap == 0 || R.state_bytes == 0) return (const void*)k_replay<true, false>;
+  return ext ? (const void*)k_replay<true, true> : (const void*)k_replay<false, true>;
+}
+
 extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_round** out) {
   if (!desc || !out || !desc->pools) return TANGRAM_EINVAL;
   if (desc->n_scenarios < 1 || desc->max_actions < 1 || desc->n_pools < 1 ||
@@ -661,6 +667,14 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
   const void* kern[3] = {cache ? (const void*)k_pool<true> : (const void*)k_pool<false>, round_kernel(cache, false, false),
                          cache || desc->side_costs > 0 ? round_kernel(cache, true, false) : round_kernel(false, false, true)};
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaFuncSetAttribute(kern[k], cudaFuncAttributeMaxDynamicSharedMemorySize, K2_DYN_SMEM);
+  if (desc->max_rounds > 0) {
+    // Here and not at the call, which may be captured; the same limit for every round, as it is the kernel's and not the
+    // round's: another thread's round must not lower it between a call's two steps.
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k)
+      e = cudaFuncSetAttribute(replay_kernel(r->R, k != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, TG_REPLAY_SMEM);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_occupancy);      // (loads it)
+  }
   if (e != cudaSuccess) { tangram_round_destroy(r); return cuda_fail(e, "cudaFuncSetAttribute"); }
   *out = r;
   return TANGRAM_OK;
@@ -981,10 +995,7 @@ static int replay_impl(tangram_round* r, const tangram_actions* a, tangram_resul
     R.max_traj = pin->max_trajectories; R.traj_node = pin->traj_node; R.mem_free = (i64*)pin->node_mem_free;
     R.pool_rw = pin->pool_out;
   }
-  // (the attribute is set here, so that a round that never replays does not load these kernels)
-  const bool ext = policy || pin || P.n_side > 0 || (P.cache_slots > 0 && P.n_nodes_total > 0);
-  void (*kern)(Params, ReplayWs) = R.rcap == 0 || R.state_bytes == 0 ? k_replay<true, false> : ext ? k_replay<true, true> : k_replay<false, true>;
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, r->replay_smem));
+  void (*kern)(Params, ReplayWs) = (void (*)(Params, ReplayWs))replay_kernel(R, policy || pin || P.n_side > 0 || has_cache(P));
   kern<<<blocks, KR_THREADS, r->replay_smem, st>>>(P, R);
   if (R.occupancy) { k_occupancy<<<P.S, 256, 0, st>>>(P.P, R.max_rounds, R.rounds_used, P.o_status, R.occupancy); r->launches += 1; }
   if (ev) CK(cudaEventRecord(ev[1], st));

@@ -165,3 +165,54 @@ def test_grants_of_calls_in_bursts_match_oracle(oracle, policy):
     assert_same(o, {k: v.cpu().numpy() for k, v in g.items()})
     assert np.all(o["n_selected"] == N) and (o["place_off"][a["pool"] == 0] > 40).any()
     rnd.destroy()
+
+
+def test_rounds_of_different_sizes_replay_from_two_threads(oracle):
+    # their replays take about 110 KB and 25 KB of shared memory per block of the same kernel; few actions, so that the host
+    # calls set the pace
+    import threading
+    import torch
+    from paper_2603_13019_b200 import binding
+    jobs = []
+    for N, pools in ((2000, (Pool(POOL_CPU, 24, 8),)), (32, (Pool(POOL_CPU, 6, 3),))):
+        w, a = random_round(N, 1, N, pools, small_durations=0.2, max_mult=4)
+        a["arrival_us"] = np.cumsum(np.random.default_rng(N).integers(0, 6000, a["pool"].shape), axis=1).astype(np.int64)
+        a["n_actions"][:] = 1
+        rnd = binding.Round(1, N, pools, round_us=10_000, max_rounds=4)
+        jobs.append((rnd, binding.to_device(a), rnd.new_result(replay=True), torch.cuda.Stream(),
+                     oracle.replay_trace(pools, a, depth=2, round_us=10_000, max_rounds=4)))
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(rnd, dev, out, stream, want):
+        call, args = rnd._lib.tangram_replay_trace, (rnd._h, rnd._actions(dev), rnd._result(out), rnd._stream(stream))
+        for k in range(300):
+            failed.extend(filter(None, [call(*args) for _ in range(64)]))    # (a loop that is mostly in the library)
+            stream.synchronize()
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed, (len(failed), failed[0])
+    for rnd, _, out, _, want in jobs:
+        assert_same(want, {k: v.cpu().numpy() for k, v in out.items()})
+        rnd.destroy()
+
+
+def test_first_replay_of_a_round_can_be_captured(oracle):
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = POOLSETS[0]
+    w, a = random_round(77, 3, 60, pools, small_durations=0.2, max_mult=4)
+    a["arrival_us"] = np.cumsum(np.random.default_rng(7).integers(0, 6000, a["pool"].shape), axis=1).astype(np.int64)
+    rnd, dev = binding.Round(3, 60, pools, round_us=10_000, max_rounds=300), binding.to_device(a)
+    out, graph = rnd.new_result(replay=True), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        rnd.replay_trace(dev, out)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert_same(oracle.replay_trace(pools, a, depth=2, round_us=10_000, max_rounds=300), {k: v.cpu().numpy() for k, v in out.items()})
+    rnd.destroy()
