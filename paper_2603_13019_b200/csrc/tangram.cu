@@ -174,8 +174,8 @@ __device__ __forceinline__ void place_and_write(const Params& P, int sc, int j, 
     int R[4];
     gpu_requests(keep, C.cg, C.rkeep, C.pnode, C.poff, R, lane);
     const u64 bytes = (u64)(R[0] + R[1] + R[2] + R[3]) * 4;
+    u8* nm = pd.n_nodes > 32 ? (u8*)slab.take_fast(pd.n_nodes) : nullptr;   // (before the list, which can be done without)
     u32* list = bytes <= WARP_WORK_BYTES ? (u32*)warp_smem() : (u32*)slab.take(bytes);   // (the selection is done with its work area)
-    u8* nm = pd.n_nodes > 32 ? (u8*)slab.take_fast(pd.n_nodes) : nullptr;
     __syncwarp();
     if (pd.n_nodes > 32 && !nm) { if (lane == 0) atomicOr(&P.o_status[sc], TG_ST_WORKSPACE); keep = 0; }
     else if (list && pd.n_nodes <= 32) place_gpu_lists<true>(pd, br, nullptr, list, R, keep, C.pnode, C.poff, lane);

@@ -220,3 +220,17 @@ def test_gpu_placement_at_the_edges_match_oracle(oracle, gpus, group, busy):
     o = oracle.schedule_batch(pools, a)
     assert_same(o, gpu_round(pools, a))
     assert o["n_selected"].sum() > gpus // 4
+
+
+@pytest.mark.parametrize("n", [2950, 3200])
+def test_requests_by_the_ten_thousands_are_placed(n):
+    # n actions of 32 replicas of one GPU each on free nodes of eight: every action gets the next four nodes.  2950: a list of
+    # all requests fits the scratch of one pool, but not beside the masks of its 11840 nodes; 3200: the list alone does not fit.
+    # Both are placed one request after the other.
+    pools = (Pool(POOL_GPU, 32 * n + 320, 8),)
+    a = dict(pool=np.zeros((2, n), np.uint8), unit=np.ones((2, n), np.uint8), level_mask=np.full((2, n), 1 << 31, np.uint32),
+             s_us=np.full((2, n), 1000, np.int64), p_us=np.full((2, n), 32_000, np.int64), arrival_us=None,
+             n_actions=np.full(2, n, np.int32), gpu_busy=None)
+    g = gpu_round(pools, a, depth=1)
+    assert np.all(g["status"] == 0) and np.all(g["n_selected"] == n) and np.all(g["alloc_units"] == 32)
+    assert np.array_equal(g["place_node"], np.tile(4 * np.arange(n), (2, 1))) and np.all(g["place_off"] == 0) and np.all(g["act_us"] == 2000)
