@@ -119,7 +119,7 @@ STATES = {
     "wide": ((Pool(POOL_CPU, 900, 300), Pool(POOL_GPU, 320, 8)), 10_000, 1.0),
     # one core per domain: every grant of more spans domains, more domains than lanes
     "spanning": ((Pool(POOL_CPU, 40, 1), Pool(POOL_GPU, 6, 2), Pool(POOL_CPU, 33, 11)), 10_000, 1.0),
-    # live state and running actions in global memory; a window shorter than a round, a concurrency limit
+    # live state in global memory; a window shorter than a round, a concurrency limit
     "global": ((Pool(POOL_CPU, 6000, 60), Pool(POOL_API, 3, 0, 4_000), Pool(POOL_API, 4, 0, 0), Pool(POOL_GPU, 16, 4)), 10_000, 1.0),
     # times beyond 32 bits: a step between two candidates that has to be decided exactly
     "long": ((Pool(POOL_CPU, 6, 3), Pool(POOL_GPU, 8, 8)), 4_000_000, 2e4),
@@ -215,4 +215,29 @@ def test_first_replay_of_a_round_can_be_captured(oracle):
     graph.replay()
     torch.cuda.synchronize()
     assert_same(oracle.replay_trace(pools, a, depth=2, round_us=10_000, max_rounds=300), {k: v.cpu().numpy() for k, v in out.items()})
+    rnd.destroy()
+
+
+@pytest.mark.parametrize("cores,group", [(2700, 60), (6000, 60)])
+@pytest.mark.parametrize("policy", [0, 2])
+def test_running_sets_in_global_memory_match_oracle(oracle, cores, group, policy):
+    # a block's shared memory has no room for the 4000 actions that may run here, nor for more than 1600 that wait (most of
+    # them do, behind GPUs that are taken); live state in shared and in global memory, with and without a sorted queue
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, cores, group), Pool(POOL_API, 1500, 0, 3_000_000), Pool(POOL_GPU, 32, 8))
+    S, N = 3, 4000
+    rng = np.random.default_rng(cores + policy)
+    elastic = rng.random((S, N)) < 0.02
+    pool = rng.choice(3, (S, N), p=[0.7, 0.28, 0.02]).astype(np.uint8)
+    a = dict(pool=pool, unit=np.where(pool == 0, rng.integers(1, 4, (S, N)), 1).astype(np.uint8),
+             level_mask=np.where(elastic, 0xB, 1).astype(np.uint32), s_us=rng.integers(200_000, 2_500_000, (S, N)).astype(np.int64),
+             p_us=np.where(elastic, rng.integers(0, 900_000, (S, N)), 0).astype(np.int64),
+             arrival_us=np.cumsum(rng.integers(0, 400, (S, N)), axis=1).astype(np.int64), n_actions=np.full(S, N, np.int32), gpu_busy=None)
+    o = oracle.replay_trace(pools, a, round_us=10_000, max_rounds=2500, policy=policy)
+    rnd = binding.Round(S, N, pools, round_us=10_000, max_rounds=2500)
+    g = rnd.replay_trace(binding.to_device(a), policy=policy)
+    torch.cuda.synchronize()
+    assert_same(o, {k: v.cpu().numpy() for k, v in g.items()})
+    assert np.all(o["n_selected"] == N)
     rnd.destroy()
