@@ -60,6 +60,8 @@ __host__ __device__ __forceinline__ size_t replay_state_bytes(const ReplayWs& R)
 #define KR_WAIT_BYTES 60          // per waiting record: three 16-byte pieces, key, queue, free list
 #define KR_RUN_BYTES 36
 #define KR_STATE_MAX 16384
+#define KR_MIN_WAIT 64
+#define KR_PER_SM 8               // blocks of 32 threads of 255 registers that an SM holds
 #define KR_SLOT_BYTES 128         // free capacity of the 32 demand slots at most
 // shared memory of a block (one warp) without the parts sized by the round
 #define KR_TABLE_BYTES 2048       // per free mask of a node: its free blocks by size, and where a chunk of every size goes

@@ -568,16 +568,25 @@ extern "C" int tangram_round_create(const tangram_round_desc* desc, tangram_roun
     bad |= cudaMalloc((void**)&R.wait, SN * sizeof(int)) != cudaSuccess;
     // what a block (one scenario at a time) keeps in shared memory: live state, running actions, waiting records
     {
-      const size_t state = replay_state_bytes(R);
-      R.state_bytes = state <= KR_STATE_MAX ? (int)state : 0;
       size_t running = 0;                                  // a running action holds a unit at least, quota calls aside
       for (int j = 0; j < P.P; ++j) running += P.pool[j].type == TG_POOL_API && P.pool[j].window_us > 0 ? (size_t)P.N : (size_t)P.pool[j].capacity;
       running = align_up(running < (size_t)P.N ? running : (size_t)P.N, 8);
+      // Resident blocks of an SM: all of its scenarios, or as many at a time as turns of KR_PER_SM take, so that the last turn is
+      // as full as the others.  With six at most, 1024 traces of 2000 actions on 256 cores and 8 GPUs took two turns, 9.9 ms,
+      // against 7.3 in one of seven (2048: 17.6 and 14.3; pinned to three nodes 17.2 and 12.3).
       size_t per_sm = ((size_t)P.S + r->n_sm - 1) / r->n_sm;
-      if (per_sm > 6) per_sm = 6;
+      const size_t turns = (per_sm + KR_PER_SM - 1) / KR_PER_SM;
+      per_sm = (per_sm + turns - 1) / turns;
       size_t room = (size_t)TG_SMEM_PER_SM / per_sm - 1024;
       if (room > TG_REPLAY_SMEM) room = TG_REPLAY_SMEM;
-      size_t left = room - KR_BASE_BYTES - (size_t)R.state_bytes;
+      size_t left = room - KR_BASE_BYTES;
+      // The live state goes to global memory where it leaves no room for KR_MIN_WAIT waiting records, each of which would be
+      // decoded from scattered columns whenever it is looked at: 1024 traces on 3712 cores, state of 16 KB beside none 28.3 ms,
+      // beside 128 26.0, in global memory 23.5 (seven blocks).  On 1024 cores 5 KB beside 96 records 5.5 ms, in global
+      // memory 5.7.
+      const size_t state = replay_state_bytes(R);
+      R.state_bytes = state <= KR_STATE_MAX && state + KR_MIN_WAIT * KR_WAIT_BYTES <= left ? (int)state : 0;
+      left -= (size_t)R.state_bytes;
       R.rcap = running * KR_RUN_BYTES <= left / 2 ? (int)running : 0;
       left -= (size_t)R.rcap * KR_RUN_BYTES;
       size_t wc = left / KR_WAIT_BYTES;

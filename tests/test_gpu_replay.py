@@ -241,3 +241,25 @@ def test_running_sets_in_global_memory_match_oracle(oracle, cores, group, policy
     assert_same(o, {k: v.cpu().numpy() for k, v in g.items()})
     assert np.all(o["n_selected"] == N)
     rnd.destroy()
+
+
+@pytest.mark.parametrize("cores", [60, 300, 1500])
+@pytest.mark.parametrize("policy", [0, 1])
+def test_replays_of_many_scenarios_match_oracle(oracle, cores, policy):
+    # 1160 scenarios, eight blocks on an SM: running actions and live state in shared memory, the state only, neither; up to
+    # 300 actions wait, more than such a block keeps in shared memory (160 at most)
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, cores, 60), Pool(POOL_GPU, 8, 4))
+    S, N, copies = 4, 300, 290
+    w, a = random_round(cores + policy, S, N, pools, small_durations=0.1, max_mult=6)
+    a["level_mask"] |= 1
+    a["arrival_us"] = np.cumsum(np.random.default_rng(cores).integers(0, 200, (S, N)), axis=1).astype(np.int64)
+    o = oracle.replay_trace(pools, a, round_us=10_000, max_rounds=1000, policy=policy)
+    rnd = binding.Round(S * copies, N, pools, round_us=10_000, max_rounds=1000)
+    many = {k: None if v is None else np.tile(v, (copies,) + (1,) * (v.ndim - 1)) for k, v in a.items()}
+    g = rnd.replay_trace(binding.to_device(many), policy=policy)
+    torch.cuda.synchronize()
+    assert_same({k: np.tile(o[k], (copies,) + (1,) * (o[k].ndim - 1)) for k in KEYS}, {k: v.cpu().numpy() for k, v in g.items()})
+    assert o["n_selected"].sum() > 0 and np.all(o["status"] == 0)
+    rnd.destroy()
