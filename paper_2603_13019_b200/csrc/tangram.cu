@@ -99,6 +99,8 @@ __device__ bool gather_candidates(const Params& P, int sc, int j, const PoolMeta
 #define WARP_TASK_BYTES 384
 #define WARP_SMEM_BYTES (WARP_WORK_BYTES + WARP_FAST_BYTES + WARP_TASK_BYTES)
 static_assert(sizeof(PoolTask) <= WARP_TASK_BYTES, "");
+// the choices of a small table in the work area (solve_prefix): behind the staged levels and all that ev_run_regs<8> uses
+static_assert((64 * 8 + 2 * EV_BLOCK + 4) * 4 <= 32 * CELL_LEVELS * 16 && 32 * CELL_LEVELS * 16 + CELL_SHARED_ROWS * 64 <= WARP_WORK_BYTES, "");
 #define K2_DYN_SMEM ((K2_THREADS / 32) * WARP_SMEM_BYTES + 16)
 __device__ __forceinline__ char* warp_smem() {
   extern __shared__ __align__(16) unsigned char k2_smem[];

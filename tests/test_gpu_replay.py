@@ -263,3 +263,19 @@ def test_replays_of_many_scenarios_match_oracle(oracle, cores, policy):
     assert_same({k: np.tile(o[k], (copies,) + (1,) * (o[k].ndim - 1)) for k in KEYS}, {k: v.cpu().numpy() for k, v in g.items()})
     assert o["n_selected"].sum() > 0 and np.all(o["status"] == 0)
     rnd.destroy()
+
+
+def test_running_and_candidates_around_256_match_oracle(oracle):
+    # up to 270 one-core actions run; a few elastic ones are decided beside them all the time, with few cores to spare
+    pools = (Pool(POOL_CPU, 270, 270),)
+    S, N = 4, 1500
+    rng = np.random.default_rng(256)
+    elastic = rng.random((S, N)) < 0.4
+    a = dict(pool=np.zeros((S, N), np.uint8), unit=np.ones((S, N), np.uint8), level_mask=np.where(elastic, 0xB, 1).astype(np.uint32),
+             s_us=np.where(elastic, rng.integers(0, 20_000, (S, N)), rng.integers(0, 2_500_000, (S, N))),
+             p_us=np.where(elastic, rng.integers(0, 400_000, (S, N)), 0), arrival_us=np.cumsum(rng.integers(0, 4_500, (S, N)), axis=1),
+             n_actions=np.full(S, N, np.int32), gpu_busy=None)
+    o = oracle.replay_trace(pools, a, depth=2, round_us=10_000, max_rounds=3000)
+    assert_same(o, gpu_replay(pools, a, 2, 10_000, 3000))
+    busy = o["occupancy"][:, :, 0]
+    assert np.all(o["n_selected"] == N) and (busy > 258).sum() > 100 and ((busy > 200) & (busy < 254)).sum() > 100

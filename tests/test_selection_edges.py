@@ -234,3 +234,20 @@ def test_requests_by_the_ten_thousands_are_placed(n):
     g = gpu_round(pools, a, depth=1)
     assert np.all(g["status"] == 0) and np.all(g["n_selected"] == n) and np.all(g["alloc_units"] == 32)
     assert np.array_equal(g["place_node"], np.tile(4 * np.arange(n), (2, 1))) and np.all(g["place_off"] == 0) and np.all(g["act_us"] == 2000)
+
+
+@pytest.mark.parametrize("m", [255, 256, 257])
+def test_shared_table_beside_the_largest_register_heaps_matches_oracle(oracle, m):
+    # 60 elastic candidates among m, ten spare units: their choices share the work area with heaps of up to 256 times (with
+    # more, both go elsewhere); some of the last ones pay to be evicted
+    pools = (Pool(POOL_CPU, m + 10, m + 10), Pool(POOL_API, 1, 0, 0))
+    a = _round(500 + m, pools, m, [1], 1, 150)
+    rows = np.random.Generator(np.random.PCG64(m)).permutation(m)[:60]
+    a["level_mask"][:, rows] = 0b1011
+    a["level_mask"][:, m - 6:m] = 0b1011
+    a["p_us"][1, m - 8:m] = 4_000_000
+    a["s_us"][2] = 0
+    a["p_us"][3, rows] = 60_000
+    o = oracle.schedule_batch(pools, a)
+    assert_same(o, gpu_round(pools, a))
+    assert (o["n_selected"] < m + 1).sum() >= 2          # (one token beside the m)
