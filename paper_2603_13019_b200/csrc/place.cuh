@@ -112,6 +112,18 @@ __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u
   }
 }
 
+// The nodes of a pool as a round keeps them (a byte of busy GPUs each), and as a replay does (a word of free ones).
+struct BusyNodes {
+  u8* m;
+  __device__ __forceinline__ u32 busy(int v) const { return m[v]; }
+  __device__ __forceinline__ void take(int v, u32 gpus) const { m[v] |= (u8)gpus; }
+};
+struct FreeNodes {
+  u32* w;
+  __device__ __forceinline__ u32 busy(int v) const { return ~w[v] & 0xffu; }
+  __device__ __forceinline__ void take(int v, u32 gpus) const { w[v] &= ~gpus; }
+};
+
 // GPU placement with a service cache (Section 5.3, evict on execution).  The rule of place_gpu, and among
 // the free blocks of the level it picks, one whose granted chunk (the block's low end) caches the
 // request's instance goes first, then the lowest (node, start).  An instance is (service, chunk size);
@@ -125,7 +137,8 @@ __device__ void place_cpu_fresh(const PoolDev& pd, int* dfree, int keep, const u
 // entries a lane each.  Bound by that chain; the entries work in shared memory (mem) where they fit, 38 nodes of two per
 // GPU in the selection's work area.  A lane that walked a node's chunks entry by entry in global memory took 3600 cycles a
 // request: 4096 x 1024 with two entries per GPU 400 us a call against 357.
-__device__ __forceinline__ void place_gpu_cache(const PoolDev& pd, u8* nm, int keep, const u8* cg, const u8* r, const int* ids,
+template <class Nodes>
+__device__ __forceinline__ void place_gpu_cache(const PoolDev& pd, const Nodes nodes, int keep, const u8* cg, const u8* r, const int* ids,
                                                 int* pnode, int* poff, u8* miss, int* scratch, const unsigned short* svc, u32* tag_row, i64* use_row,
                                                 int K, i64 now, int lane, char* mem, int mem_bytes, int* owner = nullptr) {
   const int entries = pd.n_nodes * 8 * K;
@@ -173,7 +186,7 @@ __device__ __forceinline__ void place_gpu_cache(const PoolDev& pd, u8* nm, int k
                 if ((lane >> 2) == q) hold = (w >> (8 * (lane & 3))) & 0xffu;
               }
             const int v = v0 + lane;
-            const NodeBlocks nb = node_blocks(v < n_nodes ? nm[v] | pad : 0xffu);
+            const NodeBlocks nb = node_blocks(v < n_nodes ? nodes.busy(v) | pad : 0xffu);
             // the node's smallest sufficient level, the blocks of that level, and the ones whose low end caches the tag
             const u32 s = lz <= 0 && nb.s1 ? nb.s1 : (lz <= 1 && nb.s2 ? nb.s2 : (lz <= 2 && nb.s4 ? nb.s4 : nb.s8));
             const u32 lev = lz <= 0 && nb.s1 ? 0u : (lz <= 1 && nb.s2 ? 1u : (lz <= 2 && nb.s4 ? 2u : 3u));
@@ -190,7 +203,7 @@ __device__ __forceinline__ void place_gpu_cache(const PoolDev& pd, u8* nm, int k
           const bool hit = ((best >> 29) & 1u) == 0u;
           __syncwarp();
           if (lane == 0) {
-            nm[node] |= (u8)(((1u << z) - 1u) << start);
+            nodes.take(node, ((1u << z) - 1u) << start);
             if (rep == 0) { pnode[i] = node; poff[i] = start; }
             if (tag && !hit) miss[i] = 1;
           }

@@ -979,17 +979,10 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               if (!ok) break;
               const u8* missed = nullptr;                  // candidates whose chunk did not cache their service
               if (cached) {
-                u8* nm = (u8*)slab.take_fast(pd.n_nodes);  // as busy masks
-                if (!nm) { ok = false; break; }
-#pragma unroll 1
-                for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = (u8)~Z.words[R.word0[j] + v];
-                __syncwarp();
                 const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
-                place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
+                place_gpu_cache(pd, FreeNodes{Z.words + R.word0[j]}, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
                                 P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, now, lane,
                                 warp_smem(), WARP_WORK_BYTES, ow);
-#pragma unroll 1
-                for (int v = lane; v < pd.n_nodes; v += 32) Z.words[R.word0[j] + v] = ~(u32)nm[v] & ((1u << pd.group) - 1u);
                 missed = C.rsel;
               } else if (pd.type == TG_POOL_GPU) {
                 // Section 5.3: by size, largest first, then queue position

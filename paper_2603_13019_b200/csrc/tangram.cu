@@ -166,7 +166,7 @@ __device__ __forceinline__ void place_and_write(const Params& P, int sc, int j, 
       for (int v = lane; v < pd.n_nodes; v += 32) nm[v] = busy_row ? busy_row[pd.node0 + v] : 0;
       __syncwarp();
       const size_t cbase = ((size_t)sc * P.n_nodes_total + pd.node0) * 8 * P.cache_slots;
-      place_gpu_cache(pd, nm, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
+      place_gpu_cache(pd, BusyNodes{nm}, keep, C.cg, C.rkeep, C.cidx, C.pnode, C.poff, C.rsel, C.rowcand,
                       P.a_service ? P.a_service + row : nullptr, P.cache_tag + cbase, P.cache_use + cbase, P.cache_slots, P.now, lane,
                       warp_smem(), WARP_WORK_BYTES);   // (the selection is done with its work area)
       missed = C.rsel;

@@ -204,3 +204,28 @@ def test_cfg1_with_a_service_cache_matches_oracle(oracle):
     rnd.destroy()
     for k in CACHE_KEYS:
         assert np.array_equal(o[k], g[k]), k
+
+
+@pytest.mark.gpu
+def test_replay_with_a_cache_on_more_nodes_than_the_scratch_holds_matches_oracle(oracle):
+    # 340000 nodes of one GPU: a byte for each is more than a warp's scratch (331776 bytes beside the candidates' arrays)
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_GPU, 340_000, 1),)
+    a = _arrays([(1, 1, 300, 0, 5, 2000), (1, 0b11, 300, 400, 5, 2000), (1, 1, 300, 0, 6, 2000), (1, 1, 900, 0, 5, 2000)], 1, 1,
+                arrival=[0, 0, 0, 4000])
+    a["gpu_busy"] = None
+    a["cache_tag"] = np.zeros((1, 340_000 * 8), np.uint32)
+    a["cache_use"] = np.zeros((1, 340_000 * 8), np.int64)
+    a["cache_tag"][0, 339_999 * 8] = tag(6, 1)
+    o = oracle.replay_trace(pools, a, round_us=1000, max_rounds=12, cache_slots=1)
+    rnd = binding.Round(1, 4, pools, round_us=1000, max_rounds=12, cache_slots=1)
+    dev = binding.to_device(a)
+    g = rnd.replay_trace(dev)
+    torch.cuda.synchronize()
+    for k in CACHE_KEYS[:7] + ("rounds_used", "occupancy"):
+        assert np.array_equal(o[k], g[k].cpu().numpy()), k
+    assert np.array_equal(o["cache_tag"], dev["cache_tag"].cpu().numpy().view(np.uint32))
+    assert np.array_equal(o["cache_use"], dev["cache_use"].cpu().numpy())
+    assert list(o["n_selected"]) == [4] and o["place_node"][0, 2] == 339_999
+    rnd.destroy()
