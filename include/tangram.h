@@ -223,7 +223,7 @@ int64_t tangram_kernel_launches(const tangram_round* round);
  *
  * tangram_schedule_batch_ordered runs one round (as tangram_schedule_batch) on every queue sorted that way;
  * results are written at the actions' own positions.  policy 0 is tangram_schedule_batch itself.  Its first
- * call allocates 54 B per action of device memory that the round keeps (cudaMalloc; TANGRAM_ENOMEM).
+ * call allocates 4 B per action of device memory that the round keeps (cudaMalloc; TANGRAM_ENOMEM).
  * Device buffers only; max_actions <= 16384 (TANGRAM_ETOOBIG beyond); not with cache_slots / side_costs
  * (TANGRAM_EINVAL).  Asynchronous on the stream. */
 #define TANGRAM_ORDER_FCFS 0

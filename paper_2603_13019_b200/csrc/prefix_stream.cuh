@@ -16,7 +16,7 @@
 // order, to the pool's list in `tmin`.
 //
 // The output rows behind the candidate prefix get "not scheduled" from the selection kernel, which leaves the memory
-// idle (fill_part); of an ordered round k_fill writes all rows beside the sort, on a stream of its own.
+// idle (fill_rows); of an ordered round k_fill writes all rows beside the sort, on a stream of its own.
 //
 // Partitioned arrays (order, tmin and the solver's arrays) give every (scenario, pool) its own
 // row of max_actions entries, so a position never depends on another pool's count and the

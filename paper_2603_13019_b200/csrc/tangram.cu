@@ -331,8 +331,9 @@ __global__ void __launch_bounds__(K2_THREADS, 2) k_pool(const __grid_constant__ 
 // The whole round of a small batch in one launch, one block per scenario: the first warp walks the head of the queue
 // while the others write "not scheduled" everywhere, all of them stream the rest of the queue, then every pool
 // gets a warp (wpb < n_pools of them where memory is short: the static entry).  A block's scratch is its own, so nothing depends on the number of scenarios.  What bounds a small
-// batch is latency, and one launch instead of four (and a memset) saves the gaps.  The last block to finish resets
-// the bump pointer of the arena for the next call.  1 x 64: 38.6 -> 26.8 us a call, 16 x 500 (static): 110 -> 84 us.
+// batch is latency, and one launch instead of three and a memset saves the gaps: 1 x 64 38.6 -> 26.8 us a call, 16 x 500
+// (static) 110 -> 84 us when it took the place of four.  The last block to finish resets the bump pointer of the arena for
+// the next call.
 #define TG_DONE_COUNTER 4           // word of arena_top that counts finished blocks
 template <bool SIDE, bool SORTED, bool CACHE>
 __global__ void __launch_bounds__(K2_THREADS, 2) k_round(const __grid_constant__ Params P, int wpb) {
