@@ -365,6 +365,61 @@ __device__ __forceinline__ bool replay_select(const Params& P, const ReplayWs& R
   return keep >= 0;
 }
 
+// the waiting records of a block, from `at` in its shared memory on
+template <bool LIST>
+__device__ __forceinline__ ReplayQueue<LIST> replay_queue(const ReplayWs& R, char* at) {
+  ReplayQueue<LIST> Q;
+  Q.cap = R.wcap; Q.head = 0;
+  Q.sp = (uint4*)at; Q.ta = Q.sp + Q.cap; Q.c = Q.ta + Q.cap; Q.key = (u64*)(Q.c + Q.cap);
+  Q.q = (unsigned short*)(Q.key + Q.cap); Q.free = Q.q + Q.cap;
+  return Q;
+}
+// `started` of the first n actions leave a queue that goes on in global memory (n <= Q.cap < nw): the ones of the prefix that
+// stay move up behind the others, and records from global memory take the places that the head then leaves behind.  Only
+// those are read; moving every record and every number behind them took 15000 to 260000 cycles a round, a quarter to 38 % of
+// a replay whose queue stays long (3000 actions on domains of 256 cores 32.7 -> 22.9 ms, 20000 on 256 cores 943 -> 553).
+// Out of line, and with few arguments, since the common path (the whole queue in shared memory) is slower with this text in
+// it: 256 x 20000 40.1 ms without, 40.3 out of line, 41.4 in line.
+template <bool LIST>
+__device__ __noinline__ void replay_leave(const Params& P, const ReplayWs& R, int head, int off, int sc, int n, int nw, int started, int free_slots) {
+  extern __shared__ __align__(16) unsigned char k2_smem[];
+  const int lane = threadIdx.x;
+  const u32 below = (1u << lane) - 1u;
+  const size_t row = (size_t)sc * P.N;
+  const int* wait = R.wait + row + off; const u64* wkey = R.wkey + row + off;
+  ReplayQueue<LIST> Q = replay_queue<LIST>(R, (char*)k2_smem + WARP_SMEM_BYTES + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES);
+  Q.head = head;
+  int to_end = n;
+#pragma unroll 1
+  for (int i0 = (n - 1) & ~31; i0 >= 0; i0 -= 32) {
+    const int i = i0 + lane, x = i < n ? Q.slot(i) : 0;
+    const bool gone = i < n && (Q.c[x].y & RQ_STARTED), stay = i < n && !gone;
+    const u32 gb = __ballot_sync(TG_FULL, gone), sb = __ballot_sync(TG_FULL, stay);
+    const int to = Q.at(stay ? to_end - __popc(sb >> lane) : 0);
+    uint4 sp, ta, c;
+    if (!LIST && stay) { sp = Q.sp[x]; ta = Q.ta[x]; c = Q.c[x]; }
+    if (LIST && gone) Q.free[free_slots + __popc(gb & below)] = (unsigned short)x;
+    free_slots += __popc(gb); to_end -= __popc(sb);
+    __syncwarp();
+    if (stay) { if (LIST) Q.q[to] = (unsigned short)x; else { Q.sp[to] = sp; Q.ta[to] = ta; Q.c[to] = c; } }
+    __syncwarp();
+  }
+  Q.head = Q.at(started < Q.cap ? started : 0);
+  const int first = Q.cap - started, end = min(Q.cap, nw - started);
+#pragma unroll 1
+  for (int p = first + lane; p < end; p += 32) {
+    const int a = wait[p + started];
+    int y = Q.at(p);
+    if (LIST) {
+      const int z = Q.free[free_slots - 1 - (p - first)];
+      Q.q[y] = (unsigned short)z; y = z;
+      if (R.policy) Q.key[y] = wkey[p + started];
+    }
+    replay_store(Q, y, replay_load(P, row, a), a, replay_last<LIST>(R, row, a));
+  }
+  __syncwarp();
+}
+
 // Two candidates (queue positions ba < bb < 32, in shared memory) on a pool with at most KR_PAIR_RUN actions running in all and
 // at most KR_PAIR_WAIT waiting behind the prefix: DPArrange's answer for both (lanes try b's levels, one after
 // the other a's), a's alone, and the eviction step between them, without any of the selection's arrays.  Returns how many
@@ -453,13 +508,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
   ReplayState Z;
   Z.slot = (int*)(fast + KR_FAST_BYTES);
   Z.node_of = (uint2*)(fast + KR_FAST_BYTES + KR_SLOT_BYTES);
-  ReplayQueue<EXT> Q;
-  Q.cap = R.wcap;
-  {
-    char* at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES;
-    Q.sp = (uint4*)at; Q.ta = Q.sp + Q.cap; Q.c = Q.ta + Q.cap; Q.key = (u64*)(Q.c + Q.cap);
-    Q.q = (unsigned short*)(Q.key + Q.cap); Q.free = Q.q + Q.cap;
-  }
+  ReplayQueue<EXT> Q = replay_queue<EXT>(R, fast + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES);
   char* const run_at = fast + KR_FAST_BYTES + KR_SLOT_BYTES + KR_TABLE_BYTES + align16((size_t)Q.cap * KR_WAIT_BYTES);
   char* const state_at = run_at + align16((size_t)R.rcap * KR_RUN_BYTES);
 #pragma unroll 1
@@ -1104,7 +1153,16 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
             Q.head = Q.at(started < Q.cap ? started : 0);
             nw -= started;
             __syncwarp();
-          } else if (started) {                             // a queue that goes on in global memory
+          } else if (started && n <= Q.cap) {               // a queue that goes on in global memory
+            // `wait` and `wkey` point to where queue position 0 would be, so that nothing moves there (what started since that
+            // part was last empty and what waits are different actions: it never outgrows its row)
+            replay_leave<EXT>(P, R, Q.head, (int)(wait - (R.wait + row)), sc, n, nw, started, free_slots);
+            Q.head = Q.at(started < Q.cap ? started : 0);
+            nw -= started;
+            if (EXT) free_slots += Q.cap - min(Q.cap, nw);
+            if (nw > Q.cap) { wait += started; if (EXT && R.policy) wkey += started; }
+            else { wait = R.wait + row; if (EXT && R.policy) wkey = R.wkey + row; }
+          } else if (started) {                             // ... as the prefix does: all of it moves up
             int kw = 0;
 #pragma unroll 1
             for (int i0 = 0; i0 < nw; i0 += 32) {
@@ -1137,6 +1195,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) k_replay(const __grid_constant_
               kw += __popc(b);
             }
             nw = kw;
+            if (nw <= Q.cap) { wait = R.wait + row; if (EXT && R.policy) wkey = R.wkey + row; }
           }
         }
         // 5. the next round in which something can start

@@ -279,3 +279,30 @@ def test_running_and_candidates_around_256_match_oracle(oracle):
     assert_same(o, gpu_replay(pools, a, 2, 10_000, 3000))
     busy = o["occupancy"][:, :, 0]
     assert np.all(o["n_selected"] == N) and (busy > 258).sum() > 100 and ((busy > 200) & (busy < 254)).sum() > 100
+
+
+@pytest.mark.parametrize("policy", [0, 1, 2])
+@pytest.mark.parametrize("scenarios", [2, 1160])
+def test_queues_that_stay_long_match_oracle(oracle, policy, scenarios):
+    # actions arrive in bursts, faster than they run, more than a block keeps in shared memory: the part of the queue in global memory moves on, is drained and
+    # fills again; evictions leave gaps in the prefix; a call for most of a concurrency pool holds long prefixes up
+    import torch
+    from paper_2603_13019_b200 import binding
+    pools = (Pool(POOL_CPU, 48, 16), Pool(POOL_API, 40, 0, 0), Pool(POOL_GPU, 8, 8))
+    S, N = 2, 2600
+    w, a = random_round(60 + policy, S, N, pools, ragged=False, max_mult=4, small_durations=0.5, inelastic=0.5)
+    a["level_mask"] |= 1
+    a["unit"] = np.where((a["pool"] == 1) & (np.random.default_rng(1).random((S, N)) < 0.01), 38, a["unit"]).astype(np.uint8)
+    gap = np.where(np.arange(N) % 1300 < 1200, 40, 90_000)
+    a["arrival_us"] = np.cumsum(np.random.default_rng(2).integers(0, gap, (S, N)), axis=1).astype(np.int64)
+    o = oracle.replay_trace(pools, a, round_us=10_000, max_rounds=9000, policy=policy)
+    copies = scenarios // S
+    rnd = binding.Round(scenarios, N, pools, round_us=10_000, max_rounds=9000)
+    many = {k: None if v is None else np.tile(v, (copies,) + (1,) * (v.ndim - 1)) for k, v in a.items()}
+    out = rnd.replay_trace(binding.to_device(many), policy=policy)
+    torch.cuda.synchronize()
+    for k in KEYS:
+        g = out[k].cpu().numpy()
+        assert np.array_equal(o[k], g[:S]) and np.array_equal(g, np.tile(g[:S], (copies,) + (1,) * (g.ndim - 1))), k
+    assert np.all(o["status"] == 0) and np.all(o["n_selected"] > 2500)
+    rnd.destroy()
